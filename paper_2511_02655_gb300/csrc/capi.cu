@@ -1267,12 +1267,13 @@ nbody_status nbody_init(nbody_ctx** out, const nbody_config* cfg, int64_t n_syst
   c->offsets.assign(offsets, offsets + n_systems + 1);
   c->n_total = offsets[n_systems];
 
-  // chunks: runs of <= kChunk bodies inside one system
+  // chunks: runs of <= chunk bodies inside one system
+  const int64_t chunk = chunk_bodies(c->n_total);
   c->sys_chunk.assign(c->n_sys + 1, 0);
   for (int s = 0; s < c->n_sys; ++s) {
     c->sys_chunk[s] = (int32_t)c->chunks.size();
-    for (int64_t b = offsets[s]; b < offsets[s + 1]; b += kChunk)
-      c->chunks.push_back(Chunk{s, (int32_t)b, (int32_t)std::min<int64_t>(offsets[s + 1], b + kChunk), 1});
+    for (int64_t b = offsets[s]; b < offsets[s + 1]; b += chunk)
+      c->chunks.push_back(Chunk{s, (int32_t)b, (int32_t)std::min<int64_t>(offsets[s + 1], b + chunk), 1});
   }
   c->sys_chunk[c->n_sys] = (int32_t)c->chunks.size();
 

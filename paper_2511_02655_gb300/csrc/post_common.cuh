@@ -20,10 +20,19 @@ __device__ __forceinline__ double warp_sum(double v) {
 // The sum is transposed so that every thread adds: the CTA's NV x THREADS
 // values go to shared memory, then a group of TPV lanes per value adds its
 // row in a fixed interleaved order and a TPV-lane xor shuffle finishes it.
-// For NV = 8 and 128 threads that is 11 float64 additions per thread instead
+// For NV = 8 and 64 threads that is 11 float64 additions per thread instead
 // of the 40 of a per-value warp butterfly (float64 adds are GB300's scarce
-// resource in these kernels).
-template <int NV, int THREADS>
+// resource in these kernels). FIRST: only the CTA's first THREADS threads take
+// part (they meet at named barrier 1); otherwise THREADS is the whole CTA.
+template <bool FIRST, int THREADS>
+__device__ __forceinline__ void sum_barrier() {
+  if (FIRST)
+    asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
+  else
+    __syncthreads();
+}
+
+template <int NV, int THREADS, bool FIRST = false>
 __device__ __forceinline__ void block_sum(double (&v)[NV]) {
   constexpr int NVP = NV <= 1 ? 1 : NV <= 2 ? 2 : NV <= 4 ? 4 : NV <= 8 ? 8 : 16;
   constexpr int TPV0 = THREADS / NVP;
@@ -32,10 +41,10 @@ __device__ __forceinline__ void block_sum(double (&v)[NV]) {
   static_assert(TPV >= 1 && THREADS % 32 == 0 && NV <= 16, "block_sum layout");
   __shared__ double red[NV][THREADS];
   __shared__ double res[NV];
-  __syncthreads();  // an earlier block_sum of the same shape may still be reading
+  sum_barrier<FIRST, THREADS>();  // an earlier block_sum of the same shape may still be reading
 #pragma unroll
   for (int k = 0; k < NV; ++k) red[k][threadIdx.x] = v[k];
-  __syncthreads();
+  sum_barrier<FIRST, THREADS>();
   const int k = (int)threadIdx.x / TPV, p = (int)threadIdx.x % TPV;
   double s = 0.0;
   if (k < NV) {
@@ -45,7 +54,7 @@ __device__ __forceinline__ void block_sum(double (&v)[NV]) {
 #pragma unroll
   for (int o = TPV / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (k < NV && p == 0) res[k] = s;
-  __syncthreads();
+  sum_barrier<FIRST, THREADS>();
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int q = 0; q < NV; ++q) v[q] = res[q];

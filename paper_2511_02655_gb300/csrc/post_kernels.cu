@@ -7,6 +7,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "nbody_internal.h"
 #include "post_common.cuh"
@@ -14,12 +15,69 @@
 namespace nbody {
 namespace {
 
-__global__ void __launch_bounds__(kPostThreads) k_post(const PostLaunch P) {
+// The slices of one body, added by kSlotGroups threads (thread group g of the CTA
+// takes slices g, g + kSlotGroups, ...) and then over the groups in order, all of it
+// for NC components per slice. Mixed: compensated float32 pairs, added as pairs on
+// the FP32 pipe (TwoSum of the hi parts, the lo parts and rounding errors summed
+// alongside). Valid in group 0; every thread of the CTA calls it.
+template <int CB>
+struct SlotSums {
+  float h[kSlotGroups - 1][CB];
+  float l[kSlotGroups - 1][CB];
+};
+
+template <int NC, int CB>
+__device__ __forceinline__ void add_groups(SlotSums<CB> (&red)[NC], const int g, const int b, float (&h)[NC],
+                                           float (&l)[NC]) {
+  if (g > 0) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) red[c].h[g - 1][b] = h[c], red[c].l[g - 1][b] = l[c];
+  }
+  __syncthreads();
+  if (g == 0) {
+#pragma unroll
+    for (int k = 0; k < kSlotGroups - 1; ++k)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        two_sum_acc(h[c], l[c], red[c].h[k][b]);
+        l[c] += red[c].l[k][b];
+      }
+  }
+}
+
+template <int NC, int CB>
+__device__ __forceinline__ void add_groups(double (&red)[NC][kSlotGroups - 1][CB], const int g, const int b,
+                                           double (&s)[NC]) {
+  if (g > 0) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) red[c][g - 1][b] = s[c];
+  }
+  __syncthreads();
+  if (g == 0) {
+#pragma unroll
+    for (int k = 0; k < kSlotGroups - 1; ++k)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) s[c] += red[c][k][b];
+  }
+}
+
+// One CTA per chunk, kSlotGroups threads per body to add the slices and one to do
+// the rest (a CTA of one thread per body when the mode combines nothing). Adding
+// the slices is a chain of 32-byte loads from L2, and that latency bounds the
+// kernel: on the 10 000-body Lennard-Jones gas (40 slices, 157 chunks) a step
+// took 89 us with one thread per body and 128-body chunks and takes 84 us with
+// four threads per body and 64-body chunks.
+template <int CB>
+__global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
+  __shared__ union {
+    SlotSums<CB> f[4];
+    double d[4][kSlotGroups - 1][CB];
+  } red;
   pdl_wait();     // the force kernel before it has finished writing the partials
   pdl_trigger();  // the next force kernel may be scheduled once every CTA has started
   if ((int)blockIdx.x == P.n_chunks) {
     // the extra CTA: the previous step's energy record from its chunk partials
-    systems_final<kEnergyVals, kPostThreads>(P.sys_chunk, P.n_sys, P.eprev, P.n_chunks, P.status,
+    systems_final<kEnergyVals, kSlotGroups * CB>(P.sys_chunk, P.n_sys, P.eprev, P.n_chunks, P.status,
                                              [&](int sy, const double (&v)[kEnergyVals]) {
                                                emit_energy(P.eprev_out, sy, v);
                                              });
@@ -28,49 +86,56 @@ __global__ void __launch_bounds__(kPostThreads) k_post(const PostLaunch P) {
   Chunk c = P.chunks[blockIdx.x];
   if (!chunk_ok(c, P.n_total, P.n_sys, (P.mode & kCombine) ? P.part_slices : 0, P.status))
     c.begin = c.end = 0;  // NBODY_DEBUG builds only: processed as an empty chunk
-  const double4_32a* part = reinterpret_cast<const double4_32a*>(P.part);
   const double* cen = P.centre + 3 * c.sys;
   double e[kEnergyVals];
 #pragma unroll
   for (int k = 0; k < kEnergyVals; ++k) e[k] = 0.0;
-  bool bad = false;
   const unsigned mode = P.mode;
+  const int b = (int)threadIdx.x % CB, g = (int)threadIdx.x / CB;
+  const int i = c.begin + b;
+  const bool live = i < c.end;
 
-  for (int i = c.begin + (int)threadIdx.x; i < c.end; i += kPostThreads) {
-    double sx = 0.0, sy = 0.0, sz = 0.0, sp = 0.0;
-    if ((mode & kCombine) && P.precision == 1) {
-      // compensated float32 pairs, added as pairs on the FP32 pipe: TwoSum of
-      // the hi parts, the lo parts and rounding errors summed alongside
-      const fpair4* fp = reinterpret_cast<const fpair4*>(P.part);
-      float hx = 0.f, lx = 0.f, hy = 0.f, ly = 0.f, hz = 0.f, lz = 0.f, hp = 0.f, lp = 0.f;
+  double sx = 0.0, sy = 0.0, sz = 0.0, sp = 0.0;
+  if ((mode & kCombine) && P.precision == 1) {
+    const fpair4* fp = reinterpret_cast<const fpair4*>(P.part) + i;
+    float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
+    if (live) {
 #pragma unroll 8
-      for (int s = 0; s < c.n_slices; ++s) {
-        const fpair4 q = fp[(int64_t)s * P.n_total + i];
-        two_sum_acc(hx, lx, q.xy.x), lx += q.xy.y;
-        two_sum_acc(hy, ly, q.xy.z), ly += q.xy.w;
-        two_sum_acc(hz, lz, q.zp.x), lz += q.zp.y;
-        two_sum_acc(hp, lp, q.zp.z), lp += q.zp.w;
-      }
-      sx = (double)hx + (double)lx, sy = (double)hy + (double)ly;
-      sz = (double)hz + (double)lz, sp = (double)hp + (double)lp;
-    } else if (mode & kCombine) {
-#pragma unroll 8
-      for (int s = 0; s < c.n_slices; ++s) {
-        const double4_32a q = part[(int64_t)s * P.n_total + i];
-        sx += q.x, sy += q.y, sz += q.z, sp += q.w;
+      for (int s = g; s < c.n_slices; s += kSlotGroups) {
+        const fpair4 q = fp[(int64_t)s * P.n_total];
+        two_sum_acc(h[0], l[0], q.xy.x), l[0] += q.xy.y;
+        two_sum_acc(h[1], l[1], q.xy.z), l[1] += q.xy.w;
+        two_sum_acc(h[2], l[2], q.zp.x), l[2] += q.zp.y;
+        two_sum_acc(h[3], l[3], q.zp.z), l[3] += q.zp.w;
       }
     }
-    bad |= post_body(P, mode, i, cen, sx, sy, sz, sp, e);
+    add_groups(red.f, g, b, h, l);
+    if (g == 0) {
+      sx = (double)h[0] + (double)l[0], sy = (double)h[1] + (double)l[1];
+      sz = (double)h[2] + (double)l[2], sp = (double)h[3] + (double)l[3];
+    }
+  } else if (mode & kCombine) {
+    const double4_32a* part = reinterpret_cast<const double4_32a*>(P.part) + i;
+    double s4[4] = {0.0, 0.0, 0.0, 0.0};
+    if (live) {
+#pragma unroll 8
+      for (int s = g; s < c.n_slices; s += kSlotGroups) {
+        const double4_32a q = part[(int64_t)s * P.n_total];
+        s4[0] += q.x, s4[1] += q.y, s4[2] += q.z, s4[3] += q.w;
+      }
+    }
+    add_groups(red.d, g, b, s4);
+    sx = s4[0], sy = s4[1], sz = s4[2], sp = s4[3];
   }
-  if (bad) atomicOr(P.status, kFlagNonFinite);
+  if (g == 0 && live && post_body(P, mode, i, cen, sx, sy, sz, sp, e)) atomicOr(P.status, kFlagNonFinite);
   if (mode & kVirial) {
     double kw[2] = {e[0], e[1]};
-    block_sum<2, kPostThreads>(kw);
+    if (g == 0) block_sum<2, CB, true>(kw);
     if (threadIdx.x == 0) P.epart[(int64_t)blockIdx.x * kEnergyVals + 0] = kw[0],
                           P.epart[(int64_t)blockIdx.x * kEnergyVals + 1] = kw[1];
     if (last_of(P.done, (unsigned)P.n_chunks)) {
       __threadfence();
-      systems_final<2, kPostThreads>(P.sys_chunk, P.n_sys, P.epart, P.n_chunks, P.status,
+      systems_final<2, kSlotGroups * CB>(P.sys_chunk, P.n_sys, P.epart, P.n_chunks, P.status,
                                      [&](int sy, const double (&v)[2]) {
                                        double* o = P.vout + 3 * (int64_t)sy;
                                        o[0] = v[0];
@@ -81,7 +146,7 @@ __global__ void __launch_bounds__(kPostThreads) k_post(const PostLaunch P) {
     return;
   }
   if (mode & kEnergy) {
-    block_sum<kEnergyVals, kPostThreads>(e);
+    if (g == 0) block_sum<kEnergyVals, CB, true>(e);
     if (threadIdx.x == 0) {
 #pragma unroll
       for (int k = 0; k < kEnergyVals; ++k) P.epart[(int64_t)blockIdx.x * kEnergyVals + k] = e[k];
@@ -90,7 +155,7 @@ __global__ void __launch_bounds__(kPostThreads) k_post(const PostLaunch P) {
     // eout null the partials wait for the next step's k_post
     if (P.eout && last_of(P.done, (unsigned)P.n_chunks)) {
       __threadfence();
-      systems_final<kEnergyVals, kPostThreads>(P.sys_chunk, P.n_sys, P.epart, P.n_chunks, P.status,
+      systems_final<kEnergyVals, kSlotGroups * CB>(P.sys_chunk, P.n_sys, P.epart, P.n_chunks, P.status,
                                                [&](int sy, const double (&v)[kEnergyVals]) {
                                                  emit_energy(P.eout, sy, v);
                                                });
@@ -101,27 +166,28 @@ __global__ void __launch_bounds__(kPostThreads) k_post(const PostLaunch P) {
 // Staging origin: per chunk, sum m x (3), sum m, sum x (3) into cpart[chunk][8];
 // the last CTA then forms, per system in a fixed order, the mass-weighted mean
 // position (plain mean if the mass is not positive; 0 for an empty system).
-__global__ void __launch_bounds__(kPostThreads) k_centre(const Chunk* chunks, const int32_t* sys_chunk,
+template <int CB>
+__global__ void __launch_bounds__(CB) k_centre(const Chunk* chunks, const int32_t* sys_chunk,
                                                          const int64_t* off, const int n_sys, const double* x,
                                                          const double* m, double* cpart, double* centre,
                                                          unsigned* done, const int64_t n_total, unsigned* status) {
   Chunk c = chunks[blockIdx.x];
   if (!chunk_ok(c, n_total, n_sys, 0, status)) c.begin = c.end = 0;  // NBODY_DEBUG builds only
   double v[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  for (int i = c.begin + (int)threadIdx.x; i < c.end; i += kPostThreads) {
+  for (int i = c.begin + (int)threadIdx.x; i < c.end; i += CB) {
     const double mi = m[i];
     const double x0 = x[3 * i + 0], x1 = x[3 * i + 1], x2 = x[3 * i + 2];
     v[0] += mi * x0, v[1] += mi * x1, v[2] += mi * x2, v[3] += mi;
     v[4] += x0, v[5] += x1, v[6] += x2;
   }
-  block_sum<7, kPostThreads>(v);
+  block_sum<7, CB>(v);
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int k = 0; k < 7; ++k) cpart[(int64_t)blockIdx.x * kEnergyVals + k] = v[k];
   }
   if (!last_of(done, gridDim.x)) return;
   __threadfence();
-  systems_final<7, kPostThreads>(sys_chunk, n_sys, cpart, gridDim.x, status, [&](int sy, const double (&w)[7]) {
+  systems_final<7, CB>(sys_chunk, n_sys, cpart, gridDim.x, status, [&](int sy, const double (&w)[7]) {
     const int64_t n = off[sy + 1] - off[sy];
     double c0 = 0.0, c1 = 0.0, c2 = 0.0;
     if (w[3] > 0.0 && isfinite(w[3])) {
@@ -134,28 +200,34 @@ __global__ void __launch_bounds__(kPostThreads) k_centre(const Chunk* chunks, co
   });
 }
 
-__global__ void __launch_bounds__(kPostThreads) k_adj_update(const AdjLaunch A) {
+template <int CB>
+__global__ void __launch_bounds__(kSlotGroups * CB) k_adj_update(const AdjLaunch A) {
+  __shared__ union {
+    SlotSums<CB> f[10];
+    double d[10][kSlotGroups - 1][CB];
+  } red;
   Chunk c = A.chunks[blockIdx.x];
   if (!chunk_ok(c, A.n_total, A.n_sys, A.part_slices, A.status)) c.begin = c.end = 0;  // NBODY_DEBUG builds only
-  const double4_32a* part = reinterpret_cast<const double4_32a*>(A.part);
   const double* cen = A.centre + 3 * c.sys;
   const int kw = A.g_params ? 3 : 2;  // partials (fpair4 / double4_32a) per body and slice
   double pv[2] = {0.0, 0.0};          // this thread's w.da/dG and sum m (d.w) / s^5
-  bool bad = false;
-  for (int i = c.begin + (int)threadIdx.x; i < c.end; i += kPostThreads) {
-    double a1x = 0, a1y = 0, a1z = 0, a2 = 0, gbx = 0, gby = 0, gbz = 0, gm = 0;
-    if (A.precision == 1) {
-      // compensated float32 pairs (fpair4), added as pairs on the FP32 pipe
-      const fpair4* fp = reinterpret_cast<const fpair4*>(A.part);
-      float h[10], l[10];
+  const int b = (int)threadIdx.x % CB, g = (int)threadIdx.x / CB;
+  const int i = c.begin + b;
+  const bool live = i < c.end;
+  double S[10];  // A1 (3), A2, Gb (3), Gm, Pg, Pe of the body
+  if (A.precision == 1) {
+    // compensated float32 pairs (fpair4), added as pairs on the FP32 pipe
+    const fpair4* fp = reinterpret_cast<const fpair4*>(A.part);
+    float h[10], l[10];
 #pragma unroll
-      for (int q = 0; q < 10; ++q) h[q] = l[q] = 0.f;
-      auto add = [&](const int q, const float hv, const float lv) {
-        two_sum_acc(h[q], l[q], hv);
-        l[q] += lv;
-      };
+    for (int q = 0; q < 10; ++q) h[q] = l[q] = 0.f;
+    auto add = [&](const int q, const float hv, const float lv) {
+      two_sum_acc(h[q], l[q], hv);
+      l[q] += lv;
+    };
+    if (live) {
 #pragma unroll 4
-      for (int s = 0; s < c.n_slices; ++s) {
+      for (int s = g; s < c.n_slices; s += kSlotGroups) {
         const int64_t k = kw * ((int64_t)s * A.n_total + i);
         const fpair4 p = fp[k], q = fp[k + 1];
         add(0, p.xy.x, p.xy.y), add(1, p.xy.z, p.xy.w), add(2, p.zp.x, p.zp.y), add(3, p.zp.z, p.zp.w);
@@ -165,29 +237,39 @@ __global__ void __launch_bounds__(kPostThreads) k_adj_update(const AdjLaunch A) 
           add(8, r.xy.x, r.xy.y), add(9, r.xy.z, r.xy.w);
         }
       }
-      auto d = [&](const int q) { return (double)h[q] + (double)l[q]; };
-      a1x = d(0), a1y = d(1), a1z = d(2), a2 = d(3), gbx = d(4), gby = d(5), gbz = d(6), gm = d(7);
-      if (A.g_params) pv[0] += d(8), pv[1] += d(9);
-    } else {
+    }
+    add_groups(red.f, g, b, h, l);
+#pragma unroll
+    for (int q = 0; q < 10; ++q) S[q] = g == 0 ? (double)h[q] + (double)l[q] : 0.0;
+  } else {
+    const double4_32a* part = reinterpret_cast<const double4_32a*>(A.part);
+#pragma unroll
+    for (int q = 0; q < 10; ++q) S[q] = 0.0;
+    if (live) {
 #pragma unroll 4
-      for (int s = 0; s < c.n_slices; ++s) {
+      for (int s = g; s < c.n_slices; s += kSlotGroups) {
         const int64_t k = kw * ((int64_t)s * A.n_total + i);
         const double4_32a p = part[k], q = part[k + 1];
-        a1x += p.x, a1y += p.y, a1z += p.z, a2 += p.w;
-        gbx += q.x, gby += q.y, gbz += q.z, gm += q.w;
+        S[0] += p.x, S[1] += p.y, S[2] += p.z, S[3] += p.w;
+        S[4] += q.x, S[5] += q.y, S[6] += q.z, S[7] += q.w;
         if (A.g_params) {
           const double4_32a r = part[k + 2];
-          pv[0] += r.x, pv[1] += r.y;
+          S[8] += r.x, S[9] += r.y;
         }
       }
     }
+    add_groups(red.d, g, b, S);
+  }
+  if (g == 0 && live) {
+    const double a1x = S[0], a1y = S[1], a1z = S[2], a2 = S[3], gbx = S[4], gby = S[5], gbz = S[6], gm = S[7];
+    if (A.g_params) pv[0] = S[8], pv[1] = S[9];
     const double mi = A.m[i];
     double w0 = A.lam_v[3 * i + 0], w1 = A.lam_v[3 * i + 1], w2 = A.lam_v[3 * i + 2];
     const double gx0 = A.G * (mi * a1x - a2 * w0 - 3.0 * gbx);
     const double gx1 = A.G * (mi * a1y - a2 * w1 - 3.0 * gby);
     const double gx2 = A.G * (mi * a1z - a2 * w2 - 3.0 * gbz);
     const double gmi = -A.G * gm;
-    bad |= !(isfinite(gx0) && isfinite(gx1) && isfinite(gx2) && isfinite(gmi));
+    if (!(isfinite(gx0) && isfinite(gx1) && isfinite(gx2) && isfinite(gmi))) atomicOr(A.status, kFlagNonFinite);
     const double l0 = A.lam_x[3 * i + 0] + A.coef * gx0;
     const double l1 = A.lam_x[3 * i + 1] + A.coef * gx1;
     const double l2 = A.lam_x[3 * i + 2] + A.coef * gx2;
@@ -205,16 +287,15 @@ __global__ void __launch_bounds__(kPostThreads) k_adj_update(const AdjLaunch A) 
       stage_store(A.precision, A.stage_x, i, A.x_next[3 * i + 0], A.x_next[3 * i + 1], A.x_next[3 * i + 2], mi,
                   cen, A.stage_lo);
   }
-  if (bad) atomicOr(A.status, kFlagNonFinite);
   if (!A.g_params) return;
   // dL/dG += coef sum_k w_k . da_k/dG; dL/deps += coef (-3 G eps) sum_k sum_j m_j (d.w_k) / s^5,
   // per system in a fixed order (chunk partials, then the last CTA)
-  block_sum<2, kPostThreads>(pv);
+  if (g == 0) block_sum<2, CB, true>(pv);
   if (threadIdx.x == 0) A.cpart[(int64_t)blockIdx.x * kEnergyVals + 0] = pv[0],
                         A.cpart[(int64_t)blockIdx.x * kEnergyVals + 1] = pv[1];
   if (!last_of(A.done, gridDim.x)) return;
   __threadfence();
-  systems_final<2, kPostThreads>(A.sys_chunk, A.n_sys, A.cpart, gridDim.x, A.status, [&](int sy, const double (&v)[2]) {
+  systems_final<2, kSlotGroups * CB>(A.sys_chunk, A.n_sys, A.cpart, gridDim.x, A.status, [&](int sy, const double (&v)[2]) {
     const double dG = A.coef * v[0], de = A.coef * (-3.0 * A.G * A.eps) * v[1];
     if (!(isfinite(dG) && isfinite(de))) atomicOr(A.status, kFlagNonFinite);
     A.g_params[2 * sy + 0] += dG;
@@ -222,14 +303,15 @@ __global__ void __launch_bounds__(kPostThreads) k_adj_update(const AdjLaunch A) 
   });
 }
 
-__global__ void __launch_bounds__(kPostThreads) k_stage_vec(const Chunk* chunks, int precision, const double* vec,
+template <int CB>
+__global__ void __launch_bounds__(CB) k_stage_vec(const Chunk* chunks, int precision, const double* vec,
                                                             const double* m, const double* centre, void* stage,
                                                             void* stage_lo, int as_position, const int64_t n_total,
                                                             const int n_sys, unsigned* status) {
   Chunk c = chunks[blockIdx.x];
   if (!chunk_ok(c, n_total, n_sys, 0, status)) c.begin = c.end = 0;  // NBODY_DEBUG builds only
   const double* cen = centre + 3 * c.sys;
-  for (int i = c.begin + (int)threadIdx.x; i < c.end; i += kPostThreads) {
+  for (int i = c.begin + (int)threadIdx.x; i < c.end; i += CB) {
     const double v0 = vec[3 * i + 0], v1 = vec[3 * i + 1], v2 = vec[3 * i + 2];
     if (as_position) {
       stage_store(precision, stage, i, v0, v1, v2, m[i], cen, stage_lo);
@@ -266,33 +348,53 @@ cudaError_t launch_copy4(const Copy4& C, int n_sms, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// f(std::integral_constant<int, bodies per chunk of a layout of n_total bodies>)
+template <typename F>
+static cudaError_t with_chunk(const int64_t n_total, F f) {
+  return chunk_bodies(n_total) == kChunk ? f(std::integral_constant<int, kChunk>())
+                                         : f(std::integral_constant<int, kChunkSmall>());
+}
+
 cudaError_t launch_post(const PostLaunch& P, cudaStream_t st) {
   if (P.n_chunks <= 0) return cudaSuccess;
-  return launch_pdl(k_post, (unsigned)P.n_chunks + (P.eprev_out ? 1u : 0u), kPostThreads, st, P);
+  return with_chunk(P.n_total, [&](auto cb) {
+    constexpr int CB = decltype(cb)::value;
+    // a pass that combines nothing needs one thread per body only
+    return launch_pdl(k_post<CB>, (unsigned)P.n_chunks + (P.eprev_out ? 1u : 0u),
+                      (P.mode & kCombine) ? kSlotGroups * CB : CB, st, P);
+  });
 }
 
 cudaError_t launch_centre(const Chunk* chunks, int n_chunks, const int32_t* sys_chunk, const int64_t* off, int n_sys,
                           const double* x, const double* m, double* cpart, double* centre, unsigned* done,
                           int64_t n_total, unsigned* status, cudaStream_t st) {
   if (n_sys <= 0 || n_chunks <= 0) return cudaSuccess;
-  k_centre<<<n_chunks, kPostThreads, 0, st>>>(chunks, sys_chunk, off, n_sys, x, m, cpart, centre, done, n_total,
-                                              status);
-  return cudaGetLastError();
+  return with_chunk(n_total, [&](auto cb) {
+    constexpr int CB = decltype(cb)::value;
+    k_centre<CB><<<n_chunks, CB, 0, st>>>(chunks, sys_chunk, off, n_sys, x, m, cpart, centre, done, n_total, status);
+    return cudaGetLastError();
+  });
 }
 
 cudaError_t launch_adj_update(const AdjLaunch& A, cudaStream_t st) {
   if (A.n_chunks <= 0) return cudaSuccess;
-  k_adj_update<<<A.n_chunks, kPostThreads, 0, st>>>(A);
-  return cudaGetLastError();
+  return with_chunk(A.n_total, [&](auto cb) {
+    constexpr int CB = decltype(cb)::value;
+    k_adj_update<CB><<<A.n_chunks, kSlotGroups * CB, 0, st>>>(A);
+    return cudaGetLastError();
+  });
 }
 
 cudaError_t launch_stage_vec(const Chunk* chunks, int n_chunks, int precision, const double* vec, const double* m,
                              const double* centre, void* stage, void* stage_lo, int as_position, int64_t n_total,
                              int n_sys, unsigned* status, cudaStream_t st) {
   if (n_chunks <= 0) return cudaSuccess;
-  k_stage_vec<<<n_chunks, kPostThreads, 0, st>>>(chunks, precision, vec, m, centre, stage, stage_lo, as_position,
-                                                 n_total, n_sys, status);
-  return cudaGetLastError();
+  return with_chunk(n_total, [&](auto cb) {
+    constexpr int CB = decltype(cb)::value;
+    k_stage_vec<CB><<<n_chunks, CB, 0, st>>>(chunks, precision, vec, m, centre, stage, stage_lo, as_position, n_total,
+                                             n_sys, status);
+    return cudaGetLastError();
+  });
 }
 
 }  // namespace nbody
