@@ -167,8 +167,6 @@ __global__ void __launch_bounds__(BLOCK) k_vjp_mixed(const PairLaunch L) {
   const float4* __restrict__ sx = static_cast<const float4*>(L.stage_x);
   const float4* __restrict__ sw = static_cast<const float4*>(L.stage_w);
   fpair4* __restrict__ part = reinterpret_cast<fpair4*>(L.part);
-  const float eps2 = (float)L.eps2;
-  const float r2c = L.r2_near;
   const float4* __restrict__ slo = L.stage_lo;
 
   for (;;) {
@@ -176,6 +174,7 @@ __global__ void __launch_bounds__(BLOCK) k_vjp_mixed(const PairLaunch L) {
     if (it >= L.n_items) break;
     const WorkItem w = L.items[it];
     if (!item_ok(w, L)) continue;  // NBODY_DEBUG builds only
+    const float eps2 = L.sys[w.sys].eps2, r2c = slo ? L.sys[w.sys].r2c : 0.f;
 
     float xk[R], yk[R], zk[R], mk[R], wkx[R], wky[R], wkz[R];
     Acc8f hi[R], lo[R];
@@ -435,9 +434,6 @@ __global__ void __launch_bounds__(BLOCK) k_vjp_mixed2(const PairLaunch L) {
   const float4* __restrict__ sx = static_cast<const float4*>(L.stage_x);
   const float4* __restrict__ sw = static_cast<const float4*>(L.stage_w);
   fpair4* __restrict__ part = reinterpret_cast<fpair4*>(L.part);
-  const float eps2 = (float)L.eps2;
-  const float2 e2 = make_float2(eps2, eps2);
-  const float r2c = L.r2_near;
   const float4* __restrict__ slo = L.stage_lo;
 
   auto put = [&](const int b, const int t, const float4 q, const float4 u) {
@@ -454,6 +450,8 @@ __global__ void __launch_bounds__(BLOCK) k_vjp_mixed2(const PairLaunch L) {
     if (it >= L.n_items) break;
     const WorkItem w = L.items[it];
     if (!item_ok(w, L)) continue;  // NBODY_DEBUG builds only
+    const float eps2 = L.sys[w.sys].eps2, r2c = slo ? L.sys[w.sys].r2c : 0.f;
+    const float2 e2 = make_float2(eps2, eps2);
 
     float2 nx[R], ny[R], nz[R], mk[R], wkx[R], wky[R], wkz[R];
     float hi[R][NC], lo[R][NC];

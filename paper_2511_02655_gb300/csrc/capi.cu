@@ -36,9 +36,16 @@ constexpr int64_t kTailMin = 64;   // shortest slice of a halving tail
 
 struct Tiling {
   int block = 0, ipt = 0, jtile = 0, slice = 0, n_ctas = 0;
-  int variant = 0;  // mixed kernels: 0 scalar, 1 packed float32x2, 2 packed with a 4-CTA register cap (force)
+  int variant = 0;  // mixed kernels: 0 scalar, 1 packed float32x2, 2 packed with a 4-CTA register cap (force),
+                    // 3 symmetric (every unordered pair once)
   int tail = 0;     // slicing of a system's j-range: 0 equal slices, 1 full slices and a halving tail
+                    // (symmetric: 1 cuts every other row of i-tiles into pieces a third as long)
 };
+constexpr int kSymVariant = 3;
+constexpr double kSymMinBodies = 1024.0;    // typical system size from which the symmetric pass is a candidate
+constexpr double kSymOnlyBodies = 32768.0;  // ... and from which it is the only one (mixed path)
+constexpr int64_t kMaxSymRows = 64;                      // rows of i-tiles a system is cut into at most
+constexpr size_t kMaxSymPartialBytes = size_t(4) << 30;  // cap on the symmetric pass's partial sums
 
 // Near-pair refinement radius of the mixed force kernels: 4 softening lengths
 // for gravity, 4 sigma for Lennard-Jones (the neighbour shells that carry its
@@ -120,7 +127,7 @@ struct nbody_ctx {
   int64_t launches = 0;
 
   // layout
-  std::vector<Chunk> chunks;  // force tiling's slices
+  std::vector<Chunk> chunks;  // without slots (Chunk::n_slices, stride, row0: the copies on the device)
   std::vector<int32_t> sys_chunk;
   Chunk* d_chunks = nullptr;
   Chunk* d_vchunks = nullptr;  // same chunks, VJP tiling's slice counts
@@ -129,21 +136,23 @@ struct nbody_ctx {
 
   // force work list
   Tiling ft;
-  WorkItem* d_items = nullptr;
+  void* d_items = nullptr;  // WorkItem, or SymItem for the symmetric variant
   int n_items = 0;
   int max_slices = 1;
+  size_t fpart_bytes = 0;  // partial sums of the force pass
   // VJP work list (built on first adjoint)
   Tiling vt;
-  WorkItem* d_vitems = nullptr;
+  void* d_vitems = nullptr;
   int n_vitems = 0;
   int vmax_slices = 1;
+  size_t vpart_bytes = 0;  // partial sums of the VJP pass (without the parameter sums)
   bool vjp_ready = false;
   int64_t fault_alloc = 0;  // > 0: the fault_alloc-th scratch allocation fails (NBODY_FAULT_ALLOC, tests)
   bool nvtx = false;        // NBODY_NVTX=1: NVTX ranges around the API calls and the adjoint's phases
   bool vjp_params = false;  // VJP launches also form the G and eps gradient sums
 
   // scratch
-  DevBuf stage, stage_lo, stage_w, part, centre, epart, status_counter, a_scratch;
+  DevBuf stage, stage_lo, stage_w, part, sysp, epart, status_counter, a_scratch;
   unsigned* counter = nullptr;  // [2]
   unsigned* status = nullptr;   // [1]
 
@@ -259,9 +268,33 @@ nbody_status check_dev(nbody_ctx* c, const void* p, size_t bytes, const char* na
 // ---------------------------------------------------------------------------
 // work lists
 
+constexpr int kSymBlock = 64;  // j-bodies that a warp of the symmetric pass meets in one block: pieces are whole blocks
+
 int ctas_per_sm(int prec, const Tiling& t, bool vjp, int law) {
+  if (t.variant == kSymVariant)
+    return !vjp && prec == NBODY_MIXED && t.jtile == kSymTile ? sym_force_ctas_per_sm(t.block, t.ipt, law) : 0;
   return vjp ? vjp_ctas_per_sm(prec, t.variant, t.block, t.ipt, t.jtile)
              : force_ctas_per_sm(prec, t.variant, t.block, t.ipt, t.jtile, law);
+}
+
+bool is_sym(const Tiling& t) { return t.variant == kSymVariant; }
+
+// Unordered pairs of all systems.
+double total_pairs(const nbody_ctx* c) {
+  double p = 0.0;
+  for (int s = 0; s < c->n_sys; ++s) {
+    const double n = (double)(c->offsets[s + 1] - c->offsets[s]);
+    p += 0.5 * n * n;
+  }
+  return p;
+}
+
+// Slice of a symmetric tiling that makes about `pieces` work items per persistent CTA.
+constexpr int kSymPieces = 6;
+int sym_slice(const nbody_ctx* c, const Tiling& t, int n_ctas, int pieces) {
+  const double len = total_pairs(c) / ((double)n_ctas * pieces * t.block * t.ipt);
+  const double q = kSymBlock;
+  return (int)std::min(1.0e9, std::max(q, q * std::floor(len / q + 0.5)));
 }
 
 // Slice length for tiling t: the largest power-of-two multiple of jtile that
@@ -367,28 +400,26 @@ void build_items(const nbody_ctx* c, const Tiling& t, std::vector<WorkItem>& ite
   });
 }
 
-nbody_status upload_items(nbody_ctx* c, const std::vector<WorkItem>& items, WorkItem** dst) {
+nbody_status upload_items(nbody_ctx* c, const void* items, size_t bytes, void** dst) {
   invalidate_graph(c);
   if (*dst) {
     cudaStreamSynchronize(c->stream);
     cudaFree(*dst);
     *dst = nullptr;
   }
-  const size_t bytes = std::max<size_t>(1, items.size()) * sizeof(WorkItem);
-  if (cudaMalloc(dst, bytes) != cudaSuccess) {
+  if (cudaMalloc(dst, std::max<size_t>(16, bytes)) != cudaSuccess) {
     cudaGetLastError();
+    *dst = nullptr;
     return fail(c, NBODY_ENOMEM, "cudaMalloc of the work list failed");
   }
-  if (!items.empty()) NB_CUDA(c, cudaMemcpy(*dst, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
+  if (bytes) NB_CUDA(c, cudaMemcpy(*dst, items, bytes, cudaMemcpyHostToDevice));
   // a pageable-memory cudaMemcpy may return before its DMA lands; the context
   // stream can be non-blocking, so wait for the device before any launch
   NB_CUDA(c, cudaDeviceSynchronize());
   return NBODY_OK;
 }
 
-nbody_status upload_chunks(nbody_ctx* c, const std::vector<int>& sys_slices, Chunk** dst) {
-  std::vector<Chunk> ch = c->chunks;
-  for (auto& k : ch) k.n_slices = sys_slices[k.sys];
+nbody_status upload_chunks(nbody_ctx* c, const std::vector<Chunk>& ch, Chunk** dst) {
   if (!*dst) {
     if (cudaMalloc(dst, std::max<size_t>(1, ch.size()) * sizeof(Chunk)) != cudaSuccess) {
       cudaGetLastError();
@@ -400,6 +431,70 @@ nbody_status upload_chunks(nbody_ctx* c, const std::vector<int>& sys_slices, Chu
   return NBODY_OK;
 }
 
+// Work list of the symmetric pass for tiling t (see sym_common.cuh): rows of
+// whole i-tiles, at most kMaxSymRows per system (a body has a slot per row up to
+// its own, so more rows would mean more partials to combine than pair work saved),
+// each cut into pieces of about slice x i-tile pairs. Chunks get their slots; rows
+// is the number of entries the partial buffer needs.
+void build_sym_items(const nbody_ctx* c, const Tiling& t, std::vector<SymItem>& items, std::vector<Chunk>& chunks,
+                     int& max_slots, int64_t& rows) {
+  items.clear();
+  chunks = c->chunks;
+  max_slots = 1;
+  rows = 0;
+  const int64_t itile = (int64_t)t.block * t.ipt;
+  const int64_t q = kSymBlock;
+  const double area = (double)t.slice * (double)itile;
+  std::vector<int> slots;
+  for (int s = 0; s < c->n_sys; ++s) {
+    const int64_t b = c->offsets[s], n = c->offsets[s + 1] - b;
+    if (n <= 0) continue;
+    const int64_t H = itile * ((n + itile * kMaxSymRows - 1) / (itile * kMaxSymRows)), nr = (n + H - 1) / H;
+    slots.assign((size_t)nr, 0);
+    const size_t first = items.size();
+    int most = 0;
+    for (int64_t r = 0; r < nr; ++r) {
+      const int64_t i0 = r * H, ni = std::min(H, n - i0), len = n - i0;
+      const double pairs = (double)ni * ((double)len - 0.5 * (double)ni);
+      const double want = t.tail && (r & 1) ? area / 3.0 : area;
+      int64_t p = std::max<int64_t>(1, (int64_t)(pairs / want + 0.5));
+      const int64_t step = (((len + p - 1) / p + q - 1) / q) * q;
+      p = (len + step - 1) / step;
+      slots[(size_t)r] = (int)(r + 1 + p);
+      most = std::max(most, slots[(size_t)r]);
+      for (int64_t k = 0; k < p; ++k) {
+        SymItem w{};
+        w.sys = s;
+        w.i_begin = (int32_t)(b + i0);
+        w.i_end = (int32_t)(b + i0 + ni);
+        w.j_begin = (int32_t)(b + i0 + k * step);
+        w.j_end = (int32_t)(b + std::min(n, i0 + (k + 1) * step));
+        w.slot_j = (int32_t)r;
+        w.slot_i = (int32_t)(r + 1 + k);
+        w.stride = (int32_t)n;
+        w.row0 = rows - b;
+        items.push_back(w);
+      }
+    }
+    for (int32_t k = c->sys_chunk[s]; k < c->sys_chunk[s + 1]; ++k) {
+      Chunk& ch = chunks[(size_t)k];
+      ch.n_slices = slots[(size_t)((ch.begin - b) / H)];
+      ch.stride = (int32_t)n;
+      ch.row0 = rows - b;
+    }
+    (void)first;
+    max_slots = std::max(max_slots, most);
+    rows += (int64_t)most * n;
+  }
+  // longest first, for the dynamic schedule of the persistent grid
+  auto cost = [](const SymItem& w) {
+    const int64_t ni = w.i_end - w.i_begin, nj = w.j_end - w.j_begin;
+    const int64_t own = std::max<int64_t>(0, std::min(w.i_end, w.j_end) - w.j_begin);  // j-bodies inside the row
+    return ni * nj - own * (own - 1) / 2;
+  };
+  std::stable_sort(items.begin(), items.end(), [&](const SymItem& x, const SymItem& y) { return cost(x) > cost(y); });
+}
+
 // Installs tiling t for the force (vjp=false) or VJP (vjp=true) pass.
 nbody_status install_tiling(nbody_ctx* c, Tiling t, bool vjp) {
   const int prec = c->cfg.precision;
@@ -407,26 +502,62 @@ nbody_status install_tiling(nbody_ctx* c, Tiling t, bool vjp) {
   if (occ <= 0)
     return fail(c, NBODY_EINVAL, "unsupported tiling block=%d ipt=%d jtile=%d variant=%d", t.block, t.ipt, t.jtile,
                 t.variant);
-  if (t.slice <= 0) t.slice = auto_slice(c, t, occ * c->sm_count);
-  t.slice = std::max(kSliceQuantum, (t.slice / kSliceQuantum) * kSliceQuantum);
-  std::vector<WorkItem> items;
-  std::vector<int> sys_slices;
-  int max_slices = 1;
-  build_items(c, t, items, sys_slices, max_slices);
-  t.n_ctas = std::max(1, std::min<int>(occ * c->sm_count, (int)std::max<size_t>(1, items.size())));
-  nbody_status s = upload_items(c, items, vjp ? &c->d_vitems : &c->d_items);
-  if (s) return s;
-  s = upload_chunks(c, sys_slices, vjp ? &c->d_vchunks : &c->d_chunks);
-  if (s) return s;
   const size_t per = vjp ? 64 : 32;
-  s = ensure(c, c->part, (size_t)max_slices * (size_t)c->n_total * per);
-  if (s) return s;
-  if (vjp) {
-    c->vt = t, c->n_vitems = (int)items.size(), c->vmax_slices = max_slices, c->vjp_ready = true;
+  std::vector<Chunk> chunks;
+  int n_items = 0, max_slices = 1;
+  size_t part_bytes = 0;
+  nbody_status s;
+  if (is_sym(t)) {
+    if (t.slice <= 0) t.slice = sym_slice(c, t, occ * c->sm_count, kSymPieces);
+    std::vector<SymItem> items;
+    int64_t rows = 0;
+    build_sym_items(c, t, items, chunks, max_slices, rows);
+    part_bytes = (size_t)rows * per;
+    if (part_bytes > kMaxSymPartialBytes)
+      return fail(c, NBODY_EINVAL, "symmetric tiling needs %zu bytes of partial sums", part_bytes);
+    n_items = (int)items.size();
+    if ((s = upload_items(c, items.data(), items.size() * sizeof(SymItem), vjp ? &c->d_vitems : &c->d_items))) return s;
   } else {
-    c->ft = t, c->n_items = (int)items.size(), c->max_slices = max_slices;
+    if (t.slice <= 0) t.slice = auto_slice(c, t, occ * c->sm_count);
+    t.slice = std::max(kSliceQuantum, (t.slice / kSliceQuantum) * kSliceQuantum);
+    std::vector<WorkItem> items;
+    std::vector<int> sys_slices;
+    build_items(c, t, items, sys_slices, max_slices);
+    chunks = c->chunks;
+    for (auto& k : chunks) k.n_slices = sys_slices[k.sys], k.stride = (int32_t)c->n_total, k.row0 = 0;
+    part_bytes = (size_t)max_slices * (size_t)c->n_total * per;
+    n_items = (int)items.size();
+    if ((s = upload_items(c, items.data(), items.size() * sizeof(WorkItem), vjp ? &c->d_vitems : &c->d_items))) return s;
+  }
+  t.n_ctas = std::max(1, std::min(occ * c->sm_count, std::max(1, n_items)));
+  if ((s = upload_chunks(c, chunks, vjp ? &c->d_vchunks : &c->d_chunks))) return s;
+  if ((s = ensure(c, c->part, part_bytes))) return s;
+  if (vjp) {
+    c->vt = t, c->n_vitems = n_items, c->vmax_slices = max_slices, c->vpart_bytes = part_bytes, c->vjp_ready = true;
+  } else {
+    c->ft = t, c->n_items = n_items, c->max_slices = max_slices, c->fpart_bytes = part_bytes;
   }
   return NBODY_OK;
+}
+
+SymLaunch sym_launch(nbody_ctx* c, bool phi) {
+  SymLaunch L{};
+  L.stage_x = c->stage.p;
+  L.stage_lo = static_cast<const float4*>(c->stage_lo.p);
+  L.items = static_cast<const SymItem*>(c->d_items);
+  L.n_items = c->n_items;
+  L.counter = c->counter;
+  L.part = static_cast<double*>(c->part.p);
+  L.part_rows = (int64_t)(c->part.bytes / 32);
+  L.n_total = c->n_total;
+  L.sys = static_cast<const SysParam*>(c->sysp.p);
+  L.eps2 = c->cfg.eps * c->cfg.eps;
+  L.sigma2 = c->cfg.lj_sigma * c->cfg.lj_sigma;
+  L.law = c->cfg.law;
+  L.block = c->ft.block, L.ipt = c->ft.ipt, L.n_ctas = c->ft.n_ctas;
+  L.phi = phi ? 1 : 0;
+  L.status = c->status;
+  return L;
 }
 
 // refine: the mixed force and VJP kernels may use the staged remainders (near pairs).
@@ -435,21 +566,16 @@ PairLaunch pair_launch(nbody_ctx* c, bool vjp, bool refine = true, bool phi = tr
   const bool lo = refine && c->cfg.precision == NBODY_MIXED && c->stage_lo.p;
   L.stage_lo = lo ? static_cast<const float4*>(c->stage_lo.p) : nullptr;
   L.law = vjp ? 0 : c->cfg.law;
-  const double sc2 = c->stage_scale * c->stage_scale;  // staged length units: sigma (mixed LJ) or 1
-  L.sigma2 = c->cfg.lj_sigma * c->cfg.lj_sigma * sc2;   // 1 for mixed Lennard-Jones
-  L.r2_near = 0.f;
-  if (lo)
-    L.r2_near = c->cfg.law == NBODY_LAW_LJ
-                    ? (float)(kNearRadiusSigma * kNearRadiusSigma * L.sigma2 + c->cfg.eps * c->cfg.eps * sc2)
-                    : (float)(kNearRadiusEps * kNearRadiusEps * c->cfg.eps * c->cfg.eps);
+  L.sys = static_cast<const SysParam*>(c->sysp.p);
+  L.sigma2 = c->cfg.lj_sigma * c->cfg.lj_sigma * c->stage_scale * c->stage_scale;  // 1 for mixed Lennard-Jones
   L.stage_x = c->stage.p;
   L.stage_w = c->stage_w.p;
-  L.items = vjp ? c->d_vitems : c->d_items;
+  L.items = static_cast<const WorkItem*>(vjp ? c->d_vitems : c->d_items);
   L.n_items = vjp ? c->n_vitems : c->n_items;
   L.counter = c->counter;
   L.part = static_cast<double*>(c->part.p);
   L.n_total = c->n_total;
-  L.eps2 = c->cfg.eps * c->cfg.eps * sc2;
+  L.eps2 = c->cfg.eps * c->cfg.eps;
   const Tiling& t = vjp ? c->vt : c->ft;
   L.block = t.block, L.ipt = t.ipt, L.jtile = t.jtile, L.n_ctas = t.n_ctas;
   L.variant = t.variant;
@@ -462,10 +588,11 @@ PairLaunch pair_launch(nbody_ctx* c, bool vjp, bool refine = true, bool phi = tr
   return L;
 }
 
-// Slices of partials (bytes_per_body each) the partial-sum buffer holds.
-int32_t part_slices(const nbody_ctx* c, size_t bytes_per_body) {
-  if (c->n_total <= 0) return 0;
-  return (int32_t)std::min<size_t>(INT32_MAX, c->part.bytes / ((size_t)c->n_total * bytes_per_body));
+// The all-pairs kernel of the installed tiling.
+cudaError_t launch_pairs(nbody_ctx* c, bool vjp, bool phi, cudaStream_t st) {
+  if (!vjp && is_sym(c->ft)) return launch_sym_force(sym_launch(c, phi), st);
+  const PairLaunch L = pair_launch(c, vjp, true, phi);
+  return vjp ? launch_vjp(c->cfg.precision, L, st) : launch_force(c->cfg.precision, L, st);
 }
 
 cudaEvent_t pooled_event(nbody_ctx* c) {
@@ -486,14 +613,13 @@ cudaEvent_t pooled_event(nbody_ctx* c) {
 // eager (non-capturing) stream.
 nbody_status run_pair(nbody_ctx* c, cudaStream_t st, bool vjp, bool phi = true) {
   if (c->n_total == 0) return NBODY_OK;
-  PairLaunch L = pair_launch(c, vjp, true, phi);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (c->profiling && !c->capturing) {
     e0 = pooled_event(c);
     e1 = pooled_event(c);
     if (e0 && e1) NB_CUDA(c, cudaEventRecord(e0, st));
   }
-  NB_CUDA(c, vjp ? launch_vjp(c->cfg.precision, L, st) : launch_force(c->cfg.precision, L, st));
+  NB_CUDA(c, launch_pairs(c, vjp, phi, st));
   if (e0 && e1) {
     NB_CUDA(c, cudaEventRecord(e1, st));
     c->ev_used.push_back({vjp ? 1 : 0, {e0, e1}});
@@ -527,14 +653,14 @@ PostLaunch post_launch(nbody_ctx* c, unsigned mode, double* x, double* v, const 
   P.box = c->cfg.box;
   P.stage = c->stage.p;
   P.stage_lo = c->stage_lo.p;
-  P.centre = static_cast<const double*>(c->centre.p);
+  P.sys = static_cast<const SysParam*>(c->sysp.p);
   P.epart = static_cast<double*>(c->epart.p);
   P.status = c->status;
   P.eout = nullptr;
   P.sys_chunk = c->d_sys_chunk;
   P.n_sys = c->n_sys;
   P.done = c->counter + 4;
-  P.part_slices = part_slices(c, 32);
+  P.part_rows = (int64_t)(c->part.bytes / 32);
   return P;
 }
 
@@ -547,9 +673,21 @@ nbody_status run_post(nbody_ctx* c, const PostLaunch& P, cudaStream_t st) {
 
 nbody_status run_centre(nbody_ctx* c, const double* x, const double* m, cudaStream_t st) {
   if (c->cfg.precision != NBODY_MIXED || c->n_total == 0) return NBODY_OK;
-  NB_CUDA(c, launch_centre(c->d_chunks, (int)c->chunks.size(), c->d_sys_chunk, c->d_off, c->n_sys, x, m,
-                           static_cast<double*>(c->epart.p), static_cast<double*>(c->centre.p), c->counter + 5,
-                           c->n_total, c->status, st));
+  CentreLaunch C{};
+  C.chunks = c->d_chunks;
+  C.n_chunks = (int32_t)c->chunks.size();
+  C.sys_chunk = c->d_sys_chunk;
+  C.off = c->d_off;
+  C.n_sys = c->n_sys;
+  C.x = x, C.m = m;
+  C.cpart = static_cast<double*>(c->epart.p);
+  C.sys = static_cast<SysParam*>(c->sysp.p);
+  C.law = c->cfg.law;
+  C.eps = c->cfg.eps, C.near_eps = kNearRadiusEps;
+  C.done = c->counter + 5;
+  C.n_total = c->n_total;
+  C.status = c->status;
+  NB_CUDA(c, launch_centre(C, st));
   c->launches += c->chunks.empty() ? 0 : 1;
   return NBODY_OK;
 }
@@ -685,9 +823,11 @@ nbody_status fill_synthetic(nbody_ctx* c, bool with_w) {
 // slices pay for their partial-sum traffic and the tail of the schedule
 // counts; long lists are timed on a prefix of two items per persistent CTA.
 nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
-  PairLaunch L = pair_launch(c, vjp);
   const Tiling& t = vjp ? c->vt : c->ft;
+  PairLaunch L = pair_launch(c, vjp);
+  const bool sym = is_sym(t);  // timed whole: too large layouts do not come here
   auto launch = [&](const PairLaunch& P) {
+    if (sym) return launch_pairs(c, vjp, true, c->stream);
     return vjp ? launch_vjp(c->cfg.precision, P, c->stream) : launch_force(c->cfg.precision, P, c->stream);
   };
   PostLaunch C{};
@@ -700,7 +840,8 @@ nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
   C.mode = kCombine;
   C.status = c->status;
   C.n_sys = c->n_sys;
-  C.part_slices = part_slices(c, vjp ? 64 : 32);
+  C.sys = static_cast<const SysParam*>(c->sysp.p);
+  C.part_rows = (int64_t)(c->part.bytes / (vjp ? 64 : 32));
   cudaEvent_t ev[4];
   for (auto& e : ev) NB_CUDA(c, cudaEventCreate(&e));
   auto timed = [&](const PairLaunch& P, bool combine, float* best_ms) -> cudaError_t {
@@ -724,7 +865,7 @@ nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
     return err;
   };
   PairLaunch P = L;
-  P.n_items = std::min(L.n_items, 2 * t.n_ctas);
+  P.n_items = sym ? L.n_items : std::min(L.n_items, 2 * t.n_ctas);
   float ms = 0.f;
   cudaError_t err = cudaSuccess;
   if (P.n_items < L.n_items) err = timed(P, false, &ms);
@@ -736,7 +877,9 @@ nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
   if (err != cudaSuccess) return fail(c, NBODY_ECUDA, "autotune launch failed: %s", cudaGetErrorString(err));
   // interaction slots covered by the timed items (the list is longest-first)
   double slots = 0.0;
-  {
+  if (sym) {
+    slots = 2.0 * total_pairs(c);
+  } else {
     std::vector<WorkItem> h(P.n_items);
     NB_CUDA(c, cudaMemcpy(h.data(), L.items, h.size() * sizeof(WorkItem), cudaMemcpyDeviceToHost));
     for (const auto& w : h) slots += (double)(w.i_end - w.i_begin) * (double)(w.j_end - w.j_begin);
@@ -761,7 +904,7 @@ std::string tune_key(const nbody_ctx* c, bool vjp) {
   }
   char buf[512];
   snprintf(buf, sizeof(buf),
-           "v2|%s|cc%d|sm%d|%s|prec%d|law%d|var%d|b%d|r%d|j%d|s%d|nsys%d|n%lld|lay%016llx|eps%.17g|sig%.17g|box%.17g",
+           "v3|%s|cc%d|sm%d|%s|prec%d|law%d|var%d|b%d|r%d|j%d|s%d|nsys%d|n%lld|lay%016llx|eps%.17g|sig%.17g|box%.17g",
            c->dev_name.c_str(), c->dev_cc, c->sm_count, vjp ? "vjp" : "force", g.precision, g.law, g.variant,
            vjp ? 0 : g.block, vjp ? 0 : g.i_per_thread, vjp ? 0 : g.j_tile, vjp ? 0 : g.slice, c->n_sys,
            (long long)c->n_total, (unsigned long long)h, g.eps, g.lj_sigma, g.box);
@@ -824,9 +967,39 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
     if (vjp)
       variants = g.variant ? std::vector<int>{std::min(g.variant - 1, 1)} : std::vector<int>{0, 1};
     else
-      variants = g.variant ? std::vector<int>{g.variant - 1} : std::vector<int>{0, 1, 2};
+      variants = g.variant ? std::vector<int>{g.variant - 1} : std::vector<int>{1, 2};  // (the scalar kernel never won)
     // Lennard-Jones: the packed kernel, uncapped and capped (6 CTAs per SM)
     if (!vjp && g.law == NBODY_LAW_LJ) variants = g.variant ? std::vector<int>{g.variant - 1} : std::vector<int>{1, 2};
+  }
+  // The symmetric pass is a candidate when nothing about the tiling was asked for. Typical
+  // system size: the one that an average pair belongs to.
+  double pairs = 0.0, cubes = 0.0;
+  for (int k = 0; k < c->n_sys; ++k) {
+    const double n = (double)(c->offsets[k + 1] - c->offsets[k]);
+    pairs += n * n, cubes += n * n * n;
+  }
+  const bool large = pairs > kTuneLargePairs;
+  const double typical = pairs > 0 ? cubes / pairs : 0.0;
+  const bool any_tiling = !g.variant && !g.block && !g.i_per_thread && !g.j_tile && !g.slice;
+  const bool mixed = g.precision == NBODY_MIXED;
+  const bool sym = !vjp && mixed && any_tiling && typical >= kSymMinBodies;
+  const bool sym_only = sym && typical >= kSymOnlyBodies;
+  if (sym_only && large) {
+    // nothing to choose between: its cost per pair no longer depends on the tiling
+    Tiling t;
+    t.block = 256, t.ipt = 4, t.jtile = kSymTile, t.variant = kSymVariant, t.tail = 1;
+    if (install_tiling(c, t, false) == NBODY_OK) {
+      tune_cache_store(c, vjp, c->ft);
+      return NBODY_OK;
+    }
+  }
+  if (sym && !large) {
+    for (const auto& p : std::vector<std::pair<int, int>>{{128, 2}, {128, 4}, {256, 2}, {256, 4}}) {
+      Tiling t;
+      t.block = p.first, t.ipt = p.second, t.jtile = kSymTile, t.variant = kSymVariant;
+      cands.push_back(t);
+    }
+    if (sym_only) variants.clear();
   }
   for (int var : variants)
     for (int b : blocks) {
@@ -848,19 +1021,13 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
   // Large layouts are compared on work lists of short slices (the cost per
   // interaction no longer depends on the slice length there), which keeps the
   // timed prefix short; their final slice is the automatic choice.
-  double pairs = 0.0;
-  for (int k = 0; k < c->n_sys; ++k) {
-    const double n = (double)(c->offsets[k + 1] - c->offsets[k]);
-    pairs += n * n;
-  }
-  const bool large = pairs > kTuneLargePairs;
   const char* verbose_env = getenv("NBODY_TUNE_VERBOSE");  // tuning log on stderr when set to 1
   const bool verbose = verbose_env && verbose_env[0] == '1';
   // one timed measurement of candidate t0 (large layouts: short slices, scaled by the
   // wave quantisation of the final work list, which the prefix cannot see)
   auto measure = [&](const Tiling& t0, double* cost) -> nbody_status {
     Tiling t = t0;
-    if (large && t.slice == 0) t.slice = kTuneSlice;
+    if (large && t.slice == 0) t.slice = kTuneSlice;  // (no symmetric tiling comes here)
     nbody_status r;
     if ((r = install_tiling(c, t, vjp))) return r;
     if ((r = time_tiling(c, vjp, cost))) return r;
@@ -926,7 +1093,13 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
       const int L0 = c->ft.slice;
       const int64_t n_ctas = c->ft.n_ctas;
       std::vector<int> ls = {L0 / 2, L0, L0 * 2};
-      if (c->n_sys == 1) {
+      if (is_sym(base)) {
+        ls.clear();
+        for (int k : {1, 2, 3, 4, 6, 8, 12}) {
+          const int len = sym_slice(c, base, (int)n_ctas, k);
+          if (std::find(ls.begin(), ls.end(), len) == ls.end()) ls.push_back(len);
+        }
+      } else if (c->n_sys == 1) {
         const int64_t n = c->offsets[1], tiles = (n + (int64_t)base.block * base.ipt - 1) / ((int64_t)base.block * base.ipt);
         for (int64_t W = 1; W <= 64 && ls.size() < 7; ++W) {
           const int64_t ns = W * n_ctas / tiles;  // slices per tile with tiles x ns <= W x CTAs
@@ -1002,7 +1175,7 @@ void free_ctx(nbody_ctx* c) {
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   for (auto& u : c->ev_used) cudaEventDestroy(u.second.first), cudaEventDestroy(u.second.second);
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
-  for (DevBuf* b : {&c->stage, &c->stage_lo, &c->stage_w, &c->part, &c->centre, &c->epart, &c->status_counter, &c->a_scratch,
+  for (DevBuf* b : {&c->stage, &c->stage_lo, &c->stage_w, &c->part, &c->sysp, &c->epart, &c->status_counter, &c->a_scratch,
                     &c->xw, &c->vw, &c->aw, &c->ckpt, &c->traj, &c->hx, &c->hv, &c->hm, &c->ha, &c->hlog})
     release(*b);
   if (c->h_status) cudaFreeHost(c->h_status);
@@ -1062,7 +1235,7 @@ nbody_status adjoint_sweep(nbody_ctx* c, const double* x0, const double* v0, con
     if ((s = autotune(c, true))) return s;
   }
   const int vjp_bytes = g_params ? 96 : 64;  // per body and slice: 2 or 3 double4
-  if ((s = ensure(c, c->part, (size_t)std::max(c->max_slices * 32, c->vmax_slices * vjp_bytes) * n))) return s;
+  if ((s = ensure(c, c->part, std::max(c->fpart_bytes, c->vpart_bytes / 64 * (size_t)vjp_bytes)))) return s;
 
   NB_CUDA(c, cudaMemcpyAsync(g_x0, lam_xT, n3b, cudaMemcpyDeviceToDevice, st));
   NB_CUDA(c, cudaMemcpyAsync(g_v0, lam_vT, n3b, cudaMemcpyDeviceToDevice, st));
@@ -1134,7 +1307,7 @@ nbody_status adjoint_sweep(nbody_ctx* c, const double* x0, const double* v0, con
   A.stage_x = c->stage.p;
   A.stage_w = c->stage_w.p;
   A.stage_lo = c->stage_lo.p;
-  A.centre = static_cast<const double*>(c->centre.p);
+  A.sys = static_cast<const SysParam*>(c->sysp.p);
   A.status = c->status;
   A.g_params = g_params;
   A.eps = c->cfg.eps;
@@ -1142,7 +1315,7 @@ nbody_status adjoint_sweep(nbody_ctx* c, const double* x0, const double* v0, con
   A.sys_chunk = c->d_sys_chunk;
   A.n_sys = c->n_sys;
   A.done = c->counter + 6;
-  A.part_slices = part_slices(c, g_params ? 96 : 64);
+  A.part_rows = (int64_t)(c->part.bytes / (size_t)vjp_bytes);
   const Chunk* vch = c->d_vchunks;
   const int nch = (int)c->chunks.size();
   for (int k = nseg - 1; k >= 0; --k) {
@@ -1158,12 +1331,11 @@ nbody_status adjoint_sweep(nbody_ctx* c, const double* x0, const double* v0, con
     for (int t = 0; t < top - s0; ++t)
       if ((s = step(X + (size_t)(t + 1) * n3))) return s;
     NB_CUDA(c, launch_stage_vec(vch, nch, c->cfg.precision, X + (size_t)(top - s0) * n3, m,
-                                static_cast<const double*>(c->centre.p), c->stage.p, c->stage_lo.p, 1, c->n_total,
+                                A.sys, c->stage.p, c->stage_lo.p, 1, c->n_total,
                                 c->n_sys, c->status, st));
     ++c->launches;
     if (k == nseg - 1) {
-      NB_CUDA(c, launch_stage_vec(vch, nch, c->cfg.precision, g_v0, m, static_cast<const double*>(c->centre.p),
-                                  c->stage_w.p, nullptr, 0, c->n_total, c->n_sys, c->status, st));
+      NB_CUDA(c, launch_stage_vec(vch, nch, c->cfg.precision, g_v0, m, A.sys, c->stage_w.p, nullptr, 0, c->n_total, c->n_sys, c->status, st));
       ++c->launches;
     }
     for (int t = top; t >= s0; --t) {
@@ -1273,7 +1445,7 @@ nbody_status nbody_init(nbody_ctx** out, const nbody_config* cfg, int64_t n_syst
   for (int s = 0; s < c->n_sys; ++s) {
     c->sys_chunk[s] = (int32_t)c->chunks.size();
     for (int64_t b = offsets[s]; b < offsets[s + 1]; b += chunk)
-      c->chunks.push_back(Chunk{s, (int32_t)b, (int32_t)std::min<int64_t>(offsets[s + 1], b + chunk), 1});
+      c->chunks.push_back(Chunk{s, (int32_t)b, (int32_t)std::min<int64_t>(offsets[s + 1], b + chunk), 1, 0, 0, 0});
   }
   c->sys_chunk[c->n_sys] = (int32_t)c->chunks.size();
 
@@ -1287,7 +1459,7 @@ nbody_status nbody_init(nbody_ctx** out, const nbody_config* cfg, int64_t n_syst
   const size_t stage_bytes = n * (cfg->precision == NBODY_MIXED ? sizeof(float4) : sizeof(double4_32a));
   if ((s = ensure(c, c->stage, stage_bytes))) return bail(s);
   if (cfg->precision == NBODY_MIXED && (s = ensure(c, c->stage_lo, n * sizeof(float4)))) return bail(s);
-  if ((s = ensure(c, c->centre, (size_t)c->n_sys * 3 * sizeof(double)))) return bail(s);
+  if ((s = ensure(c, c->sysp, (size_t)c->n_sys * sizeof(SysParam)))) return bail(s);
   // two sets of chunk partials: a step's energy record may be finished by the next step's k_post
   if ((s = ensure(c, c->epart, 2 * std::max<size_t>(1, c->chunks.size()) * kEnergyVals * sizeof(double)))) return bail(s);
   // [0..1] work counter, [2] status word, [4] energy ticket, [5] centre ticket, [6] adjoint-parameter ticket
@@ -1301,8 +1473,19 @@ nbody_status nbody_init(nbody_ctx** out, const nbody_config* cfg, int64_t n_syst
     return bail(fail(c, NBODY_ENOMEM, "cudaHostAlloc of the status word failed"));
   }
   *c->h_status = 0u;
-  if (cudaMemset(c->centre.p, 0, (size_t)c->n_sys * 3 * sizeof(double)) != cudaSuccess)
-    return bail(fail(c, NBODY_ECUDA, "memset failed"));
+  {
+    // unscaled staging: the FP64 path's, the tuner's, and of Lennard-Jones all but the origin
+    const double sc2 = c->stage_scale * c->stage_scale, e2 = cfg->eps * cfg->eps;
+    SysParam p{};
+    p.scale = c->stage_scale, p.mscale = p.inv_mscale = 1.0;
+    p.eps2 = (float)(e2 * sc2);
+    p.r2c = cfg->law == NBODY_LAW_LJ
+                ? (float)((kNearRadiusSigma * kNearRadiusSigma * cfg->lj_sigma * cfg->lj_sigma + e2) * sc2)
+                : (float)(kNearRadiusEps * kNearRadiusEps * e2);
+    const std::vector<SysParam> all((size_t)c->n_sys, p);
+    if (cudaMemcpy(c->sysp.p, all.data(), all.size() * sizeof(SysParam), cudaMemcpyHostToDevice) != cudaSuccess)
+      return bail(fail(c, NBODY_ECUDA, "upload of the staging parameters failed"));
+  }
   if (cudaMalloc(&c->d_off, (n_systems + 1) * sizeof(int64_t)) != cudaSuccess ||
       cudaMalloc(&c->d_sys_chunk, (n_systems + 1) * sizeof(int32_t)) != cudaSuccess) {
     cudaGetLastError();

@@ -115,8 +115,6 @@ __device__ __forceinline__ void items_mixed(const PairLaunch& L, unsigned* count
   auto& tile = sm.tile;
   const float4* __restrict__ st = static_cast<const float4*>(L.stage_x);
   fpair4* __restrict__ part = reinterpret_cast<fpair4*>(L.part);
-  const float eps2 = (float)L.eps2;
-  const float r2c = L.r2_near;
   const float4* __restrict__ lo = L.stage_lo;
 
   for (;;) {
@@ -124,6 +122,7 @@ __device__ __forceinline__ void items_mixed(const PairLaunch& L, unsigned* count
     if (it >= L.n_items) break;
     const WorkItem w = L.items[it];
     if (!item_ok(w, L)) continue;  // NBODY_DEBUG builds only
+    const float eps2 = L.sys[w.sys].eps2, r2c = lo ? L.sys[w.sys].r2c : 0.f;
 
     float xi[R], yi[R], zi[R];
     float hx[R], hy[R], hz[R], hp[R], lx[R], ly[R], lz[R], lp[R];
@@ -384,10 +383,7 @@ __device__ __forceinline__ void items_mixed2(const PairLaunch& L, unsigned* coun
   auto& tm = sm.tm;
   const float4* __restrict__ st = static_cast<const float4*>(L.stage_x);
   fpair4* __restrict__ part = reinterpret_cast<fpair4*>(L.part);
-  const float eps2 = (float)L.eps2;
-  const float2 e2 = make_float2(eps2, eps2);
   const float2 s2 = make_float2((float)L.sigma2, (float)L.sigma2);
-  const float r2c = L.r2_near;
   const float4* __restrict__ lo = L.stage_lo;
 
   for (;;) {
@@ -395,6 +391,8 @@ __device__ __forceinline__ void items_mixed2(const PairLaunch& L, unsigned* coun
     if (it >= L.n_items) break;
     const WorkItem w = L.items[it];
     if (!item_ok(w, L)) continue;  // NBODY_DEBUG builds only
+    const float eps2 = L.sys[w.sys].eps2, r2c = lo ? L.sys[w.sys].r2c : 0.f;
+    const float2 e2 = make_float2(eps2, eps2);
 
     float2 nx[R], ny[R], nz[R];
     float hx[R], hy[R], hz[R], hp[R], lx[R], ly[R], lz[R], lp[R];

@@ -24,7 +24,37 @@ struct WorkItem {
 struct Chunk {
   int32_t sys;
   int32_t begin, end;
-  int32_t n_slices;  // force/VJP slices of this system (partials to combine)
+  int32_t n_slices;  // partials to combine: slot s of body i is entry row0 + s * stride + i of the partial buffer
+  int32_t stride;
+  int32_t pad;
+  int64_t row0;
+};
+
+// Per-system staging of the mixed path. Positions are staged as (x - c) * scale
+// and masses as m * mscale, with powers of two as scales for gravity (set from
+// the largest coordinate and mass at the start of every call, k_centre): the
+// float32 pair arithmetic then has the same range whatever the caller's units are
+// and the scaling costs no rounding. Where all masses of a system are equal they
+// are staged as 1 (uniform). Lennard-Jones: scale = 1 / sigma, masses unused.
+struct __align__(16) SysParam {
+  double c[3];
+  double scale, mscale, inv_mscale;
+  float eps2, r2c;   // staged softening^2 and near-pair radius^2 (0: no refinement)
+  uint32_t uniform;
+  uint32_t pad;
+};
+
+// Work item of the symmetric force pass (sym_common.cuh): i-bodies [i_begin,
+// i_end) of one system (whole i-tiles but for the system's end) against its
+// j-bodies [j_begin, j_end), every unordered pair once. Partials of i-bodies go to
+// slot slot_i, of j-bodies to slot slot_j (row0 and stride as in Chunk).
+struct SymItem {
+  int32_t sys;
+  int32_t i_begin, i_end;
+  int32_t j_begin, j_end;
+  int32_t slot_i, slot_j;
+  int32_t stride;
+  int64_t row0;
 };
 
 // The O(N) kernels do their float64 work on GB300's FP64 pipe (about 1/75 of
@@ -74,11 +104,12 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, cudaStream_t st, Args... args) {
+inline cudaError_t launch_pdl_smem(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                                   Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -86,6 +117,11 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned bl
   cfg.attrs = at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, cudaStream_t st, Args... args) {
+  return launch_pdl_smem(kern, grid, block, 0, st, args...);
 }
 
 // Device status word bits (latched, read by nbody_sync).
@@ -122,9 +158,9 @@ struct PairLaunch {
   unsigned* counter;     // [2]: next item, CTAs done (zero between launches)
   double* part;          // [slices][N] x (force: 1, VJP: 2, or 3 with params) of fpair4 (mixed) or double4_32a (FP64)
   int64_t n_total;
-  double eps2;
+  double eps2;           // FP64 softening^2 (mixed: sys)
+  const SysParam* sys;   // mixed: staged softening and near-pair radius of each system
   const float4* stage_lo;  // mixed: float32 remainders (x - c) - hi [N], near-pair refinement
-  float r2_near;         // mixed: refine pairs with s^2 below this (0 = never)
   int variant;           // mixed kernels: 0 scalar float32, 1 packed float32x2
   int law;               // 0 softened gravity, 1 Lennard-Jones
   double sigma2;         // Lennard-Jones sigma^2
@@ -135,6 +171,22 @@ struct PairLaunch {
   int32_t part_slices;   // slices the partial buffer holds (index checks of NBODY_DEBUG builds)
   int32_t block_bodies;  // debug checks: i-bodies a work item may hold (block x ipt)
   unsigned* status;      // device status word (index checks of NBODY_DEBUG builds)
+};
+
+// Launch of the symmetric force pass (sym_kernels.cu).
+struct SymLaunch {
+  const void* stage_x;     // as in PairLaunch
+  const float4* stage_lo;
+  const SymItem* items;
+  int32_t n_items;
+  unsigned* counter;
+  double* part;            // fpair4 (mixed) or double4_32a (FP64)
+  int64_t part_rows;       // entries the partial buffer holds (index checks of NBODY_DEBUG builds)
+  int64_t n_total;
+  const SysParam* sys;
+  double eps2, sigma2;     // FP64 path
+  int law, block, ipt, n_ctas, phi;
+  unsigned* status;
 };
 
 #ifdef NBODY_DEBUG
@@ -148,18 +200,30 @@ __device__ __forceinline__ bool item_ok(const WorkItem& w, const PairLaunch& L) 
                      L.status);
 }
 
+__device__ __forceinline__ bool sym_item_ok(const SymItem& w, const SymLaunch& L) {
+  const bool rows = w.i_begin >= 0 && w.i_begin < w.i_end && w.i_end <= L.n_total && w.j_begin >= w.i_begin &&
+                    w.j_begin < w.j_end && w.j_end <= L.n_total && w.slot_i >= 0 && w.slot_j >= 0 && w.stride > 0;
+  return nb_debug_ok(rows && w.row0 + w.i_begin >= 0 &&
+                         w.row0 + (int64_t)w.slot_i * w.stride + w.i_end <= L.part_rows &&
+                         w.row0 + (int64_t)w.slot_j * w.stride + w.j_end <= L.part_rows,
+                     L.status);
+}
+
 // NBODY_DEBUG check of a chunk of an O(N) kernel: rows, system index and (when
-// part_slices > 0) its slice count against the partial-sum buffer. A chunk that
-// fails is processed as an empty one.
-__device__ __forceinline__ bool chunk_ok(const Chunk& c, const int64_t n_total, const int n_sys, const int part_slices,
-                                         unsigned* status) {
+// part_rows > 0) its slots against the entries the partial-sum buffer holds. A
+// chunk that fails is processed as an empty one.
+__device__ __forceinline__ bool chunk_ok(const Chunk& c, const int64_t n_total, const int n_sys,
+                                         const int64_t part_rows, unsigned* status) {
   return nb_debug_ok(c.begin >= 0 && c.begin < c.end && c.end <= n_total && c.end - c.begin <= kChunk && c.sys >= 0 &&
-                         c.sys < n_sys && (part_slices <= 0 || (c.n_slices >= 1 && c.n_slices <= part_slices)),
+                         c.sys < n_sys &&
+                         (part_rows <= 0 || (c.n_slices >= 1 && c.row0 + c.begin >= 0 &&
+                                             c.row0 + (int64_t)(c.n_slices - 1) * c.stride + c.end <= part_rows)),
                      status);
 }
 #else
 __device__ __forceinline__ constexpr bool item_ok(const WorkItem&, const PairLaunch&) { return true; }
-__device__ __forceinline__ constexpr bool chunk_ok(const Chunk&, int64_t, int, int, unsigned*) { return true; }
+__device__ __forceinline__ constexpr bool sym_item_ok(const SymItem&, const SymLaunch&) { return true; }
+__device__ __forceinline__ constexpr bool chunk_ok(const Chunk&, int64_t, int, int64_t, unsigned*) { return true; }
 #endif
 
 // Returns cudaErrorInvalidConfiguration for an unsupported tiling.
@@ -168,6 +232,12 @@ cudaError_t launch_vjp(int precision, const PairLaunch& L, cudaStream_t st);
 // CTAs of the force kernel that fit on one SM for the tiling (0 if unsupported).
 int force_ctas_per_sm(int precision, int variant, int block, int ipt, int jtile, int law);
 int vjp_ctas_per_sm(int precision, int variant, int block, int ipt, int jtile);
+
+// Symmetric force pass (mixed): threads per CTA (block) and i-bodies per lane (ipt) select the
+// compiled kernel; cudaErrorInvalidConfiguration / 0 if there is none.
+cudaError_t launch_sym_force(const SymLaunch& L, cudaStream_t st);
+int sym_force_ctas_per_sm(int block, int ipt, int law);
+constexpr int kSymTile = 256;  // j-bodies per shared-memory tile of the symmetric kernels
 
 // ---------------------------------------------------------------------------
 // O(N) kernels (post_kernels.cu)
@@ -197,11 +267,11 @@ struct PostLaunch {
   int precision;
   int law;                 // 0 gravity: a = G S, phi = -G S_phi; 1 Lennard-Jones: a = 24 eps S / m, phi = 4 eps S_phi / m
   double lj_eps;
-  double stage_scale;      // mixed: staged positions are (x - c) * stage_scale (1 / sigma for Lennard-Jones)
+  double stage_scale;      // Lennard-Jones: staged positions are (x - c) * stage_scale (mixed: 1 / sigma)
   double box;              // > 0: reflecting walls of [0, box]^3 applied after the drift
   void* stage;             // float4 / double4_32a [N]
   void* stage_lo;          // mixed: float4 remainders of the staged coordinates [N] (nullable)
-  const double* centre;    // [n_sys][3] staging origin (mixed)
+  const SysParam* sys;     // [n_sys] staging origin and scales
   double* epart;           // [n_chunks][kEnergyVals]
   unsigned* status;        // device status word
   double* eout;            // kEnergy: nullable [n_sys][9] record formed by the last CTA (null: partials only)
@@ -211,16 +281,32 @@ struct PostLaunch {
   const int32_t* sys_chunk;  // [n_sys + 1] chunk range of each system
   int n_sys;
   unsigned* done;          // last-CTA ticket (zero between launches)
-  int32_t part_slices;     // slices the partial buffer holds (index checks of NBODY_DEBUG builds)
+  int64_t part_rows;       // entries the partial buffer holds (index checks of NBODY_DEBUG builds)
 };
 cudaError_t launch_post(const PostLaunch& P, cudaStream_t st);
 
-// centre[s] = mass-weighted mean position of system s (plain mean if the mass is 0):
-// per-chunk sums into cpart [n_chunks][kEnergyVals], then per system in a fixed
-// order by the last CTA (ticket `done`, zero between launches).
-cudaError_t launch_centre(const Chunk* chunks, int n_chunks, const int32_t* sys_chunk, const int64_t* off, int n_sys,
-                          const double* x, const double* m, double* cpart, double* centre, unsigned* done,
-                          int64_t n_total, unsigned* status, cudaStream_t st);
+// Staging parameters of every system (mixed path): the origin c is the
+// mass-weighted mean position (plain mean if the mass is 0), and for gravity the
+// scales are set from the largest coordinate and mass. Per-chunk sums into cpart
+// [n_chunks][kEnergyVals], then per system in a fixed order by the last CTA
+// (ticket `done`, zero between launches).
+struct CentreLaunch {
+  const Chunk* chunks;
+  int32_t n_chunks;
+  const int32_t* sys_chunk;
+  const int64_t* off;
+  int n_sys;
+  const double* x;
+  const double* m;
+  double* cpart;
+  SysParam* sys;
+  int law;
+  double eps, near_eps;  // gravity: softening length, near-pair radius in softening lengths
+  unsigned* done;
+  int64_t n_total;
+  unsigned* status;
+};
+cudaError_t launch_centre(const CentreLaunch& C, cudaStream_t st);
 
 struct AdjLaunch {
   const Chunk* chunks;
@@ -238,7 +324,7 @@ struct AdjLaunch {
   void* stage_x;
   void* stage_w;
   void* stage_lo;          // mixed: float4 remainders of the staged positions (nullable)
-  const double* centre;
+  const SysParam* sys;
   unsigned* status;
   double* g_params;        // nullable [n_sys][2]: += coef (w.da/dG, w.da/deps), formed by the last CTA
   double eps;
@@ -246,7 +332,7 @@ struct AdjLaunch {
   const int32_t* sys_chunk;
   int n_sys;
   unsigned* done;          // last-CTA ticket (zero between launches)
-  int32_t part_slices;     // slices the partial buffer holds (index checks of NBODY_DEBUG builds)
+  int64_t part_rows;       // bodies' entries the partial buffer holds (index checks of NBODY_DEBUG builds)
 };
 cudaError_t launch_adj_update(const AdjLaunch& A, cudaStream_t st);
 
@@ -262,7 +348,7 @@ cudaError_t launch_copy4(const Copy4& C, int n_sms, cudaStream_t st);
 // stage w = lam (float4 / double4_32a) or positions x (as_position; with their
 // float32 remainders into stage_lo when given) for a VJP without an update
 cudaError_t launch_stage_vec(const Chunk* chunks, int n_chunks, int precision, const double* vec, const double* m,
-                             const double* centre, void* stage, void* stage_lo, int as_position, int64_t n_total,
+                             const SysParam* sys, void* stage, void* stage_lo, int as_position, int64_t n_total,
                              int n_sys, unsigned* status, cudaStream_t st);
 
 }  // namespace nbody

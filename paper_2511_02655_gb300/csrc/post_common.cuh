@@ -76,16 +76,15 @@ __device__ __forceinline__ void reflect(double& x, double& v, const double box) 
   }
 }
 
-// Staging entry of body i. Mixed: float4 ((x - c) * scale, m) rounded to
-// float32 and, when lo is given, the float32 remainders of the scaled
-// coordinates used by the near-pair refinement of the force kernels (scale is
-// 1, or 1 / sigma for Lennard-Jones). FP64: double4 (x, m).
+// Staging entry of body i. Mixed: float4 ((x - c) * scale, m * mscale) rounded to
+// float32 and, when lo is given, the float32 remainders of the scaled coordinates
+// used by the near-pair refinement (SysParam). FP64: double4 (x, m).
 __device__ __forceinline__ void stage_store(int precision, void* stage, int i, double x, double y, double z,
-                                            double m, const double* c, void* lo = nullptr, double scale = 1.0) {
+                                            double m, const SysParam& sp, void* lo = nullptr) {
   if (precision == 1) {
-    const double X = (x - c[0]) * scale, Y = (y - c[1]) * scale, Z = (z - c[2]) * scale;
+    const double X = (x - sp.c[0]) * sp.scale, Y = (y - sp.c[1]) * sp.scale, Z = (z - sp.c[2]) * sp.scale;
     const float hx = (float)X, hy = (float)Y, hz = (float)Z;
-    static_cast<float4*>(stage)[i] = make_float4(hx, hy, hz, (float)m);
+    static_cast<float4*>(stage)[i] = make_float4(hx, hy, hz, sp.uniform ? 1.f : (float)(m * sp.mscale));
     if (lo)
       static_cast<float4*>(lo)[i] =
           make_float4((float)(X - (double)hx), (float)(Y - (double)hy), (float)(Z - (double)hz), 0.f);
@@ -168,9 +167,9 @@ __device__ __forceinline__ void emit_energy(double* out, const int sy, const dou
 // summed partials (sx, sy, sz, sp) become a = G S (or the Lennard-Jones
 // scaling) and phi; then the closing half-kick, the energy or virial terms
 // (accumulated into e), the opening half-kick and drift of the next step (with
-// the walls), and the staging entry of the new position. cen is the system's
-// staging origin. Returns true if a combined value is not finite.
-__device__ __forceinline__ bool post_body(const PostLaunch& P, const unsigned mode, const int i, const double* cen,
+// the walls), and the staging entry of the new position. s holds the system's
+// staging origin and scales. Returns true if a combined value is not finite.
+__device__ __forceinline__ bool post_body(const PostLaunch& P, const unsigned mode, const int i, const SysParam& s,
                                           const double sx, const double sy, const double sz, const double sp,
                                           double (&e)[kEnergyVals]) {
   bool bad = false;
@@ -185,8 +184,9 @@ __device__ __forceinline__ bool post_body(const PostLaunch& P, const unsigned mo
   if (need_m) m = P.m[i];
   double ax = 0.0, ay = 0.0, az = 0.0, ph = 0.0;
   if (mode & kCombine) {
-    if (P.law == 0) {  // softened gravity
-      ax = P.G * sx, ay = P.G * sy, az = P.G * sz, ph = -P.G * sp;
+    if (P.law == 0) {  // softened gravity; the staged sums carry mscale / scale^2 (mscale / scale)
+      const double gp = P.G * (s.scale * s.inv_mscale), ga = gp * s.scale;
+      ax = ga * sx, ay = ga * sy, az = ga * sz, ph = -gp * sp;
     } else {  // Lennard-Jones: per unit mass of body i (sums over staged coordinates in units of sigma
               // carry one factor sigma: S = sigma * sum (u^3 - 2 u^6) d / r^2, hence the stage_scale)
       const double im = 1.0 / m, ca = 24.0 * P.lj_eps * P.stage_scale * im, cp = 4.0 * P.lj_eps * im;
@@ -228,7 +228,7 @@ __device__ __forceinline__ bool post_body(const PostLaunch& P, const unsigned mo
     }
     if (mode & (kKickEnd | kDrift)) P.v[3 * i + 0] = v0, P.v[3 * i + 1] = v1, P.v[3 * i + 2] = v2;
   }
-  if (mode & kStage) stage_store(P.precision, P.stage, i, x0, x1, x2, m, cen, P.stage_lo, P.stage_scale);
+  if (mode & kStage) stage_store(P.precision, P.stage, i, x0, x1, x2, m, s, P.stage_lo);
   return bad;
 }
 

@@ -84,9 +84,9 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
     return;
   }
   Chunk c = P.chunks[blockIdx.x];
-  if (!chunk_ok(c, P.n_total, P.n_sys, (P.mode & kCombine) ? P.part_slices : 0, P.status))
+  if (!chunk_ok(c, P.n_total, P.n_sys, (P.mode & kCombine) ? P.part_rows : 0, P.status))
     c.begin = c.end = 0;  // NBODY_DEBUG builds only: processed as an empty chunk
-  const double* cen = P.centre + 3 * c.sys;
+  const SysParam& sp = P.sys[c.sys];
   double e[kEnergyVals];
 #pragma unroll
   for (int k = 0; k < kEnergyVals; ++k) e[k] = 0.0;
@@ -95,14 +95,14 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
   const int i = c.begin + b;
   const bool live = i < c.end;
 
-  double sx = 0.0, sy = 0.0, sz = 0.0, sp = 0.0;
+  double sx = 0.0, sy = 0.0, sz = 0.0, sphi = 0.0;
   if ((mode & kCombine) && P.precision == 1) {
-    const fpair4* fp = reinterpret_cast<const fpair4*>(P.part) + i;
+    const fpair4* fp = reinterpret_cast<const fpair4*>(P.part) + (c.row0 + i);
     float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
     if (live) {
 #pragma unroll 8
       for (int s = g; s < c.n_slices; s += kSlotGroups) {
-        const fpair4 q = fp[(int64_t)s * P.n_total];
+        const fpair4 q = fp[(int64_t)s * c.stride];
         two_sum_acc(h[0], l[0], q.xy.x), l[0] += q.xy.y;
         two_sum_acc(h[1], l[1], q.xy.z), l[1] += q.xy.w;
         two_sum_acc(h[2], l[2], q.zp.x), l[2] += q.zp.y;
@@ -112,22 +112,22 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
     add_groups(red.f, g, b, h, l);
     if (g == 0) {
       sx = (double)h[0] + (double)l[0], sy = (double)h[1] + (double)l[1];
-      sz = (double)h[2] + (double)l[2], sp = (double)h[3] + (double)l[3];
+      sz = (double)h[2] + (double)l[2], sphi = (double)h[3] + (double)l[3];
     }
   } else if (mode & kCombine) {
-    const double4_32a* part = reinterpret_cast<const double4_32a*>(P.part) + i;
+    const double4_32a* part = reinterpret_cast<const double4_32a*>(P.part) + (c.row0 + i);
     double s4[4] = {0.0, 0.0, 0.0, 0.0};
     if (live) {
 #pragma unroll 8
       for (int s = g; s < c.n_slices; s += kSlotGroups) {
-        const double4_32a q = part[(int64_t)s * P.n_total];
+        const double4_32a q = part[(int64_t)s * c.stride];
         s4[0] += q.x, s4[1] += q.y, s4[2] += q.z, s4[3] += q.w;
       }
     }
     add_groups(red.d, g, b, s4);
-    sx = s4[0], sy = s4[1], sz = s4[2], sp = s4[3];
+    sx = s4[0], sy = s4[1], sz = s4[2], sphi = s4[3];
   }
-  if (g == 0 && live && post_body(P, mode, i, cen, sx, sy, sz, sp, e)) atomicOr(P.status, kFlagNonFinite);
+  if (g == 0 && live && post_body(P, mode, i, sp, sx, sy, sz, sphi, e)) atomicOr(P.status, kFlagNonFinite);
   if (mode & kVirial) {
     double kw[2] = {e[0], e[1]};
     if (g == 0) block_sum<2, CB, true>(kw);
@@ -163,32 +163,73 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
   }
 }
 
-// Staging origin: per chunk, sum m x (3), sum m, sum x (3) into cpart[chunk][8];
-// the last CTA then forms, per system in a fixed order, the mass-weighted mean
-// position (plain mean if the mass is not positive; 0 for an empty system).
+// Largest coordinate and mass of a chunk by their float64 high words (sign bit
+// off: the words order as the magnitudes) and whether its masses all equal its
+// system's first, as one 64-bit value that is carried beside the chunk's sums.
+struct Extent {
+  unsigned x, m, uniform;
+  __device__ __forceinline__ void join(const Extent& o) {
+    x = max(x, o.x), m = max(m, o.m), uniform &= o.uniform;
+  }
+  __device__ __forceinline__ void warp_join() {
+    x = __reduce_max_sync(0xffffffffu, x);
+    m = __reduce_max_sync(0xffffffffu, m);
+    uniform = __reduce_and_sync(0xffffffffu, uniform);
+  }
+  __device__ __forceinline__ double pack() const {
+    return __hiloint2double((int)x, (int)(m << 1 | uniform));
+  }
+  __device__ __forceinline__ static Extent unpack(const double d) {
+    const unsigned l = (unsigned)__double2loint(d);
+    return Extent{(unsigned)__double2hiint(d), l >> 1, l & 1u};
+  }
+};
+
+__device__ __forceinline__ unsigned high_word(const double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+
+// 2^(to - e) for the float64 with high word h of binary exponent e (1 where h is 0, tiny, infinite or NaN)
+__device__ __forceinline__ double power_of_two_scale(const unsigned h, const int to) {
+  const int e = (int)(h >> 20) - 1023;
+  return e < -900 || e > 900 ? 1.0 : ldexp(1.0, to - e);
+}
+
+// The staged coordinates of gravity stay below 2^12: with distances down to 2^-25
+// of that, s^-5 (the force gradient) stays in the float32 range at both ends.
+constexpr int kExtentExp = 10;
+
 template <int CB>
-__global__ void __launch_bounds__(CB) k_centre(const Chunk* chunks, const int32_t* sys_chunk,
-                                                         const int64_t* off, const int n_sys, const double* x,
-                                                         const double* m, double* cpart, double* centre,
-                                                         unsigned* done, const int64_t n_total, unsigned* status) {
-  Chunk c = chunks[blockIdx.x];
-  if (!chunk_ok(c, n_total, n_sys, 0, status)) c.begin = c.end = 0;  // NBODY_DEBUG builds only
+__global__ void __launch_bounds__(CB) k_centre(const CentreLaunch C) {
+  constexpr int NW = CB / 32;
+  __shared__ Extent ext[NW];
+  const int lane = (int)threadIdx.x & 31, wid = (int)threadIdx.x >> 5;
+  Chunk c = C.chunks[blockIdx.x];
+  if (!chunk_ok(c, C.n_total, C.n_sys, 0, C.status)) c.begin = c.end = 0;  // NBODY_DEBUG builds only
   double v[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  for (int i = c.begin + (int)threadIdx.x; i < c.end; i += CB) {
-    const double mi = m[i];
-    const double x0 = x[3 * i + 0], x1 = x[3 * i + 1], x2 = x[3 * i + 2];
-    v[0] += mi * x0, v[1] += mi * x1, v[2] += mi * x2, v[3] += mi;
-    v[4] += x0, v[5] += x1, v[6] += x2;
+  Extent q{0u, 0u, 1u};
+  const int i = c.begin + (int)threadIdx.x;
+  if (i < c.end) {
+    const double mi = C.m[i], m0 = C.m[C.off[c.sys]];
+    const double x0 = C.x[3 * i + 0], x1 = C.x[3 * i + 1], x2 = C.x[3 * i + 2];
+    v[0] = mi * x0, v[1] = mi * x1, v[2] = mi * x2, v[3] = mi;
+    v[4] = x0, v[5] = x1, v[6] = x2;
+    q.x = max(max(high_word(x0), high_word(x1)), high_word(x2));
+    q.m = high_word(mi);
+    q.uniform = __double_as_longlong(mi) == __double_as_longlong(m0) ? 1u : 0u;
   }
-  block_sum<7, CB>(v);
+  q.warp_join();
+  if (lane == 0) ext[wid] = q;
+  block_sum<7, CB>(v);  // its barriers also publish ext
   if (threadIdx.x == 0) {
+    for (int w = 1; w < NW; ++w) q.join(ext[w]);
+    double* o = C.cpart + (int64_t)blockIdx.x * kEnergyVals;
 #pragma unroll
-    for (int k = 0; k < 7; ++k) cpart[(int64_t)blockIdx.x * kEnergyVals + k] = v[k];
+    for (int k = 0; k < 7; ++k) o[k] = v[k];
+    o[7] = q.pack();
   }
-  if (!last_of(done, gridDim.x)) return;
+  if (!last_of(C.done, gridDim.x)) return;
   __threadfence();
-  systems_final<7, CB>(sys_chunk, n_sys, cpart, gridDim.x, status, [&](int sy, const double (&w)[7]) {
-    const int64_t n = off[sy + 1] - off[sy];
+  auto emit = [&](const int sy, const double (&w)[7], const Extent& e) {
+    const int64_t n = C.off[sy + 1] - C.off[sy];
     double c0 = 0.0, c1 = 0.0, c2 = 0.0;
     if (w[3] > 0.0 && isfinite(w[3])) {
       c0 = w[0] / w[3], c1 = w[1] / w[3], c2 = w[2] / w[3];
@@ -196,8 +237,52 @@ __global__ void __launch_bounds__(CB) k_centre(const Chunk* chunks, const int32_
       c0 = w[4] / (double)n, c1 = w[5] / (double)n, c2 = w[6] / (double)n;
     }
     if (!(isfinite(c0) && isfinite(c1) && isfinite(c2))) c0 = c1 = c2 = 0.0;
-    centre[3 * sy + 0] = c0, centre[3 * sy + 1] = c1, centre[3 * sy + 2] = c2;
-  });
+    SysParam& o = C.sys[sy];
+    o.c[0] = c0, o.c[1] = c1, o.c[2] = c2;
+    if (C.law != 0 || n <= 0) return;
+    // the softening counts as an extent, so that its staged square stays finite
+    const double s = power_of_two_scale(max(e.x, high_word(C.eps)), kExtentExp);
+    const double m0 = C.m[C.off[sy]], e2 = C.eps * s, rc = C.near_eps * e2;
+    const unsigned h0 = high_word(m0);
+    const bool uniform = e.uniform && m0 > 0.0 && h0 >= (123u << 20) && h0 <= (1923u << 20);
+    const double ms = power_of_two_scale(e.m, 0);
+    o.scale = s;
+    o.mscale = uniform ? 1.0 / m0 : ms;
+    o.inv_mscale = uniform ? m0 : 1.0 / ms;
+    o.eps2 = (float)(e2 * e2), o.r2c = (float)(rc * rc);
+    o.uniform = uniform ? 1u : 0u;
+  };
+  auto extent = [&](const int sy, const int first, const int step) {
+    Extent e{0u, 0u, 1u};
+    for (int k = C.sys_chunk[sy] + first; k < C.sys_chunk[sy + 1]; k += step)
+      e.join(Extent::unpack(__ldcg(C.cpart + (int64_t)k * kEnergyVals + 7)));
+    e.warp_join();
+    return e;
+  };
+  // up to four systems are reduced by the whole CTA, more by a warp each (as systems_final)
+  if (C.n_sys <= 4) {
+    for (int sy = 0; sy < C.n_sys; ++sy) {
+      Extent e = extent(sy, (int)threadIdx.x, CB);
+      __syncthreads();
+      if (lane == 0) ext[wid] = e;
+      __syncthreads();
+      for (int w = 0; w < NW; ++w) e.join(ext[w]);
+      systems_final<7, CB>(C.sys_chunk + sy, 1, C.cpart, gridDim.x, C.status,
+                           [&](int, const double (&w)[7]) { emit(sy, w, e); });
+    }
+    return;
+  }
+  for (int sy = wid; sy < C.n_sys; sy += NW) {
+    double w[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int k = C.sys_chunk[sy] + lane; k < C.sys_chunk[sy + 1]; k += 32) {
+#pragma unroll
+      for (int q = 0; q < 7; ++q) w[q] += __ldcg(C.cpart + (int64_t)k * kEnergyVals + q);
+    }
+#pragma unroll
+    for (int q = 0; q < 7; ++q) w[q] = warp_sum(w[q]);
+    const Extent e = extent(sy, lane, 32);
+    if (lane == 0) emit(sy, w, e);
+  }
 }
 
 template <int CB>
@@ -207,8 +292,8 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_adj_update(const AdjLaunch
     double d[10][kSlotGroups - 1][CB];
   } red;
   Chunk c = A.chunks[blockIdx.x];
-  if (!chunk_ok(c, A.n_total, A.n_sys, A.part_slices, A.status)) c.begin = c.end = 0;  // NBODY_DEBUG builds only
-  const double* cen = A.centre + 3 * c.sys;
+  if (!chunk_ok(c, A.n_total, A.n_sys, A.part_rows, A.status)) c.begin = c.end = 0;  // NBODY_DEBUG builds only
+  const SysParam& sp = A.sys[c.sys];
   const int kw = A.g_params ? 3 : 2;  // partials (fpair4 / double4_32a) per body and slice
   double pv[2] = {0.0, 0.0};          // this thread's w.da/dG and sum m (d.w) / s^5
   const int b = (int)threadIdx.x % CB, g = (int)threadIdx.x / CB;
@@ -228,7 +313,7 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_adj_update(const AdjLaunch
     if (live) {
 #pragma unroll 4
       for (int s = g; s < c.n_slices; s += kSlotGroups) {
-        const int64_t k = kw * ((int64_t)s * A.n_total + i);
+        const int64_t k = kw * (c.row0 + (int64_t)s * c.stride + i);
         const fpair4 p = fp[k], q = fp[k + 1];
         add(0, p.xy.x, p.xy.y), add(1, p.xy.z, p.xy.w), add(2, p.zp.x, p.zp.y), add(3, p.zp.z, p.zp.w);
         add(4, q.xy.x, q.xy.y), add(5, q.xy.z, q.xy.w), add(6, q.zp.x, q.zp.y), add(7, q.zp.z, q.zp.w);
@@ -248,7 +333,7 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_adj_update(const AdjLaunch
     if (live) {
 #pragma unroll 4
       for (int s = g; s < c.n_slices; s += kSlotGroups) {
-        const int64_t k = kw * ((int64_t)s * A.n_total + i);
+        const int64_t k = kw * (c.row0 + (int64_t)s * c.stride + i);
         const double4_32a p = part[k], q = part[k + 1];
         S[0] += p.x, S[1] += p.y, S[2] += p.z, S[3] += p.w;
         S[4] += q.x, S[5] += q.y, S[6] += q.z, S[7] += q.w;
@@ -261,8 +346,11 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_adj_update(const AdjLaunch
     add_groups(red.d, g, b, S);
   }
   if (g == 0 && live) {
-    const double a1x = S[0], a1y = S[1], a1z = S[2], a2 = S[3], gbx = S[4], gby = S[5], gbz = S[6], gm = S[7];
-    if (A.g_params) pv[0] = S[8], pv[1] = S[9];
+    // the staged sums carry powers of the staging scales
+    const double q = sp.scale, q2 = q * q, q3 = q2 * q, q3m = q3 * sp.inv_mscale;
+    const double a1x = q3 * S[0], a1y = q3 * S[1], a1z = q3 * S[2], a2 = q3m * S[3];
+    const double gbx = q3m * S[4], gby = q3m * S[5], gbz = q3m * S[6], gm = q2 * S[7];
+    if (A.g_params) pv[0] = q2 * sp.inv_mscale * S[8], pv[1] = q2 * q2 * sp.inv_mscale * S[9];
     const double mi = A.m[i];
     double w0 = A.lam_v[3 * i + 0], w1 = A.lam_v[3 * i + 1], w2 = A.lam_v[3 * i + 2];
     const double gx0 = A.G * (mi * a1x - a2 * w0 - 3.0 * gbx);
@@ -285,7 +373,7 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_adj_update(const AdjLaunch
     }
     if (A.x_next)
       stage_store(A.precision, A.stage_x, i, A.x_next[3 * i + 0], A.x_next[3 * i + 1], A.x_next[3 * i + 2], mi,
-                  cen, A.stage_lo);
+                  sp, A.stage_lo);
   }
   if (!A.g_params) return;
   // dL/dG += coef sum_k w_k . da_k/dG; dL/deps += coef (-3 G eps) sum_k sum_j m_j (d.w_k) / s^5,
@@ -305,16 +393,16 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_adj_update(const AdjLaunch
 
 template <int CB>
 __global__ void __launch_bounds__(CB) k_stage_vec(const Chunk* chunks, int precision, const double* vec,
-                                                            const double* m, const double* centre, void* stage,
+                                                  const double* m, const SysParam* sys, void* stage,
                                                             void* stage_lo, int as_position, const int64_t n_total,
                                                             const int n_sys, unsigned* status) {
   Chunk c = chunks[blockIdx.x];
   if (!chunk_ok(c, n_total, n_sys, 0, status)) c.begin = c.end = 0;  // NBODY_DEBUG builds only
-  const double* cen = centre + 3 * c.sys;
+  const SysParam& sp = sys[c.sys];
   for (int i = c.begin + (int)threadIdx.x; i < c.end; i += CB) {
     const double v0 = vec[3 * i + 0], v1 = vec[3 * i + 1], v2 = vec[3 * i + 2];
     if (as_position) {
-      stage_store(precision, stage, i, v0, v1, v2, m[i], cen, stage_lo);
+      stage_store(precision, stage, i, v0, v1, v2, m[i], sp, stage_lo);
     } else if (precision == 1) {
       static_cast<float4*>(stage)[i] = make_float4((float)v0, (float)v1, (float)v2, 0.f);
     } else {
@@ -365,13 +453,11 @@ cudaError_t launch_post(const PostLaunch& P, cudaStream_t st) {
   });
 }
 
-cudaError_t launch_centre(const Chunk* chunks, int n_chunks, const int32_t* sys_chunk, const int64_t* off, int n_sys,
-                          const double* x, const double* m, double* cpart, double* centre, unsigned* done,
-                          int64_t n_total, unsigned* status, cudaStream_t st) {
-  if (n_sys <= 0 || n_chunks <= 0) return cudaSuccess;
-  return with_chunk(n_total, [&](auto cb) {
+cudaError_t launch_centre(const CentreLaunch& C, cudaStream_t st) {
+  if (C.n_sys <= 0 || C.n_chunks <= 0) return cudaSuccess;
+  return with_chunk(C.n_total, [&](auto cb) {
     constexpr int CB = decltype(cb)::value;
-    k_centre<CB><<<n_chunks, CB, 0, st>>>(chunks, sys_chunk, off, n_sys, x, m, cpart, centre, done, n_total, status);
+    k_centre<CB><<<C.n_chunks, CB, 0, st>>>(C);
     return cudaGetLastError();
   });
 }
@@ -386,12 +472,12 @@ cudaError_t launch_adj_update(const AdjLaunch& A, cudaStream_t st) {
 }
 
 cudaError_t launch_stage_vec(const Chunk* chunks, int n_chunks, int precision, const double* vec, const double* m,
-                             const double* centre, void* stage, void* stage_lo, int as_position, int64_t n_total,
+                             const SysParam* sys, void* stage, void* stage_lo, int as_position, int64_t n_total,
                              int n_sys, unsigned* status, cudaStream_t st) {
   if (n_chunks <= 0) return cudaSuccess;
   return with_chunk(n_total, [&](auto cb) {
     constexpr int CB = decltype(cb)::value;
-    k_stage_vec<CB><<<n_chunks, CB, 0, st>>>(chunks, precision, vec, m, centre, stage, stage_lo, as_position, n_total,
+    k_stage_vec<CB><<<n_chunks, CB, 0, st>>>(chunks, precision, vec, m, sys, stage, stage_lo, as_position, n_total,
                                              n_sys, status);
     return cudaGetLastError();
   });

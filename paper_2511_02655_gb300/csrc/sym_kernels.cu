@@ -1,0 +1,74 @@
+// Launchers of the symmetric force pass (sym_common.cuh).
+#include <algorithm>
+
+#include "nbody_internal.h"
+#include "sym_common.cuh"
+
+namespace nbody {
+namespace {
+
+// MINB resident CTAs per SM: 16 warps per SM at R = 4 (<= 128 registers), 24 at R = 2
+// (<= 80 registers).
+template <int LAW, int W, int R, bool PHI, int MINB>
+__global__ void __launch_bounds__(W * 32, MINB) k_force_sym(const SymLaunch L) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  auto& sm = *reinterpret_cast<sym::Smem<W, R, kSymTile>*>(raw);
+  pdl_wait();
+  sym::items<LAW, W, R, kSymTile, PHI>(L, L.counter, sm);
+  pdl_trigger();
+  retire_cta(L.counter);
+}
+
+// More than 48 KB of shared memory per CTA has to be asked for, once per kernel and device.
+template <typename K>
+cudaError_t allow_smem(K kern, size_t bytes) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+template <typename K>
+int occupancy_of(K kern, int block, size_t smem) {
+  int n = 0;
+  if (allow_smem(kern, smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, block, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+}  // namespace
+
+// Compiled: warps, i-bodies per lane (and resident CTAs).
+#define NBODY_SYM_TILINGS(X) X(4, 2, 6) X(4, 4, 4) X(8, 2, 3) X(8, 4, 2)
+
+cudaError_t launch_sym_force(const SymLaunch& L, cudaStream_t st) {
+  if (L.n_ctas <= 0) return cudaErrorInvalidConfiguration;
+#define NBODY_X(W, R, MINB)                                                                              \
+  if (L.block == W * 32 && L.ipt == R) {                                                                 \
+    constexpr size_t smem = sizeof(sym::Smem<W, R, kSymTile>);                                           \
+    if (L.law == 0)                                                                                      \
+      return L.phi ? launch_pdl_smem(k_force_sym<0, W, R, true, MINB>, L.n_ctas, W * 32, smem, st, L)    \
+                   : launch_pdl_smem(k_force_sym<0, W, R, false, MINB>, L.n_ctas, W * 32, smem, st, L);  \
+    return L.phi ? launch_pdl_smem(k_force_sym<1, W, R, true, MINB>, L.n_ctas, W * 32, smem, st, L)      \
+                 : launch_pdl_smem(k_force_sym<1, W, R, false, MINB>, L.n_ctas, W * 32, smem, st, L);    \
+  }
+  NBODY_SYM_TILINGS(NBODY_X)
+#undef NBODY_X
+  return cudaErrorInvalidConfiguration;
+}
+
+int sym_force_ctas_per_sm(int block, int ipt, int law) {
+#define NBODY_X(W, R, MINB)                                                                              \
+  if (block == W * 32 && ipt == R) {                                                                     \
+    constexpr size_t smem = sizeof(sym::Smem<W, R, kSymTile>);                                           \
+    return law == 0 ? std::min(occupancy_of(k_force_sym<0, W, R, true, MINB>, W * 32, smem),             \
+                               occupancy_of(k_force_sym<0, W, R, false, MINB>, W * 32, smem))            \
+                    : std::min(occupancy_of(k_force_sym<1, W, R, true, MINB>, W * 32, smem),             \
+                               occupancy_of(k_force_sym<1, W, R, false, MINB>, W * 32, smem));           \
+  }
+  NBODY_SYM_TILINGS(NBODY_X)
+#undef NBODY_X
+  return 0;
+}
+
+}  // namespace nbody

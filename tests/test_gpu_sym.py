@@ -1,0 +1,129 @@
+"""The symmetric all-pairs passes (every unordered pair once) at the edges of their tiles.
+
+They are chosen by the tuner only, so the tiling under test is put into the tuning cache
+(NBODY_TUNE_CACHE) under the key that a first context of the same setup writes."""
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2511_02655_gb300 import inputs
+from helpers import assert_elem_close, force_rel_err, to_dev
+
+pytestmark = pytest.mark.gpu
+
+MIX_MED, MIX_MAX, MIX_PHI_MAX = 1e-6, 1e-4, 3e-5  # the mixed path's bounds (test_gpu_parity.py)
+
+
+def _forced(nb, path, tilings, use=None, **kw):
+    """A context whose tilings ({"force" | "vjp": cache line}) come from the tuning cache."""
+    if path.exists():
+        path.unlink()
+    ctx = nb.nbody_init(**kw)
+    if use:
+        use(ctx)  # first use of a kernel that is tuned late
+    ctx.close()
+    lines = []
+    for line in path.read_text().splitlines():
+        key = line.split("\t")[0]
+        for kind, t in tilings.items():
+            if f"|{kind}|" in key:
+                lines.append(key + "\t" + " ".join(str(v) for v in t))
+    path.write_text("\n".join(lines) + "\n")
+    return nb.nbody_init(**kw)
+
+
+def _masses(m, kind, seed):
+    return m if kind == "equal" else m * np.exp(0.4 * np.random.default_rng(seed).standard_normal(len(m)))
+
+
+# block, i-bodies per lane, j-tile, slice, variant, tail: i-tiles of 256, 512, 512 and 1024 bodies
+TILINGS = [(128, 2, 256, 64, 3, 0), (128, 4, 256, 192, 3, 1), (256, 2, 256, 320, 3, 0), (256, 4, 256, 64, 3, 1)]
+
+
+@pytest.mark.parametrize("tiling", TILINGS)
+@pytest.mark.parametrize("n", [1, 2, 63, 65, 257, 1025, 4999])
+@pytest.mark.parametrize("masses", ["equal", "lognormal"])
+def test_sym_forces(nb, tmp_path, monkeypatch, tiling, n, masses):
+    import torch
+    monkeypatch.setenv("NBODY_TUNE_CACHE", str(tmp_path / "tune"))
+    G, eps = 1.2, 0.05  # 4 eps = 0.2: near pairs in most tiles
+    x, v, m = inputs.plummer(n, seed=n)
+    m = _masses(m, masses, n)
+    ctx = _forced(nb, tmp_path / "tune", {"force": tiling}, G=G, eps=eps, dt=1e-3, n=n)
+    assert nb.nbody_get_tuning(ctx)["variant"] == 4
+    xt, mt = to_dev(x, m)
+    a, phi = nb.nbody_forces(ctx, xt, mt)
+    a0, _ = nb.nbody_forces(ctx, xt, mt, with_phi=False)
+    nb.nbody_sync(ctx)
+    assert torch.equal(a, a0)
+    if n == 1:
+        assert not a.any() and not phi.any()
+        return
+    a_ref, phi_ref = oracle.forces(x, m, G=G, eps=eps)
+    e = force_rel_err(a.cpu().numpy(), a_ref)
+    assert np.median(e) <= MIX_MED and e.max() <= MIX_MAX, (np.median(e), e.max())
+    assert_elem_close(phi.cpu().numpy(), phi_ref, MIX_PHI_MAX, "phi")
+
+
+@pytest.mark.parametrize("tiling", TILINGS)
+def test_sym_lennard_jones(nb, tmp_path, monkeypatch, tiling):
+    monkeypatch.setenv("NBODY_TUNE_CACHE", str(tmp_path / "tune"))
+    x, v, m, box = inputs.lj_gas(2050, seed=7, density=0.3)
+    m = _masses(m, "lognormal", 3)
+    ctx = _forced(nb, tmp_path / "tune", {"force": tiling}, law=nb.LENNARD_JONES, dt=1e-3, n=2050, lj_epsilon=1.3,
+                  lj_sigma=0.9)
+    assert nb.nbody_get_tuning(ctx)["variant"] == 4
+    a, phi = nb.nbody_forces(ctx, *to_dev(x, m))
+    nb.nbody_sync(ctx)
+    a_ref, phi_ref = oracle.lj_forces(x, m, eps_lj=1.3, sigma=0.9)
+    e = force_rel_err(a.cpu().numpy(), a_ref)
+    assert np.median(e) <= MIX_MED and e.max() <= MIX_MAX, (np.median(e), e.max())
+    assert_elem_close(phi.cpu().numpy(), phi_ref, MIX_MAX, "phi")
+
+
+@pytest.mark.parametrize("length,mass", [(1e12, 1e30), (1e-9, 1e-27), (1.0, 1.0)])
+def test_mixed_forces_in_any_units(nb, length, mass):
+    """Staging scales positions and masses by powers of two, so the float32 arithmetic stays in
+    range in any units (metres and kilograms of a planetary system included)."""
+    n = 3000
+    x, v, m = inputs.plummer(n, seed=5)
+    m = _masses(m, "lognormal", 5)
+    for variant in (0, 1, 2):
+        ctx = nb.nbody_init(G=1.0, eps=0.02 * length, dt=1e-3, n=n, variant=variant)
+        a, phi = nb.nbody_forces(ctx, *to_dev(x * length, m * mass))
+        nb.nbody_sync(ctx)
+        a_ref, phi_ref = oracle.forces(x, m, G=1.0, eps=0.02)
+        e = force_rel_err(a.cpu().numpy() * (length / mass * length), a_ref)
+        assert np.median(e) <= MIX_MED and e.max() <= MIX_MAX, (variant, np.median(e), e.max())
+        assert_elem_close(phi.cpu().numpy() * (length / mass), phi_ref, MIX_PHI_MAX, "phi")
+        ctx.close()
+
+
+def test_sym_several_systems_and_zero_masses(nb, tmp_path, monkeypatch):
+    """Systems of every kind in one list: empty, single, equal masses, unequal ones, massless bodies
+    (they feel forces and exert none), one far from the origin."""
+    import torch
+    monkeypatch.setenv("NBODY_TUNE_CACHE", str(tmp_path / "tune"))
+    sizes = [0, 1, 300, 1100, 2, 700, 0, 513]
+    ens = inputs.ensemble(len(sizes), seed=3, sizes=np.array(sizes))
+    off = [int(o) for o in ens.offsets]
+    x, m = ens.x.copy(), ens.m.copy()
+    m[off[3]:off[4]:2] = 0.0
+    m[off[5]:off[6]] *= np.exp(np.random.default_rng(1).standard_normal(700))
+    x[off[7]:off[8]] += 50.0
+    ctx = _forced(nb, tmp_path / "tune", {"force": (128, 2, 256, 128, 3, 1)}, G=1.0, eps=0.02, dt=1e-3, offsets=off)
+    assert nb.nbody_get_tuning(ctx)["variant"] == 4
+    xt, mt = to_dev(x, m)
+    a, phi = nb.nbody_forces(ctx, xt, mt)
+    a2, phi2 = nb.nbody_forces(ctx, xt, mt)
+    nb.nbody_sync(ctx)
+    assert torch.equal(a, a2) and torch.equal(phi, phi2)
+    for s, k in enumerate(sizes):
+        b, e = off[s], off[s + 1]
+        if k < 2:
+            assert not a[b:e].any()
+            continue
+        a_ref, phi_ref = oracle.forces(x[b:e], m[b:e], G=1.0, eps=0.02)
+        assert force_rel_err(a[b:e].cpu().numpy(), a_ref).max() <= MIX_MAX, s
+        assert_elem_close(phi[b:e].cpu().numpy(), phi_ref, MIX_PHI_MAX, f"phi {s}")
