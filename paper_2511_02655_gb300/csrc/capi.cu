@@ -44,6 +44,7 @@ struct Tiling {
 constexpr int kSymVariant = 3;
 constexpr double kSymMinBodies = 1024.0;    // typical system size from which the symmetric pass is a candidate
 constexpr double kSymOnlyBodies = 32768.0;  // ... and from which it is the only one (mixed path)
+constexpr double kSymMinBodies64 = 64.0, kSymOnlyBodies64 = 512.0;  // FP64 path
 constexpr int64_t kMaxSymRows = 64;                      // rows of i-tiles a system is cut into at most
 constexpr size_t kMaxSymPartialBytes = size_t(4) << 30;  // cap on the symmetric pass's partial sums
 
@@ -268,11 +269,13 @@ nbody_status check_dev(nbody_ctx* c, const void* p, size_t bytes, const char* na
 // ---------------------------------------------------------------------------
 // work lists
 
-constexpr int kSymBlock = 64;  // j-bodies that a warp of the symmetric pass meets in one block: pieces are whole blocks
+int sym_tile(int prec) { return prec == NBODY_MIXED ? kSymTile : kSymTile64; }
+// j-bodies that a warp of the symmetric pass meets in one block: pieces are whole blocks
+int sym_block(int prec) { return prec == NBODY_MIXED ? 64 : 32; }
 
 int ctas_per_sm(int prec, const Tiling& t, bool vjp, int law) {
   if (t.variant == kSymVariant)
-    return !vjp && prec == NBODY_MIXED && t.jtile == kSymTile ? sym_force_ctas_per_sm(t.block, t.ipt, law) : 0;
+    return !vjp && t.jtile == sym_tile(prec) ? sym_force_ctas_per_sm(prec, t.block, t.ipt, law) : 0;
   return vjp ? vjp_ctas_per_sm(prec, t.variant, t.block, t.ipt, t.jtile)
              : force_ctas_per_sm(prec, t.variant, t.block, t.ipt, t.jtile, law);
 }
@@ -293,7 +296,7 @@ double total_pairs(const nbody_ctx* c) {
 constexpr int kSymPieces = 6;
 int sym_slice(const nbody_ctx* c, const Tiling& t, int n_ctas, int pieces) {
   const double len = total_pairs(c) / ((double)n_ctas * pieces * t.block * t.ipt);
-  const double q = kSymBlock;
+  const double q = sym_block(c->cfg.precision);
   return (int)std::min(1.0e9, std::max(q, q * std::floor(len / q + 0.5)));
 }
 
@@ -443,7 +446,7 @@ void build_sym_items(const nbody_ctx* c, const Tiling& t, std::vector<SymItem>& 
   max_slots = 1;
   rows = 0;
   const int64_t itile = (int64_t)t.block * t.ipt;
-  const int64_t q = kSymBlock;
+  const int64_t q = sym_block(c->cfg.precision);
   const double area = (double)t.slice * (double)itile;
   std::vector<int> slots;
   for (int s = 0; s < c->n_sys; ++s) {
@@ -458,7 +461,7 @@ void build_sym_items(const nbody_ctx* c, const Tiling& t, std::vector<SymItem>& 
       const double pairs = (double)ni * ((double)len - 0.5 * (double)ni);
       const double want = t.tail && (r & 1) ? area / 3.0 : area;
       int64_t p = std::max<int64_t>(1, (int64_t)(pairs / want + 0.5));
-      const int64_t step = (((len + p - 1) / p + q - 1) / q) * q;
+      const int64_t step = std::max<int64_t>(1, (len + p * q / 2) / (p * q)) * q;  // whole blocks
       p = (len + step - 1) / step;
       slots[(size_t)r] = (int)(r + 1 + p);
       most = std::max(most, slots[(size_t)r]);
@@ -590,7 +593,7 @@ PairLaunch pair_launch(nbody_ctx* c, bool vjp, bool refine = true, bool phi = tr
 
 // The all-pairs kernel of the installed tiling.
 cudaError_t launch_pairs(nbody_ctx* c, bool vjp, bool phi, cudaStream_t st) {
-  if (!vjp && is_sym(c->ft)) return launch_sym_force(sym_launch(c, phi), st);
+  if (!vjp && is_sym(c->ft)) return launch_sym_force(c->cfg.precision, sym_launch(c, phi), st);
   const PairLaunch L = pair_launch(c, vjp, true, phi);
   return vjp ? launch_vjp(c->cfg.precision, L, st) : launch_force(c->cfg.precision, L, st);
 }
@@ -982,21 +985,25 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
   const double typical = pairs > 0 ? cubes / pairs : 0.0;
   const bool any_tiling = !g.variant && !g.block && !g.i_per_thread && !g.j_tile && !g.slice;
   const bool mixed = g.precision == NBODY_MIXED;
-  const bool sym = !vjp && mixed && any_tiling && typical >= kSymMinBodies;
-  const bool sym_only = sym && typical >= kSymOnlyBodies;
+  const bool sym = !vjp && any_tiling && typical >= (mixed ? kSymMinBodies : kSymMinBodies64);
+  const bool sym_only = sym && typical >= (mixed ? kSymOnlyBodies : kSymOnlyBodies64);
   if (sym_only && large) {
     // nothing to choose between: its cost per pair no longer depends on the tiling
     Tiling t;
-    t.block = 256, t.ipt = 4, t.jtile = kSymTile, t.variant = kSymVariant, t.tail = 1;
+    t.block = mixed ? 256 : 128, t.ipt = mixed ? 4 : 1, t.jtile = sym_tile(g.precision), t.variant = kSymVariant;
+    t.tail = 1;
     if (install_tiling(c, t, false) == NBODY_OK) {
       tune_cache_store(c, vjp, c->ft);
       return NBODY_OK;
     }
   }
   if (sym && !large) {
-    for (const auto& p : std::vector<std::pair<int, int>>{{128, 2}, {128, 4}, {256, 2}, {256, 4}}) {
+    const std::vector<std::pair<int, int>> br =
+        mixed ? std::vector<std::pair<int, int>>{{128, 2}, {128, 4}, {256, 2}, {256, 4}}
+              : std::vector<std::pair<int, int>>{{64, 1}, {128, 1}, {256, 1}, {128, 2}};
+    for (const auto& p : br) {
       Tiling t;
-      t.block = p.first, t.ipt = p.second, t.jtile = kSymTile, t.variant = kSymVariant;
+      t.block = p.first, t.ipt = p.second, t.jtile = sym_tile(g.precision), t.variant = kSymVariant;
       cands.push_back(t);
     }
     if (sym_only) variants.clear();

@@ -233,11 +233,12 @@ cudaError_t launch_vjp(int precision, const PairLaunch& L, cudaStream_t st);
 int force_ctas_per_sm(int precision, int variant, int block, int ipt, int jtile, int law);
 int vjp_ctas_per_sm(int precision, int variant, int block, int ipt, int jtile);
 
-// Symmetric force pass (mixed): threads per CTA (block) and i-bodies per lane (ipt) select the
+// Symmetric force pass: threads per CTA (block) and i-bodies per lane (ipt) select the
 // compiled kernel; cudaErrorInvalidConfiguration / 0 if there is none.
-cudaError_t launch_sym_force(const SymLaunch& L, cudaStream_t st);
-int sym_force_ctas_per_sm(int block, int ipt, int law);
-constexpr int kSymTile = 256;  // j-bodies per shared-memory tile of the symmetric kernels
+cudaError_t launch_sym_force(int precision, const SymLaunch& L, cudaStream_t st);
+int sym_force_ctas_per_sm(int precision, int block, int ipt, int law);
+constexpr int kSymTile = 256;   // j-bodies per shared-memory tile of the symmetric kernels, mixed
+constexpr int kSymTile64 = 64;  // ... and FP64
 
 // ---------------------------------------------------------------------------
 // O(N) kernels (post_kernels.cu)

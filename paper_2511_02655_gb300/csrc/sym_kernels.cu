@@ -2,6 +2,7 @@
 #include <algorithm>
 
 #include "nbody_internal.h"
+#include "sym64.cuh"
 #include "sym_common.cuh"
 
 namespace nbody {
@@ -15,6 +16,15 @@ __global__ void __launch_bounds__(W * 32, MINB) k_force_sym(const SymLaunch L) {
   auto& sm = *reinterpret_cast<sym::Smem<W, R, kSymTile>*>(raw);
   pdl_wait();
   sym::items<LAW, W, R, kSymTile, PHI>(L, L.counter, sm);
+  pdl_trigger();
+  retire_cta(L.counter);
+}
+
+template <int LAW, int W, int R, bool PHI>
+__global__ void __launch_bounds__(W * 32) k_force_sym64(const SymLaunch L) {
+  __shared__ sym64::Smem<W> sm;
+  pdl_wait();
+  sym64::items<LAW, W, R, PHI>(L, L.counter, sm);
   pdl_trigger();
   retire_cta(L.counter);
 }
@@ -40,9 +50,23 @@ int occupancy_of(K kern, int block, size_t smem) {
 
 // Compiled: warps, i-bodies per lane (and resident CTAs).
 #define NBODY_SYM_TILINGS(X) X(4, 2, 6) X(4, 4, 4) X(8, 2, 3) X(8, 4, 2)
+#define NBODY_SYM64_TILINGS(X) X(2, 1) X(4, 1) X(8, 1) X(4, 2)
 
-cudaError_t launch_sym_force(const SymLaunch& L, cudaStream_t st) {
+cudaError_t launch_sym_force(int precision, const SymLaunch& L, cudaStream_t st) {
   if (L.n_ctas <= 0) return cudaErrorInvalidConfiguration;
+  if (precision == 0) {
+#define NBODY_X(W, R)                                                                       \
+  if (L.block == W * 32 && L.ipt == R) {                                                    \
+    if (L.law == 0)                                                                         \
+      return L.phi ? launch_pdl(k_force_sym64<0, W, R, true>, L.n_ctas, W * 32, st, L)      \
+                   : launch_pdl(k_force_sym64<0, W, R, false>, L.n_ctas, W * 32, st, L);    \
+    return L.phi ? launch_pdl(k_force_sym64<1, W, R, true>, L.n_ctas, W * 32, st, L)        \
+                 : launch_pdl(k_force_sym64<1, W, R, false>, L.n_ctas, W * 32, st, L);      \
+  }
+    NBODY_SYM64_TILINGS(NBODY_X)
+#undef NBODY_X
+    return cudaErrorInvalidConfiguration;
+  }
 #define NBODY_X(W, R, MINB)                                                                              \
   if (L.block == W * 32 && L.ipt == R) {                                                                 \
     constexpr size_t smem = sizeof(sym::Smem<W, R, kSymTile>);                                           \
@@ -57,7 +81,17 @@ cudaError_t launch_sym_force(const SymLaunch& L, cudaStream_t st) {
   return cudaErrorInvalidConfiguration;
 }
 
-int sym_force_ctas_per_sm(int block, int ipt, int law) {
+int sym_force_ctas_per_sm(int precision, int block, int ipt, int law) {
+  if (precision == 0) {
+#define NBODY_X(W, R)                                                                                                 \
+  if (block == W * 32 && ipt == R)                                                                                    \
+    return law == 0                                                                                                   \
+               ? std::min(occupancy_of(k_force_sym64<0, W, R, true>, W * 32, 0), occupancy_of(k_force_sym64<0, W, R, false>, W * 32, 0))  \
+               : std::min(occupancy_of(k_force_sym64<1, W, R, true>, W * 32, 0), occupancy_of(k_force_sym64<1, W, R, false>, W * 32, 0));
+    NBODY_SYM64_TILINGS(NBODY_X)
+#undef NBODY_X
+    return 0;
+  }
 #define NBODY_X(W, R, MINB)                                                                              \
   if (block == W * 32 && ipt == R) {                                                                     \
     constexpr size_t smem = sizeof(sym::Smem<W, R, kSymTile>);                                           \

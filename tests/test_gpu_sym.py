@@ -82,6 +82,56 @@ def test_sym_lennard_jones(nb, tmp_path, monkeypatch, tiling):
     assert_elem_close(phi.cpu().numpy(), phi_ref, MIX_MAX, "phi")
 
 
+# i-tiles of 64, 128, 256 and 256 bodies
+TILINGS64 = [(64, 1, 64, 32, 3, 0), (128, 1, 64, 96, 3, 1), (256, 1, 64, 64, 3, 0), (128, 2, 64, 160, 3, 1)]
+
+
+@pytest.mark.parametrize("tiling", TILINGS64)
+@pytest.mark.parametrize("n", [65, 300, 1025, 2500])
+@pytest.mark.parametrize("length,mass", [(1.0, 1.0), (1e100, 1e30), (1e-95, 1.0)])
+def test_sym64_forces(nb, tmp_path, monkeypatch, tiling, n, length, mass):
+    """FP64 path, in units where s^2 takes the integer steps and in some where it leaves their
+    range (the oracle gets scaled copies; powers of ten, so the comparison is good to rounding)."""
+    import torch
+    monkeypatch.setenv("NBODY_TUNE_CACHE", str(tmp_path / "tune"))
+    x, v, m = inputs.plummer(n, seed=n)
+    m = _masses(m, "lognormal", n)
+    xs, ms, eps = x * length, m * mass, 0.03 * length
+    ctx = _forced(nb, tmp_path / "tune", {"force": tiling}, G=1.1, eps=eps, dt=1e-3, n=n, precision=nb.FP64)
+    assert nb.nbody_get_tuning(ctx)["variant"] == 4
+    xt, mt = to_dev(xs, ms)
+    a, phi = nb.nbody_forces(ctx, xt, mt)
+    a0, _ = nb.nbody_forces(ctx, xt, mt, with_phi=False)
+    nb.nbody_sync(ctx)
+    assert torch.equal(a, a0)
+    a_ref, phi_ref = oracle.forces(x, m, G=1.1, eps=0.03)
+    a, phi = a.cpu().numpy() * (length / mass) * length, phi.cpu().numpy() * (length / mass)
+    assert force_rel_err(a, a_ref).max() <= 1e-12
+    assert_elem_close(phi, phi_ref, 1e-12, "phi")
+
+
+@pytest.mark.parametrize("tiling", TILINGS64)
+def test_sym64_lennard_jones_and_coincident(nb, tmp_path, monkeypatch, tiling):
+    monkeypatch.setenv("NBODY_TUNE_CACHE", str(tmp_path / "tune"))
+    x, v, m, box = inputs.lj_gas(1100, seed=7, density=0.3)
+    m = _masses(m, "lognormal", 3)
+    kw = dict(law=nb.LENNARD_JONES, dt=1e-3, n=1100, lj_epsilon=1.3, lj_sigma=0.9, precision=nb.FP64)
+    ctx = _forced(nb, tmp_path / "tune", {"force": tiling}, **kw)
+    assert nb.nbody_get_tuning(ctx)["variant"] == 4
+    a, phi = nb.nbody_forces(ctx, *to_dev(x, m))
+    nb.nbody_sync(ctx)
+    a_ref, phi_ref = oracle.lj_forces(x, m, eps_lj=1.3, sigma=0.9)
+    assert force_rel_err(a.cpu().numpy(), a_ref).max() <= 1e-12
+    assert_elem_close(phi.cpu().numpy(), phi_ref, 1e-12, "phi")
+    # unsoftened coincident bodies stay a reported condition
+    ctx = _forced(nb, tmp_path / "tune", {"force": tiling}, G=1.0, eps=0.0, dt=1e-3, n=1100, precision=nb.FP64)
+    x[700] = x[3]
+    nb.nbody_forces(ctx, *to_dev(x, m))
+    with pytest.raises(nb.NBodyError) as ei:
+        nb.nbody_sync(ctx)
+    assert ei.value.status == 5
+
+
 @pytest.mark.parametrize("length,mass", [(1e12, 1e30), (1e-9, 1e-27), (1.0, 1.0)])
 def test_mixed_forces_in_any_units(nb, length, mass):
     """Staging scales positions and masses by powers of two, so the float32 arithmetic stays in
