@@ -269,13 +269,15 @@ nbody_status check_dev(nbody_ctx* c, const void* p, size_t bytes, const char* na
 // ---------------------------------------------------------------------------
 // work lists
 
-int sym_tile(int prec) { return prec == NBODY_MIXED ? kSymTile : kSymTile64; }
+int sym_tile(int prec, bool vjp) { return prec != NBODY_MIXED ? kSymTile64 : vjp ? kSymVjpTile : kSymTile; }
 // j-bodies that a warp of the symmetric pass meets in one block: pieces are whole blocks
 int sym_block(int prec) { return prec == NBODY_MIXED ? 64 : 32; }
 
 int ctas_per_sm(int prec, const Tiling& t, bool vjp, int law) {
-  if (t.variant == kSymVariant)
-    return !vjp && t.jtile == sym_tile(prec) ? sym_force_ctas_per_sm(prec, t.block, t.ipt, law) : 0;
+  if (t.variant == kSymVariant) {
+    if (t.jtile != sym_tile(prec, vjp)) return 0;
+    return vjp ? sym_vjp_ctas_per_sm(prec, t.block, t.ipt) : sym_force_ctas_per_sm(prec, t.block, t.ipt, law);
+  }
   return vjp ? vjp_ctas_per_sm(prec, t.variant, t.block, t.ipt, t.jtile)
              : force_ctas_per_sm(prec, t.variant, t.block, t.ipt, t.jtile, law);
 }
@@ -543,21 +545,24 @@ nbody_status install_tiling(nbody_ctx* c, Tiling t, bool vjp) {
   return NBODY_OK;
 }
 
-SymLaunch sym_launch(nbody_ctx* c, bool phi) {
+SymLaunch sym_launch(nbody_ctx* c, bool vjp, bool phi) {
   SymLaunch L{};
+  const Tiling& t = vjp ? c->vt : c->ft;
   L.stage_x = c->stage.p;
   L.stage_lo = static_cast<const float4*>(c->stage_lo.p);
-  L.items = static_cast<const SymItem*>(c->d_items);
-  L.n_items = c->n_items;
+  L.stage_w = c->stage_w.p;
+  L.items = static_cast<const SymItem*>(vjp ? c->d_vitems : c->d_items);
+  L.n_items = vjp ? c->n_vitems : c->n_items;
   L.counter = c->counter;
   L.part = static_cast<double*>(c->part.p);
-  L.part_rows = (int64_t)(c->part.bytes / 32);
+  L.params = vjp && c->vjp_params ? 1 : 0;
+  L.part_rows = (int64_t)(c->part.bytes / (!vjp ? 32 : L.params ? 96 : 64));
   L.n_total = c->n_total;
   L.sys = static_cast<const SysParam*>(c->sysp.p);
   L.eps2 = c->cfg.eps * c->cfg.eps;
   L.sigma2 = c->cfg.lj_sigma * c->cfg.lj_sigma;
   L.law = c->cfg.law;
-  L.block = c->ft.block, L.ipt = c->ft.ipt, L.n_ctas = c->ft.n_ctas;
+  L.block = t.block, L.ipt = t.ipt, L.n_ctas = t.n_ctas;
   L.phi = phi ? 1 : 0;
   L.status = c->status;
   return L;
@@ -593,7 +598,10 @@ PairLaunch pair_launch(nbody_ctx* c, bool vjp, bool refine = true, bool phi = tr
 
 // The all-pairs kernel of the installed tiling.
 cudaError_t launch_pairs(nbody_ctx* c, bool vjp, bool phi, cudaStream_t st) {
-  if (!vjp && is_sym(c->ft)) return launch_sym_force(c->cfg.precision, sym_launch(c, phi), st);
+  if (is_sym(vjp ? c->vt : c->ft)) {
+    const SymLaunch L = sym_launch(c, vjp, phi);
+    return vjp ? launch_sym_vjp(c->cfg.precision, L, st) : launch_sym_force(c->cfg.precision, L, st);
+  }
   const PairLaunch L = pair_launch(c, vjp, true, phi);
   return vjp ? launch_vjp(c->cfg.precision, L, st) : launch_force(c->cfg.precision, L, st);
 }
@@ -752,6 +760,22 @@ uint64_t splitmix(uint64_t& s) {
   return z ^ (z >> 31);
 }
 
+// Staging parameters without scales: the FP64 path's, the tuner's synthetic data's, and of
+// Lennard-Jones all but the origin (k_centre sets the rest at the start of every call).
+nbody_status upload_plain_staging(nbody_ctx* c) {
+  const nbody_config& g = c->cfg;
+  const double sc2 = c->stage_scale * c->stage_scale, e2 = g.eps * g.eps;
+  SysParam p{};
+  p.scale = c->stage_scale, p.mscale = p.inv_mscale = 1.0;
+  p.eps2 = (float)(e2 * sc2);
+  p.r2c = g.law == NBODY_LAW_LJ
+              ? (float)((kNearRadiusSigma * kNearRadiusSigma * g.lj_sigma * g.lj_sigma + e2) * sc2)
+              : (float)(kNearRadiusEps * kNearRadiusEps * e2);
+  const std::vector<SysParam> all((size_t)c->n_sys, p);
+  NB_CUDA(c, cudaMemcpy(c->sysp.p, all.data(), all.size() * sizeof(SysParam), cudaMemcpyHostToDevice));
+  return NBODY_OK;
+}
+
 // Fills the staging buffers with synthetic bodies so that candidate tilings
 // can be timed before any user data exists: for gravity each system is a
 // Plummer sphere (scale radius 1, total mass 1, radii truncated at 20), for
@@ -759,6 +783,7 @@ uint64_t splitmix(uint64_t& s) {
 // are typically run on, which also set how often the near-pair correction of
 // the mixed kernels fires.
 nbody_status fill_synthetic(nbody_ctx* c, bool with_w) {
+  if (nbody_status r = upload_plain_staging(c)) return r;
   const int64_t n = c->n_total;
   uint64_t seed = 12345;
   auto u01 = [&] { return ((double)(splitmix(seed) >> 11) + 0.5) * (1.0 / 9007199254740992.0); };
@@ -874,7 +899,7 @@ nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
   if (P.n_items < L.n_items) err = timed(P, false, &ms);
   if (err == cudaSuccess && (P.n_items == L.n_items || ms * (double)L.n_items / std::max(1, P.n_items) < 60.0)) {
     P = L;
-    err = timed(P, !vjp, &ms);
+    err = timed(P, !vjp || sym, &ms);  // (a gradient's slots: the force combine reads half of each entry)
   }
   for (auto& e : ev) cudaEventDestroy(e);
   if (err != cudaSuccess) return fail(c, NBODY_ECUDA, "autotune launch failed: %s", cudaGetErrorString(err));
@@ -968,7 +993,7 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
     // a variant fixed by the caller applies to the force and the VJP kernels (the
     // register-capped packed force kernel pairs with the packed VJP)
     if (vjp)
-      variants = g.variant ? std::vector<int>{std::min(g.variant - 1, 1)} : std::vector<int>{0, 1};
+      variants = g.variant ? std::vector<int>{std::min(g.variant - 1, 1)} : std::vector<int>{1};
     else
       variants = g.variant ? std::vector<int>{g.variant - 1} : std::vector<int>{1, 2};  // (the scalar kernel never won)
     // Lennard-Jones: the packed kernel, uncapped and capped (6 CTAs per SM)
@@ -983,27 +1008,30 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
   }
   const bool large = pairs > kTuneLargePairs;
   const double typical = pairs > 0 ? cubes / pairs : 0.0;
-  const bool any_tiling = !g.variant && !g.block && !g.i_per_thread && !g.j_tile && !g.slice;
+  // (a requested force tiling does not concern the VJP, a requested variant does)
+  const bool any_tiling = !g.variant && (vjp || (!g.block && !g.i_per_thread && !g.j_tile && !g.slice));
   const bool mixed = g.precision == NBODY_MIXED;
-  const bool sym = !vjp && any_tiling && typical >= (mixed ? kSymMinBodies : kSymMinBodies64);
+  const bool sym = any_tiling && typical >= (mixed ? kSymMinBodies : kSymMinBodies64);
   const bool sym_only = sym && typical >= (mixed ? kSymOnlyBodies : kSymOnlyBodies64);
   if (sym_only && large) {
     // nothing to choose between: its cost per pair no longer depends on the tiling
     Tiling t;
-    t.block = mixed ? 256 : 128, t.ipt = mixed ? 4 : 1, t.jtile = sym_tile(g.precision), t.variant = kSymVariant;
-    t.tail = 1;
-    if (install_tiling(c, t, false) == NBODY_OK) {
-      tune_cache_store(c, vjp, c->ft);
+    t.block = mixed && !vjp ? 256 : 128, t.ipt = !mixed ? 1 : vjp ? 2 : 4;
+    t.jtile = sym_tile(g.precision, vjp), t.variant = kSymVariant, t.tail = 1;
+    if (install_tiling(c, t, vjp) == NBODY_OK) {
+      tune_cache_store(c, vjp, vjp ? c->vt : c->ft);
       return NBODY_OK;
     }
   }
   if (sym && !large) {
     const std::vector<std::pair<int, int>> br =
-        mixed ? std::vector<std::pair<int, int>>{{128, 2}, {128, 4}, {256, 2}, {256, 4}}
-              : std::vector<std::pair<int, int>>{{64, 1}, {128, 1}, {256, 1}, {128, 2}};
+        mixed && vjp ? std::vector<std::pair<int, int>>{{128, 1}, {128, 2}, {256, 2}}
+        : mixed      ? std::vector<std::pair<int, int>>{{128, 2}, {128, 4}, {256, 2}, {256, 4}}
+        : vjp        ? std::vector<std::pair<int, int>>{{64, 1}, {128, 1}, {256, 1}}
+                     : std::vector<std::pair<int, int>>{{64, 1}, {128, 1}, {256, 1}, {128, 2}};
     for (const auto& p : br) {
       Tiling t;
-      t.block = p.first, t.ipt = p.second, t.jtile = sym_tile(g.precision), t.variant = kSymVariant;
+      t.block = p.first, t.ipt = p.second, t.jtile = sym_tile(g.precision, vjp), t.variant = kSymVariant;
       cands.push_back(t);
     }
     if (sym_only) variants.clear();
@@ -1090,15 +1118,20 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
   // last wave ends): with equal slices several tilings often lie within 0.2%
   // of each other, and the one the tail favours must not be cut by that noise.
   // Every setting is timed twice, interleaved, the best kept.
-  if (!vjp && g.slice == 0 && !large) {
+  if ((vjp || g.slice == 0) && !large) {
     std::vector<Tiling> settings;
     for (size_t f = 0; f < top; ++f) {
       Tiling base = timed[f].second;
+      if (vjp && !is_sym(base)) {
+        settings.push_back(base);
+        continue;
+      }
       base.slice = 0;
       base.tail = 0;
       if ((s = install_tiling(c, base, vjp))) return s;
-      const int L0 = c->ft.slice;
-      const int64_t n_ctas = c->ft.n_ctas;
+      const int L0 = (vjp ? c->vt : c->ft).slice;
+      // (a short list has fewer CTAs than the grid it is planned for)
+      const int64_t n_ctas = is_sym(base) ? (int64_t)ctas_per_sm(g.precision, base, vjp, g.law) * c->sm_count : c->ft.n_ctas;
       std::vector<int> ls = {L0 / 2, L0, L0 * 2};
       if (is_sym(base)) {
         ls.clear();
@@ -1128,7 +1161,7 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
       }
     }
     std::vector<double> lc(settings.size(), 1e300);
-    for (int round = 0; round < 2; ++round)
+    for (int round = 0; round < 2 && !settings.empty(); ++round)
       for (size_t k = 0; k < settings.size(); ++k) {
         if ((s = install_tiling(c, settings[k], vjp))) return s;
         double cost = 0;
@@ -1136,7 +1169,7 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
         if (verbose)
           fprintf(stderr, "nbody tune variant=%d block=%d ipt=%d jtile=%d slice=%d tail=%d items=%d -> %.4g ps/pair\n",
                   settings[k].variant, settings[k].block, settings[k].ipt, settings[k].jtile, settings[k].slice,
-                  settings[k].tail, c->n_items, cost * 1e12);
+                  settings[k].tail, vjp ? c->n_vitems : c->n_items, cost * 1e12);
         lc[k] = std::min(lc[k], cost);
       }
     double bc = 1e300;
@@ -1480,19 +1513,7 @@ nbody_status nbody_init(nbody_ctx** out, const nbody_config* cfg, int64_t n_syst
     return bail(fail(c, NBODY_ENOMEM, "cudaHostAlloc of the status word failed"));
   }
   *c->h_status = 0u;
-  {
-    // unscaled staging: the FP64 path's, the tuner's, and of Lennard-Jones all but the origin
-    const double sc2 = c->stage_scale * c->stage_scale, e2 = cfg->eps * cfg->eps;
-    SysParam p{};
-    p.scale = c->stage_scale, p.mscale = p.inv_mscale = 1.0;
-    p.eps2 = (float)(e2 * sc2);
-    p.r2c = cfg->law == NBODY_LAW_LJ
-                ? (float)((kNearRadiusSigma * kNearRadiusSigma * cfg->lj_sigma * cfg->lj_sigma + e2) * sc2)
-                : (float)(kNearRadiusEps * kNearRadiusEps * e2);
-    const std::vector<SysParam> all((size_t)c->n_sys, p);
-    if (cudaMemcpy(c->sysp.p, all.data(), all.size() * sizeof(SysParam), cudaMemcpyHostToDevice) != cudaSuccess)
-      return bail(fail(c, NBODY_ECUDA, "upload of the staging parameters failed"));
-  }
+  if ((s = upload_plain_staging(c))) return bail(s);
   if (cudaMalloc(&c->d_off, (n_systems + 1) * sizeof(int64_t)) != cudaSuccess ||
       cudaMalloc(&c->d_sys_chunk, (n_systems + 1) * sizeof(int32_t)) != cudaSuccess) {
     cudaGetLastError();

@@ -173,19 +173,21 @@ struct PairLaunch {
   unsigned* status;      // device status word (index checks of NBODY_DEBUG builds)
 };
 
-// Launch of the symmetric force pass (sym_kernels.cu).
+// Launch of a symmetric pass (sym_kernels.cu, sym_vjp.cu).
 struct SymLaunch {
   const void* stage_x;     // as in PairLaunch
+  const void* stage_w;
   const float4* stage_lo;
   const SymItem* items;
   int32_t n_items;
   unsigned* counter;
   double* part;            // fpair4 (mixed) or double4_32a (FP64)
-  int64_t part_rows;       // entries the partial buffer holds (index checks of NBODY_DEBUG builds)
+  int64_t part_rows;       // bodies' entries the partial buffer holds (index checks of NBODY_DEBUG builds)
   int64_t n_total;
   const SysParam* sys;
   double eps2, sigma2;     // FP64 path
   int law, block, ipt, n_ctas, phi;
+  int params;              // VJP: also the sums for the G and eps gradients
   unsigned* status;
 };
 
@@ -239,6 +241,9 @@ cudaError_t launch_sym_force(int precision, const SymLaunch& L, cudaStream_t st)
 int sym_force_ctas_per_sm(int precision, int block, int ipt, int law);
 constexpr int kSymTile = 256;   // j-bodies per shared-memory tile of the symmetric kernels, mixed
 constexpr int kSymTile64 = 64;  // ... and FP64
+cudaError_t launch_sym_vjp(int precision, const SymLaunch& L, cudaStream_t st);
+int sym_vjp_ctas_per_sm(int precision, int block, int ipt);
+constexpr int kSymVjpTile = 128;  // j-tile of the mixed symmetric VJP (FP64: kSymTile64)
 
 // ---------------------------------------------------------------------------
 // O(N) kernels (post_kernels.cu)

@@ -177,3 +177,32 @@ def test_sym_several_systems_and_zero_masses(nb, tmp_path, monkeypatch):
         a_ref, phi_ref = oracle.forces(x[b:e], m[b:e], G=1.0, eps=0.02)
         assert force_rel_err(a[b:e].cpu().numpy(), a_ref).max() <= MIX_MAX, s
         assert_elem_close(phi[b:e].cpu().numpy(), phi_ref, MIX_PHI_MAX, f"phi {s}")
+
+
+@pytest.mark.parametrize("prec,tiling", [(1, (128, 1, 128, 64, 3, 0)), (1, (128, 2, 128, 64, 3, 1)),
+                                         (1, (256, 2, 128, 192, 3, 0)), (0, (64, 1, 64, 32, 3, 0)),
+                                         (0, (128, 1, 64, 96, 3, 1)), (0, (256, 1, 64, 64, 3, 0))])
+@pytest.mark.parametrize("n", [2, 65, 513, 1100])
+def test_sym_vjp(nb, tmp_path, monkeypatch, prec, tiling, n):
+    """Gradients through a few steps, G and eps included, near pairs in most tiles (4 eps = 0.2)."""
+    import torch
+    monkeypatch.setenv("NBODY_TUNE_CACHE", str(tmp_path / "tune"))
+    G, eps, dt, T, K = 1.1, 0.05, 4e-3, 3, 2
+    x, v, m = inputs.plummer(n, seed=70 + n)
+    m = _masses(m, "lognormal", n)
+    rng = np.random.default_rng(n)
+    lx, lv = rng.standard_normal((n, 3)), 0.1 * rng.standard_normal((n, 3))
+    args = to_dev(x, v, m) + (T, K) + to_dev(lx, lv)
+    ctx = _forced(nb, tmp_path / "tune", {"vjp": tiling}, use=lambda c: nb.nbody_adjoint(c, *args), G=G, eps=eps, dt=dt,
+                  n=n, precision=prec)
+    gx, gv, gm, gp = nb.nbody_adjoint_params(ctx, *args)
+    hx, hv, hm = nb.nbody_adjoint(ctx, *args)
+    nb.nbody_sync(ctx)
+    assert torch.equal(gx, hx) and torch.equal(gv, hv) and torch.equal(gm, hm)
+    ox, ov, om, (oG, oe) = oracle.adjoint_params(x, v, m, G, eps, dt, T, lx, lv)
+    tol = 1e-4 if prec else 1e-11  # the bounds of test_gpu_adjoint.py
+    for g, o, what in ((gx, ox, "g_x0"), (gv, ov, "g_v0"), (gm, om, "g_m")):
+        assert_elem_close(g.cpu().numpy(), o, tol, what)
+    gG, ge = gp.cpu().numpy()[0]
+    scale = max(abs(oG), abs(oe) * eps)
+    assert abs(gG - oG) <= tol * scale and abs(ge - oe) * eps <= tol * scale
