@@ -222,8 +222,9 @@ nbody_status nbody_sync(nbody_ctx* ctx);
 /*
  * Tiling in use (after init / autotune): block, i_per_thread, j_tile, slice,
  * the number of persistent CTAs the force kernel launches, and the force
- * kernel variant (as in nbody_config.variant: 1 scalar, 2 packed, 3 packed capped). Any pointer
- * may be NULL.
+ * kernel variant (as in nbody_config.variant: 1 scalar, 2 packed, 3 packed capped; 4, which
+ * cannot be requested: the symmetric pass, every unordered pair once, both precisions, with
+ * block also 64). Any pointer may be NULL.
  */
 nbody_status nbody_get_tuning(const nbody_ctx* ctx, int32_t* block, int32_t* i_per_thread, int32_t* j_tile,
                               int32_t* slice, int32_t* n_ctas, int32_t* variant);
@@ -255,9 +256,10 @@ int64_t nbody_launch_count(const nbody_ctx* ctx);
 
 /*
  * Largest body count nbody_forces_noalloc accepts. Its scratch is a fixed
- * 32 MiB + 256 B __device__ array (32 bytes per body: the float32 staging
- * entry and the float32 remainders of the near-pair refinement), held on every
- * GPU that loads the library's device code, for the life of the process.
+ * 32 MiB + 8 KiB __device__ array (32 bytes per body: the float32 staging
+ * entry and the float32 remainders of the near-pair refinement; what fewer bodies
+ * leave of it takes partial sums), held on every GPU that loads the library's
+ * device code, for the life of the process.
  */
 #define NBODY_NOALLOC_MAX_BODIES 1048576
 
@@ -277,8 +279,8 @@ int64_t nbody_launch_count(const nbody_ctx* ctx);
  * float32 pairs with the near-pair refinement (pairs closer than 4 eps
  * recomputed from the staged float32 remainders), compensated float32 tile
  * sums, float64 result; the same error bounds against the float64 direct sum
- * (median <= 1e-6, max <= 1e-4 relative per body). One CTA per i-tile and no
- * j-slices, so results agree with nbody_forces to rounding, not bit for bit.
+ * (median <= 1e-6, max <= 1e-4 relative per body). The work is cut by the body
+ * count alone, so results agree with nbody_forces to rounding, not bit for bit.
  *
  * Scratch is a static __device__ array shared by every call in the process:
  * calls that overlap on the GPU (different streams, or different host threads)
@@ -288,7 +290,7 @@ int64_t nbody_launch_count(const nbody_ctx* ctx);
  * The first call on a device is a warm-up: it looks up the array's device
  * address (cudaGetSymbolAddress) with that device current, which makes the
  * CUDA runtime load the library's device code on that device if it has not
- * yet, and loading reserves the 32 MiB array and the kernels' code there (it
+ * yet, and loading reserves the scratch array and the kernels' code there (it
  * can fail with NBODY_ECUDA when the device is out of memory, and may
  * synchronise). Make that first call before the region that must not
  * allocate, and before any stream capture; later calls on that device

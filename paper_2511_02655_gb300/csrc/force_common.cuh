@@ -371,10 +371,12 @@ struct SmemMixed2 {
   int item;
 };
 
-// Work items of the packed mixed kernel, taken from `counter` until none is left;
-// each writes its slice's compensated float32 sums (fpair4) per i-body.
-template <int LAW, int BLOCK, int R, int J, bool PHI>
-__device__ __forceinline__ void items_mixed2(const PairLaunch& L, unsigned* counter, SmemMixed2<J>& sm) {
+// Work items of the packed mixed kernel, taken from next(WorkItem&) until it returns
+// false (called by all threads of the CTA; if it is called again, it is a barrier:
+// the buffers are free); each hands its slice's compensated float32 sums (fpair4) per
+// i-body to put(item, body, sums).
+template <int LAW, int BLOCK, int R, int J, bool PHI, typename Next, typename Put>
+__device__ __forceinline__ void items_mixed2(const PairLaunch& L, Next next, Put put, SmemMixed2<J>& sm) {
   static_assert(J % 4 == 0, "tiles hold whole quads of j-bodies");
   constexpr int LPT = (J + BLOCK - 1) / BLOCK;
   auto& tx = sm.tx;
@@ -382,14 +384,11 @@ __device__ __forceinline__ void items_mixed2(const PairLaunch& L, unsigned* coun
   auto& tz = sm.tz;
   auto& tm = sm.tm;
   const float4* __restrict__ st = static_cast<const float4*>(L.stage_x);
-  fpair4* __restrict__ part = reinterpret_cast<fpair4*>(L.part);
   const float2 s2 = make_float2((float)L.sigma2, (float)L.sigma2);
   const float4* __restrict__ lo = L.stage_lo;
 
-  for (;;) {
-    const int it = next_item(counter, &sm.item);  // also a barrier: the buffers are free
-    if (it >= L.n_items) break;
-    const WorkItem w = L.items[it];
+  WorkItem w;
+  while (next(w)) {
     if (!item_ok(w, L)) continue;  // NBODY_DEBUG builds only
     const float eps2 = L.sys[w.sys].eps2, r2c = lo ? L.sys[w.sys].r2c : 0.f;
     const float2 e2 = make_float2(eps2, eps2);
@@ -470,11 +469,10 @@ __device__ __forceinline__ void items_mixed2(const PairLaunch& L, unsigned* coun
       __syncthreads();
     }
 
-    fpair4* out = part + (int64_t)w.slice * L.n_total;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       if (ig[r] < w.i_end)
-        out[ig[r]] = fpair4{make_float4(hx[r], lx[r], hy[r], ly[r]), make_float4(hz[r], lz[r], hp[r], lp[r])};
+        put(w, ig[r], fpair4{make_float4(hx[r], lx[r], hy[r], ly[r]), make_float4(hz[r], lz[r], hp[r], lp[r])});
     }
   }
 }

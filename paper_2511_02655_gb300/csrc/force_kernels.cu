@@ -64,7 +64,15 @@ __global__ void __launch_bounds__(BLOCK, (MINB > 0 ? MINB
     k_force_mixed2(const PairLaunch L) {
   __shared__ fc::SmemMixed2<J> sm;
   pdl_wait();
-  fc::items_mixed2<LAW, BLOCK, R, J, PHI>(L, L.counter, sm);
+  auto next = [&](WorkItem& w) {
+    const int it = next_item(L.counter, &sm.item);
+    if (it < L.n_items) w = L.items[it];
+    return it < L.n_items;
+  };
+  auto put = [&](const WorkItem& w, const int i, const fpair4& sums) {
+    reinterpret_cast<fpair4*>(L.part)[(int64_t)w.slice * L.n_total + i] = sums;
+  };
+  fc::items_mixed2<LAW, BLOCK, R, J, PHI>(L, next, put, sm);
   pdl_trigger();
   retire_cta(L.counter);
 }

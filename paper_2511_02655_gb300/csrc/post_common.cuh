@@ -61,6 +61,130 @@ __device__ __forceinline__ void block_sum(double (&v)[NV]) {
   }
 }
 
+// The slices of one body, added by kSlotGroups threads (thread group g of the CTA
+// takes slices g, g + kSlotGroups, ...) and then over the groups in order, all of it
+// for NC components per slice. Mixed: compensated float32 pairs, added as pairs on
+// the FP32 pipe (TwoSum of the hi parts, the lo parts and rounding errors summed
+// alongside). Valid in group 0; every thread of the CTA calls it.
+template <int CB>
+struct SlotSums {
+  float h[kSlotGroups - 1][CB];
+  float l[kSlotGroups - 1][CB];
+};
+
+template <int NC, int CB>
+__device__ __forceinline__ void add_groups(SlotSums<CB> (&red)[NC], const int g, const int b, float (&h)[NC],
+                                           float (&l)[NC]) {
+  if (g > 0) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) red[c].h[g - 1][b] = h[c], red[c].l[g - 1][b] = l[c];
+  }
+  __syncthreads();
+  if (g == 0) {
+#pragma unroll
+    for (int k = 0; k < kSlotGroups - 1; ++k)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        two_sum_acc(h[c], l[c], red[c].h[k][b]);
+        l[c] += red[c].l[k][b];
+      }
+  }
+}
+
+template <int NC, int CB>
+__device__ __forceinline__ void add_groups(double (&red)[NC][kSlotGroups - 1][CB], const int g, const int b,
+                                           double (&s)[NC]) {
+  if (g > 0) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) red[c][g - 1][b] = s[c];
+  }
+  __syncthreads();
+  if (g == 0) {
+#pragma unroll
+    for (int k = 0; k < kSlotGroups - 1; ++k)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) s[c] += red[c][k][b];
+  }
+}
+
+// One slot of a body's force partials onto its sums.
+__device__ __forceinline__ void add_slot(const fpair4 q, float (&h)[4], float (&l)[4]) {
+  two_sum_acc(h[0], l[0], q.xy.x), l[0] += q.xy.y;
+  two_sum_acc(h[1], l[1], q.xy.z), l[1] += q.xy.w;
+  two_sum_acc(h[2], l[2], q.zp.x), l[2] += q.zp.y;
+  two_sum_acc(h[3], l[3], q.zp.z), l[3] += q.zp.w;
+}
+
+// Largest coordinate and mass of a chunk by their float64 high words (sign bit
+// off: the words order as the magnitudes) and whether its masses all equal its
+// system's first, as one 64-bit value that is carried beside the chunk's sums.
+struct Extent {
+  unsigned x, m, uniform;
+  __device__ __forceinline__ void join(const Extent& o) {
+    x = max(x, o.x), m = max(m, o.m), uniform &= o.uniform;
+  }
+  __device__ __forceinline__ void warp_join() {
+    x = __reduce_max_sync(0xffffffffu, x);
+    m = __reduce_max_sync(0xffffffffu, m);
+    uniform = __reduce_and_sync(0xffffffffu, uniform);
+  }
+  __device__ __forceinline__ double pack() const {
+    return __hiloint2double((int)x, (int)(m << 1 | uniform));
+  }
+  __device__ __forceinline__ static Extent unpack(const double d) {
+    const unsigned l = (unsigned)__double2loint(d);
+    return Extent{(unsigned)__double2hiint(d), l >> 1, l & 1u};
+  }
+};
+
+__device__ __forceinline__ unsigned high_word(const double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+
+// 2^(to - e) for the float64 with high word h of binary exponent e (1 where h is 0, tiny, infinite or NaN)
+__device__ __forceinline__ double power_of_two_scale(const unsigned h, const int to) {
+  const int e = (int)(h >> 20) - 1023;
+  return e < -900 || e > 900 ? 1.0 : ldexp(1.0, to - e);
+}
+
+// The staged coordinates of gravity stay below 2^12: with distances down to 2^-25
+// of that, s^-5 (the force gradient) stays in the float32 range at both ends.
+constexpr int kExtentExp = 10;
+
+// One body's terms of the staging origin's sums (sum m x, sum m, sum x) and its extent.
+__device__ __forceinline__ void centre_terms(const double x0, const double x1, const double x2, const double mi,
+                                             const double m0, double (&v)[7], Extent& q) {
+  v[0] += mi * x0, v[1] += mi * x1, v[2] += mi * x2, v[3] += mi;
+  v[4] += x0, v[5] += x1, v[6] += x2;
+  q.join(Extent{max(max(high_word(x0), high_word(x1)), high_word(x2)), high_word(mi),
+                __double_as_longlong(mi) == __double_as_longlong(m0) ? 1u : 0u});
+}
+
+// Staging parameters of a system of n bodies from those sums: the origin, and for gravity the
+// scales (m0: its first mass).
+__device__ __forceinline__ void staging_params(SysParam& o, const double (&w)[7], const Extent& e, const int64_t n,
+                                               const double m0, const bool gravity, const double eps,
+                                               const double near_eps) {
+  double c0 = 0.0, c1 = 0.0, c2 = 0.0;
+  if (w[3] > 0.0 && isfinite(w[3])) {
+    c0 = w[0] / w[3], c1 = w[1] / w[3], c2 = w[2] / w[3];
+  } else if (n > 0) {
+    c0 = w[4] / (double)n, c1 = w[5] / (double)n, c2 = w[6] / (double)n;
+  }
+  if (!(isfinite(c0) && isfinite(c1) && isfinite(c2))) c0 = c1 = c2 = 0.0;
+  o.c[0] = c0, o.c[1] = c1, o.c[2] = c2;
+  if (!gravity || n <= 0) return;
+  // the softening counts as an extent, so that its staged square stays finite
+  const double s = power_of_two_scale(max(e.x, high_word(eps)), kExtentExp);
+  const double e2 = eps * s, rc = near_eps * e2;
+  const unsigned h0 = high_word(m0);
+  const bool uniform = e.uniform && m0 > 0.0 && h0 >= (123u << 20) && h0 <= (1923u << 20);
+  const double ms = power_of_two_scale(e.m, 0);
+  o.scale = s;
+  o.mscale = uniform ? 1.0 / m0 : ms;
+  o.inv_mscale = uniform ? m0 : 1.0 / ms;
+  o.eps2 = (float)(e2 * e2), o.r2c = (float)(rc * rc);
+  o.uniform = uniform ? 1u : 0u;
+}
+
 // Reflecting walls of [0, box] ("boundary checking"): a coordinate that left
 // the box is mirrored back across the wall and its velocity component flips;
 // repeated (bounded) for steps that cross the box more than once.

@@ -15,52 +15,6 @@
 namespace nbody {
 namespace {
 
-// The slices of one body, added by kSlotGroups threads (thread group g of the CTA
-// takes slices g, g + kSlotGroups, ...) and then over the groups in order, all of it
-// for NC components per slice. Mixed: compensated float32 pairs, added as pairs on
-// the FP32 pipe (TwoSum of the hi parts, the lo parts and rounding errors summed
-// alongside). Valid in group 0; every thread of the CTA calls it.
-template <int CB>
-struct SlotSums {
-  float h[kSlotGroups - 1][CB];
-  float l[kSlotGroups - 1][CB];
-};
-
-template <int NC, int CB>
-__device__ __forceinline__ void add_groups(SlotSums<CB> (&red)[NC], const int g, const int b, float (&h)[NC],
-                                           float (&l)[NC]) {
-  if (g > 0) {
-#pragma unroll
-    for (int c = 0; c < NC; ++c) red[c].h[g - 1][b] = h[c], red[c].l[g - 1][b] = l[c];
-  }
-  __syncthreads();
-  if (g == 0) {
-#pragma unroll
-    for (int k = 0; k < kSlotGroups - 1; ++k)
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        two_sum_acc(h[c], l[c], red[c].h[k][b]);
-        l[c] += red[c].l[k][b];
-      }
-  }
-}
-
-template <int NC, int CB>
-__device__ __forceinline__ void add_groups(double (&red)[NC][kSlotGroups - 1][CB], const int g, const int b,
-                                           double (&s)[NC]) {
-  if (g > 0) {
-#pragma unroll
-    for (int c = 0; c < NC; ++c) red[c][g - 1][b] = s[c];
-  }
-  __syncthreads();
-  if (g == 0) {
-#pragma unroll
-    for (int k = 0; k < kSlotGroups - 1; ++k)
-#pragma unroll
-      for (int c = 0; c < NC; ++c) s[c] += red[c][k][b];
-  }
-}
-
 // One CTA per chunk, kSlotGroups threads per body to add the slices and one to do
 // the rest (a CTA of one thread per body when the mode combines nothing). Adding
 // the slices is a chain of 32-byte loads from L2, and that latency bounds the
@@ -101,13 +55,7 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
     float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
     if (live) {
 #pragma unroll 8
-      for (int s = g; s < c.n_slices; s += kSlotGroups) {
-        const fpair4 q = fp[(int64_t)s * c.stride];
-        two_sum_acc(h[0], l[0], q.xy.x), l[0] += q.xy.y;
-        two_sum_acc(h[1], l[1], q.xy.z), l[1] += q.xy.w;
-        two_sum_acc(h[2], l[2], q.zp.x), l[2] += q.zp.y;
-        two_sum_acc(h[3], l[3], q.zp.z), l[3] += q.zp.w;
-      }
+      for (int s = g; s < c.n_slices; s += kSlotGroups) add_slot(fp[(int64_t)s * c.stride], h, l);
     }
     add_groups(red.f, g, b, h, l);
     if (g == 0) {
@@ -163,40 +111,6 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
   }
 }
 
-// Largest coordinate and mass of a chunk by their float64 high words (sign bit
-// off: the words order as the magnitudes) and whether its masses all equal its
-// system's first, as one 64-bit value that is carried beside the chunk's sums.
-struct Extent {
-  unsigned x, m, uniform;
-  __device__ __forceinline__ void join(const Extent& o) {
-    x = max(x, o.x), m = max(m, o.m), uniform &= o.uniform;
-  }
-  __device__ __forceinline__ void warp_join() {
-    x = __reduce_max_sync(0xffffffffu, x);
-    m = __reduce_max_sync(0xffffffffu, m);
-    uniform = __reduce_and_sync(0xffffffffu, uniform);
-  }
-  __device__ __forceinline__ double pack() const {
-    return __hiloint2double((int)x, (int)(m << 1 | uniform));
-  }
-  __device__ __forceinline__ static Extent unpack(const double d) {
-    const unsigned l = (unsigned)__double2loint(d);
-    return Extent{(unsigned)__double2hiint(d), l >> 1, l & 1u};
-  }
-};
-
-__device__ __forceinline__ unsigned high_word(const double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
-
-// 2^(to - e) for the float64 with high word h of binary exponent e (1 where h is 0, tiny, infinite or NaN)
-__device__ __forceinline__ double power_of_two_scale(const unsigned h, const int to) {
-  const int e = (int)(h >> 20) - 1023;
-  return e < -900 || e > 900 ? 1.0 : ldexp(1.0, to - e);
-}
-
-// The staged coordinates of gravity stay below 2^12: with distances down to 2^-25
-// of that, s^-5 (the force gradient) stays in the float32 range at both ends.
-constexpr int kExtentExp = 10;
-
 template <int CB>
 __global__ void __launch_bounds__(CB) k_centre(const CentreLaunch C) {
   constexpr int NW = CB / 32;
@@ -207,15 +121,8 @@ __global__ void __launch_bounds__(CB) k_centre(const CentreLaunch C) {
   double v[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   Extent q{0u, 0u, 1u};
   const int i = c.begin + (int)threadIdx.x;
-  if (i < c.end) {
-    const double mi = C.m[i], m0 = C.m[C.off[c.sys]];
-    const double x0 = C.x[3 * i + 0], x1 = C.x[3 * i + 1], x2 = C.x[3 * i + 2];
-    v[0] = mi * x0, v[1] = mi * x1, v[2] = mi * x2, v[3] = mi;
-    v[4] = x0, v[5] = x1, v[6] = x2;
-    q.x = max(max(high_word(x0), high_word(x1)), high_word(x2));
-    q.m = high_word(mi);
-    q.uniform = __double_as_longlong(mi) == __double_as_longlong(m0) ? 1u : 0u;
-  }
+  if (i < c.end)
+    centre_terms(C.x[3 * i + 0], C.x[3 * i + 1], C.x[3 * i + 2], C.m[i], C.m[C.off[c.sys]], v, q);
   q.warp_join();
   if (lane == 0) ext[wid] = q;
   block_sum<7, CB>(v);  // its barriers also publish ext
@@ -230,27 +137,7 @@ __global__ void __launch_bounds__(CB) k_centre(const CentreLaunch C) {
   __threadfence();
   auto emit = [&](const int sy, const double (&w)[7], const Extent& e) {
     const int64_t n = C.off[sy + 1] - C.off[sy];
-    double c0 = 0.0, c1 = 0.0, c2 = 0.0;
-    if (w[3] > 0.0 && isfinite(w[3])) {
-      c0 = w[0] / w[3], c1 = w[1] / w[3], c2 = w[2] / w[3];
-    } else if (n > 0) {
-      c0 = w[4] / (double)n, c1 = w[5] / (double)n, c2 = w[6] / (double)n;
-    }
-    if (!(isfinite(c0) && isfinite(c1) && isfinite(c2))) c0 = c1 = c2 = 0.0;
-    SysParam& o = C.sys[sy];
-    o.c[0] = c0, o.c[1] = c1, o.c[2] = c2;
-    if (C.law != 0 || n <= 0) return;
-    // the softening counts as an extent, so that its staged square stays finite
-    const double s = power_of_two_scale(max(e.x, high_word(C.eps)), kExtentExp);
-    const double m0 = C.m[C.off[sy]], e2 = C.eps * s, rc = C.near_eps * e2;
-    const unsigned h0 = high_word(m0);
-    const bool uniform = e.uniform && m0 > 0.0 && h0 >= (123u << 20) && h0 <= (1923u << 20);
-    const double ms = power_of_two_scale(e.m, 0);
-    o.scale = s;
-    o.mscale = uniform ? 1.0 / m0 : ms;
-    o.inv_mscale = uniform ? m0 : 1.0 / ms;
-    o.eps2 = (float)(e2 * e2), o.r2c = (float)(rc * rc);
-    o.uniform = uniform ? 1u : 0u;
+    staging_params(C.sys[sy], w, e, n, n > 0 ? C.m[C.off[sy]] : 0.0, C.law == 0, C.eps, C.near_eps);
   };
   auto extent = [&](const int sy, const int first, const int step) {
     Extent e{0u, 0u, 1u};

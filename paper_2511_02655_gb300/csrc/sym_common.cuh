@@ -216,9 +216,10 @@ __device__ __forceinline__ void refine_block(const unsigned near, unsigned any, 
   }
 }
 
-// Work items, taken from `counter` until none is left.
-template <int LAW, int W, int R, int J, bool PHI>
-__device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Smem<W, R, J>& sm) {
+// Work items, taken from next(SymItem&) until it returns false (called by all threads of the
+// CTA, after a barrier of its own if it is called again).
+template <int LAW, int W, int R, int J, bool PHI, typename Next>
+__device__ __forceinline__ void items(const SymLaunch& L, Next next, Smem<W, R, J>& sm) {
   constexpr int T = W * 32, NB = J / 64, TI = T * R, LPT = (J + T - 1) / T;
   constexpr int NC = PHI ? 4 : 3;
   const int tid = (int)threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -226,10 +227,8 @@ __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Sme
   const float4* __restrict__ lo = L.stage_lo;
   fpair4* part = reinterpret_cast<fpair4*>(L.part);
 
-  for (;;) {
-    const int n = next_item(counter, &sm.item);
-    if (n >= L.n_items) break;
-    const SymItem it = L.items[n];
+  SymItem it;
+  while (next(it)) {
     if (!sym_item_ok(it, L)) continue;  // NBODY_DEBUG builds only
     const float eps2 = L.sys[it.sys].eps2, r2c = lo ? L.sys[it.sys].r2c : 0.f;
     const bool uniform = LAW == 0 && L.sys[it.sys].uniform != 0u;

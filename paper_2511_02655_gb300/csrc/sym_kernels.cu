@@ -15,7 +15,12 @@ __global__ void __launch_bounds__(W * 32, MINB) k_force_sym(const SymLaunch L) {
   extern __shared__ __align__(16) unsigned char raw[];
   auto& sm = *reinterpret_cast<sym::Smem<W, R, kSymTile>*>(raw);
   pdl_wait();
-  sym::items<LAW, W, R, kSymTile, PHI>(L, L.counter, sm);
+  auto next = [&](SymItem& it) {
+    const int n = next_item(L.counter, &sm.item);
+    if (n < L.n_items) it = L.items[n];
+    return n < L.n_items;
+  };
+  sym::items<LAW, W, R, kSymTile, PHI>(L, next, sm);
   pdl_trigger();
   retire_cta(L.counter);
 }

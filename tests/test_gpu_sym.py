@@ -206,3 +206,23 @@ def test_sym_vjp(nb, tmp_path, monkeypatch, prec, tiling, n):
     gG, ge = gp.cpu().numpy()[0]
     scale = max(abs(oG), abs(oe) * eps)
     assert abs(gG - oG) <= tol * scale and abs(ge - oe) * eps <= tol * scale
+
+
+@pytest.mark.parametrize("n", [33, 2048, 2049, 8193, 24000, 24001, 524288, 524289])
+@pytest.mark.parametrize("masses", ["equal", "lognormal"])
+def test_noalloc_work_splits(nb, n, masses):
+    """Both sides of every size at which the allocation-free entry point changes its work split,
+    against the oracle on sampled bodies."""
+    import torch
+    x, v, m = inputs.plummer(n, seed=n)
+    m = _masses(m, masses, n)
+    xt, mt = to_dev(x, m)
+    a, phi = nb.nbody_forces_noalloc(xt, mt, 1.1, 0.01, phi=torch.empty_like(mt))
+    a0, _ = nb.nbody_forces_noalloc(xt, mt, 1.1, 0.01)
+    torch.cuda.synchronize()
+    assert torch.equal(a, a0)
+    idx = inputs.sample_indices(n, 512, seed=1)
+    a_ref, phi_ref = oracle.forces_at(x, m, idx, G=1.1, eps=0.01)
+    e = force_rel_err(a.cpu().numpy()[idx], a_ref)
+    assert np.median(e) <= MIX_MED and e.max() <= MIX_MAX, (np.median(e), e.max())
+    assert_elem_close(phi.cpu().numpy()[idx], phi_ref, MIX_PHI_MAX, "phi")
