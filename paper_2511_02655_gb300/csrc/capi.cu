@@ -39,7 +39,8 @@ struct Tiling {
   int variant = 0;  // mixed kernels: 0 scalar, 1 packed float32x2, 2 packed with a 4-CTA register cap (force),
                     // 3 symmetric (every unordered pair once)
   int tail = 0;     // slicing of a system's j-range: 0 equal slices, 1 full slices and a halving tail
-                    // (symmetric: 1 cuts every other row of i-tiles into pieces a third as long)
+                    // (symmetric: 0 pieces of one length and a remainder per row of i-tiles, 1 every other
+                    // row in pieces a third as long, 2 pieces of a row as equal as whole blocks allow)
 };
 constexpr int kSymVariant = 3;
 constexpr double kSymMinBodies = 1024.0;    // typical system size from which the symmetric pass is a candidate
@@ -269,13 +270,15 @@ nbody_status check_dev(nbody_ctx* c, const void* p, size_t bytes, const char* na
 // ---------------------------------------------------------------------------
 // work lists
 
-int sym_tile(int prec, bool vjp) { return prec != NBODY_MIXED ? kSymTile64 : vjp ? kSymVjpTile : kSymTile; }
+int sym_tile(int prec, bool vjp, int block) {
+  return prec != NBODY_MIXED ? kSymTile64 : vjp ? kSymVjpTile : sym_force_tile(block / 32);
+}
 // j-bodies that a warp of the symmetric pass meets in one block: pieces are whole blocks
 int sym_block(int prec) { return prec == NBODY_MIXED ? 64 : 32; }
 
 int ctas_per_sm(int prec, const Tiling& t, bool vjp, int law) {
   if (t.variant == kSymVariant) {
-    if (t.jtile != sym_tile(prec, vjp)) return 0;
+    if (t.jtile != sym_tile(prec, vjp, t.block)) return 0;
     return vjp ? sym_vjp_ctas_per_sm(prec, t.block, t.ipt) : sym_force_ctas_per_sm(prec, t.block, t.ipt, law);
   }
   return vjp ? vjp_ctas_per_sm(prec, t.variant, t.block, t.ipt, t.jtile)
@@ -461,10 +464,12 @@ void build_sym_items(const nbody_ctx* c, const Tiling& t, std::vector<SymItem>& 
     for (int64_t r = 0; r < nr; ++r) {
       const int64_t i0 = r * H, ni = std::min(H, n - i0), len = n - i0;
       const double pairs = (double)ni * ((double)len - 0.5 * (double)ni);
-      const double want = t.tail && (r & 1) ? area / 3.0 : area;
-      int64_t p = std::max<int64_t>(1, (int64_t)(pairs / want + 0.5));
-      const int64_t step = std::max<int64_t>(1, (len + p * q / 2) / (p * q)) * q;  // whole blocks
-      p = (len + step - 1) / step;
+      const double want = t.tail == 1 && (r & 1) ? area / 3.0 : area;
+      const int64_t blocks = (len + q - 1) / q;  // pieces are whole blocks
+      int64_t p = std::max<int64_t>(1, std::min(blocks, (int64_t)(pairs / want + 0.5)));
+      const int64_t step = std::max<int64_t>(1, (2 * blocks + p) / (2 * p));
+      if (t.tail != 2) p = (blocks + step - 1) / step;
+      auto cut = [&](int64_t k) { return std::min(n, i0 + q * (t.tail == 2 ? k * blocks / p : k * step)); };
       slots[(size_t)r] = (int)(r + 1 + p);
       most = std::max(most, slots[(size_t)r]);
       for (int64_t k = 0; k < p; ++k) {
@@ -472,8 +477,8 @@ void build_sym_items(const nbody_ctx* c, const Tiling& t, std::vector<SymItem>& 
         w.sys = s;
         w.i_begin = (int32_t)(b + i0);
         w.i_end = (int32_t)(b + i0 + ni);
-        w.j_begin = (int32_t)(b + i0 + k * step);
-        w.j_end = (int32_t)(b + std::min(n, i0 + (k + 1) * step));
+        w.j_begin = (int32_t)(b + cut(k));
+        w.j_end = (int32_t)(b + cut(k + 1));
         w.slot_j = (int32_t)r;
         w.slot_i = (int32_t)(r + 1 + k);
         w.stride = (int32_t)n;
@@ -1017,7 +1022,7 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
     // nothing to choose between: its cost per pair no longer depends on the tiling
     Tiling t;
     t.block = mixed && !vjp ? 256 : 128, t.ipt = !mixed ? 1 : vjp ? 2 : 4;
-    t.jtile = sym_tile(g.precision, vjp), t.variant = kSymVariant, t.tail = 1;
+    t.jtile = sym_tile(g.precision, vjp, t.block), t.variant = kSymVariant, t.tail = 1;
     if (install_tiling(c, t, vjp) == NBODY_OK) {
       tune_cache_store(c, vjp, vjp ? c->vt : c->ft);
       return NBODY_OK;
@@ -1026,12 +1031,12 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
   if (sym && !large) {
     const std::vector<std::pair<int, int>> br =
         mixed && vjp ? std::vector<std::pair<int, int>>{{128, 1}, {128, 2}, {256, 2}}
-        : mixed      ? std::vector<std::pair<int, int>>{{128, 2}, {128, 4}, {256, 2}, {256, 4}}
+        : mixed      ? std::vector<std::pair<int, int>>{{64, 4}, {128, 2}, {128, 4}, {256, 2}, {256, 4}}
         : vjp        ? std::vector<std::pair<int, int>>{{64, 1}, {128, 1}, {256, 1}}
                      : std::vector<std::pair<int, int>>{{64, 1}, {128, 1}, {256, 1}, {128, 2}};
     for (const auto& p : br) {
       Tiling t;
-      t.block = p.first, t.ipt = p.second, t.jtile = sym_tile(g.precision, vjp), t.variant = kSymVariant;
+      t.block = p.first, t.ipt = p.second, t.jtile = sym_tile(g.precision, vjp, t.block), t.variant = kSymVariant;
       cands.push_back(t);
     }
     if (sym_only) variants.clear();
@@ -1135,7 +1140,7 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
       std::vector<int> ls = {L0 / 2, L0, L0 * 2};
       if (is_sym(base)) {
         ls.clear();
-        for (int k : {1, 2, 3, 4, 6, 8, 12}) {
+        for (int k : {1, 2, 3, 4, 6, 8}) {
           const int len = sym_slice(c, base, (int)n_ctas, k);
           if (std::find(ls.begin(), ls.end(), len) == ls.end()) ls.push_back(len);
         }
@@ -1152,7 +1157,7 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
       }
       for (int len : ls) {
         if (len < kSliceQuantum) continue;
-        for (int tail = 0; tail < 2; ++tail) {
+        for (int tail = 0; tail < (is_sym(base) ? 3 : 2); ++tail) {
           Tiling t = base;
           t.slice = len;
           t.tail = tail;

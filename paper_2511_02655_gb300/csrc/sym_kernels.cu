@@ -13,14 +13,14 @@ namespace {
 template <int LAW, int W, int R, bool PHI, int MINB>
 __global__ void __launch_bounds__(W * 32, MINB) k_force_sym(const SymLaunch L) {
   extern __shared__ __align__(16) unsigned char raw[];
-  auto& sm = *reinterpret_cast<sym::Smem<W, R, kSymTile>*>(raw);
+  auto& sm = *reinterpret_cast<sym::Smem<W, R, sym_force_tile(W)>*>(raw);
   pdl_wait();
   auto next = [&](SymItem& it) {
     const int n = next_item(L.counter, &sm.item);
     if (n < L.n_items) it = L.items[n];
     return n < L.n_items;
   };
-  sym::items<LAW, W, R, kSymTile, PHI>(L, next, sm);
+  sym::items<LAW, W, R, sym_force_tile(W), PHI>(L, next, sm);
   pdl_trigger();
   retire_cta(L.counter);
 }
@@ -54,7 +54,8 @@ int occupancy_of(K kern, int block, size_t smem) {
 }  // namespace
 
 // Compiled: warps, i-bodies per lane (and resident CTAs).
-#define NBODY_SYM_TILINGS(X) X(4, 2, 6) X(4, 4, 4) X(8, 2, 3) X(8, 4, 2)
+// (2, 4) has the i-tile of (4, 2) with half the shared-memory and shuffle work per pair.
+#define NBODY_SYM_TILINGS(X) X(2, 4, 8) X(4, 2, 6) X(4, 4, 4) X(8, 2, 3) X(8, 4, 2)
 #define NBODY_SYM64_TILINGS(X) X(2, 1) X(4, 1) X(8, 1) X(4, 2)
 
 cudaError_t launch_sym_force(int precision, const SymLaunch& L, cudaStream_t st) {
@@ -74,7 +75,7 @@ cudaError_t launch_sym_force(int precision, const SymLaunch& L, cudaStream_t st)
   }
 #define NBODY_X(W, R, MINB)                                                                              \
   if (L.block == W * 32 && L.ipt == R) {                                                                 \
-    constexpr size_t smem = sizeof(sym::Smem<W, R, kSymTile>);                                           \
+    constexpr size_t smem = sizeof(sym::Smem<W, R, sym_force_tile(W)>);                                           \
     if (L.law == 0)                                                                                      \
       return L.phi ? launch_pdl_smem(k_force_sym<0, W, R, true, MINB>, L.n_ctas, W * 32, smem, st, L)    \
                    : launch_pdl_smem(k_force_sym<0, W, R, false, MINB>, L.n_ctas, W * 32, smem, st, L);  \
@@ -99,7 +100,7 @@ int sym_force_ctas_per_sm(int precision, int block, int ipt, int law) {
   }
 #define NBODY_X(W, R, MINB)                                                                              \
   if (block == W * 32 && ipt == R) {                                                                     \
-    constexpr size_t smem = sizeof(sym::Smem<W, R, kSymTile>);                                           \
+    constexpr size_t smem = sizeof(sym::Smem<W, R, sym_force_tile(W)>);                                           \
     return law == 0 ? std::min(occupancy_of(k_force_sym<0, W, R, true, MINB>, W * 32, smem),             \
                                occupancy_of(k_force_sym<0, W, R, false, MINB>, W * 32, smem))            \
                     : std::min(occupancy_of(k_force_sym<1, W, R, true, MINB>, W * 32, smem),             \
