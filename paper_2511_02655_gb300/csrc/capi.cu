@@ -44,7 +44,7 @@ struct Tiling {
 };
 constexpr int kSymVariant = 3;
 constexpr double kSymMinBodies = 1024.0;    // typical system size from which the symmetric pass is a candidate
-constexpr double kSymOnlyBodies = 32768.0;  // ... and from which it is the only one (mixed path)
+constexpr double kSymOnlyBodies = 8192.0;  // ... and from which it is the only one (mixed path)
 constexpr double kSymMinBodies64 = 64.0, kSymOnlyBodies64 = 512.0;  // FP64 path
 constexpr int64_t kMaxSymRows = 64;                      // rows of i-tiles a system is cut into at most
 constexpr size_t kMaxSymPartialBytes = size_t(4) << 30;  // cap on the symmetric pass's partial sums
@@ -1122,10 +1122,10 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
   // together because the tail helps some more than others (it changes how the
   // last wave ends): with equal slices several tilings often lie within 0.2%
   // of each other, and the one the tail favours must not be cut by that noise.
-  // Every setting is timed twice, interleaved, the best kept.
+  // Every setting is timed once and those within 3% of the best once more.
   if ((vjp || g.slice == 0) && !large) {
     std::vector<Tiling> settings;
-    for (size_t f = 0; f < top; ++f) {
+    for (size_t f = 0; f < std::min<size_t>(top, is_sym(timed[0].second) ? 3 : 5); ++f) {
       Tiling base = timed[f].second;
       if (vjp && !is_sym(base)) {
         settings.push_back(base);
@@ -1166,8 +1166,10 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
       }
     }
     std::vector<double> lc(settings.size(), 1e300);
-    for (int round = 0; round < 2 && !settings.empty(); ++round)
+    for (int round = 0; round < 2 && !settings.empty(); ++round) {
+      const double limit = round == 0 ? 1e300 : 1.03 * *std::min_element(lc.begin(), lc.end());
       for (size_t k = 0; k < settings.size(); ++k) {
+        if (round == 1 && lc[k] > limit) continue;
         if ((s = install_tiling(c, settings[k], vjp))) return s;
         double cost = 0;
         if ((s = time_tiling(c, vjp, &cost))) return s;
@@ -1177,6 +1179,7 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
                   settings[k].tail, vjp ? c->n_vitems : c->n_items, cost * 1e12);
         lc[k] = std::min(lc[k], cost);
       }
+    }
     double bc = 1e300;
     for (size_t k = 0; k < settings.size(); ++k)
       if (lc[k] < bc) bc = lc[k], bt = settings[k];
