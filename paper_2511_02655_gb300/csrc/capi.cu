@@ -43,6 +43,7 @@ struct Tiling {
                     // row in pieces a third as long, 2 pieces of a row as equal as whole blocks allow)
 };
 constexpr int kSymVariant = 3;
+enum class Potential { kNone = 0, kBodies = 1, kEnergy = 2 };  // as sym::kPhi*
 constexpr double kSymMinBodies = 1024.0;    // typical system size from which the symmetric pass is a candidate
 constexpr double kSymOnlyBodies = 8192.0;  // ... and from which it is the only one (mixed path)
 constexpr double kSymMinBodies64 = 64.0, kSymOnlyBodies64 = 512.0;  // FP64 path
@@ -550,7 +551,7 @@ nbody_status install_tiling(nbody_ctx* c, Tiling t, bool vjp) {
   return NBODY_OK;
 }
 
-SymLaunch sym_launch(nbody_ctx* c, bool vjp, bool phi) {
+SymLaunch sym_launch(nbody_ctx* c, bool vjp, Potential phi) {
   SymLaunch L{};
   const Tiling& t = vjp ? c->vt : c->ft;
   L.stage_x = c->stage.p;
@@ -568,7 +569,7 @@ SymLaunch sym_launch(nbody_ctx* c, bool vjp, bool phi) {
   L.sigma2 = c->cfg.lj_sigma * c->cfg.lj_sigma;
   L.law = c->cfg.law;
   L.block = t.block, L.ipt = t.ipt, L.n_ctas = t.n_ctas;
-  L.phi = phi ? 1 : 0;
+  L.phi = (int)phi;
   L.status = c->status;
   return L;
 }
@@ -602,12 +603,12 @@ PairLaunch pair_launch(nbody_ctx* c, bool vjp, bool refine = true, bool phi = tr
 }
 
 // The all-pairs kernel of the installed tiling.
-cudaError_t launch_pairs(nbody_ctx* c, bool vjp, bool phi, cudaStream_t st) {
+cudaError_t launch_pairs(nbody_ctx* c, bool vjp, Potential phi, cudaStream_t st) {
   if (is_sym(vjp ? c->vt : c->ft)) {
     const SymLaunch L = sym_launch(c, vjp, phi);
     return vjp ? launch_sym_vjp(c->cfg.precision, L, st) : launch_sym_force(c->cfg.precision, L, st);
   }
-  const PairLaunch L = pair_launch(c, vjp, true, phi);
+  const PairLaunch L = pair_launch(c, vjp, true, phi != Potential::kNone);
   return vjp ? launch_vjp(c->cfg.precision, L, st) : launch_force(c->cfg.precision, L, st);
 }
 
@@ -627,7 +628,7 @@ cudaEvent_t pooled_event(nbody_ctx* c) {
 
 // Launches an all-pairs kernel, bracketed by an event pair when profiling an
 // eager (non-capturing) stream.
-nbody_status run_pair(nbody_ctx* c, cudaStream_t st, bool vjp, bool phi = true) {
+nbody_status run_pair(nbody_ctx* c, cudaStream_t st, bool vjp, Potential phi) {
   if (c->n_total == 0) return NBODY_OK;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (c->profiling && !c->capturing) {
@@ -644,10 +645,10 @@ nbody_status run_pair(nbody_ctx* c, cudaStream_t st, bool vjp, bool phi = true) 
   return NBODY_OK;
 }
 
-// phi: whether the potential is needed (an energy record, a phi output); only
-// the packed mixed kernel can skip it, the others always form it.
-nbody_status run_force(nbody_ctx* c, cudaStream_t st, bool phi) { return run_pair(c, st, false, phi); }
-nbody_status run_vjp(nbody_ctx* c, cudaStream_t st) { return run_pair(c, st, true); }
+// phi: the potential that is needed; one-sided kernels form every body's for an energy record too, and
+// only the packed mixed one and the symmetric ones can leave it out
+nbody_status run_force(nbody_ctx* c, cudaStream_t st, Potential phi) { return run_pair(c, st, false, phi); }
+nbody_status run_vjp(nbody_ctx* c, cudaStream_t st) { return run_pair(c, st, true, Potential::kNone); }
 
 
 PostLaunch post_launch(nbody_ctx* c, unsigned mode, double* x, double* v, const double* m, double* a, double* phi) {
@@ -673,6 +674,7 @@ PostLaunch post_launch(nbody_ctx* c, unsigned mode, double* x, double* v, const 
   P.epart = static_cast<double*>(c->epart.p);
   P.status = c->status;
   P.eout = nullptr;
+  P.u_weight = is_sym(c->ft) ? 1.0 : 0.5;  // energy passes: Potential::kEnergy
   P.sys_chunk = c->d_sys_chunk;
   P.n_sys = c->n_sys;
   P.done = c->counter + 4;
@@ -716,7 +718,7 @@ nbody_status enqueue_step(nbody_ctx* c, double* x, double* v, const double* m, d
   if ((s = run_centre(c, x, m, st))) return s;
   if (!a_valid) {
     if ((s = run_post(c, post_launch(c, kStage, x, v, m, a, nullptr), st))) return s;
-    if ((s = run_force(c, st, false))) return s;
+    if ((s = run_force(c, st, Potential::kNone))) return s;
     if ((s = run_post(c, post_launch(c, kCombine, x, v, m, a, nullptr), st))) return s;
   }
   if (n_steps == 0) return NBODY_OK;
@@ -734,7 +736,7 @@ nbody_status enqueue_step(nbody_ctx* c, double* x, double* v, const double* m, d
   int rec = 0;
   for (int k = 0; k < n_steps; ++k) {
     const bool rec_now = elog && every > 0 && (k + 1) % every == 0;
-    if ((s = run_force(c, st, rec_now))) return s;
+    if ((s = run_force(c, st, rec_now ? Potential::kEnergy : Potential::kNone))) return s;
     unsigned mode = kCombine | kKickEnd;
     if (rec_now) mode |= kEnergy;
     if (k + 1 < n_steps) mode |= kDrift | kStage;
@@ -860,7 +862,7 @@ nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
   PairLaunch L = pair_launch(c, vjp);
   const bool sym = is_sym(t);  // timed whole: too large layouts do not come here
   auto launch = [&](const PairLaunch& P) {
-    if (sym) return launch_pairs(c, vjp, true, c->stream);
+    if (sym) return launch_pairs(c, vjp, Potential::kBodies, c->stream);
     return vjp ? launch_vjp(c->cfg.precision, P, c->stream) : launch_force(c->cfg.precision, P, c->stream);
   };
   PostLaunch C{};
@@ -1308,7 +1310,7 @@ nbody_status adjoint_sweep(nbody_ctx* c, const double* x0, const double* v0, con
   NB_CUDA(c, cudaMemcpyAsync(xw, x0, n3b, cudaMemcpyDeviceToDevice, st));
   NB_CUDA(c, cudaMemcpyAsync(vw, v0, n3b, cudaMemcpyDeviceToDevice, st));
   if ((s = run_post(c, post_launch(c, kStage, xw, vw, m, aw, nullptr), st))) return s;
-  if ((s = run_force(c, st, false))) return s;
+  if ((s = run_force(c, st, Potential::kNone))) return s;
   if ((s = run_post(c, post_launch(c, kCombine, xw, vw, m, aw, nullptr), st))) return s;
 
   // one KDK step on (xw, vw, aw), optionally copying x after the drift
@@ -1317,7 +1319,7 @@ nbody_status adjoint_sweep(nbody_ctx* c, const double* x0, const double* v0, con
     PostLaunch P = post_launch(c, kDrift | kStage, xw, vw, m, aw, nullptr);
     P.x_copy = xcopy;
     if ((r = run_post(c, P, st))) return r;
-    if ((r = run_force(c, st, false))) return r;
+    if ((r = run_force(c, st, Potential::kNone))) return r;
     return run_post(c, post_launch(c, kCombine | kKickEnd, xw, vw, m, aw, nullptr), st);
   };
 
@@ -1565,7 +1567,7 @@ nbody_status nbody_forces(nbody_ctx* c, const double* x, const double* m, double
   double* xm = const_cast<double*>(x);
   if ((s = run_centre(c, x, m, c->stream))) return s;
   if ((s = run_post(c, post_launch(c, kStage, xm, nullptr, m, a, nullptr), c->stream))) return s;
-  if ((s = run_force(c, c->stream, phi != nullptr))) return s;
+  if ((s = run_force(c, c->stream, phi ? Potential::kBodies : Potential::kNone))) return s;
   return run_post(c, post_launch(c, kCombine, xm, nullptr, m, a, phi), c->stream);
 }
 
@@ -1653,7 +1655,7 @@ nbody_status nbody_energy(nbody_ctx* c, const double* x, const double* v, const 
   double* as = static_cast<double*>(c->a_scratch.p);
   if ((s = run_centre(c, x, m, c->stream))) return s;
   if ((s = run_post(c, post_launch(c, kStage, xm, vm, m, as, nullptr), c->stream))) return s;
-  if ((s = run_force(c, c->stream, true))) return s;
+  if ((s = run_force(c, c->stream, Potential::kEnergy))) return s;
   // the last CTA writes every system's record (systems without bodies get zeros)
   PostLaunch P = post_launch(c, kCombine | kEnergy, xm, vm, m, as, nullptr);
   P.eout = out;
@@ -1676,7 +1678,7 @@ nbody_status nbody_virial(nbody_ctx* c, const double* x, const double* v, const 
   double* as = static_cast<double*>(c->a_scratch.p);
   if ((s = run_centre(c, x, m, c->stream))) return s;
   if ((s = run_post(c, post_launch(c, kStage, xm, vm, m, as, nullptr), c->stream))) return s;
-  if ((s = run_force(c, c->stream, false))) return s;
+  if ((s = run_force(c, c->stream, Potential::kNone))) return s;
   PostLaunch P = post_launch(c, kCombine | kVirial, xm, vm, m, as, nullptr);
   P.vout = out;
   return run_post(c, P, c->stream);

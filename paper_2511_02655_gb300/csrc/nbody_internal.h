@@ -186,7 +186,8 @@ struct SymLaunch {
   int64_t n_total;
   const SysParam* sys;
   double eps2, sigma2;     // FP64 path
-  int law, block, ipt, n_ctas, phi;
+  int law, block, ipt, n_ctas;
+  int phi;                 // potential: 0 none, 1 of every body, 2 for an energy record (sym::kPhi*)
   int params;              // VJP: also the sums for the G and eps gradients
   unsigned* status;
 };
@@ -281,6 +282,7 @@ struct PostLaunch {
   const SysParam* sys;     // [n_sys] staging origin and scales
   double* epart;           // [n_chunks][kEnergyVals]
   unsigned* status;        // device status word
+  double u_weight;         // kEnergy: U = u_weight sum m phi (1/2, or 1 if phi holds each pair once)
   double* eout;            // kEnergy: nullable [n_sys][9] record formed by the last CTA (null: partials only)
   const double* eprev;     // nullable: chunk partials [n_chunks][kEnergyVals] of the previous step's record,
   double* eprev_out;       //   finished into eprev_out [n_sys][9] by one extra CTA (blockIdx.x == n_chunks)

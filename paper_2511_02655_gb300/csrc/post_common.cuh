@@ -333,7 +333,7 @@ __device__ __forceinline__ bool post_body(const PostLaunch& P, const unsigned mo
     }
     if (mode & kEnergy) {
       e[0] += 0.5 * m * (v0 * v0 + v1 * v1 + v2 * v2);
-      e[1] += 0.5 * m * ph;
+      e[1] += P.u_weight * m * ph;
       e[2] += m * v0, e[3] += m * v1, e[4] += m * v2;
       e[5] += m * (x1 * v2 - x2 * v1);
       e[6] += m * (x2 * v0 - x0 * v2);

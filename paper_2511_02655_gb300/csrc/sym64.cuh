@@ -14,6 +14,7 @@
 
 #include "nbody_internal.h"
 #include "pair_common.cuh"
+#include "sym_common.cuh"
 
 namespace nbody {
 namespace sym64 {
@@ -98,7 +99,7 @@ __device__ __forceinline__ double rcp_f64(const double r2) {
 
 // Pair weights: the force on the i-body is wj d, on the j-body -wi d; t is the potential term
 // (times the other body's mass for gravity). FAST: s^2 is in range.
-template <int LAW, bool FAST, bool PHI>
+template <int LAW, bool FAST, int PHI>
 __device__ __forceinline__ void weights(const double r2, const double s2, const double mj, const double mi, double& wj,
                                         double& wi, double& t) {
   if (LAW == 0) {
@@ -135,7 +136,7 @@ constexpr int kUnroll = 4;
 // The 32 steps of one block. FAST: returns whether the lane met an s^2 out of range, in which case
 // the sums are void and the block is to be repeated without FAST (there is no branch per pair, so
 // that the pairs of several steps overlap).
-template <int LAW, bool SYM, bool MASK, bool PHI, bool FAST, int R>
+template <int LAW, bool SYM, bool MASK, int PHI, bool FAST, int R>
 __device__ __forceinline__ bool block32(const double (&q)[4][kTile / 32][64], const int b, const int jg0, const int lane,
                                         const int ig0, const double (&xi)[R], const double (&yi)[R],
                                         const double (&zi)[R], const double (&mi)[R], const double eps2,
@@ -159,26 +160,27 @@ __device__ __forceinline__ bool block32(const double (&q)[4][kTile / 32][64], co
       ax[r] = fma(dx, wj, ax[r]);
       ay[r] = fma(dy, wj, ay[r]);
       az[r] = fma(dz, wj, az[r]);
+      if (MASK && PHI == sym::kPhiEnergy) t *= 0.5;
       if (PHI) pp[r] = LAW == 0 ? fma(mj, t, pp[r]) : pp[r] + t;
       if (SYM) {
         jx = fma(-dx, wi, jx);
         jy = fma(-dy, wi, jy);
         jz = fma(-dz, wi, jz);
-        if (PHI) jp = LAW == 0 ? fma(mi[r], t, jp) : jp + t;
+        if (PHI == sym::kPhiBoth) jp = LAW == 0 ? fma(mi[r], t, jp) : jp + t;
       }
     }
     if (SYM) {
       jx = __shfl_sync(0xffffffffu, jx, src);
       jy = __shfl_sync(0xffffffffu, jy, src);
       jz = __shfl_sync(0xffffffffu, jz, src);
-      if (PHI) jp = __shfl_sync(0xffffffffu, jp, src);
+      if (PHI == sym::kPhiBoth) jp = __shfl_sync(0xffffffffu, jp, src);
     }
   }
   return out;
 }
 
 // A block with FAST, repeated without it where any lane met an s^2 out of range.
-template <int LAW, bool SYM, bool MASK, bool PHI, int R>
+template <int LAW, bool SYM, bool MASK, int PHI, int R>
 __device__ __forceinline__ void block(const double (&q)[4][kTile / 32][64], const int b, const int jg0, const int lane,
                                       const int ig0, const double (&xi)[R], const double (&yi)[R],
                                       const double (&zi)[R], const double (&mi)[R], const double eps2, const double s2,
@@ -200,9 +202,9 @@ __device__ __forceinline__ void block(const double (&q)[4][kTile / 32][64], cons
 }
 
 // Work items, taken from `counter` until none is left.
-template <int LAW, int W, int R, bool PHI>
+template <int LAW, int W, int R, int PHI>
 __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Smem<W>& sm) {
-  constexpr int T = W * 32, TI = T * R, NC = PHI ? 4 : 3;
+  constexpr int T = W * 32, TI = T * R, NC = PHI == sym::kPhiBoth ? 4 : 3;  // sums of a j-body
   const int tid = (int)threadIdx.x, lane = tid & 31, w = tid >> 5;
   const double4_32a* __restrict__ st = static_cast<const double4_32a*>(L.stage_x);
   double4_32a* part = reinterpret_cast<double4_32a*>(L.part);
@@ -254,7 +256,7 @@ __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Sme
           }
           const int p = 32 * b + lane;
           sm.jacc[w][0][p] = jx, sm.jacc[w][1][p] = jy, sm.jacc[w][2][p] = jz;
-          if (PHI) sm.jacc[w][3][p] = jp;
+          if (PHI == sym::kPhiBoth) sm.jacc[w][3][p] = jp;
         }
         __syncthreads();
         for (int t = tid; t < kTile; t += T) {

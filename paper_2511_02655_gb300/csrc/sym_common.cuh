@@ -48,16 +48,22 @@ struct Smem {
   int item;
 };
 
+// Potential: none, of both bodies, or for an energy record, which needs only sum m phi: each pair's
+// term counted once, at its i-body (and half in the one-sided blocks, which hold a pair twice), one
+// operation and two shuffles less; U is then the whole sum, not half of it.
+enum { kPhiNone = 0, kPhiBoth = 1, kPhiEnergy = 2 };
+
 // One step: the lane's j-pair against its R i-bodies. SYM: also the j-pair's sums;
 // MASK: the self pair is left out (jg: global index of the pair's first body); EQ: equal
 // masses, left out of the sums (staged as 1). mn: the smallest s^2 met.
-template <int LAW, bool SYM, bool MASK, bool PHI, bool EQ, int R>
+template <int LAW, bool SYM, bool MASK, int PHI, bool EQ, int R>
 __device__ __forceinline__ void step(const float4 X, const float4 Z, const int jg, const int ig0, const float2 (&nx)[R],
                                      const float2 (&ny)[R], const float2 (&nz)[R], const float2 (&mi)[R],
                                      const float2 e2, float2 (&ax)[R], float2 (&ay)[R], float2 (&az)[R],
                                      float2 (&pp)[R], float2& jx, float2& jy, float2& jz, float2& jp, float& mn) {
   const float2 xj = make_float2(X.x, X.y), yj = make_float2(X.z, X.w);
   const float2 zj = make_float2(Z.x, Z.y), mj = make_float2(Z.z, Z.w);
+  constexpr bool HALF = MASK && PHI == kPhiEnergy;  // these blocks hold both orders of a pair
   mn = 3.0e38f;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
@@ -76,13 +82,14 @@ __device__ __forceinline__ void step(const float4 X, const float4 Z, const int j
       ax[r] = __ffma2_rn(dx, wj, ax[r]);
       ay[r] = __ffma2_rn(dy, wj, ay[r]);
       az[r] = __ffma2_rn(dz, wj, az[r]);
-      if (PHI) pp[r] = EQ ? __fadd2_rn(pp[r], inv) : __ffma2_rn(mj, inv, pp[r]);
+      const float2 one = HALF ? __fmul2_rn(inv, make_float2(0.5f, 0.5f)) : inv;
+      if (PHI) pp[r] = EQ ? __fadd2_rn(pp[r], one) : __ffma2_rn(mj, one, pp[r]);
       if (SYM) {
         const float2 wi = EQ ? i3 : __fmul2_rn(i3, mi[r]);
         jx = __ffma2_rn(dx, wi, jx);
         jy = __ffma2_rn(dy, wi, jy);
         jz = __ffma2_rn(dz, wi, jz);
-        if (PHI) jp = EQ ? __fadd2_rn(jp, inv) : __ffma2_rn(mi[r], inv, jp);
+        if (PHI == kPhiBoth) jp = EQ ? __fadd2_rn(jp, inv) : __ffma2_rn(mi[r], inv, jp);
       }
     } else {  // u = sigma^2 / r^2 (positions staged in units of sigma)
       const float2 u3 = __fmul2_rn(inv, __fmul2_rn(inv, inv));
@@ -98,8 +105,8 @@ __device__ __forceinline__ void step(const float4 X, const float4 Z, const int j
       }
       if (PHI) {
         const float2 p = __ffma2_rn(u3, make_float2(-1.f, -1.f), u6);
-        pp[r] = __fadd2_rn(pp[r], p);
-        if (SYM) jp = __fadd2_rn(jp, p);
+        pp[r] = HALF ? __ffma2_rn(p, make_float2(0.5f, 0.5f), pp[r]) : __fadd2_rn(pp[r], p);
+        if (SYM && PHI == kPhiBoth) jp = __fadd2_rn(jp, p);
       }
     }
   }
@@ -111,7 +118,7 @@ constexpr int kUnroll = 4;
 
 // The 32 steps of one 64-body block. Returns the lane's bit mask of steps that met
 // a near pair (s^2 below r2c).
-template <int LAW, bool SYM, bool MASK, bool PHI, bool EQ, int R>
+template <int LAW, bool SYM, bool MASK, int PHI, bool EQ, int R>
 __device__ __forceinline__ unsigned block64(const float4* bxy, const float4* bzm, const int jg0, const int lane,
                                             const int ig0, const float2 (&nx)[R], const float2 (&ny)[R],
                                             const float2 (&nz)[R], const float2 (&mi)[R], const float2 e2,
@@ -132,7 +139,7 @@ __device__ __forceinline__ unsigned block64(const float4* bxy, const float4* bzm
     if (mn < r2c) near |= 1u << k;
     if (SYM) {
       pass(jx), pass(jy), pass(jz);
-      if (PHI) pass(jp);
+      if (PHI == kPhiBoth) pass(jp);
     }
   }
   return near;
@@ -160,7 +167,7 @@ __device__ __forceinline__ void pair_terms(const float r2, float& f, float& p) {
 // them, a force pass at 10 000 bodies fell from over 85 us to 65). The i-sums are corrected in registers, the
 // j-sums in the warp's shared entries; lanes that meet the same j-pair in a round take
 // turns in lane order.
-template <int LAW, bool SYM, bool PHI, int R, int NB>
+template <int LAW, bool SYM, int PHI, int R, int NB>
 __device__ __forceinline__ void refine_block(unsigned near, const float4* bxy, const float4* bzm, const int b,
                                              const int jg0, const int j_end, const int lane, const int ig0,
                                              const int i_end, const float2 (&nx)[R], const float2 (&ny)[R],
@@ -204,7 +211,8 @@ __device__ __forceinline__ void refine_block(unsigned near, const float4* bxy, c
         if (LAW == 1) m = 1.f;
         const float uj = fu * mj, vj = fr * mj;
         const float tx = fmaf(ex, vj, -(dx * uj)), ty = fmaf(ey, vj, -(dy * uj)), tz = fmaf(ez, vj, -(dz * uj));
-        const float tp = PHI ? fmaf(mj, pr, -(mj * pu)) : 0.f;
+        const float half = PHI == kPhiEnergy && !SYM ? 0.5f : 1.f;
+        const float tp = PHI ? half * fmaf(mj, pr, -(mj * pu)) : 0.f;
 #pragma unroll
         for (int q = 0; q < R; ++q)
           if (r == q) {
@@ -214,7 +222,7 @@ __device__ __forceinline__ void refine_block(unsigned near, const float4* bxy, c
         if (SYM) {
           const float ui = fu * m, vi = fr * m;
           const float sx = fmaf(ex, vi, -(dx * ui)), sy = fmaf(ey, vi, -(dy * ui)), sz = fmaf(ez, vi, -(dz * ui));
-          const float sp = PHI ? fmaf(m, pr, -(m * pu)) : 0.f;
+          const float sp = PHI == kPhiBoth ? fmaf(m, pr, -(m * pu)) : 0.f;
           if (h)
             cx.y += sx, cy.y += sy, cz.y += sz, cp.y += sp;
           else
@@ -230,7 +238,7 @@ __device__ __forceinline__ void refine_block(unsigned near, const float4* bxy, c
         if (on && turn == t) {
           auto add = [&](float2& s, const float2 c) { s.x += c.x, s.y += c.y; };
           add(jacc[0][b][p], cx), add(jacc[1][b][p], cy), add(jacc[2][b][p], cz);
-          if (PHI) add(jacc[3][b][p], cp);
+          if (PHI == kPhiBoth) add(jacc[3][b][p], cp);
         }
         __syncwarp();
       }
@@ -240,10 +248,10 @@ __device__ __forceinline__ void refine_block(unsigned near, const float4* bxy, c
 
 // Work items, taken from next(SymItem&) until it returns false (called by all threads of the
 // CTA, after a barrier of its own if it is called again).
-template <int LAW, int W, int R, int J, bool PHI, typename Next>
+template <int LAW, int W, int R, int J, int PHI, typename Next>
 __device__ __forceinline__ void items(const SymLaunch& L, Next next, Smem<W, R, J>& sm) {
   constexpr int T = W * 32, NB = J / 64, TI = T * R, LPT = (J + T - 1) / T;
-  constexpr int NC = PHI ? 4 : 3;
+  constexpr int NC = PHI ? 4 : 3, NCJ = PHI == kPhiBoth ? 4 : 3;  // sums of an i-body, of a j-body
   const int tid = (int)threadIdx.x, lane = tid & 31, w = tid >> 5;
   const float4* __restrict__ st = static_cast<const float4*>(L.stage_x);
   const float4* __restrict__ lo = L.stage_lo;
@@ -323,7 +331,7 @@ __device__ __forceinline__ void items(const SymLaunch& L, Next next, Smem<W, R, 
             }
           }
           sm.jacc[w][0][b][lane] = jx, sm.jacc[w][1][b][lane] = jy, sm.jacc[w][2][b][lane] = jz;
-          if (PHI) sm.jacc[w][3][b][lane] = jp;
+          if (PHI == kPhiBoth) sm.jacc[w][3][b][lane] = jp;
           if (__any_sync(0xffffffffu, near != 0u)) {
             __syncwarp();
             if (both)
@@ -350,7 +358,7 @@ __device__ __forceinline__ void items(const SymLaunch& L, Next next, Smem<W, R, 
             if (add) oxy = __ldcg(&oj[j].xy), ozp = __ldcg(&oj[j].zp);
             float h[4] = {oxy.x, oxy.z, ozp.x, ozp.z}, l[4] = {oxy.y, oxy.w, ozp.y, ozp.w};
 #pragma unroll
-            for (int c = 0; c < NC; ++c)
+            for (int c = 0; c < NCJ; ++c)
 #pragma unroll
               for (int u = 0; u < W; ++u) {
                 const float v = (&sm.jacc[u][c][t >> 6][(t & 63) >> 1].x)[t & 1];

@@ -1,5 +1,6 @@
 // Launchers of the symmetric force pass (sym_common.cuh).
 #include <algorithm>
+#include <type_traits>
 
 #include "nbody_internal.h"
 #include "sym64.cuh"
@@ -10,7 +11,7 @@ namespace {
 
 // MINB resident CTAs per SM: 16 warps per SM at R = 4 (<= 128 registers), 24 at R = 2
 // (<= 80 registers).
-template <int LAW, int W, int R, bool PHI, int MINB>
+template <int LAW, int W, int R, int PHI, int MINB>
 __global__ void __launch_bounds__(W * 32, MINB) k_force_sym(const SymLaunch L) {
   extern __shared__ __align__(16) unsigned char raw[];
   auto& sm = *reinterpret_cast<sym::Smem<W, R, sym_force_tile(W)>*>(raw);
@@ -25,7 +26,7 @@ __global__ void __launch_bounds__(W * 32, MINB) k_force_sym(const SymLaunch L) {
   retire_cta(L.counter);
 }
 
-template <int LAW, int W, int R, bool PHI>
+template <int LAW, int W, int R, int PHI>
 __global__ void __launch_bounds__(W * 32) k_force_sym64(const SymLaunch L) {
   __shared__ sym64::Smem<W> sm;
   pdl_wait();
@@ -58,57 +59,59 @@ int occupancy_of(K kern, int block, size_t smem) {
 #define NBODY_SYM_TILINGS(X) X(2, 4, 8) X(4, 2, 6) X(4, 4, 4) X(8, 2, 3) X(8, 4, 2)
 #define NBODY_SYM64_TILINGS(X) X(2, 1) X(4, 1) X(8, 1) X(4, 2)
 
-cudaError_t launch_sym_force(int precision, const SymLaunch& L, cudaStream_t st) {
-  if (L.n_ctas <= 0) return cudaErrorInvalidConfiguration;
-  if (precision == 0) {
-#define NBODY_X(W, R)                                                                       \
-  if (L.block == W * 32 && L.ipt == R) {                                                    \
-    if (L.law == 0)                                                                         \
-      return L.phi ? launch_pdl(k_force_sym64<0, W, R, true>, L.n_ctas, W * 32, st, L)      \
-                   : launch_pdl(k_force_sym64<0, W, R, false>, L.n_ctas, W * 32, st, L);    \
-    return L.phi ? launch_pdl(k_force_sym64<1, W, R, true>, L.n_ctas, W * 32, st, L)        \
-                 : launch_pdl(k_force_sym64<1, W, R, false>, L.n_ctas, W * 32, st, L);      \
-  }
-    NBODY_SYM64_TILINGS(NBODY_X)
-#undef NBODY_X
-    return cudaErrorInvalidConfiguration;
-  }
-#define NBODY_X(W, R, MINB)                                                                              \
-  if (L.block == W * 32 && L.ipt == R) {                                                                 \
-    constexpr size_t smem = sizeof(sym::Smem<W, R, sym_force_tile(W)>);                                           \
-    if (L.law == 0)                                                                                      \
-      return L.phi ? launch_pdl_smem(k_force_sym<0, W, R, true, MINB>, L.n_ctas, W * 32, smem, st, L)    \
-                   : launch_pdl_smem(k_force_sym<0, W, R, false, MINB>, L.n_ctas, W * 32, smem, st, L);  \
-    return L.phi ? launch_pdl_smem(k_force_sym<1, W, R, true, MINB>, L.n_ctas, W * 32, smem, st, L)      \
-                 : launch_pdl_smem(k_force_sym<1, W, R, false, MINB>, L.n_ctas, W * 32, smem, st, L);    \
-  }
-  NBODY_SYM_TILINGS(NBODY_X)
-#undef NBODY_X
-  return cudaErrorInvalidConfiguration;
+// f(law, potential) as integral constants
+template <typename F>
+static auto with_modes(const int law, const int phi, F f) {
+  using std::integral_constant;
+  auto with_law = [&](auto l) {
+    return phi == sym::kPhiBoth     ? f(l, integral_constant<int, sym::kPhiBoth>())
+           : phi == sym::kPhiEnergy ? f(l, integral_constant<int, sym::kPhiEnergy>())
+                                    : f(l, integral_constant<int, sym::kPhiNone>());
+  };
+  return law == 0 ? with_law(integral_constant<int, 0>()) : with_law(integral_constant<int, 1>());
 }
 
+cudaError_t launch_sym_force(int precision, const SymLaunch& L, cudaStream_t st) {
+  if (L.n_ctas <= 0) return cudaErrorInvalidConfiguration;
+  return with_modes(L.law, L.phi, [&](auto law, auto phi) -> cudaError_t {
+    constexpr int LAW = decltype(law)::value, PHI = decltype(phi)::value;
+    if (precision == 0) {
+#define NBODY_X(W, R) \
+  if (L.block == W * 32 && L.ipt == R) return launch_pdl(k_force_sym64<LAW, W, R, PHI>, L.n_ctas, W * 32, st, L);
+      NBODY_SYM64_TILINGS(NBODY_X)
+#undef NBODY_X
+      return cudaErrorInvalidConfiguration;
+    }
+#define NBODY_X(W, R, MINB)            \
+  if (L.block == W * 32 && L.ipt == R) \
+    return launch_pdl_smem(k_force_sym<LAW, W, R, PHI, MINB>, L.n_ctas, W * 32, sizeof(sym::Smem<W, R, sym_force_tile(W)>), st, L);
+    NBODY_SYM_TILINGS(NBODY_X)
+#undef NBODY_X
+    return cudaErrorInvalidConfiguration;
+  });
+}
+
+// the occupancy that every potential mode of the tiling reaches
 int sym_force_ctas_per_sm(int precision, int block, int ipt, int law) {
-  if (precision == 0) {
-#define NBODY_X(W, R)                                                                                                 \
-  if (block == W * 32 && ipt == R)                                                                                    \
-    return law == 0                                                                                                   \
-               ? std::min(occupancy_of(k_force_sym64<0, W, R, true>, W * 32, 0), occupancy_of(k_force_sym64<0, W, R, false>, W * 32, 0))  \
-               : std::min(occupancy_of(k_force_sym64<1, W, R, true>, W * 32, 0), occupancy_of(k_force_sym64<1, W, R, false>, W * 32, 0));
-    NBODY_SYM64_TILINGS(NBODY_X)
+  int least = 1 << 20;
+  for (int mode : {sym::kPhiNone, sym::kPhiBoth, sym::kPhiEnergy})
+    least = std::min(least, with_modes(law, mode, [&](auto l, auto phi) -> int {
+              constexpr int LAW = decltype(l)::value, PHI = decltype(phi)::value;
+              if (precision == 0) {
+#define NBODY_X(W, R) \
+  if (block == W * 32 && ipt == R) return occupancy_of(k_force_sym64<LAW, W, R, PHI>, W * 32, 0);
+                NBODY_SYM64_TILINGS(NBODY_X)
 #undef NBODY_X
-    return 0;
-  }
-#define NBODY_X(W, R, MINB)                                                                              \
-  if (block == W * 32 && ipt == R) {                                                                     \
-    constexpr size_t smem = sizeof(sym::Smem<W, R, sym_force_tile(W)>);                                           \
-    return law == 0 ? std::min(occupancy_of(k_force_sym<0, W, R, true, MINB>, W * 32, smem),             \
-                               occupancy_of(k_force_sym<0, W, R, false, MINB>, W * 32, smem))            \
-                    : std::min(occupancy_of(k_force_sym<1, W, R, true, MINB>, W * 32, smem),             \
-                               occupancy_of(k_force_sym<1, W, R, false, MINB>, W * 32, smem));           \
-  }
-  NBODY_SYM_TILINGS(NBODY_X)
+                return 0;
+              }
+#define NBODY_X(W, R, MINB)        \
+  if (block == W * 32 && ipt == R) \
+    return occupancy_of(k_force_sym<LAW, W, R, PHI, MINB>, W * 32, sizeof(sym::Smem<W, R, sym_force_tile(W)>));
+              NBODY_SYM_TILINGS(NBODY_X)
 #undef NBODY_X
-  return 0;
+              return 0;
+            }));
+  return least;
 }
 
 }  // namespace nbody
