@@ -169,6 +169,7 @@ __global__ void __launch_bounds__(BLOCK) k_vjp_mixed(const PairLaunch L) {
   fpair4* __restrict__ part = reinterpret_cast<fpair4*>(L.part);
   const float4* __restrict__ slo = L.stage_lo;
 
+  pdl_wait();
   for (;;) {
     const int it = next_item(L.counter, &s_item);
     if (it >= L.n_items) break;
@@ -281,6 +282,7 @@ __global__ void __launch_bounds__(BLOCK) k_vjp_mixed(const PairLaunch L) {
       }
     }
   }
+  pdl_trigger();
   retire_cta(L.counter);
 }
 
@@ -295,6 +297,7 @@ __global__ void __launch_bounds__(BLOCK) k_vjp_fp64(const PairLaunch L) {
   double4_32a* __restrict__ part = reinterpret_cast<double4_32a*>(L.part);
   const double eps2 = L.eps2;
 
+  pdl_wait();
   for (;;) {
     const int it = next_item(L.counter, &s_item);
     if (it >= L.n_items) break;
@@ -369,6 +372,7 @@ __global__ void __launch_bounds__(BLOCK) k_vjp_fp64(const PairLaunch L) {
       }
     }
   }
+  pdl_trigger();
   retire_cta(L.counter);
 }
 
@@ -445,6 +449,7 @@ __global__ void __launch_bounds__(BLOCK) k_vjp_mixed2(const PairLaunch L) {
     twx[b][t] = 0.f, twy[b][t] = 0.f, twz[b][t] = 0.f;
   };
 
+  pdl_wait();
   for (;;) {
     const int it = next_item(L.counter, &s_item);
     if (it >= L.n_items) break;
@@ -598,6 +603,7 @@ __global__ void __launch_bounds__(BLOCK) k_vjp_mixed2(const PairLaunch L) {
       }
     }
   }
+  pdl_trigger();
   retire_cta(L.counter);
 }
 
@@ -619,18 +625,17 @@ cudaError_t launch_vjp(int precision, const PairLaunch& L, cudaStream_t st) {
 #define NBODY_X(B, R, J)                                                 \
   if (L.block == B && L.ipt == R && L.jtile == J) {                      \
     if (precision == 1 && L.variant == 1 && L.params)                    \
-      k_vjp_mixed2<B, R, J, true><<<L.n_ctas, B, 0, st>>>(L);            \
+      return launch_pdl(k_vjp_mixed2<B, R, J, true>, L.n_ctas, B, st, L); \
     else if (precision == 1 && L.variant == 1)                           \
-      k_vjp_mixed2<B, R, J, false><<<L.n_ctas, B, 0, st>>>(L);           \
+      return launch_pdl(k_vjp_mixed2<B, R, J, false>, L.n_ctas, B, st, L); \
     else if (precision == 1 && L.params)                                 \
-      k_vjp_mixed<B, R, J, true><<<L.n_ctas, B, 0, st>>>(L);             \
+      return launch_pdl(k_vjp_mixed<B, R, J, true>, L.n_ctas, B, st, L); \
     else if (precision == 1)                                             \
-      k_vjp_mixed<B, R, J, false><<<L.n_ctas, B, 0, st>>>(L);            \
+      return launch_pdl(k_vjp_mixed<B, R, J, false>, L.n_ctas, B, st, L); \
     else if (L.params)                                                   \
-      k_vjp_fp64<B, R, J, true><<<L.n_ctas, B, 0, st>>>(L);              \
+      return launch_pdl(k_vjp_fp64<B, R, J, true>, L.n_ctas, B, st, L); \
     else                                                                 \
-      k_vjp_fp64<B, R, J, false><<<L.n_ctas, B, 0, st>>>(L);             \
-    return cudaGetLastError();                                           \
+      return launch_pdl(k_vjp_fp64<B, R, J, false>, L.n_ctas, B, st, L); \
   }
   NBODY_VJP_TILINGS(NBODY_X)
 #undef NBODY_X

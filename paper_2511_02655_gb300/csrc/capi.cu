@@ -1313,28 +1313,34 @@ nbody_status adjoint_sweep(nbody_ctx* c, const double* x0, const double* v0, con
   if ((s = run_force(c, st, Potential::kNone))) return s;
   if ((s = run_post(c, post_launch(c, kCombine, xw, vw, m, aw, nullptr), st))) return s;
 
-  // one KDK step on (xw, vw, aw), optionally copying x after the drift
-  auto step = [&](double* xcopy) -> nbody_status {
+  // `steps` KDK steps on (xw, vw, aw); the positions after step t go to copies + t * n3 as well if
+  // copies is given. The closing half-kick of a step and the opening one of the next, with its drift and
+  // staging, are one kernel, so a step is two launches.
+  auto run_steps = [&](int steps, double* copies) -> nbody_status {
     nbody_status r;
+    if (steps <= 0) return NBODY_OK;
     PostLaunch P = post_launch(c, kDrift | kStage, xw, vw, m, aw, nullptr);
-    P.x_copy = xcopy;
+    P.x_copy = copies;
     if ((r = run_post(c, P, st))) return r;
-    if ((r = run_force(c, st, Potential::kNone))) return r;
-    return run_post(c, post_launch(c, kCombine | kKickEnd, xw, vw, m, aw, nullptr), st);
+    for (int t = 0; t < steps; ++t) {
+      if ((r = run_force(c, st, Potential::kNone))) return r;
+      const bool more = t + 1 < steps;
+      P = post_launch(c, kCombine | kKickEnd | (more ? kDrift | kStage : 0u), xw, vw, m, aw, nullptr);
+      if (more && copies) P.x_copy = copies + (size_t)(t + 1) * n3;
+      if ((r = run_post(c, P, st))) return r;
+    }
+    return NBODY_OK;
   };
 
   // forward pass: checkpoints (x, v, a) at the start of every segment; it stops at
   // the last checkpoint, since the reverse sweep recomputes the last segment anyway
   std::unique_ptr<NvtxRange> fwd(new NvtxRange(c->nvtx, "forward"));
-  const int last_ckpt = (nseg - 1) * K;
-  for (int t = 0; t <= last_ckpt; ++t) {
-    if (t % K == 0) {
-      double* cp = ck + (size_t)(t / K) * 3 * n3;
-      NB_CUDA(c, cudaMemcpyAsync(cp, xw, n3b, cudaMemcpyDeviceToDevice, st));
-      NB_CUDA(c, cudaMemcpyAsync(cp + n3, vw, n3b, cudaMemcpyDeviceToDevice, st));
-      NB_CUDA(c, cudaMemcpyAsync(cp + 2 * n3, aw, n3b, cudaMemcpyDeviceToDevice, st));
-    }
-    if (t < last_ckpt && (s = step(nullptr))) return s;
+  for (int k = 0; k < nseg; ++k) {
+    double* cp = ck + (size_t)k * 3 * n3;
+    NB_CUDA(c, cudaMemcpyAsync(cp, xw, n3b, cudaMemcpyDeviceToDevice, st));
+    NB_CUDA(c, cudaMemcpyAsync(cp + n3, vw, n3b, cudaMemcpyDeviceToDevice, st));
+    NB_CUDA(c, cudaMemcpyAsync(cp + 2 * n3, aw, n3b, cudaMemcpyDeviceToDevice, st));
+    if (k + 1 < nseg && (s = run_steps(K, nullptr))) return s;
   }
 
   fwd.reset();
@@ -1378,8 +1384,7 @@ nbody_status adjoint_sweep(nbody_ctx* c, const double* x0, const double* v0, con
     // positions s0 .. top; a segment's end state is the next segment's start, whose
     // VJP that segment has already taken, so only the last segment steps to its end
     const int top = (k == nseg - 1) ? s1 : s1 - 1;
-    for (int t = 0; t < top - s0; ++t)
-      if ((s = step(X + (size_t)(t + 1) * n3))) return s;
+    if ((s = run_steps(top - s0, X + n3))) return s;
     NB_CUDA(c, launch_stage_vec(vch, nch, c->cfg.precision, X + (size_t)(top - s0) * n3, m,
                                 A.sys, c->stage.p, c->stage_lo.p, 1, c->n_total,
                                 c->n_sys, c->status, st));

@@ -122,7 +122,6 @@ __global__ void __launch_bounds__(kSumThreads) k_na_sums(const double* x, const 
   constexpr int NW = kSumThreads / 32;
   __shared__ Extent ext[NW];
   pdl_wait();
-  pdl_trigger();
   const Scratch S = scratch_of(scratch, n);
   double v[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   Extent q{0u, 0u, 1u};
@@ -146,7 +145,6 @@ __global__ void __launch_bounds__(256) k_na_stage(const double* x, const double*
                                                   const double eps, unsigned char* scratch) {
   __shared__ SysParam sp;
   pdl_wait();
-  pdl_trigger();
   const Scratch S = scratch_of(scratch, n);
   if (threadIdx.x < 32) {
     double w[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};

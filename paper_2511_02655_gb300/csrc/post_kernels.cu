@@ -28,7 +28,6 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
     double d[4][kSlotGroups - 1][CB];
   } red;
   pdl_wait();     // the force kernel before it has finished writing the partials
-  pdl_trigger();  // the next force kernel may be scheduled once every CTA has started
   if ((int)blockIdx.x == P.n_chunks) {
     // the extra CTA: the previous step's energy record from its chunk partials
     systems_final<kEnergyVals, kSlotGroups * CB>(P.sys_chunk, P.n_sys, P.eprev, P.n_chunks, P.status,
@@ -116,6 +115,7 @@ __global__ void __launch_bounds__(CB) k_centre(const CentreLaunch C) {
   constexpr int NW = CB / 32;
   __shared__ Extent ext[NW];
   const int lane = (int)threadIdx.x & 31, wid = (int)threadIdx.x >> 5;
+  pdl_wait();
   Chunk c = C.chunks[blockIdx.x];
   if (!chunk_ok(c, C.n_total, C.n_sys, 0, C.status)) c.begin = c.end = 0;  // NBODY_DEBUG builds only
   double v[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
@@ -178,6 +178,7 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_adj_update(const AdjLaunch
     SlotSums<CB> f[10];
     double d[10][kSlotGroups - 1][CB];
   } red;
+  pdl_wait();     // the VJP kernel has finished writing the partials
   Chunk c = A.chunks[blockIdx.x];
   if (!chunk_ok(c, A.n_total, A.n_sys, A.part_rows, A.status)) c.begin = c.end = 0;  // NBODY_DEBUG builds only
   const SysParam& sp = A.sys[c.sys];
@@ -283,6 +284,7 @@ __global__ void __launch_bounds__(CB) k_stage_vec(const Chunk* chunks, int preci
                                                   const double* m, const SysParam* sys, void* stage,
                                                             void* stage_lo, int as_position, const int64_t n_total,
                                                             const int n_sys, unsigned* status) {
+  pdl_wait();
   Chunk c = chunks[blockIdx.x];
   if (!chunk_ok(c, n_total, n_sys, 0, status)) c.begin = c.end = 0;  // NBODY_DEBUG builds only
   const SysParam& sp = sys[c.sys];
@@ -344,8 +346,7 @@ cudaError_t launch_centre(const CentreLaunch& C, cudaStream_t st) {
   if (C.n_sys <= 0 || C.n_chunks <= 0) return cudaSuccess;
   return with_chunk(C.n_total, [&](auto cb) {
     constexpr int CB = decltype(cb)::value;
-    k_centre<CB><<<C.n_chunks, CB, 0, st>>>(C);
-    return cudaGetLastError();
+    return launch_pdl(k_centre<CB>, C.n_chunks, CB, st, C);
   });
 }
 
@@ -353,8 +354,7 @@ cudaError_t launch_adj_update(const AdjLaunch& A, cudaStream_t st) {
   if (A.n_chunks <= 0) return cudaSuccess;
   return with_chunk(A.n_total, [&](auto cb) {
     constexpr int CB = decltype(cb)::value;
-    k_adj_update<CB><<<A.n_chunks, kSlotGroups * CB, 0, st>>>(A);
-    return cudaGetLastError();
+    return launch_pdl(k_adj_update<CB>, A.n_chunks, kSlotGroups * CB, st, A);
   });
 }
 
@@ -364,9 +364,8 @@ cudaError_t launch_stage_vec(const Chunk* chunks, int n_chunks, int precision, c
   if (n_chunks <= 0) return cudaSuccess;
   return with_chunk(n_total, [&](auto cb) {
     constexpr int CB = decltype(cb)::value;
-    k_stage_vec<CB><<<n_chunks, CB, 0, st>>>(chunks, precision, vec, m, sys, stage, stage_lo, as_position, n_total,
-                                             n_sys, status);
-    return cudaGetLastError();
+    return launch_pdl(k_stage_vec<CB>, n_chunks, CB, st, chunks, precision, vec, m, sys, stage, stage_lo, as_position,
+                      n_total, n_sys, status);
   });
 }
 
