@@ -135,6 +135,9 @@ struct nbody_ctx {
   Chunk* d_chunks = nullptr;
   Chunk* d_vchunks = nullptr;  // same chunks, VJP tiling's slice counts
   int32_t* d_sys_chunk = nullptr;
+  int n_cchunks = 0;           // chunks of kChunk bodies of the staging origin's sums
+  Chunk* d_cchunks = nullptr;
+  int32_t* d_csys_chunk = nullptr;
   int64_t* d_off = nullptr;
 
   // force work list
@@ -692,9 +695,9 @@ nbody_status run_post(nbody_ctx* c, const PostLaunch& P, cudaStream_t st) {
 nbody_status run_centre(nbody_ctx* c, const double* x, const double* m, cudaStream_t st) {
   if (c->cfg.precision != NBODY_MIXED || c->n_total == 0) return NBODY_OK;
   CentreLaunch C{};
-  C.chunks = c->d_chunks;
-  C.n_chunks = (int32_t)c->chunks.size();
-  C.sys_chunk = c->d_sys_chunk;
+  C.chunks = c->d_cchunks;
+  C.n_chunks = c->n_cchunks;
+  C.sys_chunk = c->d_csys_chunk;
   C.off = c->d_off;
   C.n_sys = c->n_sys;
   C.x = x, C.m = m;
@@ -1232,6 +1235,8 @@ void free_ctx(nbody_ctx* c) {
   if (c->d_chunks) cudaFree(c->d_chunks);
   if (c->d_vchunks) cudaFree(c->d_vchunks);
   if (c->d_sys_chunk) cudaFree(c->d_sys_chunk);
+  if (c->d_cchunks) cudaFree(c->d_cchunks);
+  if (c->d_csys_chunk) cudaFree(c->d_csys_chunk);
   if (c->d_off) cudaFree(c->d_off);
   if (c->d_items) cudaFree(c->d_items);
   if (c->d_vitems) cudaFree(c->d_vitems);
@@ -1494,15 +1499,21 @@ nbody_status nbody_init(nbody_ctx** out, const nbody_config* cfg, int64_t n_syst
   c->offsets.assign(offsets, offsets + n_systems + 1);
   c->n_total = offsets[n_systems];
 
-  // chunks: runs of <= chunk bodies inside one system
-  const int64_t chunk = chunk_bodies(c->n_total);
-  c->sys_chunk.assign(c->n_sys + 1, 0);
-  for (int s = 0; s < c->n_sys; ++s) {
-    c->sys_chunk[s] = (int32_t)c->chunks.size();
-    for (int64_t b = offsets[s]; b < offsets[s + 1]; b += chunk)
-      c->chunks.push_back(Chunk{s, (int32_t)b, (int32_t)std::min<int64_t>(offsets[s + 1], b + chunk), 1, 0, 0, 0});
-  }
-  c->sys_chunk[c->n_sys] = (int32_t)c->chunks.size();
+  // chunks: runs of <= `bodies` bodies inside one system, and each system's range of them
+  auto cut = [&](int64_t bodies, std::vector<Chunk>& chunks, std::vector<int32_t>& sys_chunk) {
+    sys_chunk.assign(c->n_sys + 1, 0);
+    for (int s = 0; s < c->n_sys; ++s) {
+      sys_chunk[s] = (int32_t)chunks.size();
+      for (int64_t b = offsets[s]; b < offsets[s + 1]; b += bodies)
+        chunks.push_back(Chunk{s, (int32_t)b, (int32_t)std::min<int64_t>(offsets[s + 1], b + bodies), 1, 0, 0, 0});
+    }
+    sys_chunk[c->n_sys] = (int32_t)chunks.size();
+  };
+  cut(chunk_bodies(c->n_total), c->chunks, c->sys_chunk);
+  std::vector<Chunk> cchunks;
+  std::vector<int32_t> csys_chunk;
+  cut(kChunk, cchunks, csys_chunk);
+  c->n_cchunks = (int)cchunks.size();
 
   nbody_status s;
   auto bail = [&](nbody_status st) {
@@ -1530,14 +1541,18 @@ nbody_status nbody_init(nbody_ctx** out, const nbody_config* cfg, int64_t n_syst
   *c->h_status = 0u;
   if ((s = upload_plain_staging(c))) return bail(s);
   if (cudaMalloc(&c->d_off, (n_systems + 1) * sizeof(int64_t)) != cudaSuccess ||
-      cudaMalloc(&c->d_sys_chunk, (n_systems + 1) * sizeof(int32_t)) != cudaSuccess) {
+      cudaMalloc(&c->d_sys_chunk, (n_systems + 1) * sizeof(int32_t)) != cudaSuccess ||
+      cudaMalloc(&c->d_csys_chunk, (n_systems + 1) * sizeof(int32_t)) != cudaSuccess) {
     cudaGetLastError();
     return bail(fail(c, NBODY_ENOMEM, "cudaMalloc of layout tables failed"));
   }
   if (cudaMemcpy(c->d_off, offsets, (n_systems + 1) * sizeof(int64_t), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(c->d_sys_chunk, c->sys_chunk.data(), (n_systems + 1) * sizeof(int32_t), cudaMemcpyHostToDevice) !=
+          cudaSuccess ||
+      cudaMemcpy(c->d_csys_chunk, csys_chunk.data(), (n_systems + 1) * sizeof(int32_t), cudaMemcpyHostToDevice) !=
           cudaSuccess)
     return bail(fail(c, NBODY_ECUDA, "upload of layout tables failed"));
+  if ((s = upload_chunks(c, cchunks, &c->d_cchunks))) return bail(s);
 
   const bool fixed_variant = cfg->precision == NBODY_FP64 || cfg->variant != 0 || cfg->law == NBODY_LAW_LJ;
   if (c->n_total > 0 && (cfg->block == 0 || cfg->i_per_thread == 0 || cfg->j_tile == 0 || !fixed_variant)) {

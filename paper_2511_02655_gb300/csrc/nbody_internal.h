@@ -58,17 +58,17 @@ struct SymItem {
 };
 
 // The O(N) kernels do their float64 work on GB300's FP64 pipe (about 1/75 of
-// the FP32 rate), so that part of their time is the float64 operations per SM:
-// chunks of 64 bodies spread even small systems (10 000 bodies: 157 CTAs) over
-// every SM. Above kManyBodies every SM has several chunks anyway and 128 bodies
-// per chunk halve the chunk partials that one CTA sums into a record. The rest of
-// the time is the latency of reading each body's partials; a combining CTA has
-// kSlotGroups threads per body, each adding every kSlotGroups-th slice, so a
-// body's loads are in flight together.
-constexpr int kChunkSmall = 64, kChunk = 128;  // bodies per chunk (at most kChunk)
-constexpr int64_t kManyBodies = 32768;
-constexpr int kSlotGroups = 4;                 // threads per body that add its slices
-inline int chunk_bodies(int64_t n_total) { return n_total > kManyBodies ? kChunk : kChunkSmall; }
+// the FP32 rate), so that part of their time is the float64 operations per SM: the
+// smaller the system, the fewer bodies a chunk has, so that its CTAs cover every
+// SM (1024 bodies: 64 CTAs). The rest of the time is the latency of reading each
+// body's partials; a combining CTA has several threads per body (slot groups), each
+// adding every groups-th slice, so that a body's loads are in flight together.
+// Larger systems fill the SMs anyway, and their larger chunks leave fewer chunk
+// partials for one CTA to sum into a record.
+constexpr int kChunk = 128;  // bodies per chunk at most, and of the staging origin's sums
+inline int chunk_bodies(int64_t n_total) {
+  return n_total <= 4096 ? 16 : n_total <= 16384 ? 32 : n_total <= 32768 ? 64 : kChunk;
+}
 constexpr int kEnergyVals = 8;      // K, U, Px, Py, Pz, Lx, Ly, Lz per chunk
 constexpr int kAdjVals = 8;         // VJP partial values per body per slice
 

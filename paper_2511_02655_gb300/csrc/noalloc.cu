@@ -267,8 +267,8 @@ __global__ void __launch_bounds__(128, 3) k_na_force_one(const int n, const int 
 // four threads per body, as in the O(N) kernels of the context path.
 __global__ void __launch_bounds__(256) k_na_combine(const SymPlan P, const int n, const int slices, const double G,
                                                     double* a, double* phi, unsigned char* scratch) {
-  constexpr int CB = 64;
-  __shared__ SlotSums<CB> red[4];
+  constexpr int CB = 64, SG = 4;
+  __shared__ SlotSums<CB, SG> red[4];
   pdl_wait();
   pdl_trigger();
   const Scratch S = scratch_of(scratch, n);
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(256) k_na_combine(const SymPlan P, const int n
     const int ns = P.H > 0 ? P.slots(i / P.H) : slices;
     const fpair4* p = S.part + i;
 #pragma unroll 8
-    for (int s = g; s < ns; s += kSlotGroups) add_slot(p[(int64_t)s * n], h, l);
+    for (int s = g; s < ns; s += SG) add_slot(p[(int64_t)s * n], h, l);
   }
   add_groups(red, g, b, h, l);
   if (g != 0 || i >= n) return;

@@ -61,19 +61,19 @@ __device__ __forceinline__ void block_sum(double (&v)[NV]) {
   }
 }
 
-// The slices of one body, added by kSlotGroups threads (thread group g of the CTA
-// takes slices g, g + kSlotGroups, ...) and then over the groups in order, all of it
+// The slices of one body, added by SG threads (thread group g of the CTA
+// takes slices g, g + SG, ...) and then over the groups in order, all of it
 // for NC components per slice. Mixed: compensated float32 pairs, added as pairs on
 // the FP32 pipe (TwoSum of the hi parts, the lo parts and rounding errors summed
 // alongside). Valid in group 0; every thread of the CTA calls it.
-template <int CB>
+template <int CB, int SG>
 struct SlotSums {
-  float h[kSlotGroups - 1][CB];
-  float l[kSlotGroups - 1][CB];
+  float h[SG - 1][CB];
+  float l[SG - 1][CB];
 };
 
-template <int NC, int CB>
-__device__ __forceinline__ void add_groups(SlotSums<CB> (&red)[NC], const int g, const int b, float (&h)[NC],
+template <int NC, int CB, int SG>
+__device__ __forceinline__ void add_groups(SlotSums<CB, SG> (&red)[NC], const int g, const int b, float (&h)[NC],
                                            float (&l)[NC]) {
   if (g > 0) {
 #pragma unroll
@@ -82,7 +82,7 @@ __device__ __forceinline__ void add_groups(SlotSums<CB> (&red)[NC], const int g,
   __syncthreads();
   if (g == 0) {
 #pragma unroll
-    for (int k = 0; k < kSlotGroups - 1; ++k)
+    for (int k = 0; k < SG - 1; ++k)
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         two_sum_acc(h[c], l[c], red[c].h[k][b]);
@@ -91,8 +91,8 @@ __device__ __forceinline__ void add_groups(SlotSums<CB> (&red)[NC], const int g,
   }
 }
 
-template <int NC, int CB>
-__device__ __forceinline__ void add_groups(double (&red)[NC][kSlotGroups - 1][CB], const int g, const int b,
+template <int NC, int CB, int SG1>
+__device__ __forceinline__ void add_groups(double (&red)[NC][SG1][CB], const int g, const int b,
                                            double (&s)[NC]) {
   if (g > 0) {
 #pragma unroll
@@ -101,7 +101,7 @@ __device__ __forceinline__ void add_groups(double (&red)[NC][kSlotGroups - 1][CB
   __syncthreads();
   if (g == 0) {
 #pragma unroll
-    for (int k = 0; k < kSlotGroups - 1; ++k)
+    for (int k = 0; k < SG1; ++k)
 #pragma unroll
       for (int c = 0; c < NC; ++c) s[c] += red[c][k][b];
   }
@@ -287,6 +287,23 @@ __device__ __forceinline__ void emit_energy(double* out, const int sy, const dou
   for (int k = 2; k < kEnergyVals; ++k) o[k + 1] = v[k];
 }
 
+// What post_body reads of body i, loaded before the slices are added, so that these
+// loads and the slices' are in flight together (x, v, m and a are distinct arrays).
+struct BodyIn {
+  double x0 = 0.0, x1 = 0.0, x2 = 0.0, v0 = 0.0, v1 = 0.0, v2 = 0.0, m = 0.0, a0 = 0.0, a1 = 0.0, a2 = 0.0;
+};
+__device__ __forceinline__ BodyIn load_body(const PostLaunch& P, const unsigned mode, const int i) {
+  BodyIn b;
+  const bool need_x = mode & (kKickEnd | kEnergy | kDrift | kStage | kVirial);
+  const bool need_v = mode & (kKickEnd | kEnergy | kDrift | kVirial);
+  if (need_x) b.x0 = P.x[3 * i + 0], b.x1 = P.x[3 * i + 1], b.x2 = P.x[3 * i + 2];
+  if (need_v) b.v0 = P.v[3 * i + 0], b.v1 = P.v[3 * i + 1], b.v2 = P.v[3 * i + 2];
+  if (need_x || (mode & kCombine && P.law != 0)) b.m = P.m[i];
+  if (!(mode & kCombine) && (mode & (kKickEnd | kDrift)))
+    b.a0 = P.a[3 * i + 0], b.a1 = P.a[3 * i + 1], b.a2 = P.a[3 * i + 2];
+  return b;
+}
+
 // The O(N) work of one body i in the PostMode bits of `mode`: with kCombine its
 // summed partials (sx, sy, sz, sp) become a = G S (or the Lennard-Jones
 // scaling) and phi; then the closing half-kick, the energy or virial terms
@@ -294,18 +311,11 @@ __device__ __forceinline__ void emit_energy(double* out, const int sy, const dou
 // the walls), and the staging entry of the new position. s holds the system's
 // staging origin and scales. Returns true if a combined value is not finite.
 __device__ __forceinline__ bool post_body(const PostLaunch& P, const unsigned mode, const int i, const SysParam& s,
-                                          const double sx, const double sy, const double sz, const double sp,
-                                          double (&e)[kEnergyVals]) {
+                                          const BodyIn& in, const double sx, const double sy, const double sz,
+                                          const double sp, double (&e)[kEnergyVals]) {
   bool bad = false;
-  // every load of the body first, so that they are in flight together (x, v, m
-  // and a are distinct arrays; nothing below is stored before it is read)
-  const bool need_x = mode & (kKickEnd | kEnergy | kDrift | kStage | kVirial);
-  const bool need_v = mode & (kKickEnd | kEnergy | kDrift | kVirial);
-  const bool need_m = need_x || (mode & kCombine && P.law != 0);
-  double x0 = 0.0, x1 = 0.0, x2 = 0.0, v0 = 0.0, v1 = 0.0, v2 = 0.0, m = 0.0;
-  if (need_x) x0 = P.x[3 * i + 0], x1 = P.x[3 * i + 1], x2 = P.x[3 * i + 2];
-  if (need_v) v0 = P.v[3 * i + 0], v1 = P.v[3 * i + 1], v2 = P.v[3 * i + 2];
-  if (need_m) m = P.m[i];
+  double x0 = in.x0, x1 = in.x1, x2 = in.x2, v0 = in.v0, v1 = in.v1, v2 = in.v2;
+  const double m = in.m;
   double ax = 0.0, ay = 0.0, az = 0.0, ph = 0.0;
   if (mode & kCombine) {
     if (P.law == 0) {  // softened gravity; the staged sums carry mscale / scale^2 (mscale / scale)
@@ -320,7 +330,7 @@ __device__ __forceinline__ bool post_body(const PostLaunch& P, const unsigned mo
     if (P.phi) P.phi[i] = ph;
     bad = !(isfinite(ax) && isfinite(ay) && isfinite(az) && isfinite(ph));
   } else if (mode & (kKickEnd | kDrift)) {
-    ax = P.a[3 * i + 0], ay = P.a[3 * i + 1], az = P.a[3 * i + 2];
+    ax = in.a0, ay = in.a1, az = in.a2;
   }
   if (mode & kVirial) {
     e[0] += 0.5 * m * (v0 * v0 + v1 * v1 + v2 * v2);

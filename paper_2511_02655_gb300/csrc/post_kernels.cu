@@ -15,28 +15,35 @@
 namespace nbody {
 namespace {
 
-// One CTA per chunk, kSlotGroups threads per body to add the slices and one to do
-// the rest (a CTA of one thread per body when the mode combines nothing). Adding
-// the slices is a chain of 32-byte loads from L2, and that latency bounds the
-// kernel: on the 10 000-body Lennard-Jones gas (40 slices, 157 chunks) a step
-// took 89 us with one thread per body and 128-body chunks and takes 84 us with
-// four threads per body and 64-body chunks.
+// Threads that add a chunk's terms: its bodies', or a whole warp (others hold zeros)
 template <int CB>
-__global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
+constexpr unsigned kSumThreads = CB < 32 ? 32 : CB;
+
+// One CTA per chunk, SG threads per body to add the slices and one to do
+// the rest (a CTA of one thread per body when the mode combines nothing). Adding
+// the slices is a chain of 32-byte loads from L2, and that latency and the FP64 pipe
+// bound the kernel: on the 10 000-body Lennard-Jones gas (40 slices) a step took 89 us
+// with one thread per body and 128-body chunks and 84 us with four and 64; with
+// 32-body chunks, eight threads and the body's own loads ahead of the slices' it went
+// from 70.5 to 69.1 us (on top of a faster force pass); 1024 bodies: 13.7 to 12.2 us.
+// At 65 536 bodies eight threads cost 1% (1024-thread CTAs), so chunks of 128 keep four.
+template <int CB, int SG>
+__global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
   __shared__ union {
-    SlotSums<CB> f[4];
-    double d[4][kSlotGroups - 1][CB];
+    SlotSums<CB, SG> f[4];
+    double d[4][SG - 1][CB];
   } red;
-  pdl_wait();     // the force kernel before it has finished writing the partials
+  Chunk c{};  // (the chunk list is as old as the context: read while the kernel before finishes)
+  if ((int)blockIdx.x < P.n_chunks) c = P.chunks[blockIdx.x];
+  pdl_wait();  // the force kernel before it has finished writing the partials
   if ((int)blockIdx.x == P.n_chunks) {
     // the extra CTA: the previous step's energy record from its chunk partials
-    systems_final<kEnergyVals, kSlotGroups * CB>(P.sys_chunk, P.n_sys, P.eprev, P.n_chunks, P.status,
+    systems_final<kEnergyVals, SG * CB>(P.sys_chunk, P.n_sys, P.eprev, P.n_chunks, P.status,
                                              [&](int sy, const double (&v)[kEnergyVals]) {
                                                emit_energy(P.eprev_out, sy, v);
                                              });
     return;
   }
-  Chunk c = P.chunks[blockIdx.x];
   if (!chunk_ok(c, P.n_total, P.n_sys, (P.mode & kCombine) ? P.part_rows : 0, P.status))
     c.begin = c.end = 0;  // NBODY_DEBUG builds only: processed as an empty chunk
   const SysParam& sp = P.sys[c.sys];
@@ -46,7 +53,9 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
   const unsigned mode = P.mode;
   const int b = (int)threadIdx.x % CB, g = (int)threadIdx.x / CB;
   const int i = c.begin + b;
-  const bool live = i < c.end;
+  const bool live = i < c.end && g < SG;  // (a chunk of 16 has half a warp without bodies in a pass that combines nothing)
+  BodyIn in;
+  if (g == 0 && live) in = load_body(P, mode, i);
 
   double sx = 0.0, sy = 0.0, sz = 0.0, sphi = 0.0;
   if ((mode & kCombine) && P.precision == 1) {
@@ -54,7 +63,7 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
     float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
     if (live) {
 #pragma unroll 8
-      for (int s = g; s < c.n_slices; s += kSlotGroups) add_slot(fp[(int64_t)s * c.stride], h, l);
+      for (int s = g; s < c.n_slices; s += SG) add_slot(fp[(int64_t)s * c.stride], h, l);
     }
     add_groups(red.f, g, b, h, l);
     if (g == 0) {
@@ -66,7 +75,7 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
     double s4[4] = {0.0, 0.0, 0.0, 0.0};
     if (live) {
 #pragma unroll 8
-      for (int s = g; s < c.n_slices; s += kSlotGroups) {
+      for (int s = g; s < c.n_slices; s += SG) {
         const double4_32a q = part[(int64_t)s * c.stride];
         s4[0] += q.x, s4[1] += q.y, s4[2] += q.z, s4[3] += q.w;
       }
@@ -74,15 +83,15 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
     add_groups(red.d, g, b, s4);
     sx = s4[0], sy = s4[1], sz = s4[2], sphi = s4[3];
   }
-  if (g == 0 && live && post_body(P, mode, i, sp, sx, sy, sz, sphi, e)) atomicOr(P.status, kFlagNonFinite);
+  if (g == 0 && live && post_body(P, mode, i, sp, in, sx, sy, sz, sphi, e)) atomicOr(P.status, kFlagNonFinite);
   if (mode & kVirial) {
     double kw[2] = {e[0], e[1]};
-    if (g == 0) block_sum<2, CB, true>(kw);
+    if (threadIdx.x < kSumThreads<CB>) block_sum<2, kSumThreads<CB>, true>(kw);
     if (threadIdx.x == 0) P.epart[(int64_t)blockIdx.x * kEnergyVals + 0] = kw[0],
                           P.epart[(int64_t)blockIdx.x * kEnergyVals + 1] = kw[1];
     if (last_of(P.done, (unsigned)P.n_chunks)) {
       __threadfence();
-      systems_final<2, kSlotGroups * CB>(P.sys_chunk, P.n_sys, P.epart, P.n_chunks, P.status,
+      systems_final<2, SG * CB>(P.sys_chunk, P.n_sys, P.epart, P.n_chunks, P.status,
                                      [&](int sy, const double (&v)[2]) {
                                        double* o = P.vout + 3 * (int64_t)sy;
                                        o[0] = v[0];
@@ -93,7 +102,7 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
     return;
   }
   if (mode & kEnergy) {
-    if (g == 0) block_sum<kEnergyVals, CB, true>(e);
+    if (threadIdx.x < kSumThreads<CB>) block_sum<kEnergyVals, kSumThreads<CB>, true>(e);
     if (threadIdx.x == 0) {
 #pragma unroll
       for (int k = 0; k < kEnergyVals; ++k) P.epart[(int64_t)blockIdx.x * kEnergyVals + k] = e[k];
@@ -102,7 +111,7 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
     // eout null the partials wait for the next step's k_post
     if (P.eout && last_of(P.done, (unsigned)P.n_chunks)) {
       __threadfence();
-      systems_final<kEnergyVals, kSlotGroups * CB>(P.sys_chunk, P.n_sys, P.epart, P.n_chunks, P.status,
+      systems_final<kEnergyVals, SG * CB>(P.sys_chunk, P.n_sys, P.epart, P.n_chunks, P.status,
                                                [&](int sy, const double (&v)[kEnergyVals]) {
                                                  emit_energy(P.eout, sy, v);
                                                });
@@ -110,8 +119,8 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_post(const PostLaunch P) {
   }
 }
 
-template <int CB>
-__global__ void __launch_bounds__(CB) k_centre(const CentreLaunch C) {
+__global__ void __launch_bounds__(kChunk) k_centre(const CentreLaunch C) {
+  constexpr int CB = kChunk;
   constexpr int NW = CB / 32;
   __shared__ Extent ext[NW];
   const int lane = (int)threadIdx.x & 31, wid = (int)threadIdx.x >> 5;
@@ -172,14 +181,14 @@ __global__ void __launch_bounds__(CB) k_centre(const CentreLaunch C) {
   }
 }
 
-template <int CB>
-__global__ void __launch_bounds__(kSlotGroups * CB) k_adj_update(const AdjLaunch A) {
+template <int CB, int SG>
+__global__ void __launch_bounds__(SG * CB) k_adj_update(const AdjLaunch A) {
   __shared__ union {
-    SlotSums<CB> f[10];
-    double d[10][kSlotGroups - 1][CB];
+    SlotSums<CB, SG> f[10];
+    double d[10][SG - 1][CB];
   } red;
-  pdl_wait();     // the VJP kernel has finished writing the partials
   Chunk c = A.chunks[blockIdx.x];
+  pdl_wait();  // the VJP kernel has finished writing the partials
   if (!chunk_ok(c, A.n_total, A.n_sys, A.part_rows, A.status)) c.begin = c.end = 0;  // NBODY_DEBUG builds only
   const SysParam& sp = A.sys[c.sys];
   const int kw = A.g_params ? 3 : 2;  // partials (fpair4 / double4_32a) per body and slice
@@ -200,7 +209,7 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_adj_update(const AdjLaunch
     };
     if (live) {
 #pragma unroll 4
-      for (int s = g; s < c.n_slices; s += kSlotGroups) {
+      for (int s = g; s < c.n_slices; s += SG) {
         const int64_t k = kw * (c.row0 + (int64_t)s * c.stride + i);
         const fpair4 p = fp[k], q = fp[k + 1];
         add(0, p.xy.x, p.xy.y), add(1, p.xy.z, p.xy.w), add(2, p.zp.x, p.zp.y), add(3, p.zp.z, p.zp.w);
@@ -220,7 +229,7 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_adj_update(const AdjLaunch
     for (int q = 0; q < 10; ++q) S[q] = 0.0;
     if (live) {
 #pragma unroll 4
-      for (int s = g; s < c.n_slices; s += kSlotGroups) {
+      for (int s = g; s < c.n_slices; s += SG) {
         const int64_t k = kw * (c.row0 + (int64_t)s * c.stride + i);
         const double4_32a p = part[k], q = part[k + 1];
         S[0] += p.x, S[1] += p.y, S[2] += p.z, S[3] += p.w;
@@ -266,12 +275,12 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_adj_update(const AdjLaunch
   if (!A.g_params) return;
   // dL/dG += coef sum_k w_k . da_k/dG; dL/deps += coef (-3 G eps) sum_k sum_j m_j (d.w_k) / s^5,
   // per system in a fixed order (chunk partials, then the last CTA)
-  if (g == 0) block_sum<2, CB, true>(pv);
+  if (threadIdx.x < kSumThreads<CB>) block_sum<2, kSumThreads<CB>, true>(pv);
   if (threadIdx.x == 0) A.cpart[(int64_t)blockIdx.x * kEnergyVals + 0] = pv[0],
                         A.cpart[(int64_t)blockIdx.x * kEnergyVals + 1] = pv[1];
   if (!last_of(A.done, gridDim.x)) return;
   __threadfence();
-  systems_final<2, kSlotGroups * CB>(A.sys_chunk, A.n_sys, A.cpart, gridDim.x, A.status, [&](int sy, const double (&v)[2]) {
+  systems_final<2, SG * CB>(A.sys_chunk, A.n_sys, A.cpart, gridDim.x, A.status, [&](int sy, const double (&v)[2]) {
     const double dG = A.coef * v[0], de = A.coef * (-3.0 * A.G * A.eps) * v[1];
     if (!(isfinite(dG) && isfinite(de))) atomicOr(A.status, kFlagNonFinite);
     A.g_params[2 * sy + 0] += dG;
@@ -280,7 +289,7 @@ __global__ void __launch_bounds__(kSlotGroups * CB) k_adj_update(const AdjLaunch
 }
 
 template <int CB>
-__global__ void __launch_bounds__(CB) k_stage_vec(const Chunk* chunks, int precision, const double* vec,
+__global__ void __launch_bounds__(kSumThreads<CB>) k_stage_vec(const Chunk* chunks, int precision, const double* vec,
                                                   const double* m, const SysParam* sys, void* stage,
                                                             void* stage_lo, int as_position, const int64_t n_total,
                                                             const int n_sys, unsigned* status) {
@@ -288,7 +297,7 @@ __global__ void __launch_bounds__(CB) k_stage_vec(const Chunk* chunks, int preci
   Chunk c = chunks[blockIdx.x];
   if (!chunk_ok(c, n_total, n_sys, 0, status)) c.begin = c.end = 0;  // NBODY_DEBUG builds only
   const SysParam& sp = sys[c.sys];
-  for (int i = c.begin + (int)threadIdx.x; i < c.end; i += CB) {
+  for (int i = c.begin + (int)threadIdx.x; i < c.end; i += (int)kSumThreads<CB>) {
     const double v0 = vec[3 * i + 0], v1 = vec[3 * i + 1], v2 = vec[3 * i + 2];
     if (as_position) {
       stage_store(precision, stage, i, v0, v1, v2, m[i], sp, stage_lo);
@@ -325,36 +334,39 @@ cudaError_t launch_copy4(const Copy4& C, int n_sms, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// f(std::integral_constant<int, bodies per chunk of a layout of n_total bodies>)
+// f(bodies per chunk of a layout of n_total bodies, slot groups of k_post, of k_adj_update), as
+// integral constants (the latter has ten sums per body to pass through shared memory)
 template <typename F>
 static cudaError_t with_chunk(const int64_t n_total, F f) {
-  return chunk_bodies(n_total) == kChunk ? f(std::integral_constant<int, kChunk>())
-                                         : f(std::integral_constant<int, kChunkSmall>());
+  using std::integral_constant;
+  switch (chunk_bodies(n_total)) {
+    case 16: return f(integral_constant<int, 16>(), integral_constant<int, 16>(), integral_constant<int, 16>());
+    case 32: return f(integral_constant<int, 32>(), integral_constant<int, 8>(), integral_constant<int, 8>());
+    case 64: return f(integral_constant<int, 64>(), integral_constant<int, 8>(), integral_constant<int, 8>());
+    default: return f(integral_constant<int, kChunk>(), integral_constant<int, 4>(), integral_constant<int, 4>());
+  }
 }
 
 cudaError_t launch_post(const PostLaunch& P, cudaStream_t st) {
   if (P.n_chunks <= 0) return cudaSuccess;
-  return with_chunk(P.n_total, [&](auto cb) {
-    constexpr int CB = decltype(cb)::value;
+  return with_chunk(P.n_total, [&](auto cb, auto sg, auto) {
+    constexpr int CB = decltype(cb)::value, SG = decltype(sg)::value;
     // a pass that combines nothing needs one thread per body only
-    return launch_pdl(k_post<CB>, (unsigned)P.n_chunks + (P.eprev_out ? 1u : 0u),
-                      (P.mode & kCombine) ? kSlotGroups * CB : CB, st, P);
+    return launch_pdl(k_post<CB, SG>, (unsigned)P.n_chunks + (P.eprev_out ? 1u : 0u),
+                      (P.mode & kCombine) ? SG * CB : (int)kSumThreads<CB>, st, P);
   });
 }
 
 cudaError_t launch_centre(const CentreLaunch& C, cudaStream_t st) {
   if (C.n_sys <= 0 || C.n_chunks <= 0) return cudaSuccess;
-  return with_chunk(C.n_total, [&](auto cb) {
-    constexpr int CB = decltype(cb)::value;
-    return launch_pdl(k_centre<CB>, C.n_chunks, CB, st, C);
-  });
+  return launch_pdl(k_centre, C.n_chunks, kChunk, st, C);
 }
 
 cudaError_t launch_adj_update(const AdjLaunch& A, cudaStream_t st) {
   if (A.n_chunks <= 0) return cudaSuccess;
-  return with_chunk(A.n_total, [&](auto cb) {
-    constexpr int CB = decltype(cb)::value;
-    return launch_pdl(k_adj_update<CB>, A.n_chunks, kSlotGroups * CB, st, A);
+  return with_chunk(A.n_total, [&](auto cb, auto, auto sg) {
+    constexpr int CB = decltype(cb)::value, SG = decltype(sg)::value;
+    return launch_pdl(k_adj_update<CB, SG>, A.n_chunks, SG * CB, st, A);
   });
 }
 
@@ -362,9 +374,9 @@ cudaError_t launch_stage_vec(const Chunk* chunks, int n_chunks, int precision, c
                              const SysParam* sys, void* stage, void* stage_lo, int as_position, int64_t n_total,
                              int n_sys, unsigned* status, cudaStream_t st) {
   if (n_chunks <= 0) return cudaSuccess;
-  return with_chunk(n_total, [&](auto cb) {
+  return with_chunk(n_total, [&](auto cb, auto, auto) {
     constexpr int CB = decltype(cb)::value;
-    return launch_pdl(k_stage_vec<CB>, n_chunks, CB, st, chunks, precision, vec, m, sys, stage, stage_lo, as_position,
+    return launch_pdl(k_stage_vec<CB>, n_chunks, (int)kSumThreads<CB>, st, chunks, precision, vec, m, sys, stage, stage_lo, as_position,
                       n_total, n_sys, status);
   });
 }
