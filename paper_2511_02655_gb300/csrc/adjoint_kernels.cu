@@ -170,8 +170,9 @@ __global__ void __launch_bounds__(BLOCK) k_vjp_mixed(const PairLaunch L) {
   const float4* __restrict__ slo = L.stage_lo;
 
   pdl_wait();
+  ItemSource source{L.counter, &s_item};
   for (;;) {
-    const int it = next_item(L.counter, &s_item);
+    const int it = source.next();
     if (it >= L.n_items) break;
     const WorkItem w = L.items[it];
     if (!item_ok(w, L)) continue;  // NBODY_DEBUG builds only
@@ -298,8 +299,9 @@ __global__ void __launch_bounds__(BLOCK) k_vjp_fp64(const PairLaunch L) {
   const double eps2 = L.eps2;
 
   pdl_wait();
+  ItemSource source{L.counter, &s_item};
   for (;;) {
-    const int it = next_item(L.counter, &s_item);
+    const int it = source.next();
     if (it >= L.n_items) break;
     const WorkItem w = L.items[it];
     if (!item_ok(w, L)) continue;  // NBODY_DEBUG builds only
@@ -450,8 +452,9 @@ __global__ void __launch_bounds__(BLOCK) k_vjp_mixed2(const PairLaunch L) {
   };
 
   pdl_wait();
+  ItemSource source{L.counter, &s_item};
   for (;;) {
-    const int it = next_item(L.counter, &s_item);
+    const int it = source.next();
     if (it >= L.n_items) break;
     const WorkItem w = L.items[it];
     if (!item_ok(w, L)) continue;  // NBODY_DEBUG builds only

@@ -117,8 +117,9 @@ __device__ __forceinline__ void items_mixed(const PairLaunch& L, unsigned* count
   fpair4* __restrict__ part = reinterpret_cast<fpair4*>(L.part);
   const float4* __restrict__ lo = L.stage_lo;
 
+  ItemSource source{counter, &sm.item};
   for (;;) {
-    const int it = next_item(counter, &sm.item);  // also a barrier: the buffers are free
+    const int it = source.next();  // also a barrier: the buffers are free
     if (it >= L.n_items) break;
     const WorkItem w = L.items[it];
     if (!item_ok(w, L)) continue;  // NBODY_DEBUG builds only
@@ -522,8 +523,9 @@ __device__ __forceinline__ void items_fp64(const PairLaunch& L, unsigned* counte
   const double eps2 = L.eps2;
   const double s2 = L.sigma2;
 
+  ItemSource source{counter, &sm.item};
   for (;;) {
-    const int it = next_item(counter, &sm.item);
+    const int it = source.next();
     if (it >= L.n_items) break;
     const WorkItem w = L.items[it];
     if (!item_ok(w, L)) continue;  // NBODY_DEBUG builds only

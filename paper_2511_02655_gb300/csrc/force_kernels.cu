@@ -64,8 +64,9 @@ __global__ void __launch_bounds__(BLOCK, (MINB > 0 ? MINB
     k_force_mixed2(const PairLaunch L) {
   __shared__ fc::SmemMixed2<J> sm;
   pdl_wait();
+  ItemSource source{L.counter, &sm.item};
   auto next = [&](WorkItem& w) {
-    const int it = next_item(L.counter, &sm.item);
+    const int it = source.next();
     if (it < L.n_items) w = L.items[it];
     return it < L.n_items;
   };

@@ -81,15 +81,27 @@ __device__ __forceinline__ void correct_pair(const float4 q, const int jg, const
   }
 }
 
-// Persistent-kernel work distribution: CTAs take items from counter[0]; the
-// last CTA to finish zeroes both counters for the next launch. No CTA waits
+// Persistent-kernel work distribution: a CTA's first item is its own index (no
+// round trip to L2 before the work starts), further ones come from counter[0];
+// the last CTA to finish zeroes both counters for the next launch. No CTA waits
 // on another, so no wait can hang.
-__device__ __forceinline__ int next_item(unsigned* counter, int* s_item) {
-  __syncthreads();  // everyone is done with the previous item and s_item
-  if (threadIdx.x == 0) *s_item = (int)atomicAdd(&counter[0], 1u);
-  __syncthreads();
-  return *s_item;
-}
+struct ItemSource {
+  unsigned* counter;
+  int* s_item;  // shared memory
+  bool first = true;
+  // called by every thread of the CTA; from the second call on a barrier: everyone is done
+  // with the previous item
+  __device__ __forceinline__ int next() {
+    if (first) {
+      first = false;
+      return (int)blockIdx.x;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) *s_item = (int)(atomicAdd(&counter[0], 1u) + gridDim.x);
+    __syncthreads();
+    return *s_item;
+  }
+};
 
 __device__ __forceinline__ void retire_cta(unsigned* counter) {
   if (threadIdx.x == 0) {

@@ -210,8 +210,9 @@ __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Sme
   double4_32a* part = reinterpret_cast<double4_32a*>(L.part);
   const double eps2 = L.eps2, s2 = L.sigma2;
 
+  ItemSource source{counter, &sm.item};
   for (;;) {
-    const int n = next_item(counter, &sm.item);
+    const int n = source.next();
     if (n >= L.n_items) break;
     const SymItem it = L.items[n];
     if (!sym_item_ok(it, L)) continue;  // NBODY_DEBUG builds only

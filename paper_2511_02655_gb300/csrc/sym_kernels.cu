@@ -16,8 +16,9 @@ __global__ void __launch_bounds__(W * 32, MINB) k_force_sym(const SymLaunch L) {
   extern __shared__ __align__(16) unsigned char raw[];
   auto& sm = *reinterpret_cast<sym::Smem<W, R, sym_force_tile(W)>*>(raw);
   pdl_wait();
+  ItemSource source{L.counter, &sm.item};
   auto next = [&](SymItem& it) {
-    const int n = next_item(L.counter, &sm.item);
+    const int n = source.next();
     if (n < L.n_items) it = L.items[n];
     return n < L.n_items;
   };

@@ -206,8 +206,9 @@ __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Sme
   fpair4* part = reinterpret_cast<fpair4*>(L.part);
   const float2 zero = make_float2(0.f, 0.f);
 
+  ItemSource source{counter, &sm.item};
   for (;;) {
-    const int n = next_item(counter, &sm.item);
+    const int n = source.next();
     if (n >= L.n_items) break;
     const SymItem it = L.items[n];
     if (!sym_item_ok(it, L)) continue;  // NBODY_DEBUG builds only
@@ -411,8 +412,9 @@ __device__ __forceinline__ void items64(const SymLaunch& L, unsigned* counter, S
   double4_32a* part = reinterpret_cast<double4_32a*>(L.part);
   const double eps2 = L.eps2;
 
+  ItemSource source{counter, &sm.item};
   for (;;) {
-    const int n = next_item(counter, &sm.item);
+    const int n = source.next();
     if (n >= L.n_items) break;
     const SymItem it = L.items[n];
     if (!sym_item_ok(it, L)) continue;  // NBODY_DEBUG builds only
