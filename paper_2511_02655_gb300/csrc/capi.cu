@@ -128,6 +128,7 @@ struct nbody_ctx {
   std::vector<int64_t> offsets;
   std::string err = "no error";
   int64_t launches = 0;
+  uint32_t epoch = 0;  // number of the current call (SysParam::uniform); 0 while tuning
 
   // layout
   std::vector<Chunk> chunks;  // without slots (Chunk::n_slices, stride, row0: the copies on the device)
@@ -573,6 +574,7 @@ SymLaunch sym_launch(nbody_ctx* c, bool vjp, Potential phi) {
   L.law = c->cfg.law;
   L.block = t.block, L.ipt = t.ipt, L.n_ctas = t.n_ctas;
   L.phi = (int)phi;
+  L.epoch = c->epoch;
   L.status = c->status;
   return L;
 }
@@ -654,7 +656,9 @@ nbody_status run_force(nbody_ctx* c, cudaStream_t st, Potential phi) { return ru
 nbody_status run_vjp(nbody_ctx* c, cudaStream_t st) { return run_pair(c, st, true, Potential::kNone); }
 
 
-PostLaunch post_launch(nbody_ctx* c, unsigned mode, double* x, double* v, const double* m, double* a, double* phi) {
+// first_stage: the call's first staging (FP64: unequal masses are noted)
+PostLaunch post_launch(nbody_ctx* c, unsigned mode, double* x, double* v, const double* m, double* a, double* phi,
+                       bool first_stage = false) {
   PostLaunch P{};
   P.chunks = c->d_chunks;
   P.n_chunks = (int32_t)c->chunks.size();
@@ -673,7 +677,11 @@ PostLaunch post_launch(nbody_ctx* c, unsigned mode, double* x, double* v, const 
   P.box = c->cfg.box;
   P.stage = c->stage.p;
   P.stage_lo = c->stage_lo.p;
-  P.sys = static_cast<const SysParam*>(c->sysp.p);
+  P.sys = static_cast<SysParam*>(c->sysp.p);
+  // (one-sided kernels keep the masses in their sums: no system counts as uniform for them)
+  P.epoch = c->epoch;
+  P.off = is_sym(c->ft) ? c->d_off : nullptr;
+  if (c->cfg.precision == NBODY_FP64 && is_sym(c->ft) && c->cfg.law == NBODY_LAW_GRAVITY && first_stage) P.mode |= kMasses;
   P.epart = static_cast<double*>(c->epart.p);
   P.status = c->status;
   P.eout = nullptr;
@@ -692,7 +700,9 @@ nbody_status run_post(nbody_ctx* c, const PostLaunch& P, cudaStream_t st) {
   return NBODY_OK;
 }
 
+// Starts a call: its number (never 0), and on the mixed path the staging parameters.
 nbody_status run_centre(nbody_ctx* c, const double* x, const double* m, cudaStream_t st) {
+  if (++c->epoch == 0) c->epoch = 1;
   if (c->cfg.precision != NBODY_MIXED || c->n_total == 0) return NBODY_OK;
   CentreLaunch C{};
   C.chunks = c->d_cchunks;
@@ -720,12 +730,12 @@ nbody_status enqueue_step(nbody_ctx* c, double* x, double* v, const double* m, d
   nbody_status s;
   if ((s = run_centre(c, x, m, st))) return s;
   if (!a_valid) {
-    if ((s = run_post(c, post_launch(c, kStage, x, v, m, a, nullptr), st))) return s;
+    if ((s = run_post(c, post_launch(c, kStage, x, v, m, a, nullptr, true), st))) return s;
     if ((s = run_force(c, st, Potential::kNone))) return s;
     if ((s = run_post(c, post_launch(c, kCombine, x, v, m, a, nullptr), st))) return s;
   }
   if (n_steps == 0) return NBODY_OK;
-  if ((s = run_post(c, post_launch(c, kDrift | kStage, x, v, m, a, nullptr), st))) return s;
+  if ((s = run_post(c, post_launch(c, kDrift | kStage, x, v, m, a, nullptr, a_valid != 0), st))) return s;
   const int every = c->cfg.energy_every;
   // With up to four systems a step's energy record, except the call's last, is
   // finished by one extra CTA of the next step's k_post (same fixed-order sum)
@@ -878,7 +888,7 @@ nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
   C.mode = kCombine;
   C.status = c->status;
   C.n_sys = c->n_sys;
-  C.sys = static_cast<const SysParam*>(c->sysp.p);
+  C.sys = static_cast<SysParam*>(c->sysp.p);
   C.part_rows = (int64_t)(c->part.bytes / (vjp ? 64 : 32));
   cudaEvent_t ev[4];
   for (auto& e : ev) NB_CUDA(c, cudaEventCreate(&e));
@@ -1314,7 +1324,7 @@ nbody_status adjoint_sweep(nbody_ctx* c, const double* x0, const double* v0, con
   if ((s = run_centre(c, x0, m, st))) return s;
   NB_CUDA(c, cudaMemcpyAsync(xw, x0, n3b, cudaMemcpyDeviceToDevice, st));
   NB_CUDA(c, cudaMemcpyAsync(vw, v0, n3b, cudaMemcpyDeviceToDevice, st));
-  if ((s = run_post(c, post_launch(c, kStage, xw, vw, m, aw, nullptr), st))) return s;
+  if ((s = run_post(c, post_launch(c, kStage, xw, vw, m, aw, nullptr, true), st))) return s;
   if ((s = run_force(c, st, Potential::kNone))) return s;
   if ((s = run_post(c, post_launch(c, kCombine, xw, vw, m, aw, nullptr), st))) return s;
 
@@ -1586,7 +1596,7 @@ nbody_status nbody_forces(nbody_ctx* c, const double* x, const double* m, double
   if ((s = check_dev(c, phi, (size_t)c->n_total * sizeof(double), "phi", true))) return s;
   double* xm = const_cast<double*>(x);
   if ((s = run_centre(c, x, m, c->stream))) return s;
-  if ((s = run_post(c, post_launch(c, kStage, xm, nullptr, m, a, nullptr), c->stream))) return s;
+  if ((s = run_post(c, post_launch(c, kStage, xm, nullptr, m, a, nullptr, true), c->stream))) return s;
   if ((s = run_force(c, c->stream, phi ? Potential::kBodies : Potential::kNone))) return s;
   return run_post(c, post_launch(c, kCombine, xm, nullptr, m, a, phi), c->stream);
 }
@@ -1674,7 +1684,7 @@ nbody_status nbody_energy(nbody_ctx* c, const double* x, const double* v, const 
   double* vm = const_cast<double*>(v);
   double* as = static_cast<double*>(c->a_scratch.p);
   if ((s = run_centre(c, x, m, c->stream))) return s;
-  if ((s = run_post(c, post_launch(c, kStage, xm, vm, m, as, nullptr), c->stream))) return s;
+  if ((s = run_post(c, post_launch(c, kStage, xm, vm, m, as, nullptr, true), c->stream))) return s;
   if ((s = run_force(c, c->stream, Potential::kEnergy))) return s;
   // the last CTA writes every system's record (systems without bodies get zeros)
   PostLaunch P = post_launch(c, kCombine | kEnergy, xm, vm, m, as, nullptr);
@@ -1697,7 +1707,7 @@ nbody_status nbody_virial(nbody_ctx* c, const double* x, const double* v, const 
   double* vm = const_cast<double*>(v);
   double* as = static_cast<double*>(c->a_scratch.p);
   if ((s = run_centre(c, x, m, c->stream))) return s;
-  if ((s = run_post(c, post_launch(c, kStage, xm, vm, m, as, nullptr), c->stream))) return s;
+  if ((s = run_post(c, post_launch(c, kStage, xm, vm, m, as, nullptr, true), c->stream))) return s;
   if ((s = run_force(c, c->stream, Potential::kNone))) return s;
   PostLaunch P = post_launch(c, kCombine | kVirial, xm, vm, m, as, nullptr);
   P.vout = out;

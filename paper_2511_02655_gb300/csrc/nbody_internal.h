@@ -40,7 +40,8 @@ struct __align__(16) SysParam {
   double c[3];
   double scale, mscale, inv_mscale;
   float eps2, r2c;   // staged softening^2 and near-pair radius^2 (0: no refinement)
-  uint32_t uniform;
+  uint32_t uniform;  // mixed: 1 if all masses are equal (staged as 1). FP64: the number of the last call that
+                     // met unequal masses (checked when a call first stages; PostLaunch::epoch)
   uint32_t pad;
 };
 
@@ -192,6 +193,7 @@ struct SymLaunch {
   double eps2, sigma2;     // FP64 path
   int law, block, ipt, n_ctas;
   int phi;                 // potential: 0 none, 1 of every body, 2 for an energy record (sym::kPhi*)
+  uint32_t epoch;          // FP64: number of the call (SysParam::uniform)
   int params;              // VJP: also the sums for the G and eps gradients
   unsigned* status;
 };
@@ -260,6 +262,7 @@ enum PostMode : unsigned {
   kEnergy = 4u,    // per-chunk partial energies / momenta at (x, v)
   kDrift = 8u,     // v += dt/2 a; x += dt v (opening half-kick + drift of the next step)
   kStage = 16u,    // staging tile entry from x (after the drift, if any)
+  kMasses = 64u,   // FP64, with kStage: note unequal masses in SysParam::uniform
   kVirial = 32u,   // per-chunk partial K and Clausius virial W = sum m x.a (not with kEnergy)
 };
 
@@ -283,7 +286,9 @@ struct PostLaunch {
   double box;              // > 0: reflecting walls of [0, box]^3 applied after the drift
   void* stage;             // float4 / double4_32a [N]
   void* stage_lo;          // mixed: float4 remainders of the staged coordinates [N] (nullable)
-  const SysParam* sys;     // [n_sys] staging origin and scales
+  SysParam* sys;           // [n_sys] staging origin and scales
+  uint32_t epoch;          // FP64: number of the call
+  const int64_t* off;      // [n_sys + 1] first body of each system
   double* epart;           // [n_chunks][kEnergyVals]
   unsigned* status;        // device status word
   double u_weight;         // kEnergy: U = u_weight sum m phi (1/2, or 1 if phi holds each pair once)

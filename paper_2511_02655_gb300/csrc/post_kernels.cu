@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
   }
   if (!chunk_ok(c, P.n_total, P.n_sys, (P.mode & kCombine) ? P.part_rows : 0, P.status))
     c.begin = c.end = 0;  // NBODY_DEBUG builds only: processed as an empty chunk
-  const SysParam& sp = P.sys[c.sys];
+  SysParam& sp = P.sys[c.sys];
   double e[kEnergyVals];
 #pragma unroll
   for (int k = 0; k < kEnergyVals; ++k) e[k] = 0.0;
@@ -56,6 +56,15 @@ __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
   const bool live = i < c.end && g < SG;  // (a chunk of 16 has half a warp without bodies in a pass that combines nothing)
   BodyIn in;
   if (g == 0 && live) in = load_body(P, mode, i);
+  double m_all = 1.0;  // FP64 gravity: the mass that a system's bodies share is left out of the sums
+  if (P.precision == 0 && P.law == 0 && P.off && (mode & (kCombine | kMasses))) {
+    const double m0 = P.m[P.off[c.sys]];
+    if (mode & kMasses) {
+      if (g == 0 && live && __double_as_longlong(in.m) != __double_as_longlong(m0)) sp.uniform = P.epoch;
+    } else if (sp.uniform != P.epoch) {
+      m_all = m0;
+    }
+  }
 
   double sx = 0.0, sy = 0.0, sz = 0.0, sphi = 0.0;
   if ((mode & kCombine) && P.precision == 1) {
@@ -81,7 +90,7 @@ __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
       }
     }
     add_groups(red.d, g, b, s4);
-    sx = s4[0], sy = s4[1], sz = s4[2], sphi = s4[3];
+    sx = m_all * s4[0], sy = m_all * s4[1], sz = m_all * s4[2], sphi = m_all * s4[3];
   }
   if (g == 0 && live && post_body(P, mode, i, sp, in, sx, sy, sz, sphi, e)) atomicOr(P.status, kFlagNonFinite);
   if (mode & kVirial) {

@@ -4,13 +4,15 @@
 // Bound: GB300's FP64 pipe, two lanes per clock and SM against 128 of the FP32 and
 // 64 of the integer pipe. Everything that is not a float64 operation is therefore
 // free up to dozens of operations, and the pair is written for the fewest float64
-// ones: 17 per unordered pair of softened gravity (8.5 per interaction; 3 more with
-// both potentials) where the one-sided kernel with the library's rsqrt takes about
-// 20 per interaction. N = 12 002 with potentials: 4.67 ms
-// with the one-sided kernel, 2.57 ms here (20 operations a pair take 2.29 ms at the
-// pipe's rate). The error against 64-bit sums is no larger (3.3e-16 and 1.8e-16
-// relative): s^-3 is good to 1 ulp, 0.2 ulp on average.
+// ones: 16 per unordered pair of softened gravity (8 per interaction; 3 more with
+// both potentials, 2 fewer where all masses of a system are equal) where the one-sided
+// kernel with the library's rsqrt takes about 20 per interaction. N = 12 002 with
+// potentials and unequal masses: 4.67 ms with the one-sided kernel, 2.43 ms here (19
+// operations a pair take 2.18 ms at the pipe's rate). The error against 64-bit sums is
+// no larger (3.3e-16 and 1.6e-16 relative): s^-3 is good to 1.5 ulp, 0.25 ulp on average.
 #pragma once
+
+#include <type_traits>
 
 #include "nbody_internal.h"
 #include "pair_common.cuh"
@@ -71,12 +73,17 @@ __device__ __forceinline__ Root root_of(const double r2) {
   t.ef = small_to_float(t.e);
   return t;
 }
-// s^-3 and s^-2 from the start values: two and two float64 operations
+// s^-3 from the start values: one float64 operation. y^3 (1 + p), p = e^2 (15/8 + 35/16 e) >= 0 below
+// 2^-30, is the double y^3 plus p times its 53-bit mantissa in units of the last place, an integer
+// addition (a carry runs into the exponent, as it should); the linear term 3/2 y^3 is exact.
 __device__ __forceinline__ double inv3_of(const Root& t) {
   const float p = (t.ef * t.ef) * fmaf(2.1875f, t.ef, 1.875f);
-  const double c = fma(1.5, t.e, float_to_double(p)), y3 = int_scaled(t.M3, 51 + 3 * t.q);
-  return fma(y3, c, y3);
+  const uint64_t m = t.M3 << (__clzll((long long)t.M3) - 11);
+  const float fm = __uint_as_float(((127u + 52u) << 23) | ((uint32_t)(m >> 29) & 0x7fffffu));
+  const long long y3 = __double_as_longlong(int_scaled(t.M3, 51 + 3 * t.q)) + __float2int_rn(p * fm);
+  return fma(int_scaled(3u * t.M3, 52 + 3 * t.q), t.e, __longlong_as_double(y3));
 }
+// s^-2: two float64 operations
 __device__ __forceinline__ double inv2_of(const Root& t) {
   const float p = (t.ef * t.ef) * (1.f + t.ef);
   const double c = t.e + float_to_double(p), y2 = int_scaled(t.M2, 34 + 2 * t.q);
@@ -99,17 +106,17 @@ __device__ __forceinline__ double rcp_f64(const double r2) {
 
 // Pair weights: the force on the i-body is wj d, on the j-body -wi d; t is the potential term
 // (times the other body's mass for gravity). FAST: s^2 is in range.
-template <int LAW, bool FAST, int PHI>
+template <int LAW, bool FAST, int PHI, bool EQ>
 __device__ __forceinline__ void weights(const double r2, const double s2, const double mj, const double mi, double& wj,
                                         double& wi, double& t) {
   if (LAW == 0) {
     if (FAST) {
       const double i3 = inv3_of(root_of(r2));
-      wj = mj * i3, wi = mi * i3;
+      wj = EQ ? i3 : mj * i3, wi = EQ ? i3 : mi * i3;
       if (PHI) t = i3 * r2;
     } else {
       const double inv = rsqrt(r2), i2 = inv * inv;
-      wj = (mj * inv) * i2, wi = (mi * inv) * i2;
+      wj = EQ ? inv * i2 : (mj * inv) * i2, wi = EQ ? wj : (mi * inv) * i2;
       if (PHI) t = inv;
     }
   } else {  // u = sigma^2 / r^2
@@ -136,7 +143,7 @@ constexpr int kUnroll = 4;
 // The 32 steps of one block. FAST: returns whether the lane met an s^2 out of range, in which case
 // the sums are void and the block is to be repeated without FAST (there is no branch per pair, so
 // that the pairs of several steps overlap).
-template <int LAW, bool SYM, bool MASK, int PHI, bool FAST, int R>
+template <int LAW, bool SYM, bool MASK, int PHI, bool EQ, bool FAST, int R>
 __device__ __forceinline__ bool block32(const double (&q)[4][kTile / 32][64], const int b, const int jg0, const int lane,
                                         const int ig0, const double (&xi)[R], const double (&yi)[R],
                                         const double (&zi)[R], const double (&mi)[R], const double eps2,
@@ -155,18 +162,18 @@ __device__ __forceinline__ bool block32(const double (&q)[4][kTile / 32][64], co
       const bool self = MASK && jg0 + (p & 31) == ig0 + 32 * r;
       if (FAST) out |= !self && !in_range(r2);
       double wj, wi, t = 0.0;
-      weights<LAW, FAST, PHI>(r2, s2, mj, mi[r], wj, wi, t);
+      weights<LAW, FAST, PHI, EQ>(r2, s2, mj, mi[r], wj, wi, t);
       if (self) wj = 0.0, t = 0.0;
       ax[r] = fma(dx, wj, ax[r]);
       ay[r] = fma(dy, wj, ay[r]);
       az[r] = fma(dz, wj, az[r]);
       if (MASK && PHI == sym::kPhiEnergy) t *= 0.5;
-      if (PHI) pp[r] = LAW == 0 ? fma(mj, t, pp[r]) : pp[r] + t;
+      if (PHI) pp[r] = LAW == 0 && !EQ ? fma(mj, t, pp[r]) : pp[r] + t;
       if (SYM) {
         jx = fma(-dx, wi, jx);
         jy = fma(-dy, wi, jy);
         jz = fma(-dz, wi, jz);
-        if (PHI == sym::kPhiBoth) jp = LAW == 0 ? fma(mi[r], t, jp) : jp + t;
+        if (PHI == sym::kPhiBoth) jp = LAW == 0 && !EQ ? fma(mi[r], t, jp) : jp + t;
       }
     }
     if (SYM) {
@@ -180,7 +187,7 @@ __device__ __forceinline__ bool block32(const double (&q)[4][kTile / 32][64], co
 }
 
 // A block with FAST, repeated without it where any lane met an s^2 out of range.
-template <int LAW, bool SYM, bool MASK, int PHI, int R>
+template <int LAW, bool SYM, bool MASK, int PHI, bool EQ, int R>
 __device__ __forceinline__ void block(const double (&q)[4][kTile / 32][64], const int b, const int jg0, const int lane,
                                       const int ig0, const double (&xi)[R], const double (&yi)[R],
                                       const double (&zi)[R], const double (&mi)[R], const double eps2, const double s2,
@@ -189,11 +196,11 @@ __device__ __forceinline__ void block(const double (&q)[4][kTile / 32][64], cons
   double bx[R], by[R], bz[R], bp[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) bx[r] = ax[r], by[r] = ay[r], bz[r] = az[r], bp[r] = pp[r];
-  const bool out = block32<LAW, SYM, MASK, PHI, true, R>(q, b, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, bx, by, bz, bp,
+  const bool out = block32<LAW, SYM, MASK, PHI, EQ, true, R>(q, b, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, bx, by, bz, bp,
                                                          jx, jy, jz, jp);
   if (__any_sync(0xffffffffu, out)) {
     jx = jy = jz = jp = 0.0;
-    block32<LAW, SYM, MASK, PHI, false, R>(q, b, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp, jx, jy, jz,
+    block32<LAW, SYM, MASK, PHI, EQ, false, R>(q, b, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp, jx, jy, jz,
                                            jp);
   } else {
 #pragma unroll
@@ -221,6 +228,9 @@ __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Sme
     // Padding, i and j on opposite sides so that their difference is not 0. Gravity: massless and
     // far beyond the item's bodies, but in range; Lennard-Jones (no masses in the sums): so far
     // that u^3 is exactly 0.
+    // Equal masses are left out of the sums: bodies count 1, padding 0, and blocks without padding
+    // need no products with them.
+    const bool uniform = LAW == 0 && L.sys[it.sys].uniform != L.epoch;
     const double4_32a q0 = st[it.i_begin];
     const double pad = LAW == 0 ? 1.0e30 * (1.0 + fabs(q0.x) + fabs(q0.y) + fabs(q0.z)) : 3.0e89;
 
@@ -231,7 +241,7 @@ __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Sme
       for (int r = 0; r < R; ++r) {
         const int ig = ig0 + 32 * r;
         const double4_32a v = ig < it.i_end ? st[ig] : make_double4_32a(-pad, -pad, -pad, 0.0);
-        xi[r] = v.x, yi[r] = v.y, zi[r] = v.z, mi[r] = v.w;
+        xi[r] = v.x, yi[r] = v.y, zi[r] = v.z, mi[r] = uniform && ig < it.i_end ? 1.0 : v.w;
         ax[r] = ay[r] = az[r] = pp[r] = 0.0;
       }
       const int js = max(it.j_begin, i0);
@@ -241,19 +251,27 @@ __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Sme
           const double4_32a v = jt + t < it.j_end ? st[jt + t] : make_double4_32a(pad, pad, pad, 0.0);
           double* d = &sm.q[0][t >> 5][t & 31];
           constexpr int S = (kTile / 32) * 64;
-          d[0] = d[32] = v.x, d[S] = d[S + 32] = v.y, d[2 * S] = d[2 * S + 32] = v.z, d[3 * S] = d[3 * S + 32] = v.w;
+          d[0] = d[32] = v.x, d[S] = d[S + 32] = v.y, d[2 * S] = d[2 * S + 32] = v.z, d[3 * S] = d[3 * S + 32] = uniform && jt + t < it.j_end ? 1.0 : v.w;
         }
         __syncthreads();
         for (int b = 0; b < kTile / 32; ++b) {
           const int jg0 = jt + 32 * b;
           double jx = 0.0, jy = 0.0, jz = 0.0, jp = 0.0;
           if (jg0 < it.j_end && wi0 < it.i_end) {
-            if (jg0 >= wi0 + 32 * R)
-              block<LAW, true, false, PHI, R>(sm.q, b, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp, jx,
-                                                jy, jz, jp);
-            else if (jg0 + 32 > wi0)
-              block<LAW, false, true, PHI, R>(sm.q, b, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp, jx,
-                                                jy, jz, jp);
+            const bool both = jg0 >= wi0 + 32 * R;
+            auto run = [&](auto eq) {
+              constexpr bool EQ = decltype(eq)::value;
+              if (both)
+                block<LAW, true, false, PHI, EQ, R>(sm.q, b, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp,
+                                                    jx, jy, jz, jp);
+              else if (jg0 + 32 > wi0)
+                block<LAW, false, true, PHI, EQ, R>(sm.q, b, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp,
+                                                    jx, jy, jz, jp);
+            };
+            if (LAW == 0 && uniform && jg0 + 32 <= it.j_end && wi0 + 32 * R <= it.i_end)
+              run(std::integral_constant<bool, LAW == 0>());
+            else
+              run(std::false_type());
           }
           const int p = 32 * b + lane;
           sm.jacc[w][0][p] = jx, sm.jacc[w][1][p] = jy, sm.jacc[w][2][p] = jz;

@@ -89,13 +89,14 @@ TILINGS64 = [(64, 1, 64, 32, 3, 0), (128, 1, 64, 96, 3, 1), (256, 1, 64, 64, 3, 
 @pytest.mark.parametrize("tiling", TILINGS64)
 @pytest.mark.parametrize("n", [65, 300, 1025, 2500])
 @pytest.mark.parametrize("length,mass", [(1.0, 1.0), (1e100, 1e30), (1e-95, 1.0)])
-def test_sym64_forces(nb, tmp_path, monkeypatch, tiling, n, length, mass):
+@pytest.mark.parametrize("masses", ["equal", "lognormal"])
+def test_sym64_forces(nb, tmp_path, monkeypatch, tiling, n, length, mass, masses):
     """FP64 path, in units where s^2 takes the integer steps and in some where it leaves their
     range (the oracle gets scaled copies; powers of ten, so the comparison is good to rounding)."""
     import torch
     monkeypatch.setenv("NBODY_TUNE_CACHE", str(tmp_path / "tune"))
     x, v, m = inputs.plummer(n, seed=n)
-    m = _masses(m, "lognormal", n)
+    m = _masses(m, masses, n)
     xs, ms, eps = x * length, m * mass, 0.03 * length
     ctx = _forced(nb, tmp_path / "tune", {"force": tiling}, G=1.1, eps=eps, dt=1e-3, n=n, precision=nb.FP64)
     assert nb.nbody_get_tuning(ctx)["variant"] == 4
@@ -108,6 +109,30 @@ def test_sym64_forces(nb, tmp_path, monkeypatch, tiling, n, length, mass):
     a, phi = a.cpu().numpy() * (length / mass) * length, phi.cpu().numpy() * (length / mass)
     assert force_rel_err(a, a_ref).max() <= 1e-12
     assert_elem_close(phi, phi_ref, 1e-12, "phi")
+
+
+def test_sym64_masses_change_between_calls(nb):
+    """Equal masses are recognised anew in every call, replayed graphs included."""
+    import torch
+    n, G, eps, dt = 700, 1.0, 0.05, 1e-3
+    x, v, m = inputs.plummer(n, seed=8)
+    m2 = _masses(m, "lognormal", 8)
+    ctx = nb.nbody_init(G=G, eps=eps, dt=dt, n=n, precision=nb.FP64, energy_every=2, flags=nb.FLAG_GRAPH)
+    assert nb.nbody_get_tuning(ctx)["variant"] == 4
+    xt, vt, mt = to_dev(x, v, m)
+    at = torch.empty_like(xt)
+    log = torch.empty((1, 1, 9), dtype=torch.float64, device="cuda")
+    for masses in (m, m2, m, m2, m2):
+        for t, src in ((xt, x), (vt, v), (mt, masses)):
+            t.copy_(torch.from_numpy(src))
+        nb.nbody_step(ctx, xt, vt, mt, at, False, 2, log)
+        a, _ = nb.nbody_forces(ctx, xt, mt)
+        nb.nbody_sync(ctx)
+        xr, vr, ar, lr = oracle.kdk(x, v, masses, G, eps, dt, 2, energy_every=2)
+        assert np.abs(xt.cpu().numpy() - xr).max() <= 1e-13
+        assert force_rel_err(at.cpu().numpy(), ar).max() <= 1e-12
+        assert force_rel_err(a.cpu().numpy(), ar).max() <= 1e-12
+        np.testing.assert_allclose(log.cpu().numpy()[0, 0, 0:3], lr[0, 0:3], rtol=1e-12)
 
 
 @pytest.mark.parametrize("tiling", TILINGS64)
