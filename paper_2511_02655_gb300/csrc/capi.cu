@@ -44,7 +44,7 @@ struct Tiling {
 };
 constexpr int kSymVariant = 3;
 enum class Potential { kNone = 0, kBodies = 1, kEnergy = 2 };  // as sym::kPhi*
-constexpr double kSymMinBodies = 1024.0;    // typical system size from which the symmetric pass is a candidate
+constexpr double kSymMinBodies = 3000.0;    // typical system size from which the symmetric pass is a candidate
 constexpr double kSymOnlyBodies = 8192.0;  // ... and from which it is the only one (mixed path)
 constexpr double kSymMinBodies64 = 64.0, kSymOnlyBodies64 = 512.0;  // FP64 path
 constexpr int64_t kMaxSymRows = 64;                      // rows of i-tiles a system is cut into at most
@@ -275,15 +275,13 @@ nbody_status check_dev(nbody_ctx* c, const void* p, size_t bytes, const char* na
 // ---------------------------------------------------------------------------
 // work lists
 
-int sym_tile(int prec, bool vjp, int block) {
-  return prec != NBODY_MIXED ? kSymTile64 : vjp ? kSymVjpTile : sym_force_tile(block / 32);
-}
+int sym_tile(int prec, bool vjp) { return prec != NBODY_MIXED ? kSymTile64 : vjp ? kSymVjpTile : kSymTile; }
 // j-bodies that a warp of the symmetric pass meets in one block: pieces are whole blocks
 int sym_block(int prec) { return prec == NBODY_MIXED ? 64 : 32; }
 
 int ctas_per_sm(int prec, const Tiling& t, bool vjp, int law) {
   if (t.variant == kSymVariant) {
-    if (t.jtile != sym_tile(prec, vjp, t.block)) return 0;
+    if (t.jtile != sym_tile(prec, vjp)) return 0;
     return vjp ? sym_vjp_ctas_per_sm(prec, t.block, t.ipt) : sym_force_ctas_per_sm(prec, t.block, t.ipt, law);
   }
   return vjp ? vjp_ctas_per_sm(prec, t.variant, t.block, t.ipt, t.jtile)
@@ -302,12 +300,53 @@ double total_pairs(const nbody_ctx* c) {
   return p;
 }
 
-// Slice of a symmetric tiling that makes about `pieces` work items per persistent CTA.
+// The symmetric pass cuts a system of n bodies into rows of H bodies (whole i-tiles, at most
+// kMaxSymRows rows: a body has a slot per row up to its own, so more rows would mean more partials
+// to combine than pair work saved) and row r into pieces of about `area` pairs.
+struct SymRows {
+  int64_t n, H, rows, block;  // block: pieces are whole blocks of j-bodies
+  SymRows(const nbody_ctx* c, const Tiling& t, int64_t bodies) : n(bodies), block(sym_block(c->cfg.precision)) {
+    const int64_t itile = (int64_t)t.block * t.ipt;
+    H = itile * ((n + itile * kMaxSymRows - 1) / (itile * kMaxSymRows));
+    rows = (n + H - 1) / H;
+  }
+  int64_t blocks(int64_t r) const { return (n - r * H + block - 1) / block; }
+  // pieces of row r, and for a tail other than 2 the blocks of each (the last may have fewer)
+  int64_t pieces(int64_t r, double area, int tail, int64_t* step) const {
+    const double ni = (double)std::min(H, n - r * H), pairs = ni * ((double)(n - r * H) - 0.5 * ni);
+    const double want = tail == 1 && (r & 1) ? area / 3.0 : area;
+    const int64_t nb = blocks(r), p = std::max<int64_t>(1, std::min(nb, (int64_t)(pairs / want + 0.5)));
+    *step = std::max<int64_t>(1, (2 * nb + p) / (2 * p));
+    return tail == 2 ? p : (nb + *step - 1) / *step;
+  }
+};
+
+// Slice of a symmetric tiling (t.tail as set) that makes at most `pieces` work items per CTA of a
+// full grid, as many as that allows: one item more than CTAs would cost a whole second round.
 constexpr int kSymPieces = 6;
 int sym_slice(const nbody_ctx* c, const Tiling& t, int n_ctas, int pieces) {
-  const double len = total_pairs(c) / ((double)n_ctas * pieces * t.block * t.ipt);
-  const double q = sym_block(c->cfg.precision);
-  return (int)std::min(1.0e9, std::max(q, q * std::floor(len / q + 0.5)));
+  const double itile = (double)t.block * t.ipt;
+  auto fits = [&](int64_t slice) {
+    const int64_t most = (int64_t)pieces * n_ctas;
+    int64_t items = 0, step, last = 0, own = 0;  // own: items of a system of `last` bodies
+    for (int s = 0; s < c->n_sys && items <= most; ++s) {
+      const int64_t n = c->offsets[s + 1] - c->offsets[s];
+      if (n != last) {
+        const SymRows R(c, t, n);
+        own = 0, last = n;
+        for (int64_t r = 0; r < R.rows; ++r) own += R.pieces(r, (double)slice * itile, t.tail, &step);
+      }
+      items += own;
+    }
+    return items <= most;
+  };
+  int64_t lo = 1, hi = 1;  // the least slice that fits lies in (lo, hi], or no slice does (every row one piece)
+  while (!fits(hi) && hi < (int64_t)1 << 30) lo = hi, hi *= 2;
+  while (hi - lo > std::max<int64_t>(1, lo / 256)) {
+    const int64_t mid = (lo + hi) / 2;
+    (fits(mid) ? hi : lo) = mid;
+  }
+  return (int)std::min<int64_t>(hi, 1 << 30);
 }
 
 // Slice length for tiling t: the largest power-of-two multiple of jtile that
@@ -444,37 +483,29 @@ nbody_status upload_chunks(nbody_ctx* c, const std::vector<Chunk>& ch, Chunk** d
   return NBODY_OK;
 }
 
-// Work list of the symmetric pass for tiling t (see sym_common.cuh): rows of
-// whole i-tiles, at most kMaxSymRows per system (a body has a slot per row up to
-// its own, so more rows would mean more partials to combine than pair work saved),
-// each cut into pieces of about slice x i-tile pairs. Chunks get their slots; rows
-// is the number of entries the partial buffer needs.
+// Work list of the symmetric pass for tiling t (see sym_common.cuh, SymRows), pieces of
+// about slice x i-tile pairs. Chunks get their slots; rows is the number of entries the
+// partial buffer needs.
 void build_sym_items(const nbody_ctx* c, const Tiling& t, std::vector<SymItem>& items, std::vector<Chunk>& chunks,
                      int& max_slots, int64_t& rows) {
   items.clear();
   chunks = c->chunks;
   max_slots = 1;
   rows = 0;
-  const int64_t itile = (int64_t)t.block * t.ipt;
-  const int64_t q = sym_block(c->cfg.precision);
-  const double area = (double)t.slice * (double)itile;
+  const double area = (double)t.slice * (double)t.block * t.ipt;
   std::vector<int> slots;
   for (int s = 0; s < c->n_sys; ++s) {
     const int64_t b = c->offsets[s], n = c->offsets[s + 1] - b;
     if (n <= 0) continue;
-    const int64_t H = itile * ((n + itile * kMaxSymRows - 1) / (itile * kMaxSymRows)), nr = (n + H - 1) / H;
-    slots.assign((size_t)nr, 0);
-    const size_t first = items.size();
+    const SymRows R(c, t, n);
+    const int64_t H = R.H;
+    slots.assign((size_t)R.rows, 0);
     int most = 0;
-    for (int64_t r = 0; r < nr; ++r) {
-      const int64_t i0 = r * H, ni = std::min(H, n - i0), len = n - i0;
-      const double pairs = (double)ni * ((double)len - 0.5 * (double)ni);
-      const double want = t.tail == 1 && (r & 1) ? area / 3.0 : area;
-      const int64_t blocks = (len + q - 1) / q;  // pieces are whole blocks
-      int64_t p = std::max<int64_t>(1, std::min(blocks, (int64_t)(pairs / want + 0.5)));
-      const int64_t step = std::max<int64_t>(1, (2 * blocks + p) / (2 * p));
-      if (t.tail != 2) p = (blocks + step - 1) / step;
-      auto cut = [&](int64_t k) { return std::min(n, i0 + q * (t.tail == 2 ? k * blocks / p : k * step)); };
+    for (int64_t r = 0; r < R.rows; ++r) {
+      const int64_t i0 = r * H, ni = std::min(H, n - i0);
+      int64_t step;
+      const int64_t p = R.pieces(r, area, t.tail, &step);
+      auto cut = [&](int64_t k) { return std::min(n, i0 + R.block * (t.tail == 2 ? k * R.blocks(r) / p : k * step)); };
       slots[(size_t)r] = (int)(r + 1 + p);
       most = std::max(most, slots[(size_t)r]);
       for (int64_t k = 0; k < p; ++k) {
@@ -497,7 +528,6 @@ void build_sym_items(const nbody_ctx* c, const Tiling& t, std::vector<SymItem>& 
       ch.stride = (int32_t)n;
       ch.row0 = rows - b;
     }
-    (void)first;
     max_slots = std::max(max_slots, most);
     rows += (int64_t)most * n;
   }
@@ -791,6 +821,7 @@ nbody_status upload_plain_staging(nbody_ctx* c) {
   p.r2c = g.law == NBODY_LAW_LJ
               ? (float)((kNearRadiusSigma * kNearRadiusSigma * g.lj_sigma * g.lj_sigma + e2) * sc2)
               : (float)(kNearRadiusEps * kNearRadiusEps * e2);
+  p.uniform = g.precision == NBODY_MIXED && g.law == NBODY_LAW_GRAVITY;  // (the synthetic systems': equal masses)
   const std::vector<SysParam> all((size_t)c->n_sys, p);
   NB_CUDA(c, cudaMemcpy(c->sysp.p, all.data(), all.size() * sizeof(SysParam), cudaMemcpyHostToDevice));
   return NBODY_OK;
@@ -843,7 +874,7 @@ nbody_status fill_synthetic(nbody_ctx* c, bool with_w) {
       const double X = pos[3 * i] * c->stage_scale, Y = pos[3 * i + 1] * c->stage_scale,
                    Z = pos[3 * i + 2] * c->stage_scale;
       const float hx = (float)X, hy = (float)Y, hz = (float)Z;
-      h[i] = make_float4(hx, hy, hz, (float)mass[i]);
+      h[i] = make_float4(hx, hy, hz, c->cfg.law == NBODY_LAW_GRAVITY ? 1.f : (float)mass[i]);  // as SysParam::uniform says
       hl[i] = make_float4((float)(X - hx), (float)(Y - hy), (float)(Z - hz), 0.f);
     }
     NB_CUDA(c, cudaMemcpy(c->stage.p, h.data(), n * sizeof(float4), cudaMemcpyHostToDevice));
@@ -875,7 +906,7 @@ nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
   PairLaunch L = pair_launch(c, vjp);
   const bool sym = is_sym(t);  // timed whole: too large layouts do not come here
   auto launch = [&](const PairLaunch& P) {
-    if (sym) return launch_pairs(c, vjp, Potential::kBodies, c->stream);
+    if (sym) return launch_pairs(c, vjp, Potential::kEnergy, c->stream);  // (between the other two in cost)
     return vjp ? launch_vjp(c->cfg.precision, P, c->stream) : launch_force(c->cfg.precision, P, c->stream);
   };
   PostLaunch C{};
@@ -1037,22 +1068,34 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
     // nothing to choose between: its cost per pair no longer depends on the tiling
     Tiling t;
     t.block = mixed && !vjp ? 256 : 128, t.ipt = !mixed ? 1 : vjp ? 2 : 4;
-    t.jtile = sym_tile(g.precision, vjp, t.block), t.variant = kSymVariant, t.tail = 1;
+    t.jtile = sym_tile(g.precision, vjp), t.variant = kSymVariant, t.tail = 1;
     if (install_tiling(c, t, vjp) == NBODY_OK) {
       tune_cache_store(c, vjp, vjp ? c->vt : c->ft);
       return NBODY_OK;
     }
   }
+  // Work lists of the symmetric tilings: one item per CTA of a full grid (or a few), cut evenly or
+  // with shorter pieces for the end of the schedule. They are timed with the refined slicings below.
+  std::vector<Tiling> sym_settings;
   if (sym && !large) {
     const std::vector<std::pair<int, int>> br =
         mixed && vjp ? std::vector<std::pair<int, int>>{{128, 1}, {128, 2}, {256, 2}}
-        : mixed      ? std::vector<std::pair<int, int>>{{64, 4}, {128, 2}, {128, 4}, {256, 2}, {256, 4}}
+        : mixed      ? std::vector<std::pair<int, int>>{{128, 2}, {128, 4}, {256, 2}, {256, 4}}
         : vjp        ? std::vector<std::pair<int, int>>{{64, 1}, {128, 1}, {256, 1}}
                      : std::vector<std::pair<int, int>>{{64, 1}, {128, 1}, {256, 1}, {128, 2}};
     for (const auto& p : br) {
       Tiling t;
-      t.block = p.first, t.ipt = p.second, t.jtile = sym_tile(g.precision, vjp, t.block), t.variant = kSymVariant;
-      cands.push_back(t);
+      t.block = p.first, t.ipt = p.second, t.jtile = sym_tile(g.precision, vjp), t.variant = kSymVariant;
+      const int n_ctas = ctas_per_sm(g.precision, t, vjp, g.law) * c->sm_count;
+      if (n_ctas <= 0) continue;
+      for (const auto& tk : std::vector<std::pair<int, int>>{
+               {2, 1}, {2, 2}, {2, 3}, {2, 4}, {2, 6}, {0, 1}, {0, 2}, {0, 4}, {0, 6}, {1, 2}, {1, 4}, {1, 6}}) {
+        t.tail = tk.first;
+        t.slice = sym_slice(c, t, n_ctas, tk.second);
+        if (sym_settings.empty() || sym_settings.back().tail != t.tail || sym_settings.back().block != t.block ||
+            sym_settings.back().ipt != t.ipt || sym_settings.back().slice != t.slice)
+          sym_settings.push_back(t);
+      }
     }
     if (sym_only) variants.clear();
   }
@@ -1069,7 +1112,8 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
         }
       }
     }
-  if (cands.empty()) return fail(c, NBODY_EINVAL, "no compiled tiling matches the requested parameters");
+  if (cands.empty() && sym_settings.empty())
+    return fail(c, NBODY_EINVAL, "no compiled tiling matches the requested parameters");
   nbody_status s = fill_synthetic(c, vjp);
   if (s) return s;
   if ((s = ensure(c, c->a_scratch, (size_t)c->n_total * 3 * sizeof(double)))) return s;
@@ -1082,7 +1126,7 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
   // wave quantisation of the final work list, which the prefix cannot see)
   auto measure = [&](const Tiling& t0, double* cost) -> nbody_status {
     Tiling t = t0;
-    if (large && t.slice == 0) t.slice = kTuneSlice;  // (no symmetric tiling comes here)
+    if (large && t.slice == 0) t.slice = kTuneSlice;
     nbody_status r;
     if ((r = install_tiling(c, t, vjp))) return r;
     if ((r = time_tiling(c, vjp, cost))) return r;
@@ -1112,12 +1156,13 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
     if ((s = measure(t0, &cost))) return s;
     timed.push_back({cost, t0});
   }
-  if (timed.empty()) return fail(c, NBODY_EINVAL, "no compiled tiling matches the requested parameters");
+  if (timed.empty() && sym_settings.empty())
+    return fail(c, NBODY_EINVAL, "no compiled tiling matches the requested parameters");
   // the candidates within 8% of the best (at most five) are timed twice more, interleaved, and
   // keep their best time: single timings differ by 1-3% from run to run
   std::stable_sort(timed.begin(), timed.end(),
                    [](const std::pair<double, Tiling>& a, const std::pair<double, Tiling>& b) { return a.first < b.first; });
-  size_t top = 1;
+  size_t top = std::min<size_t>(1, timed.size());
   while (top < timed.size() && top < 5 && timed[top].first <= 1.08 * timed[0].first) ++top;
   for (int round = 0; round < 2 && top > 1; ++round)
     for (size_t k = 0; k < top; ++k) {
@@ -1128,7 +1173,7 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
   // order the re-timed candidates; the first is the choice unless the slice refinement finds better
   std::stable_sort(timed.begin(), timed.begin() + top,
                    [](const std::pair<double, Tiling>& a, const std::pair<double, Tiling>& b) { return a.first < b.first; });
-  Tiling bt = timed[0].second;
+  Tiling bt = timed.empty() ? sym_settings[0] : timed[0].second;
   // slice-length refinement of all those tilings (up to five): the automatic
   // choice, half and twice it, and (one system) the lengths whose work list
   // fills a whole number of waves of the persistent grid (equal items, a
@@ -1139,27 +1184,20 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
   // of each other, and the one the tail favours must not be cut by that noise.
   // Every setting is timed once and those within 3% of the best once more.
   if ((vjp || g.slice == 0) && !large) {
-    std::vector<Tiling> settings;
-    for (size_t f = 0; f < std::min<size_t>(top, is_sym(timed[0].second) ? 3 : 5); ++f) {
+    std::vector<Tiling> settings = sym_settings;
+    for (size_t f = 0; f < top; ++f) {
       Tiling base = timed[f].second;
-      if (vjp && !is_sym(base)) {
+      if (vjp) {
         settings.push_back(base);
         continue;
       }
       base.slice = 0;
       base.tail = 0;
       if ((s = install_tiling(c, base, vjp))) return s;
-      const int L0 = (vjp ? c->vt : c->ft).slice;
-      // (a short list has fewer CTAs than the grid it is planned for)
-      const int64_t n_ctas = is_sym(base) ? (int64_t)ctas_per_sm(g.precision, base, vjp, g.law) * c->sm_count : c->ft.n_ctas;
+      const int L0 = c->ft.slice;
+      const int64_t n_ctas = c->ft.n_ctas;
       std::vector<int> ls = {L0 / 2, L0, L0 * 2};
-      if (is_sym(base)) {
-        ls.clear();
-        for (int k : {1, 2, 3, 4, 6, 8}) {
-          const int len = sym_slice(c, base, (int)n_ctas, k);
-          if (std::find(ls.begin(), ls.end(), len) == ls.end()) ls.push_back(len);
-        }
-      } else if (c->n_sys == 1) {
+      if (c->n_sys == 1) {
         const int64_t n = c->offsets[1], tiles = (n + (int64_t)base.block * base.ipt - 1) / ((int64_t)base.block * base.ipt);
         for (int64_t W = 1; W <= 64 && ls.size() < 7; ++W) {
           const int64_t ns = W * n_ctas / tiles;  // slices per tile with tiles x ns <= W x CTAs
@@ -1172,7 +1210,7 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
       }
       for (int len : ls) {
         if (len < kSliceQuantum) continue;
-        for (int tail = 0; tail < (is_sym(base) ? 3 : 2); ++tail) {
+        for (int tail = 0; tail < 2; ++tail) {
           Tiling t = base;
           t.slice = len;
           t.tail = tail;

@@ -248,7 +248,6 @@ cudaError_t launch_sym_force(int precision, const SymLaunch& L, cudaStream_t st)
 int sym_force_ctas_per_sm(int precision, int block, int ipt, int law);
 constexpr int kSymTile = 256;   // j-bodies per shared-memory tile of the symmetric kernels, mixed
 constexpr int kSymTile64 = 64;  // ... and FP64
-constexpr int sym_force_tile(int warps) { return warps <= 2 ? kSymTile / 2 : kSymTile; }
 cudaError_t launch_sym_vjp(int precision, const SymLaunch& L, cudaStream_t st);
 int sym_vjp_ctas_per_sm(int precision, int block, int ipt);
 constexpr int kSymVjpTile = 128;  // j-tile of the mixed symmetric VJP (FP64: kSymTile64)

@@ -14,7 +14,7 @@ namespace {
 template <int LAW, int W, int R, int PHI, int MINB>
 __global__ void __launch_bounds__(W * 32, MINB) k_force_sym(const SymLaunch L) {
   extern __shared__ __align__(16) unsigned char raw[];
-  auto& sm = *reinterpret_cast<sym::Smem<W, R, sym_force_tile(W)>*>(raw);
+  auto& sm = *reinterpret_cast<sym::Smem<W, R, kSymTile>*>(raw);
   pdl_wait();
   ItemSource source{L.counter, &sm.item};
   auto next = [&](SymItem& it) {
@@ -22,7 +22,7 @@ __global__ void __launch_bounds__(W * 32, MINB) k_force_sym(const SymLaunch L) {
     if (n < L.n_items) it = L.items[n];
     return n < L.n_items;
   };
-  sym::items<LAW, W, R, sym_force_tile(W), PHI>(L, next, sm);
+  sym::items<LAW, W, R, kSymTile, PHI>(L, next, sm);
   pdl_trigger();
   retire_cta(L.counter);
 }
@@ -56,8 +56,7 @@ int occupancy_of(K kern, int block, size_t smem) {
 }  // namespace
 
 // Compiled: warps, i-bodies per lane (and resident CTAs).
-// (2, 4) has the i-tile of (4, 2) with half the shared-memory and shuffle work per pair.
-#define NBODY_SYM_TILINGS(X) X(2, 4, 8) X(4, 2, 6) X(4, 4, 4) X(8, 2, 3) X(8, 4, 2)
+#define NBODY_SYM_TILINGS(X) X(4, 2, 6) X(4, 4, 4) X(8, 2, 3) X(8, 4, 2)
 #define NBODY_SYM64_TILINGS(X) X(2, 1) X(4, 1) X(8, 1) X(4, 2)
 
 // f(law, potential) as integral constants
@@ -85,7 +84,7 @@ cudaError_t launch_sym_force(int precision, const SymLaunch& L, cudaStream_t st)
     }
 #define NBODY_X(W, R, MINB)            \
   if (L.block == W * 32 && L.ipt == R) \
-    return launch_pdl_smem(k_force_sym<LAW, W, R, PHI, MINB>, L.n_ctas, W * 32, sizeof(sym::Smem<W, R, sym_force_tile(W)>), st, L);
+    return launch_pdl_smem(k_force_sym<LAW, W, R, PHI, MINB>, L.n_ctas, W * 32, sizeof(sym::Smem<W, R, kSymTile>), st, L);
     NBODY_SYM_TILINGS(NBODY_X)
 #undef NBODY_X
     return cudaErrorInvalidConfiguration;
@@ -107,7 +106,7 @@ int sym_force_ctas_per_sm(int precision, int block, int ipt, int law) {
               }
 #define NBODY_X(W, R, MINB)        \
   if (block == W * 32 && ipt == R) \
-    return occupancy_of(k_force_sym<LAW, W, R, PHI, MINB>, W * 32, sizeof(sym::Smem<W, R, sym_force_tile(W)>));
+    return occupancy_of(k_force_sym<LAW, W, R, PHI, MINB>, W * 32, sizeof(sym::Smem<W, R, kSymTile>));
               NBODY_SYM_TILINGS(NBODY_X)
 #undef NBODY_X
               return 0;
