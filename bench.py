@@ -37,16 +37,31 @@ if ROOT not in sys.path:
 METRIC = "body-body interactions/s, mixed vs FP64 path at ≤1e-4 force err; % FP32 roofline"
 UNIT = "interactions/s"
 WORKLOAD = dict(n=65536, G=1.0, eps=0.005, dt=5e-4, seed=2)
-# float32-pipe operations per interaction in the mixed force kernel:
-# 3 FADD (d) + 3 FFMA (s^2) + 3 FMUL (m/s, 1/s^2, m/s^3) + 3 FFMA (a) + 1 FADD (phi); MUFU.RSQ not counted
-OPS_PER_INTERACTION = 13
+
+
+def ops_per_interaction(sym, law="gravity", equal_masses=True, record=True):
+    """float32-pipe operations per interaction in the mixed force kernels (MUFU not counted).
+
+    One-sided: 3 FADD (d) + 3 FFMA (s^2) + 3 FMUL (m/s, 1/s^2, m/s^3) + 3 FFMA (a) + 1 FADD (phi);
+    Lennard-Jones 16. Symmetric pass, per unordered pair (two interactions): 3 FADD + 3 FFMA + 2 FMUL
+    (1/s^2, 1/s^3) + 2 FMUL (the masses, unless all are equal) + 6 FFMA (both bodies' forces), one more
+    for an energy record; Lennard-Jones 17 and two more."""
+    if law == "lj":
+        return (17 + 2 * record) / 2 if sym else 14 + 2 * record
+    return (14 + 2 * (not equal_masses) + record) / 2 if sym else 12 + record
+
+
+def is_symmetric(nb, ctx):
+    return nb.nbody_get_slicing(ctx)["tail"] >= 2
+
+
 FP32_LANES_PER_SM = 128
 SM_MAX_MHZ = 2070.0
 L2_FLUSH_BYTES = 256 << 20
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "force_mixed_n65536_full.md")
 # sources of the timed force kernel: its traffic figure is valid while their hash matches
 FORCE_SRCS = [os.path.join(ROOT, "paper_2511_02655_gb300", "csrc", f)
-              for f in ("force_kernels.cu", "force_common.cuh", "pair_common.cuh", "nbody_internal.h")]
+              for f in ("sym_kernels.cu", "sym_common.cuh", "pair_common.cuh", "nbody_internal.h")]
 
 
 def parse():
@@ -288,6 +303,7 @@ def aux_two_spheres(dev, stream):
     nb.nbody_sync(ctx)
     xf, af = xt.cpu().numpy(), at.cpu().numpy()
     tuning = nb.nbody_get_tuning(ctx)
+    ops = ops_per_interaction(is_symmetric(nb, ctx), equal_masses=False, record=False)
     ctx.close()
     del xt, vt, mt, at
     threads = oracle.default_threads()
@@ -296,7 +312,7 @@ def aux_two_spheres(dev, stream):
     (ref1, _), t1 = _timed(lambda: oracle.forces_at(xf, m, idx1, G=G, eps=eps, threads=threads))
     rate = 2.0 * ks * n / (t0 + t1)
     return {"interactions_per_s": float(n) * n * k / sec, "steps": k, "force_kernel_ms": kms / kl,
-            "frac_fp32_roofline_force_kernel": (OPS_PER_INTERACTION - 1) * float(n) * n / (kms / kl * 1e-3) / 1e12
+            "frac_fp32_roofline_force_kernel": ops * float(n) * n / (kms / kl * 1e-3) / 1e12
                                                / fp32_peak_tops(),
             "tuning": tuning,
             "force_err_vs_oracle": {"step_0": _err_stats(rel_force_error(a0[idx0], ref0)),
@@ -424,10 +440,9 @@ def aux_lj(dev, stream):
         nb.nbody_sync(ctx)
         kernel = None
         if prec == nb.MIXED:  # the force kernel alone: CUDA events around it in 200 eagerly issued steps
-            tun = nb.nbody_get_tuning(ctx)
-            ce = nb.nbody_init(law=nb.LENNARD_JONES, precision=prec, n=n, dt=dt, box=box, energy_every=1,
-                               block=tun["block"], i_per_thread=tun["i_per_thread"], j_tile=tun["j_tile"],
-                               variant=tun["variant"])
+            ce = nb.nbody_init(law=nb.LENNARD_JONES, precision=prec, n=n, dt=dt, box=box, energy_every=1)
+            tun = nb.nbody_get_tuning(ce)
+            ops = ops_per_interaction(is_symmetric(nb, ce), law="lj")
             xe, ve, ae = (torch.from_numpy(a).to(dev) for a in (x, v, np.zeros_like(x)))
             le = torch.empty((200, 1, 9), dtype=torch.float64, device=dev)
             nb.nbody_step(ce, xe, ve, mt, ae, False, 20, le[:20])
@@ -439,8 +454,8 @@ def aux_lj(dev, stream):
             ce.close()
             us = ms * 1e3 / max(1, k)
             kernel = {"tuning": tun, "force_kernel_us": us, "eager_step_us": eager / 200 * 1e6,
-                      "ops_per_interaction": 16,
-                      "frac_fp32_roofline_force_kernel": 16.0 * n * n / (us * 1e-6) / (fp32_peak_tops() * 1e12)}
+                      "ops_per_interaction": ops,
+                      "frac_fp32_roofline_force_kernel": ops * n * n / (us * 1e-6) / (fp32_peak_tops() * 1e12)}
         e = logt.cpu().numpy()[:, 0, 0]
         xf, af = xt.cpu().numpy(), at.cpu().numpy()
         idx = inputs.sample_indices(n, 2048, seed=29)
@@ -699,7 +714,9 @@ def run_ours(args):
     # ---- dominant kernel vs its roofline (FP32 pipe, derived from SM count and max clock): the force
     # kernel of the timed steps (with the potential: every step records its energy)
     kernel_s = force_ms * 1e-3 / max(1, force_launches)
-    achieved = OPS_PER_INTERACTION * interactions / kernel_s / 1e12
+    sym = is_symmetric(nb, ctx)
+    ops = ops_per_interaction(sym)
+    achieved = ops * interactions / kernel_s / 1e12
     peak = fp32_peak_tops()
     traffic = traffic_per_launch()
 
@@ -721,12 +738,10 @@ def run_ours(args):
     ctx64.close()
 
     # ---- end to end through the host-memory entry point (pinned buffers, copies inside the timing):
-    # a context with the same tiling that replays its step as a CUDA graph; L2 flushed between
+    # a context of its own tuning that replays its step as a CUDA graph; L2 flushed between
     # steps outside the timing, each call timed on the host clock (it returns after its sync)
     ke = max(3, min(K, 50))
-    ctx_h = nb.nbody_init(G=G, eps=eps, dt=dt, precision=nb.MIXED, n=n, energy_every=1, flags=nb.FLAG_GRAPH,
-                          block=tuning["block"], i_per_thread=tuning["i_per_thread"], j_tile=tuning["j_tile"],
-                          slice=tuning["slice"], variant=tuning["variant"])
+    ctx_h = nb.nbody_init(G=G, eps=eps, dt=dt, precision=nb.MIXED, n=n, energy_every=1, flags=nb.FLAG_GRAPH)
     xh = xt.cpu().pin_memory()
     vh = vt.cpu().pin_memory()
     mh = mt.cpu().pin_memory()
@@ -783,8 +798,9 @@ def run_ours(args):
             },
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tops/s (FP32 pipe)",
                          "frac": achieved / peak, "traffic": traffic,
-                         "kernel": "k_force_mixed2 (packed float32x2 pair arithmetic with the potential)",
-                         "ops_per_interaction": OPS_PER_INTERACTION,
+                         "kernel": "k_force_sym (every unordered pair once, packed float32x2, energy record)" if sym
+                                   else "k_force_mixed2 (packed float32x2 pair arithmetic with the potential)",
+                         "ops_per_interaction": ops,
                          "kernel_ms": kernel_s * 1e3,
                          "peak_basis": f"{torch.cuda.get_device_properties(dev).multi_processor_count} SMs x "
                                        f"{FP32_LANES_PER_SM} FP32 lanes x {SM_MAX_MHZ:.0f} MHz"},

@@ -222,9 +222,11 @@ nbody_status nbody_sync(nbody_ctx* ctx);
 /*
  * Tiling in use (after init / autotune): block, i_per_thread, j_tile, slice,
  * the number of persistent CTAs the force kernel launches, and the force
- * kernel variant (as in nbody_config.variant: 1 scalar, 2 packed, 3 packed capped; 4, which
- * cannot be requested: the symmetric pass, every unordered pair once, both precisions, with
- * block also 64). Any pointer may be NULL.
+ * kernel variant (as in nbody_config.variant: 1 scalar, 2 packed, 3 packed capped). Any pointer
+ * may be NULL. The values can be handed back to nbody_init. Where the tuner chose the
+ * symmetric pass (every unordered pair evaluated once; both precisions), which cannot
+ * be requested, the nearest one-sided tiling and the longest piece's j-bodies as slice are
+ * reported; nbody_get_slicing tells the two apart.
  */
 nbody_status nbody_get_tuning(const nbody_ctx* ctx, int32_t* block, int32_t* i_per_thread, int32_t* j_tile,
                               int32_t* slice, int32_t* n_ctas, int32_t* variant);
@@ -232,7 +234,7 @@ nbody_status nbody_get_tuning(const nbody_ctx* ctx, int32_t* block, int32_t* i_p
 /*
  * Work-list shape of the force pass (after init / autotune): tail = 0 when
  * each system's j-range is cut into equal slices, 1 when it ends in a tail of
- * halving slices; the number of work items and the largest slice count of any
+ * halving slices, 2 and more for the symmetric pass; the number of work items and the largest slice count of any
  * system. Any pointer may be NULL.
  */
 nbody_status nbody_get_slicing(const nbody_ctx* ctx, int32_t* tail, int32_t* n_items, int32_t* max_slices);

@@ -351,7 +351,8 @@ def nbody_get_tuning(ctx: Context) -> dict:
 
 
 def nbody_get_slicing(ctx: Context) -> dict:
-    """Work-list shape of the force pass: tail (0 equal slices, 1 halving tail), n_items, max_slices."""
+    """Work-list shape of the force pass: tail (0 equal slices, 1 halving tail, 2.. symmetric pass), n_items,
+    max_slices."""
     sl = [ctypes.c_int32() for _ in range(3)]
     _check(load().nbody_get_slicing(ctx._h, *[ctypes.byref(v) for v in sl]), ctx)
     return dict(zip(("tail", "n_items", "max_slices"), (v.value for v in sl)))

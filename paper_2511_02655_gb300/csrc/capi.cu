@@ -43,6 +43,7 @@ struct Tiling {
                     // row in pieces a third as long, 2 pieces of a row as equal as whole blocks allow)
 };
 constexpr int kSymVariant = 3;
+constexpr int kSymTail = 2;  // nbody_get_slicing: tail modes of the symmetric pass are reported from here on
 enum class Potential { kNone = 0, kBodies = 1, kEnergy = 2 };  // as sym::kPhi*
 constexpr double kSymMinBodies = 3000.0;    // typical system size from which the symmetric pass is a candidate
 constexpr double kSymOnlyBodies = 8192.0;  // ... and from which it is the only one (mixed path)
@@ -147,6 +148,7 @@ struct nbody_ctx {
   int n_items = 0;
   int max_slices = 1;
   size_t fpart_bytes = 0;  // partial sums of the force pass
+  int sym_longest = 0;     // symmetric force list: j-bodies of its longest piece
   // VJP work list (built on first adjoint)
   Tiling vt;
   void* d_vitems = nullptr;
@@ -561,6 +563,10 @@ nbody_status install_tiling(nbody_ctx* c, Tiling t, bool vjp) {
     if (part_bytes > kMaxSymPartialBytes)
       return fail(c, NBODY_EINVAL, "symmetric tiling needs %zu bytes of partial sums", part_bytes);
     n_items = (int)items.size();
+    if (!vjp) {
+      c->sym_longest = 1;
+      for (const SymItem& w : items) c->sym_longest = std::max(c->sym_longest, w.j_end - w.j_begin);
+    }
     if ((s = upload_items(c, items.data(), items.size() * sizeof(SymItem), vjp ? &c->d_vitems : &c->d_items))) return s;
   } else {
     if (t.slice <= 0) t.slice = auto_slice(c, t, occ * c->sm_count);
@@ -1840,18 +1846,29 @@ nbody_status nbody_sync(nbody_ctx* c) {
 nbody_status nbody_get_tuning(const nbody_ctx* c, int32_t* block, int32_t* ipt, int32_t* jtile, int32_t* slice,
                               int32_t* n_ctas, int32_t* variant) {
   if (!c) return NBODY_EINVAL;
-  if (block) *block = c->ft.block;
-  if (ipt) *ipt = c->ft.ipt;
-  if (jtile) *jtile = c->ft.jtile;
-  if (slice) *slice = c->ft.slice;
-  if (n_ctas) *n_ctas = c->ft.n_ctas;
-  if (variant) *variant = c->ft.variant + 1;
+  // A symmetric tiling cannot be requested, but what is reported can always be handed back to
+  // nbody_init: the one-sided tiling nearest to it (packed on the mixed path).
+  Tiling t = c->ft;
+  if (is_sym(t)) {
+    const bool mixed = c->cfg.precision == NBODY_MIXED;
+    t.block = std::max(128, t.block);
+    t.jtile = mixed ? 256 : 128;
+    t.variant = mixed ? 1 : 0;
+    if (mixed && c->cfg.law == NBODY_LAW_LJ) t.block = 128, t.ipt = 2;
+    t.slice = c->sym_longest;
+  }
+  if (block) *block = t.block;
+  if (ipt) *ipt = t.ipt;
+  if (jtile) *jtile = t.jtile;
+  if (slice) *slice = t.slice;
+  if (n_ctas) *n_ctas = t.n_ctas;
+  if (variant) *variant = t.variant + 1;
   return NBODY_OK;
 }
 
 nbody_status nbody_get_slicing(const nbody_ctx* c, int32_t* tail, int32_t* n_items, int32_t* max_slices) {
   if (!c) return NBODY_EINVAL;
-  if (tail) *tail = c->ft.tail;
+  if (tail) *tail = is_sym(c->ft) ? kSymTail + c->ft.tail : c->ft.tail;
   if (n_items) *n_items = c->n_items;
   if (max_slices) *max_slices = c->max_slices;
   return NBODY_OK;

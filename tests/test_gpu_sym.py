@@ -51,7 +51,7 @@ def test_sym_forces(nb, tmp_path, monkeypatch, tiling, n, masses):
     x, v, m = inputs.plummer(n, seed=n)
     m = _masses(m, masses, n)
     ctx = _forced(nb, tmp_path / "tune", {"force": tiling}, G=G, eps=eps, dt=1e-3, n=n)
-    assert nb.nbody_get_tuning(ctx)["variant"] == 4
+    assert nb.nbody_get_slicing(ctx)["tail"] >= 2
     xt, mt = to_dev(x, m)
     a, phi = nb.nbody_forces(ctx, xt, mt)
     a0, _ = nb.nbody_forces(ctx, xt, mt, with_phi=False)
@@ -73,7 +73,7 @@ def test_sym_lennard_jones(nb, tmp_path, monkeypatch, tiling):
     m = _masses(m, "lognormal", 3)
     ctx = _forced(nb, tmp_path / "tune", {"force": tiling}, law=nb.LENNARD_JONES, dt=1e-3, n=2050, lj_epsilon=1.3,
                   lj_sigma=0.9)
-    assert nb.nbody_get_tuning(ctx)["variant"] == 4
+    assert nb.nbody_get_slicing(ctx)["tail"] >= 2
     a, phi = nb.nbody_forces(ctx, *to_dev(x, m))
     nb.nbody_sync(ctx)
     a_ref, phi_ref = oracle.lj_forces(x, m, eps_lj=1.3, sigma=0.9)
@@ -99,7 +99,7 @@ def test_sym64_forces(nb, tmp_path, monkeypatch, tiling, n, length, mass, masses
     m = _masses(m, masses, n)
     xs, ms, eps = x * length, m * mass, 0.03 * length
     ctx = _forced(nb, tmp_path / "tune", {"force": tiling}, G=1.1, eps=eps, dt=1e-3, n=n, precision=nb.FP64)
-    assert nb.nbody_get_tuning(ctx)["variant"] == 4
+    assert nb.nbody_get_slicing(ctx)["tail"] >= 2
     xt, mt = to_dev(xs, ms)
     a, phi = nb.nbody_forces(ctx, xt, mt)
     a0, _ = nb.nbody_forces(ctx, xt, mt, with_phi=False)
@@ -118,7 +118,7 @@ def test_sym64_masses_change_between_calls(nb):
     x, v, m = inputs.plummer(n, seed=8)
     m2 = _masses(m, "lognormal", 8)
     ctx = nb.nbody_init(G=G, eps=eps, dt=dt, n=n, precision=nb.FP64, energy_every=2, flags=nb.FLAG_GRAPH)
-    assert nb.nbody_get_tuning(ctx)["variant"] == 4
+    assert nb.nbody_get_slicing(ctx)["tail"] >= 2
     xt, vt, mt = to_dev(x, v, m)
     at = torch.empty_like(xt)
     log = torch.empty((1, 1, 9), dtype=torch.float64, device="cuda")
@@ -142,7 +142,7 @@ def test_sym64_lennard_jones_and_coincident(nb, tmp_path, monkeypatch, tiling):
     m = _masses(m, "lognormal", 3)
     kw = dict(law=nb.LENNARD_JONES, dt=1e-3, n=1100, lj_epsilon=1.3, lj_sigma=0.9, precision=nb.FP64)
     ctx = _forced(nb, tmp_path / "tune", {"force": tiling}, **kw)
-    assert nb.nbody_get_tuning(ctx)["variant"] == 4
+    assert nb.nbody_get_slicing(ctx)["tail"] >= 2
     a, phi = nb.nbody_forces(ctx, *to_dev(x, m))
     nb.nbody_sync(ctx)
     a_ref, phi_ref = oracle.lj_forces(x, m, eps_lj=1.3, sigma=0.9)
@@ -175,6 +175,24 @@ def test_mixed_forces_in_any_units(nb, length, mass):
         ctx.close()
 
 
+@pytest.mark.parametrize("law", [0, 1])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_reported_tiling_can_be_requested(nb, law, prec):
+    """Whatever the tuner chose, what nbody_get_tuning reports is a valid request."""
+    n = 4500
+    x, v, m, box = inputs.lj_gas(n, seed=3) if law else inputs.plummer(n, seed=3) + (0.0,)
+    kw = dict(law=law, precision=prec, n=n, dt=1e-3, eps=0.0 if law else 0.02)
+    ctx = nb.nbody_init(**kw)
+    a, _ = nb.nbody_forces(ctx, *to_dev(x, m))
+    assert nb.nbody_get_slicing(ctx)["tail"] >= 2 or prec == 1
+    t = nb.nbody_get_tuning(ctx)
+    again = nb.nbody_init(block=t["block"], i_per_thread=t["i_per_thread"], j_tile=t["j_tile"], slice=t["slice"],
+                          variant=t["variant"], **kw)
+    b, _ = nb.nbody_forces(again, *to_dev(x, m))
+    nb.nbody_sync(again)
+    assert force_rel_err(b.cpu().numpy(), a.cpu().numpy()).max() <= (1e-4 if prec else 1e-12)
+
+
 def test_sym_several_systems_and_zero_masses(nb, tmp_path, monkeypatch):
     """Systems of every kind in one list: empty, single, equal masses, unequal ones, massless bodies
     (they feel forces and exert none), one far from the origin."""
@@ -188,7 +206,7 @@ def test_sym_several_systems_and_zero_masses(nb, tmp_path, monkeypatch):
     m[off[5]:off[6]] *= np.exp(np.random.default_rng(1).standard_normal(700))
     x[off[7]:off[8]] += 50.0
     ctx = _forced(nb, tmp_path / "tune", {"force": (128, 2, 256, 128, 3, 1)}, G=1.0, eps=0.02, dt=1e-3, offsets=off)
-    assert nb.nbody_get_tuning(ctx)["variant"] == 4
+    assert nb.nbody_get_slicing(ctx)["tail"] >= 2
     xt, mt = to_dev(x, m)
     a, phi = nb.nbody_forces(ctx, xt, mt)
     a2, phi2 = nb.nbody_forces(ctx, xt, mt)
