@@ -69,6 +69,8 @@ class _Config(ctypes.Structure):
 def load():
     """Loads libnbody.so (built by ``paper_2511_02655_gb300.build``); raises if it is missing."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -159,14 +161,29 @@ def _check(status: int, ctx=None):
         raise NBodyError(status, nbody_last_error(ctx))
 
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
+
+
+# Small systems are bound by the host: of the 18 us that nbody_forces took here, the C call is 8 (12
+# now, measured at 300 and 1024 bodies). A Stream object per call (3 us), an import statement
+# per argument and ctypes objects for the addresses were the difference.
+def _current_stream(device: int) -> int:
+    """Handle of the current CUDA stream of a device."""
+    torch = _torch()
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return raw(device) if raw else torch.cuda.current_stream(device).cuda_stream
 
 
 def _bind_stream(ctx: Context):
-    torch = _torch()
-    s = torch.cuda.current_stream().cuda_stream
+    s = _current_stream(_torch().cuda.current_device())
     if s != ctx._stream:
         _check(load().nbody_set_stream(ctx._h, ctx_ptr(s)), ctx)
         ctx._stream = s
@@ -185,11 +202,11 @@ def _dev(t, name, shape, ctx: Context, allow_none=False):
     torch = _torch()
     if not isinstance(t, torch.Tensor) or not t.is_cuda or t.dtype != torch.float64:
         raise TypeError(f"{name} must be a CUDA float64 tensor")
-    if tuple(t.shape) != tuple(shape):
+    if t.shape != shape:
         raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    return ctx_ptr(t.data_ptr())
+    return t.data_ptr() or None
 
 
 def nbody_init(*, G=1.0, eps=0.0, dt=0.0, precision=MIXED, offsets=None, n=None, energy_every=0, block=0,
@@ -403,11 +420,14 @@ def nbody_forces_noalloc(x, m, G, eps, a=None, phi=None):
     check(a, "a", (n, 3))
     if phi is not None:
         check(phi, "phi", (n,))
-    stream = torch.cuda.current_stream(x.device).cuda_stream
-    with torch.cuda.device(x.device):
-        st = load().nbody_forces_noalloc(ctx_ptr(x.data_ptr()), ctx_ptr(m.data_ptr()), n, float(G), float(eps),
-                                         ctx_ptr(a.data_ptr()), ctx_ptr(phi.data_ptr()) if phi is not None else None,
-                                         ctx_ptr(stream))
+    dev = x.device.index
+    args = (x.data_ptr() or None, m.data_ptr() or None, n, float(G), float(eps), a.data_ptr() or None,
+            phi.data_ptr() or None if phi is not None else None, _current_stream(dev) or None)
+    if dev == torch.cuda.current_device():
+        st = load().nbody_forces_noalloc(*args)
+    else:
+        with torch.cuda.device(dev):
+            st = load().nbody_forces_noalloc(*args)
     _check(st)
     return a, phi
 
