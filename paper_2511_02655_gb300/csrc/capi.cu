@@ -323,25 +323,28 @@ struct SymRows {
   }
 };
 
+// Work items of a symmetric tiling with the given slice, counted up to `most` and a little beyond.
+int64_t sym_item_count(const nbody_ctx* c, const Tiling& t, int64_t slice, int64_t most) {
+  const double area = (double)slice * t.block * t.ipt;
+  int64_t items = 0, step, last = 0, own = 0;  // own: items of a system of `last` bodies
+  for (int s = 0; s < c->n_sys && items <= most; ++s) {
+    const int64_t n = c->offsets[s + 1] - c->offsets[s];
+    if (n != last) {
+      const SymRows R(c, t, n);
+      own = 0, last = n;
+      for (int64_t r = 0; r < R.rows; ++r) own += R.pieces(r, area, t.tail, &step);
+    }
+    items += own;
+  }
+  return items;
+}
+
 // Slice of a symmetric tiling (t.tail as set) that makes at most `pieces` work items per CTA of a
 // full grid, as many as that allows: one item more than CTAs would cost a whole second round.
 constexpr int kSymPieces = 6;
 int sym_slice(const nbody_ctx* c, const Tiling& t, int n_ctas, int pieces) {
-  const double itile = (double)t.block * t.ipt;
-  auto fits = [&](int64_t slice) {
-    const int64_t most = (int64_t)pieces * n_ctas;
-    int64_t items = 0, step, last = 0, own = 0;  // own: items of a system of `last` bodies
-    for (int s = 0; s < c->n_sys && items <= most; ++s) {
-      const int64_t n = c->offsets[s + 1] - c->offsets[s];
-      if (n != last) {
-        const SymRows R(c, t, n);
-        own = 0, last = n;
-        for (int64_t r = 0; r < R.rows; ++r) own += R.pieces(r, (double)slice * itile, t.tail, &step);
-      }
-      items += own;
-    }
-    return items <= most;
-  };
+  const int64_t most = (int64_t)pieces * n_ctas;
+  auto fits = [&](int64_t slice) { return sym_item_count(c, t, slice, most) <= most; };
   int64_t lo = 1, hi = 1;  // the least slice that fits lies in (lo, hi], or no slice does (every row one piece)
   while (!fits(hi) && hi < (int64_t)1 << 30) lo = hi, hi *= 2;
   while (hi - lo > std::max<int64_t>(1, lo / 256)) {
@@ -609,6 +612,12 @@ SymLaunch sym_launch(nbody_ctx* c, bool vjp, Potential phi) {
   L.sigma2 = c->cfg.lj_sigma * c->cfg.lj_sigma;
   L.law = c->cfg.law;
   L.block = t.block, L.ipt = t.ipt, L.n_ctas = t.n_ctas;
+  // Short FP64 lists leave a scheduler with one warp or none, too few to hide a pair's chain of
+  // float64 and integer operations: blocks are shared by 2 or 4 warps up to 16 warps per SM. Energy step
+  // of 512 bodies 31.8 -> 20.9 us, of 1024 33.0 -> 29.6 (4 warps), of 1400 48.4 -> 47.6 (2); a
+  // gradient step of 512 bodies 95 -> 63 us. The list of 2048 bodies has 14 warps per SM unshared.
+  const int64_t warps = (int64_t)L.n_items * (t.block / 32), room = 16 * (int64_t)c->sm_count;
+  L.split = 4 * warps <= room ? 4 : 2 * warps <= room ? 2 : 1;
   L.phi = (int)phi;
   L.epoch = c->epoch;
   L.status = c->status;
@@ -1098,6 +1107,10 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
                {2, 1}, {2, 2}, {2, 3}, {2, 4}, {2, 6}, {0, 1}, {0, 2}, {0, 4}, {0, 6}, {1, 2}, {1, 4}, {1, 6}}) {
         t.tail = tk.first;
         t.slice = sym_slice(c, t, n_ctas, tk.second);
+        // FP64 lists of few large items need an even placement on the SMs, which the timing here has
+        // and a step, whose CTAs start while the last kernel's retire, has not: 1400 bodies in 144 items
+        // of 256 threads tie with 506 of 64 here, in a step they take 51.8 us against 47.7.
+        if (!mixed && p.first > 64 && sym_item_count(c, t, t.slice, c->sm_count) < c->sm_count) continue;
         if (sym_settings.empty() || sym_settings.back().tail != t.tail || sym_settings.back().block != t.block ||
             sym_settings.back().ipt != t.ipt || sym_settings.back().slice != t.slice)
           sym_settings.push_back(t);

@@ -192,6 +192,7 @@ struct SymLaunch {
   const SysParam* sys;
   double eps2, sigma2;     // FP64 path
   int law, block, ipt, n_ctas;
+  int split;               // FP64 force: warps that share a block's work (1, 2, 4; where compiled)
   int phi;                 // potential: 0 none, 1 of every body, 2 for an energy record (sym::kPhi*)
   uint32_t epoch;          // FP64: number of the call (SysParam::uniform)
   int params;              // VJP: also the sums for the G and eps gradients

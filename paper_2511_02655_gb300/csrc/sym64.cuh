@@ -140,11 +140,12 @@ struct Smem {
 // integer operations, and small systems have few warps per scheduler to hide it.
 constexpr int kUnroll = 4;
 
-// The 32 steps of one block. FAST: returns whether the lane met an s^2 out of range, in which case
+// The 32 steps of one block, or the 32 / KS from k0 on of a warp that shares it with KS - 1 others. FAST: returns whether the lane met an s^2 out of range, in which case
 // the sums are void and the block is to be repeated without FAST (there is no branch per pair, so
 // that the pairs of several steps overlap).
-template <int LAW, bool SYM, bool MASK, int PHI, bool EQ, bool FAST, int R>
-__device__ __forceinline__ bool block32(const double (&q)[4][kTile / 32][64], const int b, const int jg0, const int lane,
+template <int LAW, bool SYM, bool MASK, int PHI, bool EQ, bool FAST, int R, int KS>
+__device__ __forceinline__ bool block32(const double (&q)[4][kTile / 32][64], const int b, const int k0, const int jg0,
+                                        const int lane,
                                         const int ig0, const double (&xi)[R], const double (&yi)[R],
                                         const double (&zi)[R], const double (&mi)[R], const double eps2,
                                         const double s2, double (&ax)[R], double (&ay)[R], double (&az)[R],
@@ -152,8 +153,8 @@ __device__ __forceinline__ bool block32(const double (&q)[4][kTile / 32][64], co
   const int src = (lane + 1) & 31;
   bool out = false;
 #pragma unroll(FAST ? kUnroll / R : 1)
-  for (int k = 0; k < 32; ++k) {
-    const int p = lane + k;
+  for (int k = 0; k < 32 / KS; ++k) {
+    const int p = lane + k0 + k;
     const double xj = q[0][b][p], yj = q[1][b][p], zj = q[2][b][p], mj = q[3][b][p];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -187,8 +188,9 @@ __device__ __forceinline__ bool block32(const double (&q)[4][kTile / 32][64], co
 }
 
 // A block with FAST, repeated without it where any lane met an s^2 out of range.
-template <int LAW, bool SYM, bool MASK, int PHI, bool EQ, int R>
-__device__ __forceinline__ void block(const double (&q)[4][kTile / 32][64], const int b, const int jg0, const int lane,
+template <int LAW, bool SYM, bool MASK, int PHI, bool EQ, int R, int KS>
+__device__ __forceinline__ void block(const double (&q)[4][kTile / 32][64], const int b, const int k0, const int jg0,
+                                      const int lane,
                                       const int ig0, const double (&xi)[R], const double (&yi)[R],
                                       const double (&zi)[R], const double (&mi)[R], const double eps2, const double s2,
                                       double (&ax)[R], double (&ay)[R], double (&az)[R], double (&pp)[R], double& jx,
@@ -196,11 +198,11 @@ __device__ __forceinline__ void block(const double (&q)[4][kTile / 32][64], cons
   double bx[R], by[R], bz[R], bp[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) bx[r] = ax[r], by[r] = ay[r], bz[r] = az[r], bp[r] = pp[r];
-  const bool out = block32<LAW, SYM, MASK, PHI, EQ, true, R>(q, b, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, bx, by, bz, bp,
+  const bool out = block32<LAW, SYM, MASK, PHI, EQ, true, R, KS>(q, b, k0, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, bx, by, bz, bp,
                                                          jx, jy, jz, jp);
   if (__any_sync(0xffffffffu, out)) {
     jx = jy = jz = jp = 0.0;
-    block32<LAW, SYM, MASK, PHI, EQ, false, R>(q, b, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp, jx, jy, jz,
+    block32<LAW, SYM, MASK, PHI, EQ, false, R, KS>(q, b, k0, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp, jx, jy, jz,
                                            jp);
   } else {
 #pragma unroll
@@ -209,10 +211,13 @@ __device__ __forceinline__ void block(const double (&q)[4][kTile / 32][64], cons
 }
 
 // Work items, taken from `counter` until none is left.
-template <int LAW, int W, int R, int PHI>
-__device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Smem<W>& sm) {
-  constexpr int T = W * 32, TI = T * R, NC = PHI == sym::kPhiBoth ? 4 : 3;  // sums of a j-body
-  const int tid = (int)threadIdx.x, lane = tid & 31, w = tid >> 5;
+// KS warps share the W warps' i-bodies and blocks, each a range of the rotation's steps (short lists,
+// SymLaunch::split): the j-sums need nothing new, as the CTA's warps' sums are added anyway, the i-sums
+// are added at the end of the i-tile.
+template <int LAW, int W, int R, int PHI, int KS>
+__device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Smem<W * KS>& sm) {
+  constexpr int T = W * KS * 32, TI = W * 32 * R, NC = PHI == sym::kPhiBoth ? 4 : 3;  // sums of a j-body
+  const int tid = (int)threadIdx.x, lane = tid & 31, w = tid >> 5, wi = w % W, k0 = w / W * (32 / KS);
   const double4_32a* __restrict__ st = static_cast<const double4_32a*>(L.stage_x);
   double4_32a* part = reinterpret_cast<double4_32a*>(L.part);
   const double eps2 = L.eps2, s2 = L.sigma2;
@@ -236,7 +241,7 @@ __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Sme
 
     for (int i0 = it.i_begin; i0 < it.i_end; i0 += TI) {
       double xi[R], yi[R], zi[R], mi[R], ax[R], ay[R], az[R], pp[R];
-      const int wi0 = i0 + w * 32 * R, ig0 = wi0 + lane;
+      const int wi0 = i0 + wi * 32 * R, ig0 = wi0 + lane;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const int ig = ig0 + 32 * r;
@@ -262,10 +267,10 @@ __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Sme
             auto run = [&](auto eq) {
               constexpr bool EQ = decltype(eq)::value;
               if (both)
-                block<LAW, true, false, PHI, EQ, R>(sm.q, b, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp,
+                block<LAW, true, false, PHI, EQ, R, KS>(sm.q, b, k0, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp,
                                                     jx, jy, jz, jp);
               else if (jg0 + 32 > wi0)
-                block<LAW, false, true, PHI, EQ, R>(sm.q, b, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp,
+                block<LAW, false, true, PHI, EQ, R, KS>(sm.q, b, k0, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp,
                                                     jx, jy, jz, jp);
             };
             if (LAW == 0 && uniform && jg0 + 32 <= it.j_end && wi0 + 32 * R <= it.i_end)
@@ -273,7 +278,7 @@ __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Sme
             else
               run(std::false_type());
           }
-          const int p = 32 * b + lane;
+          const int p = 32 * b + ((lane + k0 + 32 / KS) & 31);  // whose sums have travelled here
           sm.jacc[w][0][p] = jx, sm.jacc[w][1][p] = jy, sm.jacc[w][2][p] = jz;
           if (PHI == sym::kPhiBoth) sm.jacc[w][3][p] = jp;
         }
@@ -289,13 +294,31 @@ __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Sme
 #pragma unroll
           for (int c = 0; c < NC; ++c)
 #pragma unroll
-            for (int u = 0; u < W; ++u) s[c] += sm.jacc[u][c][t];
+            for (int u = 0; u < W * KS; ++u) s[c] += sm.jacc[u][c][t];
           oj[j] = make_double4_32a(s[0], s[1], s[2], s[3]);
         }
       }
+      if (KS > 1) {  // the i-sums of the warps that share the bodies, through the j-sums' space
+        static_assert(R <= kTile / 32, "");
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int p = 32 * r + lane;
+          sm.jacc[w][0][p] = ax[r], sm.jacc[w][1][p] = ay[r], sm.jacc[w][2][p] = az[r], sm.jacc[w][3][p] = pp[r];
+        }
+        __syncthreads();
+        if (w < W)
+#pragma unroll
+          for (int u = 1; u < KS; ++u)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+              const int p = 32 * r + lane, o = w + u * W;
+              ax[r] += sm.jacc[o][0][p], ay[r] += sm.jacc[o][1][p], az[r] += sm.jacc[o][2][p], pp[r] += sm.jacc[o][3][p];
+            }
+      }
 #pragma unroll
       for (int r = 0; r < R; ++r)
-        if (ig0 + 32 * r < it.i_end) oi[ig0 + 32 * r] = make_double4_32a(ax[r], ay[r], az[r], pp[r]);
+        if (w < W && ig0 + 32 * r < it.i_end) oi[ig0 + 32 * r] = make_double4_32a(ax[r], ay[r], az[r], pp[r]);
       __syncthreads();  // the tile and the j-sums are free for the next i-tile
     }
   }

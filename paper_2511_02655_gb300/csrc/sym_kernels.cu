@@ -27,11 +27,13 @@ __global__ void __launch_bounds__(W * 32, MINB) k_force_sym(const SymLaunch L) {
   retire_cta(L.counter);
 }
 
-template <int LAW, int W, int R, int PHI>
-__global__ void __launch_bounds__(W * 32) k_force_sym64(const SymLaunch L) {
-  __shared__ sym64::Smem<W> sm;
+// With 4 warps to a block of the work 24 warps per SM are resident at most (short lists): left to
+// itself the compiler keeps to 64 registers and spills.
+template <int LAW, int W, int R, int PHI, int KS>
+__global__ void __launch_bounds__(W * KS * 32, KS < 4 ? 0 : std::max(1, 24 / (W * KS))) k_force_sym64(const SymLaunch L) {
+  __shared__ sym64::Smem<W * KS> sm;
   pdl_wait();
-  sym64::items<LAW, W, R, PHI>(L, L.counter, sm);
+  sym64::items<LAW, W, R, PHI, KS>(L, L.counter, sm);
   pdl_trigger();
   retire_cta(L.counter);
 }
@@ -58,6 +60,8 @@ int occupancy_of(K kern, int block, size_t smem) {
 // Compiled: warps, i-bodies per lane (and resident CTAs).
 #define NBODY_SYM_TILINGS(X) X(4, 2, 6) X(4, 4, 4) X(8, 2, 3) X(8, 4, 2)
 #define NBODY_SYM64_TILINGS(X) X(2, 1) X(4, 1) X(8, 1) X(4, 2)
+// ... of which these also exist with 2 and 4 warps to a block of the work (SymLaunch::split)
+#define NBODY_SYM64_SPLITS(X) X(2, 1) X(4, 1)
 
 // f(law, potential) as integral constants
 template <typename F>
@@ -76,8 +80,15 @@ cudaError_t launch_sym_force(int precision, const SymLaunch& L, cudaStream_t st)
   return with_modes(L.law, L.phi, [&](auto law, auto phi) -> cudaError_t {
     constexpr int LAW = decltype(law)::value, PHI = decltype(phi)::value;
     if (precision == 0) {
+#define NBODY_X(W, R)                                                                                              \
+  if (L.block == W * 32 && L.ipt == R && L.split == 4)                                                             \
+    return launch_pdl(k_force_sym64<LAW, W, R, PHI, 4>, L.n_ctas, W * 128, st, L);                                 \
+  if (L.block == W * 32 && L.ipt == R && L.split == 2)                                                             \
+    return launch_pdl(k_force_sym64<LAW, W, R, PHI, 2>, L.n_ctas, W * 64, st, L);
+      NBODY_SYM64_SPLITS(NBODY_X)
+#undef NBODY_X
 #define NBODY_X(W, R) \
-  if (L.block == W * 32 && L.ipt == R) return launch_pdl(k_force_sym64<LAW, W, R, PHI>, L.n_ctas, W * 32, st, L);
+  if (L.block == W * 32 && L.ipt == R) return launch_pdl(k_force_sym64<LAW, W, R, PHI, 1>, L.n_ctas, W * 32, st, L);
       NBODY_SYM64_TILINGS(NBODY_X)
 #undef NBODY_X
       return cudaErrorInvalidConfiguration;
@@ -99,7 +110,7 @@ int sym_force_ctas_per_sm(int precision, int block, int ipt, int law) {
               constexpr int LAW = decltype(l)::value, PHI = decltype(phi)::value;
               if (precision == 0) {
 #define NBODY_X(W, R) \
-  if (block == W * 32 && ipt == R) return occupancy_of(k_force_sym64<LAW, W, R, PHI>, W * 32, 0);
+  if (block == W * 32 && ipt == R) return occupancy_of(k_force_sym64<LAW, W, R, PHI, 1>, W * 32, 0);
                 NBODY_SYM64_TILINGS(NBODY_X)
 #undef NBODY_X
                 return 0;

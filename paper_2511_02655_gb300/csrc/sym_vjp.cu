@@ -18,12 +18,12 @@ __global__ void __launch_bounds__(W * 32, MINB) k_vjp_sym(const SymLaunch L) {
   retire_cta(L.counter);
 }
 
-template <int W, bool P>
-__global__ void __launch_bounds__(W * 32) k_vjp_sym64(const SymLaunch L) {
+template <int W, bool P, int KS>
+__global__ void __launch_bounds__(W * KS * 32) k_vjp_sym64(const SymLaunch L) {
   extern __shared__ __align__(16) unsigned char raw[];
-  auto& sm = *reinterpret_cast<symv::Smem64<W, P>*>(raw);
+  auto& sm = *reinterpret_cast<symv::Smem64<W * KS, P>*>(raw);
   pdl_wait();
-  symv::items64<W, P>(L, L.counter, sm);
+  symv::items64<W, P, KS>(L, L.counter, sm);
   pdl_trigger();
   retire_cta(L.counter);
 }
@@ -41,9 +41,9 @@ int occupancy_of(K kern, int block, size_t smem) {
 
 }  // namespace
 
-// Compiled: warps, i-bodies per lane, resident CTAs (mixed); warps (FP64)
+// Compiled: warps, i-bodies per lane, resident CTAs (mixed); warps and warps to a block of the work (FP64, SymLaunch::split)
 #define NBODY_SYM_VJP_TILINGS(X) X(4, 1, 5) X(4, 2, 3) X(8, 2, 1)
-#define NBODY_SYM_VJP64_TILINGS(X) X(2) X(4) X(8)
+#define NBODY_SYM_VJP64_TILINGS(X) X(2, 1) X(2, 2) X(2, 4) X(4, 1) X(4, 2) X(4, 4) X(8, 1)
 
 cudaError_t launch_sym_vjp(int precision, const SymLaunch& L, cudaStream_t st) {
   if (L.n_ctas <= 0) return cudaErrorInvalidConfiguration;
@@ -57,10 +57,12 @@ cudaError_t launch_sym_vjp(int precision, const SymLaunch& L, cudaStream_t st) {
 #undef NBODY_X
     return cudaErrorInvalidConfiguration;
   }
-#define NBODY_X(W)                                                                                                    \
-  if (L.block == W * 32 && L.ipt == 1)                                                                                \
-    return L.params ? launch_pdl_smem(k_vjp_sym64<W, true>, L.n_ctas, W * 32, sizeof(symv::Smem64<W, true>), st, L)   \
-                    : launch_pdl_smem(k_vjp_sym64<W, false>, L.n_ctas, W * 32, sizeof(symv::Smem64<W, false>), st, L);
+#define NBODY_X(W, KS)                                                                                              \
+  if (L.block == W * 32 && L.ipt == 1 && (L.split == KS || W == 8))                                                 \
+    return L.params ? launch_pdl_smem(k_vjp_sym64<W, true, KS>, L.n_ctas, W * KS * 32,                              \
+                                      sizeof(symv::Smem64<W * KS, true>), st, L)                                    \
+                    : launch_pdl_smem(k_vjp_sym64<W, false, KS>, L.n_ctas, W * KS * 32,                             \
+                                      sizeof(symv::Smem64<W * KS, false>), st, L);
   NBODY_SYM_VJP64_TILINGS(NBODY_X)
 #undef NBODY_X
   return cudaErrorInvalidConfiguration;
@@ -76,13 +78,19 @@ int sym_vjp_ctas_per_sm(int precision, int block, int ipt) {
 #undef NBODY_X
     return 0;
   }
-#define NBODY_X(W)                                                                               \
-  if (block == W * 32 && ipt == 1)                                                               \
-    return std::min(occupancy_of(k_vjp_sym64<W, true>, W * 32, sizeof(symv::Smem64<W, true>)),   \
-                    occupancy_of(k_vjp_sym64<W, false>, W * 32, sizeof(symv::Smem64<W, false>)));
+  // (of the unsplit kernel; the shared ones are for lists that leave most of the chip free anyway,
+  // and asking for them here allows their shared memory as well)
+  int n = 0;
+#define NBODY_X(W, KS)                                                                                            \
+  if (block == W * 32 && ipt == 1) {                                                                              \
+    const int k = std::min(occupancy_of(k_vjp_sym64<W, true, KS>, W * KS * 32, sizeof(symv::Smem64<W * KS, true>)),   \
+                           occupancy_of(k_vjp_sym64<W, false, KS>, W * KS * 32, sizeof(symv::Smem64<W * KS, false>))); \
+    if (k <= 0) return 0;                                                                                         \
+    if (KS == 1) n = k;                                                                                           \
+  }
   NBODY_SYM_VJP64_TILINGS(NBODY_X)
 #undef NBODY_X
-  return 0;
+  return n;
 }
 
 }  // namespace nbody

@@ -341,16 +341,16 @@ struct Body64 {
   double x, y, z, m, wx, wy, wz;
 };
 
-template <bool SYM, bool MASK, bool P, bool FAST>
-__device__ __forceinline__ bool block32(const double (&q)[7][kSymTile64 / 32][64], const int b, const int jg0,
+template <bool SYM, bool MASK, bool P, bool FAST, int KS>
+__device__ __forceinline__ bool block32(const double (&q)[7][kSymTile64 / 32][64], const int b, const int k0, const int jg0,
                                         const int lane, const int ig, const Body64& B, const double eps2,
                                         double (&si)[P ? 10 : 8], double (&sj)[P ? 10 : 8]) {
   constexpr int NC = P ? 10 : 8;
   const int src = (lane + 1) & 31;
   bool out = false;
 #pragma unroll(FAST ? 2 : 1)
-  for (int k = 0; k < 32; ++k) {
-    const int p = lane + k;
+  for (int k = 0; k < 32 / KS; ++k) {
+    const int p = lane + k0 + k;
     const double dx = q[0][b][p] - B.x, dy = q[1][b][p] - B.y, dz = q[2][b][p] - B.z, mj = q[3][b][p];
     const double wxj = q[4][b][p], wyj = q[5][b][p], wzj = q[6][b][p];
     const double r2 = fma(dx, dx, fma(dy, dy, fma(dz, dz, eps2)));
@@ -386,27 +386,27 @@ __device__ __forceinline__ bool block32(const double (&q)[7][kSymTile64 / 32][64
   return out;
 }
 
-template <bool SYM, bool MASK, bool P>
-__device__ __forceinline__ void block(const double (&q)[7][kSymTile64 / 32][64], const int b, const int jg0,
+template <bool SYM, bool MASK, bool P, int KS>
+__device__ __forceinline__ void block(const double (&q)[7][kSymTile64 / 32][64], const int b, const int k0, const int jg0,
                                       const int lane, const int ig, const Body64& B, const double eps2,
                                       double (&si)[P ? 10 : 8], double (&sj)[P ? 10 : 8]) {
   constexpr int NC = P ? 10 : 8;
   double s0[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) s0[c] = si[c], si[c] = 0.0;
-  if (__any_sync(0xffffffffu, block32<SYM, MASK, P, true>(q, b, jg0, lane, ig, B, eps2, si, sj))) {
+  if (__any_sync(0xffffffffu, block32<SYM, MASK, P, true, KS>(q, b, k0, jg0, lane, ig, B, eps2, si, sj))) {
 #pragma unroll
     for (int c = 0; c < NC; ++c) si[c] = sj[c] = 0.0;
-    block32<SYM, MASK, P, false>(q, b, jg0, lane, ig, B, eps2, si, sj);
+    block32<SYM, MASK, P, false, KS>(q, b, k0, jg0, lane, ig, B, eps2, si, sj);
   }
 #pragma unroll
   for (int c = 0; c < NC; ++c) si[c] += s0[c];
 }
 
-template <int W, bool P>
-__device__ __forceinline__ void items64(const SymLaunch& L, unsigned* counter, Smem64<W, P>& sm) {
-  constexpr int T = W * 32, TI = T, NC = P ? 10 : 8, KW = P ? 3 : 2, J = kSymTile64;
-  const int tid = (int)threadIdx.x, lane = tid & 31, w = tid >> 5;
+template <int W, bool P, int KS>
+__device__ __forceinline__ void items64(const SymLaunch& L, unsigned* counter, Smem64<W * KS, P>& sm) {
+  constexpr int T = W * KS * 32, TI = W * 32, NC = P ? 10 : 8, KW = P ? 3 : 2, J = kSymTile64;
+  const int tid = (int)threadIdx.x, lane = tid & 31, w = tid >> 5, wi = w % W, k0 = w / W * (32 / KS);
   const double4_32a* __restrict__ st = static_cast<const double4_32a*>(L.stage_x);
   const double4_32a* __restrict__ sw = static_cast<const double4_32a*>(L.stage_w);
   double4_32a* part = reinterpret_cast<double4_32a*>(L.part);
@@ -424,7 +424,7 @@ __device__ __forceinline__ void items64(const SymLaunch& L, unsigned* counter, S
     const double pad = 1.0e30 * (1.0 + fabs(q0.x) + fabs(q0.y) + fabs(q0.z));  // as in sym64::items
 
     for (int i0 = it.i_begin; i0 < it.i_end; i0 += TI) {
-      const int wi0 = i0 + w * 32, ig = wi0 + lane;
+      const int wi0 = i0 + wi * 32, ig = wi0 + lane;
       const bool live = ig < it.i_end;
       Body64 B{-pad, -pad, -pad, 0.0, 0.0, 0.0, 0.0};
       if (live) {
@@ -453,12 +453,12 @@ __device__ __forceinline__ void items64(const SymLaunch& L, unsigned* counter, S
           for (int c = 0; c < NC; ++c) sj[c] = 0.0;
           if (jg0 < it.j_end && wi0 < it.i_end) {
             if (jg0 >= wi0 + 32)
-              block<true, false, P>(sm.q, b, jg0, lane, ig, B, eps2, si, sj);
+              block<true, false, P, KS>(sm.q, b, k0, jg0, lane, ig, B, eps2, si, sj);
             else if (jg0 + 32 > wi0)
-              block<false, true, P>(sm.q, b, jg0, lane, ig, B, eps2, si, sj);
+              block<false, true, P, KS>(sm.q, b, k0, jg0, lane, ig, B, eps2, si, sj);
           }
 #pragma unroll
-          for (int c = 0; c < NC; ++c) sm.jacc[w][c][32 * b + lane] = sj[c];
+          for (int c = 0; c < NC; ++c) sm.jacc[w][c][32 * b + ((lane + k0 + 32 / KS) & 31)] = sj[c];
         }
         __syncthreads();
         for (int t = tid; t < J; t += T) {
@@ -469,12 +469,23 @@ __device__ __forceinline__ void items64(const SymLaunch& L, unsigned* counter, S
           for (int c = 0; c < NC; ++c) {
             double s = add ? o[c] : 0.0;
 #pragma unroll
-            for (int u = 0; u < W; ++u) s += sm.jacc[u][c][t];
+            for (int u = 0; u < W * KS; ++u) s += sm.jacc[u][c][t];
             o[c] = s;
           }
         }
       }
-      if (live) {
+      if (KS > 1) {  // as in sym64::items
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < NC; ++c) sm.jacc[w][c][lane] = si[c];
+        __syncthreads();
+        if (w < W)
+#pragma unroll
+          for (int u = 1; u < KS; ++u)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) si[c] += sm.jacc[w + u * W][c][lane];
+      }
+      if (live && w < W) {
         double* o = oi + 4 * KW * (int64_t)ig;
 #pragma unroll
         for (int c = 0; c < NC; ++c) o[c] = si[c];

@@ -111,6 +111,41 @@ def test_sym64_forces(nb, tmp_path, monkeypatch, tiling, n, length, mass, masses
     assert_elem_close(phi, phi_ref, 1e-12, "phi")
 
 
+@pytest.mark.parametrize("n,split", [(65, 4), (700, 4), (1400, 2), (2050, 1)])
+@pytest.mark.parametrize("law", [0, 1])
+def test_sym64_shared_blocks(nb, tmp_path, monkeypatch, law, n, split):
+    """Lists short enough that 4, 2 or 1 warps share a block's rotation: forces, potentials and gradients."""
+    import torch
+    monkeypatch.setenv("NBODY_TUNE_CACHE", str(tmp_path / "tune"))
+    rows = -(-n // 64)
+    items = sum((n - 64 * r + 31) // 32 for r in range(rows))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert split == (4 if 8 * items <= 16 * sms else 2 if 4 * items <= 16 * sms else 1)
+    x, v, m = inputs.lj_gas(n, seed=3)[:3] if law else inputs.plummer(n, seed=n)
+    m = _masses(m, "lognormal", n)
+    kw = dict(law=1, dt=1e-3, n=n, lj_epsilon=1.3, lj_sigma=0.9) if law else dict(G=1.1, eps=0.03, dt=1e-3, n=n)
+    rng = np.random.default_rng(n)
+    lx, lv = rng.standard_normal((n, 3)), 0.1 * rng.standard_normal((n, 3))
+    args = to_dev(x, v, m) + (2, 2) + to_dev(lx, lv)
+    lines = {"force": (64, 1, 64, 1, 3, 0)}
+    if not law:
+        lines["vjp"] = (64, 1, 64, 1, 3, 0)
+    ctx = _forced(nb, tmp_path / "tune", lines, precision=nb.FP64,
+                  **({} if law else {"use": lambda c: nb.nbody_adjoint(c, *args)}), **kw)
+    a, phi = nb.nbody_forces(ctx, *to_dev(x, m))
+    nb.nbody_sync(ctx)
+    assert nb.nbody_get_slicing(ctx)["n_items"] == items
+    ref = oracle.lj_forces(x, m, eps_lj=1.3, sigma=0.9) if law else oracle.forces(x, m, G=1.1, eps=0.03)
+    tol = 1e-10 if law else 1e-12
+    assert force_rel_err(a.cpu().numpy(), ref[0]).max() <= tol
+    assert_elem_close(phi.cpu().numpy(), ref[1], tol, "phi")
+    if not law:
+        gx, gv, gm = nb.nbody_adjoint(ctx, *args)
+        nb.nbody_sync(ctx)
+        for got, want, name in zip((gx, gv, gm), oracle.adjoint(x, v, m, 1.1, 0.03, 1e-3, 2, lx, lv), ("x", "v", "m")):
+            assert_elem_close(got.cpu().numpy(), want, 1e-11, name)
+
+
 def test_sym64_masses_change_between_calls(nb):
     """Equal masses are recognised anew in every call, replayed graphs included."""
     import torch
