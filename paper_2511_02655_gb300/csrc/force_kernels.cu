@@ -22,6 +22,8 @@
 // and compensated float32 pairs on the mixed path; the O(N) post kernel adds
 // the slices in a fixed order, so results are deterministic.
 // Self pairs are masked in the tiles that overlap the item's own i-range.
+// These kernels meet every pair from both ends. They serve requested tilings and systems below 3000
+// bodies (FP64: 64, beside the other up to 512); elsewhere sym_kernels.cu meets it once.
 #include <algorithm>
 
 #include "force_common.cuh"
