@@ -21,6 +21,7 @@
 
 #include "../../include/nbody.h"
 #include "nbody_internal.h"
+#include "work_lists.h"
 
 using namespace nbody;
 
@@ -34,21 +35,11 @@ constexpr int kTuneSlice = 8192;
 constexpr int kSliceQuantum = 4;  // slice lengths are multiples of this many bodies
 constexpr int64_t kTailMin = 64;   // shortest slice of a halving tail
 
-struct Tiling {
-  int block = 0, ipt = 0, jtile = 0, slice = 0, n_ctas = 0;
-  int variant = 0;  // mixed kernels: 0 scalar, 1 packed float32x2, 2 packed with a 4-CTA register cap (force),
-                    // 3 symmetric (every unordered pair once)
-  int tail = 0;     // slicing of a system's j-range: 0 equal slices, 1 full slices and a halving tail
-                    // (symmetric: 0 pieces of one length and a remainder per row of i-tiles, 1 every other
-                    // row in pieces a third as long, 2 pieces of a row as equal as whole blocks allow)
-};
-constexpr int kSymVariant = 3;
 constexpr int kSymTail = 2;  // nbody_get_slicing: tail modes of the symmetric pass are reported from here on
 enum class Potential { kNone = 0, kBodies = 1, kEnergy = 2 };  // as sym::kPhi*
 constexpr double kSymMinBodies = 3000.0;    // typical system size from which the symmetric pass is a candidate
 constexpr double kSymOnlyBodies = 8192.0;  // ... and from which it is the only one (mixed path)
 constexpr double kSymMinBodies64 = 64.0, kSymOnlyBodies64 = 512.0;  // FP64 path
-constexpr int64_t kMaxSymRows = 64;                      // rows of i-tiles a system is cut into at most
 constexpr size_t kMaxSymPartialBytes = size_t(4) << 30;  // cap on the symmetric pass's partial sums
 
 // Near-pair refinement radius of the mixed force kernels: 4 softening lengths
@@ -113,7 +104,7 @@ bool allocation_holds(const void* p, size_t bytes, size_t* avail) {
 }
 }  // namespace nbody
 
-struct nbody_ctx {
+struct nbody_ctx : SymLayout {
   nbody_config cfg{};
   // mixed Lennard-Jones: positions are staged in units of sigma, (x - c) / sigma,
   // so that u = sigma^2 / r^2 is the reciprocal itself; 1 everywhere else
@@ -124,16 +115,11 @@ struct nbody_ctx {
   int dev_cc = 0;
   cudaStream_t stream = nullptr;
   cudaStream_t cap_stream = nullptr;  // private stream used only to capture graphs
-  int64_t n_total = 0;
-  int n_sys = 0;
-  std::vector<int64_t> offsets;
   std::string err = "no error";
   int64_t launches = 0;
   uint32_t epoch = 0;  // number of the current call (SysParam::uniform); 0 while tuning
 
   // layout
-  std::vector<Chunk> chunks;  // without slots (Chunk::n_slices, stride, row0: the copies on the device)
-  std::vector<int32_t> sys_chunk;
   Chunk* d_chunks = nullptr;
   Chunk* d_vchunks = nullptr;  // same chunks, VJP tiling's slice counts
   int32_t* d_sys_chunk = nullptr;
@@ -278,9 +264,6 @@ nbody_status check_dev(nbody_ctx* c, const void* p, size_t bytes, const char* na
 // work lists
 
 int sym_tile(int prec, bool vjp) { return prec != NBODY_MIXED ? kSymTile64 : vjp ? kSymVjpTile : kSymTile; }
-// j-bodies that a warp of the symmetric pass meets in one block: pieces are whole blocks
-int sym_block(int prec) { return prec == NBODY_MIXED ? 64 : 32; }
-
 int ctas_per_sm(int prec, const Tiling& t, bool vjp, int law) {
   if (t.variant == kSymVariant) {
     if (t.jtile != sym_tile(prec, vjp)) return 0;
@@ -288,70 +271,6 @@ int ctas_per_sm(int prec, const Tiling& t, bool vjp, int law) {
   }
   return vjp ? vjp_ctas_per_sm(prec, t.variant, t.block, t.ipt, t.jtile)
              : force_ctas_per_sm(prec, t.variant, t.block, t.ipt, t.jtile, law);
-}
-
-bool is_sym(const Tiling& t) { return t.variant == kSymVariant; }
-
-// Unordered pairs of all systems.
-double total_pairs(const nbody_ctx* c) {
-  double p = 0.0;
-  for (int s = 0; s < c->n_sys; ++s) {
-    const double n = (double)(c->offsets[s + 1] - c->offsets[s]);
-    p += 0.5 * n * n;
-  }
-  return p;
-}
-
-// The symmetric pass cuts a system of n bodies into rows of H bodies (whole i-tiles, at most
-// kMaxSymRows rows: a body has a slot per row up to its own, so more rows would mean more partials
-// to combine than pair work saved) and row r into pieces of about `area` pairs.
-struct SymRows {
-  int64_t n, H, rows, block;  // block: pieces are whole blocks of j-bodies
-  SymRows(const nbody_ctx* c, const Tiling& t, int64_t bodies) : n(bodies), block(sym_block(c->cfg.precision)) {
-    const int64_t itile = (int64_t)t.block * t.ipt;
-    H = itile * ((n + itile * kMaxSymRows - 1) / (itile * kMaxSymRows));
-    rows = (n + H - 1) / H;
-  }
-  int64_t blocks(int64_t r) const { return (n - r * H + block - 1) / block; }
-  // pieces of row r, and for a tail other than 2 the blocks of each (the last may have fewer)
-  int64_t pieces(int64_t r, double area, int tail, int64_t* step) const {
-    const double ni = (double)std::min(H, n - r * H), pairs = ni * ((double)(n - r * H) - 0.5 * ni);
-    const double want = tail == 1 && (r & 1) ? area / 3.0 : area;
-    const int64_t nb = blocks(r), p = std::max<int64_t>(1, std::min(nb, (int64_t)(pairs / want + 0.5)));
-    *step = std::max<int64_t>(1, (2 * nb + p) / (2 * p));
-    return tail == 2 ? p : (nb + *step - 1) / *step;
-  }
-};
-
-// Work items of a symmetric tiling with the given slice, counted up to `most` and a little beyond.
-int64_t sym_item_count(const nbody_ctx* c, const Tiling& t, int64_t slice, int64_t most) {
-  const double area = (double)slice * t.block * t.ipt;
-  int64_t items = 0, step, last = 0, own = 0;  // own: items of a system of `last` bodies
-  for (int s = 0; s < c->n_sys && items <= most; ++s) {
-    const int64_t n = c->offsets[s + 1] - c->offsets[s];
-    if (n != last) {
-      const SymRows R(c, t, n);
-      own = 0, last = n;
-      for (int64_t r = 0; r < R.rows; ++r) own += R.pieces(r, area, t.tail, &step);
-    }
-    items += own;
-  }
-  return items;
-}
-
-// Slice of a symmetric tiling (t.tail as set) that makes at most `pieces` work items per CTA of a
-// full grid, as many as that allows: one item more than CTAs would cost a whole second round.
-constexpr int kSymPieces = 6;
-int sym_slice(const nbody_ctx* c, const Tiling& t, int n_ctas, int pieces) {
-  const int64_t most = (int64_t)pieces * n_ctas;
-  auto fits = [&](int64_t slice) { return sym_item_count(c, t, slice, most) <= most; };
-  int64_t lo = 1, hi = 1;  // the least slice that fits lies in (lo, hi], or no slice does (every row one piece)
-  while (!fits(hi) && hi < (int64_t)1 << 30) lo = hi, hi *= 2;
-  while (hi - lo > std::max<int64_t>(1, lo / 256)) {
-    const int64_t mid = (lo + hi) / 2;
-    (fits(mid) ? hi : lo) = mid;
-  }
-  return (int)std::min<int64_t>(hi, 1 << 30);
 }
 
 // Slice length for tiling t: the largest power-of-two multiple of jtile that
@@ -488,63 +407,6 @@ nbody_status upload_chunks(nbody_ctx* c, const std::vector<Chunk>& ch, Chunk** d
   return NBODY_OK;
 }
 
-// Work list of the symmetric pass for tiling t (see sym_common.cuh, SymRows), pieces of
-// about slice x i-tile pairs. Chunks get their slots; rows is the number of entries the
-// partial buffer needs.
-void build_sym_items(const nbody_ctx* c, const Tiling& t, std::vector<SymItem>& items, std::vector<Chunk>& chunks,
-                     int& max_slots, int64_t& rows) {
-  items.clear();
-  chunks = c->chunks;
-  max_slots = 1;
-  rows = 0;
-  const double area = (double)t.slice * (double)t.block * t.ipt;
-  std::vector<int> slots;
-  for (int s = 0; s < c->n_sys; ++s) {
-    const int64_t b = c->offsets[s], n = c->offsets[s + 1] - b;
-    if (n <= 0) continue;
-    const SymRows R(c, t, n);
-    const int64_t H = R.H;
-    slots.assign((size_t)R.rows, 0);
-    int most = 0;
-    for (int64_t r = 0; r < R.rows; ++r) {
-      const int64_t i0 = r * H, ni = std::min(H, n - i0);
-      int64_t step;
-      const int64_t p = R.pieces(r, area, t.tail, &step);
-      auto cut = [&](int64_t k) { return std::min(n, i0 + R.block * (t.tail == 2 ? k * R.blocks(r) / p : k * step)); };
-      slots[(size_t)r] = (int)(r + 1 + p);
-      most = std::max(most, slots[(size_t)r]);
-      for (int64_t k = 0; k < p; ++k) {
-        SymItem w{};
-        w.sys = s;
-        w.i_begin = (int32_t)(b + i0);
-        w.i_end = (int32_t)(b + i0 + ni);
-        w.j_begin = (int32_t)(b + cut(k));
-        w.j_end = (int32_t)(b + cut(k + 1));
-        w.slot_j = (int32_t)r;
-        w.slot_i = (int32_t)(r + 1 + k);
-        w.stride = (int32_t)n;
-        w.row0 = rows - b;
-        items.push_back(w);
-      }
-    }
-    for (int32_t k = c->sys_chunk[s]; k < c->sys_chunk[s + 1]; ++k) {
-      Chunk& ch = chunks[(size_t)k];
-      ch.n_slices = slots[(size_t)((ch.begin - b) / H)];
-      ch.stride = (int32_t)n;
-      ch.row0 = rows - b;
-    }
-    max_slots = std::max(max_slots, most);
-    rows += (int64_t)most * n;
-  }
-  // longest first, for the dynamic schedule of the persistent grid
-  auto cost = [](const SymItem& w) {
-    const int64_t ni = w.i_end - w.i_begin, nj = w.j_end - w.j_begin;
-    const int64_t own = std::max<int64_t>(0, std::min(w.i_end, w.j_end) - w.j_begin);  // j-bodies inside the row
-    return ni * nj - own * (own - 1) / 2;
-  };
-  std::stable_sort(items.begin(), items.end(), [&](const SymItem& x, const SymItem& y) { return cost(x) > cost(y); });
-}
-
 // Installs tiling t for the force (vjp=false) or VJP (vjp=true) pass.
 nbody_status install_tiling(nbody_ctx* c, Tiling t, bool vjp) {
   const int prec = c->cfg.precision;
@@ -558,10 +420,11 @@ nbody_status install_tiling(nbody_ctx* c, Tiling t, bool vjp) {
   size_t part_bytes = 0;
   nbody_status s;
   if (is_sym(t)) {
-    if (t.slice <= 0) t.slice = sym_slice(c, t, occ * c->sm_count, kSymPieces);
+    if (t.slice <= 0) t.slice = sym_slice(*c, t, occ * c->sm_count, kSymPieces);
     std::vector<SymItem> items;
     int64_t rows = 0;
-    build_sym_items(c, t, items, chunks, max_slices, rows);
+    if (!build_sym_items(*c, t, items, chunks, max_slices, rows))
+      return fail(c, NBODY_EINVAL, "symmetric work list: a chunk of bodies crosses two rows");
     part_bytes = (size_t)rows * per;
     if (part_bytes > kMaxSymPartialBytes)
       return fail(c, NBODY_EINVAL, "symmetric tiling needs %zu bytes of partial sums", part_bytes);
@@ -972,7 +835,7 @@ nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
   // interaction slots covered by the timed items (the list is longest-first)
   double slots = 0.0;
   if (sym) {
-    slots = 2.0 * total_pairs(c);
+    slots = 2.0 * total_pairs(*c);
   } else {
     std::vector<WorkItem> h(P.n_items);
     NB_CUDA(c, cudaMemcpy(h.data(), L.items, h.size() * sizeof(WorkItem), cudaMemcpyDeviceToHost));
@@ -1106,11 +969,11 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
       for (const auto& tk : std::vector<std::pair<int, int>>{
                {2, 1}, {2, 2}, {2, 3}, {2, 4}, {2, 6}, {0, 1}, {0, 2}, {0, 4}, {0, 6}, {1, 2}, {1, 4}, {1, 6}}) {
         t.tail = tk.first;
-        t.slice = sym_slice(c, t, n_ctas, tk.second);
+        t.slice = sym_slice(*c, t, n_ctas, tk.second);
         // FP64 lists of few large items need an even placement on the SMs, which the timing here has
         // and a step, whose CTAs start while the last kernel's retire, has not: 1400 bodies in 144 items
         // of 256 threads tie with 506 of 64 here, in a step they take 51.8 us against 47.7.
-        if (!mixed && p.first > 64 && sym_item_count(c, t, t.slice, c->sm_count) < c->sm_count) continue;
+        if (!mixed && p.first > 64 && sym_item_count(*c, t, t.slice, c->sm_count) < c->sm_count) continue;
         if (sym_settings.empty() || sym_settings.back().tail != t.tail || sym_settings.back().block != t.block ||
             sym_settings.back().ipt != t.ipt || sym_settings.back().slice != t.slice)
           sym_settings.push_back(t);
@@ -1566,20 +1429,11 @@ nbody_status nbody_init(nbody_ctx** out, const nbody_config* cfg, int64_t n_syst
   c->offsets.assign(offsets, offsets + n_systems + 1);
   c->n_total = offsets[n_systems];
 
-  // chunks: runs of <= `bodies` bodies inside one system, and each system's range of them
-  auto cut = [&](int64_t bodies, std::vector<Chunk>& chunks, std::vector<int32_t>& sys_chunk) {
-    sys_chunk.assign(c->n_sys + 1, 0);
-    for (int s = 0; s < c->n_sys; ++s) {
-      sys_chunk[s] = (int32_t)chunks.size();
-      for (int64_t b = offsets[s]; b < offsets[s + 1]; b += bodies)
-        chunks.push_back(Chunk{s, (int32_t)b, (int32_t)std::min<int64_t>(offsets[s + 1], b + bodies), 1, 0, 0, 0});
-    }
-    sys_chunk[c->n_sys] = (int32_t)chunks.size();
-  };
-  cut(chunk_bodies(c->n_total), c->chunks, c->sys_chunk);
+  c->j_block = cfg->precision == NBODY_MIXED ? 64 : 32;
+  cut_chunks(*c, chunk_bodies(c->n_total), c->chunks, c->sys_chunk);
   std::vector<Chunk> cchunks;
   std::vector<int32_t> csys_chunk;
-  cut(kChunk, cchunks, csys_chunk);
+  cut_chunks(*c, kChunk, cchunks, csys_chunk);
   c->n_cchunks = (int)cchunks.size();
 
   nbody_status s;

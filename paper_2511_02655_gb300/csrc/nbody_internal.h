@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "work_lists.h"
+
 namespace nbody {
 
 // One unit of all-pairs work: i-bodies [i_begin, i_end) of one system against
@@ -17,17 +19,6 @@ struct WorkItem {
   int32_t j_begin, j_end;
   int32_t slice;
   int32_t n_slices;
-};
-
-// A contiguous run of bodies of one system, the unit of the O(N) kernels and
-// of the fixed-order energy reduction.
-struct Chunk {
-  int32_t sys;
-  int32_t begin, end;
-  int32_t n_slices;  // partials to combine: slot s of body i is entry row0 + s * stride + i of the partial buffer
-  int32_t stride;
-  int32_t pad;
-  int64_t row0;
 };
 
 // Per-system staging of the mixed path. Positions are staged as (x - c) * scale
@@ -45,31 +36,6 @@ struct __align__(16) SysParam {
   uint32_t pad;
 };
 
-// Work item of the symmetric force pass (sym_common.cuh): i-bodies [i_begin,
-// i_end) of one system (whole i-tiles but for the system's end) against its
-// j-bodies [j_begin, j_end), every unordered pair once. Partials of i-bodies go to
-// slot slot_i, of j-bodies to slot slot_j (row0 and stride as in Chunk).
-struct SymItem {
-  int32_t sys;
-  int32_t i_begin, i_end;
-  int32_t j_begin, j_end;
-  int32_t slot_i, slot_j;
-  int32_t stride;
-  int64_t row0;
-};
-
-// The O(N) kernels do their float64 work on GB300's FP64 pipe (about 1/75 of
-// the FP32 rate), so that part of their time is the float64 operations per SM: the
-// smaller the system, the fewer bodies a chunk has, so that its CTAs cover every
-// SM (1024 bodies: 64 CTAs). The rest of the time is the latency of reading each
-// body's partials; a combining CTA has several threads per body (slot groups), each
-// adding every groups-th slice, so that a body's loads are in flight together.
-// Larger systems fill the SMs anyway, and their larger chunks leave fewer chunk
-// partials for one CTA to sum into a record.
-constexpr int kChunk = 128;  // bodies per chunk at most, and of the staging origin's sums
-inline int chunk_bodies(int64_t n_total) {
-  return n_total <= 4096 ? 16 : n_total <= 16384 ? 32 : n_total <= 32768 ? 64 : kChunk;
-}
 constexpr int kEnergyVals = 8;      // K, U, Px, Py, Pz, Lx, Ly, Lz per chunk
 constexpr int kAdjVals = 8;         // VJP partial values per body per slice
 
