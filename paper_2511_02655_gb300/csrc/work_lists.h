@@ -102,7 +102,7 @@ struct SymRows {
   int64_t n, H, rows, block;  // block: pieces are whole blocks of j-bodies
   SymRows(const SymLayout& c, const Tiling& t, int64_t bodies) : n(bodies), block(c.j_block) {
     const int64_t unit = std::max<int64_t>((int64_t)t.block * t.ipt, chunk_bodies(c.n_total));
-    H = unit * ((n + unit * kMaxSymRows - 1) / (unit * kMaxSymRows));
+    H = unit * std::max<int64_t>(1, (n + unit * kMaxSymRows - 1) / (unit * kMaxSymRows));  // (an empty system has no row)
     rows = (n + H - 1) / H;
   }
   int64_t blocks(int64_t r) const { return (n - r * H + block - 1) / block; }
