@@ -111,6 +111,9 @@ typedef struct {
  * Environment: NBODY_TUNE_CACHE=<file> keeps the tuner's choices (force and
  * VJP) across runs, keyed by device, configuration and layout;
  * NBODY_TUNE_VERBOSE=1 prints the candidates' costs on stderr;
+ * NBODY_SYM_PARTIAL_MB=k lowers the cap on the partial sums of the symmetric
+ * passes (4096 MiB each for force and VJP, half as much again for a VJP with
+ * parameter sums): lists that need more are left out of the choice;
  * NBODY_FAULT_ALLOC=k makes the k-th scratch allocation of the context report
  * NBODY_ENOMEM (for testing failure paths); NBODY_NVTX=1 wraps the context's
  * API calls (and the adjoint's forward and reverse phases) in NVTX ranges.

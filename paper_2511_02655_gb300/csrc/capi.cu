@@ -40,7 +40,7 @@ enum class Potential { kNone = 0, kBodies = 1, kEnergy = 2 };  // as sym::kPhi*
 constexpr double kSymMinBodies = 3000.0;    // typical system size from which the symmetric pass is a candidate
 constexpr double kSymOnlyBodies = 8192.0;  // ... and from which it is the only one (mixed path)
 constexpr double kSymMinBodies64 = 64.0, kSymOnlyBodies64 = 512.0;  // FP64 path
-constexpr size_t kMaxSymPartialBytes = size_t(4) << 30;  // cap on the symmetric pass's partial sums
+constexpr size_t kMaxSymPartialBytes = size_t(4) << 30;  // cap on the symmetric passes' partial sums
 
 // Near-pair refinement radius of the mixed force kernels: 4 softening lengths
 // for gravity, 4 sigma for Lennard-Jones (the neighbour shells that carry its
@@ -142,6 +142,7 @@ struct nbody_ctx : SymLayout {
   int vmax_slices = 1;
   size_t vpart_bytes = 0;  // partial sums of the VJP pass (without the parameter sums)
   bool vjp_ready = false;
+  size_t sym_cap = kMaxSymPartialBytes;  // NBODY_SYM_PARTIAL_MB=k lowers it
   int64_t fault_alloc = 0;  // > 0: the fault_alloc-th scratch allocation fails (NBODY_FAULT_ALLOC, tests)
   bool nvtx = false;        // NBODY_NVTX=1: NVTX ranges around the API calls and the adjoint's phases
   bool vjp_params = false;  // VJP launches also form the G and eps gradient sums
@@ -407,6 +408,11 @@ nbody_status upload_chunks(nbody_ctx* c, const std::vector<Chunk>& ch, Chunk** d
   return NBODY_OK;
 }
 
+// Whether `rows` entries of partial sums stay below the cap (a gradient's without the parameter sums).
+bool sym_fits(const nbody_ctx* c, int64_t rows, bool vjp) {
+  return rows <= (int64_t)(c->sym_cap / (vjp ? 64 : 32));
+}
+
 // Installs tiling t for the force (vjp=false) or VJP (vjp=true) pass.
 nbody_status install_tiling(nbody_ctx* c, Tiling t, bool vjp) {
   const int prec = c->cfg.precision;
@@ -426,7 +432,7 @@ nbody_status install_tiling(nbody_ctx* c, Tiling t, bool vjp) {
     if (!build_sym_items(*c, t, items, chunks, max_slices, rows))
       return fail(c, NBODY_EINVAL, "symmetric work list: a chunk of bodies crosses two rows");
     part_bytes = (size_t)rows * per;
-    if (part_bytes > kMaxSymPartialBytes)
+    if (!sym_fits(c, rows, vjp))
       return fail(c, NBODY_EINVAL, "symmetric tiling needs %zu bytes of partial sums", part_bytes);
     n_items = (int)items.size();
     if (!vjp) {
@@ -973,13 +979,15 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
         // FP64 lists of few large items need an even placement on the SMs, which the timing here has
         // and a step, whose CTAs start while the last kernel's retire, has not: 1400 bodies in 144 items
         // of 256 threads tie with 506 of 64 here, in a step they take 51.8 us against 47.7.
+        if (!sym_fits(c, sym_part_rows(*c, t), vjp)) continue;
         if (!mixed && p.first > 64 && sym_item_count(*c, t, t.slice, c->sm_count) < c->sm_count) continue;
         if (sym_settings.empty() || sym_settings.back().tail != t.tail || sym_settings.back().block != t.block ||
             sym_settings.back().ipt != t.ipt || sym_settings.back().slice != t.slice)
           sym_settings.push_back(t);
       }
     }
-    if (sym_only) variants.clear();
+    // (layouts of so many bodies that no list of theirs stays below the cap keep the one-sided pass)
+    if (sym_only && !sym_settings.empty()) variants.clear();
   }
   for (int var : variants)
     for (int b : blocks) {
@@ -1422,6 +1430,8 @@ nbody_status nbody_init(nbody_ctx** out, const nbody_config* cfg, int64_t n_syst
   // host-side fault injection for tests: NBODY_FAULT_ALLOC=k makes the k-th scratch
   // allocation of this context report NBODY_ENOMEM (no device fault is involved)
   if (const char* fa = getenv("NBODY_FAULT_ALLOC")) c->fault_alloc = std::max<int64_t>(0, atoll(fa));
+  if (const char* mb = getenv("NBODY_SYM_PARTIAL_MB"))
+    c->sym_cap = std::min<size_t>(kMaxSymPartialBytes, (size_t)std::max(0, atoi(mb)) << 20);
   if (const char* nv = getenv("NBODY_NVTX")) c->nvtx = nv[0] == '1';
   NvtxRange range_init(c->nvtx, "nbody_init");
   c->stream = static_cast<cudaStream_t>(cuda_stream);

@@ -132,6 +132,24 @@ inline int64_t sym_item_count(const SymLayout& c, const Tiling& t, int64_t slice
   return items;
 }
 
+// Entries of partial sums that a symmetric tiling needs (t.slice as set): a system's bodies times the slots
+// of its most used row.
+inline int64_t sym_part_rows(const SymLayout& c, const Tiling& t) {
+  const double area = (double)t.slice * (double)t.block * t.ipt;
+  int64_t rows = 0, step, last = 0, own = 0;  // own: entries of a system of `last` bodies
+  for (int s = 0; s < c.n_sys; ++s) {
+    const int64_t n = c.offsets[s + 1] - c.offsets[s];
+    if (n != last) {
+      const SymRows R(c, t, n);
+      int64_t most = 0;
+      for (int64_t r = 0; r < R.rows; ++r) most = std::max(most, r + 1 + R.pieces(r, area, t.tail, &step));
+      own = most * n, last = n;
+    }
+    rows += own;
+  }
+  return rows;
+}
+
 // Slice of a symmetric tiling (t.tail as set) that makes at most `pieces` work items per CTA of a
 // full grid, as many as that allows: one item more than CTAs would cost a whole second round.
 constexpr int kSymPieces = 6;

@@ -65,3 +65,55 @@ def test_sym64_rows_hold_whole_chunks(nb, tmp_path, monkeypatch, sizes):
             gG, ge = gp[s].cpu().numpy()
             scale = max(abs(oG), abs(oe) * eps)
             assert abs(gG - oG) <= 10 * tol * scale and abs(ge - oe) * eps <= 10 * tol * scale, (tail, s)
+
+
+@pytest.mark.parametrize("prec,n,cap_mb,sym", [(1, 9000, 0, False), (0, 700, 0, False), (0, 2500, 1, True),
+                                               (1, 9000, 5, True)])
+def test_layouts_over_the_memory_cap_still_run(nb, monkeypatch, prec, n, cap_mb, sym):
+    """Lists over the cap of the symmetric passes' partial sums are left out; where none is below it, the
+    one-sided pass serves sizes at which it is no candidate otherwise."""
+    monkeypatch.setenv("NBODY_SYM_PARTIAL_MB", str(cap_mb))
+    G, eps, dt = 1.1, 0.05, 1e-3
+    x, v, m = inputs.plummer(n, seed=n)
+    rng = np.random.default_rng(n)
+    lx, lv = rng.standard_normal((n, 3)), 0.1 * rng.standard_normal((n, 3))
+    ctx = nb.nbody_init(G=G, eps=eps, dt=dt, n=n, precision=prec)
+    slicing = nb.nbody_get_slicing(ctx)
+    assert (slicing["tail"] >= 2) == sym
+    assert not sym or slicing["max_slices"] * n * 32 <= cap_mb << 20
+    a, phi = nb.nbody_forces(ctx, *to_dev(x, m))
+    got = nb.nbody_adjoint(ctx, *to_dev(x, v, m), 1, 1, *to_dev(lx, lv))
+    nb.nbody_sync(ctx)
+    ftol, gtol = (1e-4, 1e-4) if prec else (1e-11, 1e-10)
+    a_ref, phi_ref = oracle.forces(x, m, G=G, eps=eps)
+    assert force_rel_err(a.cpu().numpy(), a_ref).max() <= ftol
+    assert_elem_close(phi.cpu().numpy(), phi_ref, ftol, "phi")
+    for g, o, what in zip(got, oracle.adjoint(x, v, m, G, eps, dt, 1, lx, lv), ("g_x0", "g_v0", "g_m")):
+        assert_elem_close(g.cpu().numpy(), o, gtol, what)
+
+
+@pytest.mark.parametrize("systems,gradient", [(128, False), (64, True)])
+def test_many_large_systems_are_accepted(nb, systems, gradient):
+    """Layouts some of whose lists need more than the cap of 4 GiB (systems of 16 384 bodies)."""
+    k, G, eps, dt = 16384, 1.1, 0.05, 1e-3
+    x1, v1, m1 = inputs.plummer(k, seed=5)
+    scale = 1.0 + 0.01 * np.arange(systems)[:, None, None]
+    x, v = ((scale * t[None]).reshape(-1, 3) for t in (x1, v1))
+    m = np.tile(m1, systems)
+    ctx = nb.nbody_init(G=G, eps=eps, dt=dt, offsets=[k * s for s in range(systems + 1)])
+    xt, vt, mt = to_dev(x, v, m)
+    a, _ = nb.nbody_forces(ctx, xt, mt, with_phi=False)
+    nb.nbody_sync(ctx)
+    idx = inputs.sample_indices(k, 128, seed=1)
+    for s in (0, systems // 2, systems - 1):
+        sl = slice(k * s, k * (s + 1))
+        a_ref, _ = oracle.forces_at(x[sl], m[sl], idx, G=G, eps=eps)
+        assert force_rel_err(a[sl].cpu().numpy()[idx], a_ref).max() <= 1e-4
+    if gradient:
+        rng = np.random.default_rng(1)
+        lx, lv = rng.standard_normal(x.shape), 0.1 * rng.standard_normal(x.shape)
+        got = nb.nbody_adjoint(ctx, xt, vt, mt, 1, 1, *to_dev(lx, lv))
+        nb.nbody_sync(ctx)
+        sl = slice(k * (systems - 1), k * systems)
+        for g, o, what in zip(got, oracle.adjoint(x[sl], v[sl], m[sl], G, eps, dt, 1, lx[sl], lv[sl]), ("x", "v", "m")):
+            assert_elem_close(g[sl].cpu().numpy(), o, 1e-4, what)

@@ -29,6 +29,7 @@ extern "C" int check(const int64_t* sizes, int n_sys, int j_block, int block, in
   int64_t rows;
   if (!build_sym_items(c, t, items, chunks, max_slots, rows)) return 1;
   if (sym_item_count(c, t, slice, 1 << 30) != (int64_t)items.size()) return 3;  // (empty systems included)
+  if (rows != sym_part_rows(c, t)) return 2;
   std::vector<int> written((size_t)rows);
   std::vector<int64_t> met((size_t)c.n_total);
   for (const SymItem& w : items) {
