@@ -144,6 +144,7 @@ struct nbody_ctx : SymLayout {
   bool vjp_ready = false;
   size_t sym_cap = kMaxSymPartialBytes;  // NBODY_SYM_PARTIAL_MB=k lowers it
   int64_t fault_alloc = 0;  // > 0: the fault_alloc-th scratch allocation fails (NBODY_FAULT_ALLOC, tests)
+  bool fault_hit = false;   // ... has failed
   bool nvtx = false;        // NBODY_NVTX=1: NVTX ranges around the API calls and the adjoint's phases
   bool vjp_params = false;  // VJP launches also form the G and eps gradient sums
 
@@ -215,8 +216,10 @@ nbody_status ensure(nbody_ctx* c, DevBuf& b, size_t bytes) {
     b.bytes = 0;
   }
   if (bytes == 0) bytes = 16;
-  if (c->fault_alloc > 0 && --c->fault_alloc == 0)
+  if (c->fault_alloc > 0 && --c->fault_alloc == 0) {
+    c->fault_hit = true;
     return fail(c, NBODY_ENOMEM, "injected allocation failure (NBODY_FAULT_ALLOC) for %zu bytes", bytes);
+  }
   cudaError_t e = cudaMalloc(&b.p, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -377,34 +380,23 @@ void build_items(const nbody_ctx* c, const Tiling& t, std::vector<WorkItem>& ite
   });
 }
 
-nbody_status upload_items(nbody_ctx* c, const void* items, size_t bytes, void** dst) {
-  invalidate_graph(c);
-  if (*dst) {
-    cudaStreamSynchronize(c->stream);
-    cudaFree(*dst);
-    *dst = nullptr;
-  }
-  if (cudaMalloc(dst, std::max<size_t>(16, bytes)) != cudaSuccess) {
+// A new device buffer with a copy of [src, src + bytes) (*dst stays NULL on failure).
+nbody_status upload(nbody_ctx* c, const void* src, size_t bytes, void** dst) {
+  *dst = nullptr;
+  void* p = nullptr;
+  if (cudaMalloc(&p, std::max<size_t>(16, bytes)) != cudaSuccess) {
     cudaGetLastError();
-    *dst = nullptr;
-    return fail(c, NBODY_ENOMEM, "cudaMalloc of the work list failed");
+    return fail(c, NBODY_ENOMEM, "cudaMalloc of a work or chunk list failed");
   }
-  if (bytes) NB_CUDA(c, cudaMemcpy(*dst, items, bytes, cudaMemcpyHostToDevice));
+  cudaError_t e = bytes ? cudaMemcpy(p, src, bytes, cudaMemcpyHostToDevice) : cudaSuccess;
   // a pageable-memory cudaMemcpy may return before its DMA lands; the context
   // stream can be non-blocking, so wait for the device before any launch
-  NB_CUDA(c, cudaDeviceSynchronize());
-  return NBODY_OK;
-}
-
-nbody_status upload_chunks(nbody_ctx* c, const std::vector<Chunk>& ch, Chunk** dst) {
-  if (!*dst) {
-    if (cudaMalloc(dst, std::max<size_t>(1, ch.size()) * sizeof(Chunk)) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(c, NBODY_ENOMEM, "cudaMalloc of the chunk list failed");
-    }
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  if (e != cudaSuccess) {
+    cudaFree(p);
+    return fail(c, NBODY_ECUDA, "upload of a work or chunk list failed: %s", cudaGetErrorString(e));
   }
-  if (!ch.empty()) NB_CUDA(c, cudaMemcpy(*dst, ch.data(), ch.size() * sizeof(Chunk), cudaMemcpyHostToDevice));
-  NB_CUDA(c, cudaDeviceSynchronize());
+  *dst = p;
   return NBODY_OK;
 }
 
@@ -422,46 +414,62 @@ nbody_status install_tiling(nbody_ctx* c, Tiling t, bool vjp) {
                 t.variant);
   const size_t per = vjp ? 64 : 32;
   std::vector<Chunk> chunks;
-  int n_items = 0, max_slices = 1;
+  std::vector<SymItem> sym_items;
+  std::vector<WorkItem> items;
+  int n_items = 0, max_slices = 1, longest = 1;
   size_t part_bytes = 0;
-  nbody_status s;
   if (is_sym(t)) {
     if (t.slice <= 0) t.slice = sym_slice(*c, t, occ * c->sm_count, kSymPieces);
-    std::vector<SymItem> items;
     int64_t rows = 0;
-    if (!build_sym_items(*c, t, items, chunks, max_slices, rows))
+    if (!build_sym_items(*c, t, sym_items, chunks, max_slices, rows))
       return fail(c, NBODY_EINVAL, "symmetric work list: a chunk of bodies crosses two rows");
     part_bytes = (size_t)rows * per;
     if (!sym_fits(c, rows, vjp))
       return fail(c, NBODY_EINVAL, "symmetric tiling needs %zu bytes of partial sums", part_bytes);
-    n_items = (int)items.size();
-    if (!vjp) {
-      c->sym_longest = 1;
-      for (const SymItem& w : items) c->sym_longest = std::max(c->sym_longest, w.j_end - w.j_begin);
-    }
-    if ((s = upload_items(c, items.data(), items.size() * sizeof(SymItem), vjp ? &c->d_vitems : &c->d_items))) return s;
+    n_items = (int)sym_items.size();
+    for (const SymItem& w : sym_items) longest = std::max(longest, w.j_end - w.j_begin);
   } else {
     if (t.slice <= 0) t.slice = auto_slice(c, t, occ * c->sm_count);
     t.slice = std::max(kSliceQuantum, (t.slice / kSliceQuantum) * kSliceQuantum);
-    std::vector<WorkItem> items;
     std::vector<int> sys_slices;
     build_items(c, t, items, sys_slices, max_slices);
     chunks = c->chunks;
     for (auto& k : chunks) k.n_slices = sys_slices[k.sys], k.stride = (int32_t)c->n_total, k.row0 = 0;
     part_bytes = (size_t)max_slices * (size_t)c->n_total * per;
     n_items = (int)items.size();
-    if ((s = upload_items(c, items.data(), items.size() * sizeof(WorkItem), vjp ? &c->d_vitems : &c->d_items))) return s;
   }
   t.n_ctas = std::max(1, std::min(occ * c->sm_count, std::max(1, n_items)));
-  if ((s = upload_chunks(c, chunks, vjp ? &c->d_vchunks : &c->d_chunks))) return s;
-  if ((s = ensure(c, c->part, part_bytes))) return s;
+
+  // The new lists and the partial sums come first: when one of them cannot be had, the pass keeps the
+  // tiling and the list it had (they have to match: the two kinds of items differ in size).
+  invalidate_graph(c);
+  void *d_list = nullptr, *d_chunks = nullptr;
+  nbody_status s = is_sym(t) ? upload(c, sym_items.data(), sym_items.size() * sizeof(SymItem), &d_list)
+                             : upload(c, items.data(), items.size() * sizeof(WorkItem), &d_list);
+  if (!s) s = upload(c, chunks.data(), chunks.size() * sizeof(Chunk), &d_chunks);
+  if (!s) s = ensure(c, c->part, part_bytes);
+  if (s) {
+    cudaFree(d_list);
+    cudaFree(d_chunks);
+    return s;
+  }
+  cudaStreamSynchronize(c->stream);  // nothing reads the old lists any more
+  cudaFree(vjp ? c->d_vitems : c->d_items);
+  cudaFree(vjp ? c->d_vchunks : c->d_chunks);
   if (vjp) {
+    c->d_vitems = d_list, c->d_vchunks = static_cast<Chunk*>(d_chunks);
     c->vt = t, c->n_vitems = n_items, c->vmax_slices = max_slices, c->vpart_bytes = part_bytes, c->vjp_ready = true;
   } else {
+    c->d_items = d_list, c->d_chunks = static_cast<Chunk*>(d_chunks);
     c->ft = t, c->n_items = n_items, c->max_slices = max_slices, c->fpart_bytes = part_bytes;
+    c->sym_longest = longest;
   }
   return NBODY_OK;
 }
+
+// The force pass's partial sums, before anything is launched: growing the buffer for a gradient may have
+// failed and left none.
+nbody_status ensure_part(nbody_ctx* c) { return ensure(c, c->part, c->fpart_bytes); }
 
 SymLaunch sym_launch(nbody_ctx* c, bool vjp, Potential phi) {
   SymLaunch L{};
@@ -961,6 +969,9 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
   // Work lists of the symmetric tilings: one item per CTA of a full grid (or a few), cut evenly or
   // with shorter pieces for the end of the schedule. They are timed with the refined slicings below.
   std::vector<Tiling> sym_settings;
+  size_t room = 0, device = 0;  // memory that a list's partial sums can have
+  NB_CUDA(c, cudaMemGetInfo(&room, &device));
+  room += c->part.bytes;
   if (sym && !large) {
     const std::vector<std::pair<int, int>> br =
         mixed && vjp ? std::vector<std::pair<int, int>>{{128, 1}, {128, 2}, {256, 2}}
@@ -979,14 +990,15 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
         // FP64 lists of few large items need an even placement on the SMs, which the timing here has
         // and a step, whose CTAs start while the last kernel's retire, has not: 1400 bodies in 144 items
         // of 256 threads tie with 506 of 64 here, in a step they take 51.8 us against 47.7.
-        if (!sym_fits(c, sym_part_rows(*c, t), vjp)) continue;
+        const int64_t rows = sym_part_rows(*c, t);
+        if (!sym_fits(c, rows, vjp) || (size_t)rows * (vjp ? 64 : 32) > room) continue;
         if (!mixed && p.first > 64 && sym_item_count(*c, t, t.slice, c->sm_count) < c->sm_count) continue;
         if (sym_settings.empty() || sym_settings.back().tail != t.tail || sym_settings.back().block != t.block ||
             sym_settings.back().ipt != t.ipt || sym_settings.back().slice != t.slice)
           sym_settings.push_back(t);
       }
     }
-    // (layouts of so many bodies that no list of theirs stays below the cap keep the one-sided pass)
+    // (where no list has room, as in layouts of very many bodies, the one-sided pass remains)
     if (sym_only && !sym_settings.empty()) variants.clear();
   }
   for (int var : variants)
@@ -1032,22 +1044,24 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
               (vjp ? c->vt : c->ft).slice, (vjp ? c->vt : c->ft).n_ctas, vjp ? c->n_vitems : c->n_items, *cost * 1e12);
     return NBODY_OK;
   };
+  // a candidate that finds no memory is left out (an injected failure is for the caller)
+  auto no_room = [&](nbody_status r) { return r == NBODY_ENOMEM && !c->fault_hit; };
   std::vector<std::pair<double, Tiling>> timed;
   // one untimed pass first, so that the GPU has left its idle clocks before the first candidate is timed
   for (const Tiling& t0 : cands) {
     if (ctas_per_sm(g.precision, t0, vjp, g.law) <= 0) continue;
     double cost = 0;
-    if ((s = measure(t0, &cost))) return s;
+    if ((s = measure(t0, &cost)) && !no_room(s)) return s;
     break;
   }
   for (const Tiling& t0 : cands) {
     if (ctas_per_sm(g.precision, t0, vjp, g.law) <= 0) continue;
     double cost = 0;
-    if ((s = measure(t0, &cost))) return s;
-    timed.push_back({cost, t0});
+    if ((s = measure(t0, &cost)) && !no_room(s)) return s;
+    if (!s) timed.push_back({cost, t0});
   }
   if (timed.empty() && sym_settings.empty())
-    return fail(c, NBODY_EINVAL, "no compiled tiling matches the requested parameters");
+    return s ? s : fail(c, NBODY_EINVAL, "no compiled tiling matches the requested parameters");
   // the candidates within 8% of the best (at most five) are timed twice more, interleaved, and
   // keep their best time: single timings differ by 1-3% from run to run
   std::stable_sort(timed.begin(), timed.end(),
@@ -1057,7 +1071,8 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
   for (int round = 0; round < 2 && top > 1; ++round)
     for (size_t k = 0; k < top; ++k) {
       double cost = 0;
-      if ((s = measure(timed[k].second, &cost))) return s;
+      if ((s = measure(timed[k].second, &cost)) && !no_room(s)) return s;
+      if (s) continue;
       timed[k].first = std::min(timed[k].first, cost);
     }
   // order the re-timed candidates; the first is the choice unless the slice refinement finds better
@@ -1083,7 +1098,8 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
       }
       base.slice = 0;
       base.tail = 0;
-      if ((s = install_tiling(c, base, vjp))) return s;
+      if ((s = install_tiling(c, base, vjp)) && !no_room(s)) return s;
+      if (s) continue;
       const int L0 = c->ft.slice;
       const int64_t n_ctas = c->ft.n_ctas;
       std::vector<int> ls = {L0 / 2, L0, L0 * 2};
@@ -1113,7 +1129,8 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
       const double limit = round == 0 ? 1e300 : 1.03 * *std::min_element(lc.begin(), lc.end());
       for (size_t k = 0; k < settings.size(); ++k) {
         if (round == 1 && lc[k] > limit) continue;
-        if ((s = install_tiling(c, settings[k], vjp))) return s;
+        if ((s = install_tiling(c, settings[k], vjp)) && !no_room(s)) return s;
+        if (s) continue;
         double cost = 0;
         if ((s = time_tiling(c, vjp, &cost))) return s;
         if (verbose)
@@ -1225,7 +1242,10 @@ nbody_status adjoint_sweep(nbody_ctx* c, const double* x0, const double* v0, con
   if (!c->vjp_ready) {
     // VJP tiling: tuned once per context (synchronises the stream)
     NB_CUDA(c, cudaStreamSynchronize(st));
-    if ((s = autotune(c, true))) return s;
+    if ((s = autotune(c, true))) {
+      c->vjp_ready = false;  // whatever candidate was installed last: the next call tunes again
+      return s;
+    }
   }
   const int vjp_bytes = g_params ? 96 : 64;  // per body and slice: 2 or 3 double4
   if ((s = ensure(c, c->part, std::max(c->fpart_bytes, c->vpart_bytes / 64 * (size_t)vjp_bytes)))) return s;
@@ -1483,7 +1503,9 @@ nbody_status nbody_init(nbody_ctx** out, const nbody_config* cfg, int64_t n_syst
       cudaMemcpy(c->d_csys_chunk, csys_chunk.data(), (n_systems + 1) * sizeof(int32_t), cudaMemcpyHostToDevice) !=
           cudaSuccess)
     return bail(fail(c, NBODY_ECUDA, "upload of layout tables failed"));
-  if ((s = upload_chunks(c, cchunks, &c->d_cchunks))) return bail(s);
+  void* d_cchunks = nullptr;
+  if ((s = upload(c, cchunks.data(), cchunks.size() * sizeof(Chunk), &d_cchunks))) return bail(s);
+  c->d_cchunks = static_cast<Chunk*>(d_cchunks);
 
   const bool fixed_variant = cfg->precision == NBODY_FP64 || cfg->variant != 0 || cfg->law == NBODY_LAW_LJ;
   if (c->n_total > 0 && (cfg->block == 0 || cfg->i_per_thread == 0 || cfg->j_tile == 0 || !fixed_variant)) {
@@ -1515,6 +1537,7 @@ nbody_status nbody_forces(nbody_ctx* c, const double* x, const double* m, double
   nbody_status s;
   if ((s = check_state_args(c, x, nullptr, m, a, false, true))) return s;
   if ((s = check_dev(c, phi, (size_t)c->n_total * sizeof(double), "phi", true))) return s;
+  if ((s = ensure_part(c))) return s;
   double* xm = const_cast<double*>(x);
   if ((s = run_centre(c, x, m, c->stream))) return s;
   if ((s = run_post(c, post_launch(c, kStage, xm, nullptr, m, a, nullptr, true), c->stream))) return s;
@@ -1550,6 +1573,7 @@ namespace {
 nbody_status step_validated(nbody_ctx* c, double* x, double* v, const double* m, double* a, int32_t a_valid,
                             int32_t n_steps, double* energy_log) {
   nbody_status s;
+  if ((s = ensure_part(c))) return s;
   if (!(c->cfg.flags & NBODY_FLAG_GRAPH)) return enqueue_step(c, x, v, m, a, a_valid, n_steps, energy_log, c->stream);
 
   // CUDA-graph replay: capture the whole call once per argument set, replay afterwards.
@@ -1600,6 +1624,7 @@ nbody_status nbody_energy(nbody_ctx* c, const double* x, const double* v, const 
     return NBODY_OK;
   }
   if ((s = check_state_args(c, x, v, m, nullptr, true, false))) return s;
+  if ((s = ensure_part(c))) return s;
   if ((s = ensure(c, c->a_scratch, (size_t)c->n_total * 3 * sizeof(double)))) return s;
   double* xm = const_cast<double*>(x);
   double* vm = const_cast<double*>(v);
@@ -1623,6 +1648,7 @@ nbody_status nbody_virial(nbody_ctx* c, const double* x, const double* v, const 
     return NBODY_OK;
   }
   if ((s = check_state_args(c, x, v, m, nullptr, true, false))) return s;
+  if ((s = ensure_part(c))) return s;
   if ((s = ensure(c, c->a_scratch, (size_t)c->n_total * 3 * sizeof(double)))) return s;
   double* xm = const_cast<double*>(x);
   double* vm = const_cast<double*>(v);

@@ -76,3 +76,41 @@ def test_first_allocation_fails_in_init(nb, monkeypatch):
     with pytest.raises(nb.NBodyError) as ei:
         nb.nbody_init(G=1.0, eps=0.02, dt=1e-3, precision=nb.FP64, n=100)
     assert ei.value.status == 2
+
+
+@pytest.mark.parametrize("prec,n", [(0, 1500), (1, 3500)])
+def test_context_survives_a_failed_gradient(nb, monkeypatch, prec, n):
+    """An allocation that fails in the first gradient call (scratch, or partial sums of a candidate of the VJP
+    tuner) leaves list, tiling and buffers of both passes matching: forces are what they were, and the
+    gradient is right when asked for again."""
+    import torch
+    x, v, m = inputs.plummer(n, seed=45)
+    rng = np.random.default_rng(n)
+    lx, lv = rng.standard_normal((n, 3)), 0.1 * rng.standard_normal((n, 3))
+    args = to_dev(x, v, m) + (2, 1) + to_dev(lx, lv)
+    want = oracle.adjoint(x, v, m, 1.0, 0.02, 1e-3, 2, lx, lv)
+    failed = 0
+    for k in range(1, 200):
+        monkeypatch.setenv("NBODY_FAULT_ALLOC", str(k))
+        try:
+            ctx = nb.nbody_init(G=1.0, eps=0.02, dt=1e-3, precision=prec, n=n)
+        except nb.NBodyError as e:
+            assert e.status == 2
+            continue
+        a, _ = nb.nbody_forces(ctx, args[0], args[2])
+        try:
+            nb.nbody_adjoint(ctx, *args)
+            done = True
+        except nb.NBodyError as e:
+            assert e.status == 2 and "injected" in str(e)
+            done, failed = False, failed + 1
+        b, _ = nb.nbody_forces(ctx, args[0], args[2])
+        got = nb.nbody_adjoint(ctx, *args)
+        nb.nbody_sync(ctx)
+        ctx.close()
+        assert torch.equal(a, b), k
+        for g, o in zip(got, want):
+            assert np.abs(g.cpu().numpy() - o).max() <= (1e-4 if prec else 1e-11) * np.abs(o).max(), k
+        if done:
+            break
+    assert done and failed >= 3  # weights' staging, work copies, checkpoints at least
