@@ -117,7 +117,7 @@ struct nbody_ctx : SymLayout {
   cudaStream_t cap_stream = nullptr;  // private stream used only to capture graphs
   std::string err = "no error";
   int64_t launches = 0;
-  uint32_t epoch = 0;  // number of the current call (SysParam::uniform); 0 while tuning
+  uint32_t epoch = 0;  // number of the current call (SysParam::uniform), 0 before the first
 
   // layout
   Chunk* d_chunks = nullptr;
@@ -622,10 +622,21 @@ nbody_status run_post(nbody_ctx* c, const PostLaunch& P, cudaStream_t st) {
   return NBODY_OK;
 }
 
-// Starts a call: its number (never 0), and on the mixed path the staging parameters.
+// Starts a call: its number (never 0), and on the mixed path the staging parameters. A captured call keeps its
+// number in every replay, so the marks of unequal masses that carry it are taken off first (one memset node; a
+// replay with unequal masses would leave them to one with equal masses, whose sums then differ in rounding).
 nbody_status run_centre(nbody_ctx* c, const double* x, const double* m, cudaStream_t st) {
   if (++c->epoch == 0) c->epoch = 1;
-  if (c->cfg.precision != NBODY_MIXED || c->n_total == 0) return NBODY_OK;
+  if (c->n_total == 0) return NBODY_OK;
+  if (c->cfg.precision != NBODY_MIXED) {
+    if (c->cfg.law != NBODY_LAW_GRAVITY || !is_sym(c->ft)) return NBODY_OK;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
+    if (capture == cudaStreamCaptureStatusActive)
+      NB_CUDA(c, cudaMemset2DAsync(&static_cast<SysParam*>(c->sysp.p)->uniform, sizeof(SysParam), 0, sizeof(uint32_t),
+                                   (size_t)c->n_sys, st));
+    return NBODY_OK;
+  }
   CentreLaunch C{};
   C.chunks = c->d_cchunks;
   C.n_chunks = c->n_cchunks;

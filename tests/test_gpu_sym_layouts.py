@@ -117,3 +117,48 @@ def test_many_large_systems_are_accepted(nb, systems, gradient):
         sl = slice(k * (systems - 1), k * systems)
         for g, o, what in zip(got, oracle.adjoint(x[sl], v[sl], m[sl], G, eps, dt, 1, lx[sl], lv[sl]), ("x", "v", "m")):
             assert_elem_close(g[sl].cpu().numpy(), o, 1e-4, what)
+
+
+@pytest.mark.parametrize("capture", ["context", "caller"])
+def test_sym64_replays_do_not_depend_on_earlier_masses(nb, tmp_path, monkeypatch, capture):
+    """A replay with equal masses right after one with unequal masses gives the bits of an eager call."""
+    import torch
+    monkeypatch.setenv("NBODY_TUNE_CACHE", str(tmp_path / "tune"))
+    n, systems, dt = 500, 3, 1e-3
+    ens = inputs.ensemble(systems, seed=8, sizes=np.full(systems, n))
+    kw = dict(G=1.1, eps=0.05, dt=dt, offsets=[int(o) for o in ens.offsets], precision=nb.FP64)
+    eager = nb.nbody_init(**kw)
+    assert nb.nbody_get_slicing(eager)["tail"] >= 2
+    replayed = nb.nbody_init(flags=nb.FLAG_GRAPH if capture == "context" else 0, **kw)
+    unequal = _masses(ens.m, "lognormal", 8)
+    first_unequal = ens.m.copy()
+    first_unequal[:n] = unequal[:n]
+
+    def buffers():
+        xt, vt, mt = to_dev(ens.x, ens.v, ens.m)
+        return xt, vt, mt, torch.empty_like(xt)
+
+    def load(b, masses):
+        for t, src in zip(b, (ens.x, ens.v, masses)):
+            t.copy_(torch.from_numpy(src))
+
+    def step(ctx, b):
+        nb.nbody_step(ctx, *b, False, 2)
+
+    r, e = buffers(), buffers()
+    graph = torch.cuda.CUDAGraph()
+    if capture == "caller":
+        side = torch.cuda.Stream()
+        with torch.cuda.stream(side):
+            step(replayed, r)
+        side.synchronize()
+        with torch.cuda.graph(graph, stream=side, capture_error_mode="thread_local"):
+            step(replayed, r)
+    for masses in (unequal, ens.m, first_unequal, ens.m, unequal, first_unequal):
+        load(r, masses), load(e, masses)
+        torch.cuda.synchronize()
+        graph.replay() if capture == "caller" else step(replayed, r)
+        step(eager, e)
+        torch.cuda.synchronize()
+        for got, want in zip(r, e):
+            assert torch.equal(got, want)
