@@ -271,7 +271,7 @@ cudaError_t launch_post(const PostLaunch& P, cudaStream_t st);
 
 // Staging parameters of every system (mixed path): the origin c is the
 // mass-weighted mean position (plain mean if the mass is 0), and for gravity the
-// scales are set from the largest coordinate and mass. Per-chunk sums into cpart
+// scales are set from the extent, the softening and the largest mass. Per-chunk sums into cpart
 // [n_chunks][kEnergyVals], then per system in a fixed order by the last CTA
 // (ticket `done`, zero between launches).
 struct CentreLaunch {

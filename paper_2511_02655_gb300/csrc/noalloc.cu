@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(kSumThreads) k_na_sums(const double* x, const 
   Extent q{0u, 0u, 1u};
   const double m0 = m[0];
   for (int64_t i = (int64_t)blockIdx.x * kSumThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kSumThreads)
-    centre_terms(x[3 * i], x[3 * i + 1], x[3 * i + 2], m[i], m0, v, q);
+    centre_terms(x[3 * i], x[3 * i + 1], x[3 * i + 2], m[i], x, m0, v, q);
   q.warp_join();
   if (threadIdx.x % 32 == 0) ext[threadIdx.x / 32] = q;
   block_sum<7, kSumThreads>(v);  // its barriers also publish ext
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(256) k_na_stage(const double* x, const double*
     for (int c = 0; c < 7; ++c) w[c] = warp_sum(w[c]);
     e.warp_join();
     if (threadIdx.x == 0) {
-      staging_params(sp, w, e, n, m[0], true, eps, kNearRadiusEps);
+      staging_params(sp, w, e, n, x, m[0], true, eps, kNearRadiusEps);
       if (blockIdx.x == 0) *S.sys = sp;
     }
   }

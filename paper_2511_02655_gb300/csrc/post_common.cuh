@@ -115,8 +115,8 @@ __device__ __forceinline__ void add_slot(const fpair4 q, float (&h)[4], float (&
   two_sum_acc(h[3], l[3], q.zp.z), l[3] += q.zp.w;
 }
 
-// Largest coordinate and mass of a chunk by their float64 high words (sign bit
-// off: the words order as the magnitudes) and whether its masses all equal its
+// Largest distance along an axis from the system's first body and largest mass of a chunk by their
+// float64 high words (sign bit off: the words order as the magnitudes) and whether its masses all equal its
 // system's first, as one 64-bit value that is carried beside the chunk's sums.
 struct Extent {
   unsigned x, m, uniform;
@@ -139,29 +139,36 @@ struct Extent {
 
 __device__ __forceinline__ unsigned high_word(const double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
 
-// 2^(to - e) for the float64 with high word h of binary exponent e (1 where h is 0, tiny, infinite or NaN)
-__device__ __forceinline__ double power_of_two_scale(const unsigned h, const int to) {
-  const int e = (int)(h >> 20) - 1023;
-  return e < -900 || e > 900 ? 1.0 : ldexp(1.0, to - e);
+// Binary exponent of the float64 with high word h, and whether it is one to scale by (not 0, tiny, infinite or NaN).
+__device__ __forceinline__ int exponent_of(const unsigned h) { return (int)(h >> 20) - 1023; }
+__device__ __forceinline__ bool scalable(const int e) { return e >= -900 && e <= 900; }
+
+// Staged lengths of gravity. The farthest body of a system lies below 2^12 from its origin: the powers of
+// distances from there down to 2^-25, s^-5 (the force gradient) included, stay in float32's range. Where that
+// would stage the softening below 2^-24, it is lifted to 2^-24 as far as the farthest body stays below 2^22, and
+// beyond that as far as the lengths are not staged longer than they are: far from the rest, an escaper loses the
+// last bits of its gradient's powers before near pairs' turn infinite. Without softening the nearest distance is
+// not known, and a system is not staged smaller than it is up to that size.
+constexpr int kFarExp = 10, kFarthestExp = 20, kNearExp = -24;
+__device__ __forceinline__ int staging_exponent(const int far, const int eps) {  // (binary exponents)
+  const int room = kFarthestExp - far, near = scalable(eps) ? kNearExp - eps : min(0, room);
+  return max(kFarExp - far, max(min(near, room), min(near, 0)));
 }
 
-// The staged coordinates of gravity stay below 2^12: with distances down to 2^-25
-// of that, s^-5 (the force gradient) stays in the float32 range at both ends.
-constexpr int kExtentExp = 10;
-
-// One body's terms of the staging origin's sums (sum m x, sum m, sum x) and its extent.
+// One body's terms of the staging origin's sums (sum m x, sum m, sum x) and its extent about the
+// system's first body (position f, mass m0).
 __device__ __forceinline__ void centre_terms(const double x0, const double x1, const double x2, const double mi,
-                                             const double m0, double (&v)[7], Extent& q) {
+                                             const double* f, const double m0, double (&v)[7], Extent& q) {
   v[0] += mi * x0, v[1] += mi * x1, v[2] += mi * x2, v[3] += mi;
   v[4] += x0, v[5] += x1, v[6] += x2;
-  q.join(Extent{max(max(high_word(x0), high_word(x1)), high_word(x2)), high_word(mi),
+  q.join(Extent{max(max(high_word(x0 - f[0]), high_word(x1 - f[1])), high_word(x2 - f[2])), high_word(mi),
                 __double_as_longlong(mi) == __double_as_longlong(m0) ? 1u : 0u});
 }
 
 // Staging parameters of a system of n bodies from those sums: the origin, and for gravity the
-// scales (m0: its first mass).
+// scales (f, m0: its first body).
 __device__ __forceinline__ void staging_params(SysParam& o, const double (&w)[7], const Extent& e, const int64_t n,
-                                               const double m0, const bool gravity, const double eps,
+                                               const double* f, const double m0, const bool gravity, const double eps,
                                                const double near_eps) {
   double c0 = 0.0, c1 = 0.0, c2 = 0.0;
   if (w[3] > 0.0 && isfinite(w[3])) {
@@ -172,12 +179,17 @@ __device__ __forceinline__ void staging_params(SysParam& o, const double (&w)[7]
   if (!(isfinite(c0) && isfinite(c1) && isfinite(c2))) c0 = c1 = c2 = 0.0;
   o.c[0] = c0, o.c[1] = c1, o.c[2] = c2;
   if (!gravity || n <= 0) return;
-  // the softening counts as an extent, so that its staged square stays finite
-  const double s = power_of_two_scale(max(e.x, high_word(eps)), kExtentExp);
+  // no body is farther from the origin than twice the larger of these (the origin's own distance from the
+  // first body counts where negative masses put it outside); the softening counts as an extent, so that
+  // its staged square stays finite
+  const unsigned off = max(max(high_word(c0 - f[0]), high_word(c1 - f[1])), high_word(c2 - f[2]));
+  const int far = exponent_of(max(max(e.x, off), high_word(eps)));
+  const double s = scalable(far) ? ldexp(1.0, staging_exponent(far, exponent_of(high_word(eps)))) : 1.0;
   const double e2 = eps * s, rc = near_eps * e2;
   const unsigned h0 = high_word(m0);
   const bool uniform = e.uniform && m0 > 0.0 && h0 >= (123u << 20) && h0 <= (1923u << 20);
-  const double ms = power_of_two_scale(e.m, 0);
+  const int em = exponent_of(e.m);
+  const double ms = scalable(em) ? ldexp(1.0, -em) : 1.0;
   o.scale = s;
   o.mscale = uniform ? 1.0 / m0 : ms;
   o.inv_mscale = uniform ? m0 : 1.0 / ms;

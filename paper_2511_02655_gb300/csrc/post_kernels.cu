@@ -139,8 +139,10 @@ __global__ void __launch_bounds__(kChunk) k_centre(const CentreLaunch C) {
   double v[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   Extent q{0u, 0u, 1u};
   const int i = c.begin + (int)threadIdx.x;
-  if (i < c.end)
-    centre_terms(C.x[3 * i + 0], C.x[3 * i + 1], C.x[3 * i + 2], C.m[i], C.m[C.off[c.sys]], v, q);
+  if (i < c.end) {
+    const int64_t first = C.off[c.sys];
+    centre_terms(C.x[3 * i + 0], C.x[3 * i + 1], C.x[3 * i + 2], C.m[i], C.x + 3 * first, C.m[first], v, q);
+  }
   q.warp_join();
   if (lane == 0) ext[wid] = q;
   block_sum<7, CB>(v);  // its barriers also publish ext
@@ -154,8 +156,8 @@ __global__ void __launch_bounds__(kChunk) k_centre(const CentreLaunch C) {
   if (!last_of(C.done, gridDim.x)) return;
   __threadfence();
   auto emit = [&](const int sy, const double (&w)[7], const Extent& e) {
-    const int64_t n = C.off[sy + 1] - C.off[sy];
-    staging_params(C.sys[sy], w, e, n, n > 0 ? C.m[C.off[sy]] : 0.0, C.law == 0, C.eps, C.near_eps);
+    const int64_t first = C.off[sy], n = C.off[sy + 1] - first;
+    staging_params(C.sys[sy], w, e, n, C.x + 3 * first, n > 0 ? C.m[first] : 0.0, C.law == 0, C.eps, C.near_eps);
   };
   auto extent = [&](const int sy, const int first, const int step) {
     Extent e{0u, 0u, 1u};

