@@ -21,6 +21,11 @@ namespace symv {
 
 constexpr int kTile = kSymVjpTile;  // j-bodies per shared-memory tile, mixed
 
+// Padding: s^-3 underflows to 0 there, which is all that these sums need of it. (The force pass's distance, at
+// which the reciprocal root itself is 0, would let d.w overflow from |w| = 2e18 on: times the padding's mass 0
+// a NaN in the sums of every body of a partial tile. Here it takes 1e20, as in the one-sided kernels.)
+constexpr float kPad = 1.0e18f;
+
 template <int W, int R, bool P>
 struct Smem {
   static constexpr int NC = P ? 10 : 8;
@@ -225,7 +230,7 @@ __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Sme
       for (int r = 0; r < R; ++r) {
         const int ig = ig0 + 32 * r;
         const bool ok = ig < it.i_end;
-        const float4 q = ok ? st[ig] : make_float4(-sym::kPad, -sym::kPad, -sym::kPad, 0.f);
+        const float4 q = ok ? st[ig] : make_float4(-kPad, -kPad, -kPad, 0.f);
         const float4 u = ok ? sw[ig] : make_float4(0.f, 0.f, 0.f, 0.f);
         B.nx[r] = make_float2(-q.x, -q.x), B.ny[r] = make_float2(-q.y, -q.y), B.nz[r] = make_float2(-q.z, -q.z);
         B.nm[r] = make_float2(-q.w, -q.w);
@@ -240,7 +245,7 @@ __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Sme
         for (int k = 0; k < LPT; ++k) {
           const int t = tid + k * T, j = jt + t;
           if (t < kTile) {
-            const float4 q = j < it.j_end ? st[j] : make_float4(sym::kPad, sym::kPad, sym::kPad, 0.f);
+            const float4 q = j < it.j_end ? st[j] : make_float4(kPad, kPad, kPad, 0.f);
             const float4 u = j < it.j_end ? sw[j] : make_float4(0.f, 0.f, 0.f, 0.f);
             const int b = t >> 6, p = (t & 63) >> 1, h = t & 1;
             float* a = &sm.xy[b][p].x + h;

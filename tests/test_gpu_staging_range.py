@@ -78,3 +78,13 @@ def test_core_beside_a_distant_test_body(nb, tmp_path, monkeypatch, variant, far
         assert force_rel_err(b.cpu().numpy()[core], a_ref[core]).max() <= 1e-4
     _check_gradient(nb, x, v, m, 1.0, eps, 1e-4 if eps == 1e-3 else 1e-9, lx, lv, variant,
                     tmp_path / "tune", monkeypatch, core)
+
+
+@pytest.mark.parametrize("variant", [SYM, 0, 2])
+@pytest.mark.parametrize("n", [65, 300])
+def test_large_weights(nb, tmp_path, monkeypatch, variant, n):
+    """Weights of 1e19 beside the padding of partial tiles."""
+    x, v, m = inputs.plummer(n, seed=7)
+    rng = np.random.default_rng(8)
+    lx, lv = 1e19 * rng.standard_normal((n, 3)), 1e19 * rng.standard_normal((n, 3))
+    _check_gradient(nb, x, v, m, 1.1, 0.05, 1e-2, lx, lv, variant, tmp_path / "tune", monkeypatch)
