@@ -67,15 +67,15 @@ __global__ void __launch_bounds__(BLOCK, (MINB > 0 ? MINB
   __shared__ fc::SmemMixed2<J> sm;
   pdl_wait();
   ItemSource source{L.counter, &sm.item};
-  auto next = [&](WorkItem& w) {
+  auto next = [&] {
     const int it = source.next();
-    if (it < L.n_items) w = L.items[it];
-    return it < L.n_items;
+    return it < L.n_items ? it : -1;
   };
+  auto item = [&](const int it) { return L.items[it]; };
   auto put = [&](const WorkItem& w, const int i, const fpair4& sums) {
     reinterpret_cast<fpair4*>(L.part)[(int64_t)w.slice * L.n_total + i] = sums;
   };
-  fc::items_mixed2<LAW, BLOCK, R, J, PHI>(L, next, put, sm);
+  fc::items_mixed2<LAW, BLOCK, R, J, PHI>(L, next, item, put, sm);
   pdl_trigger();
   retire_cta(L.counter);
 }

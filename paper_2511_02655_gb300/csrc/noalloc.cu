@@ -242,12 +242,14 @@ __global__ void __launch_bounds__(128, 3) k_na_force_one(const int n, const int 
   L.stage_x = S.st, L.stage_lo = S.lo, L.sys = S.sys, L.n_total = n, L.sigma2 = 1.0;
   L.part_slices = 1 << 20, L.block_bodies = 256;
   bool done = false;
-  auto next = [&](WorkItem& w) {
-    if (done) return false;
+  auto next = [&] {
+    const int it = done ? -1 : (int)blockIdx.x;
     done = true;
-    const int tiles = (n + 255) / 256, t = (int)blockIdx.x % tiles, s = (int)blockIdx.x / tiles;
-    w = WorkItem{0, t * 256, min(n, t * 256 + 256), s * len, min(n, (s + 1) * len), s, s + 1};
-    return true;
+    return it;
+  };
+  auto item = [&](const int it) {
+    const int tiles = (n + 255) / 256, t = it % tiles, s = it / tiles;
+    return WorkItem{0, t * 256, min(n, t * 256 + 256), s * len, min(n, (s + 1) * len), s, s + 1};
   };
   auto put = [&](const WorkItem& w, const int i, const fpair4& q) {
     if (!DIRECT) {
@@ -260,7 +262,7 @@ __global__ void __launch_bounds__(128, 3) k_na_force_one(const int n, const int 
     a[3 * (int64_t)i + 2] = ga * ((double)q.zp.x + (double)q.zp.y);
     if (PHI) phi[i] = -gp * ((double)q.zp.z + (double)q.zp.w);
   };
-  fc::items_mixed2<0, 128, 2, kOneTile, PHI>(L, next, put, sm);
+  fc::items_mixed2<0, 128, 2, kOneTile, PHI>(L, next, item, put, sm);
 }
 
 // a and phi from the slots (row height H > 0: a symmetric plan's, else `slices` for every body):
