@@ -36,6 +36,10 @@ constexpr int kSliceQuantum = 4;  // slice lengths are multiples of this many bo
 constexpr int64_t kTailMin = 64;   // shortest slice of a halving tail
 
 constexpr int kSymTail = 2;  // nbody_get_slicing: tail modes of the symmetric pass are reported from here on
+// One-sided passes of at most this many slots per body are followed by O(N) kernels on chunks of kChunk bodies:
+// a body's slots are too few to be shared by many threads, and many small chunks of many systems only make more CTAs
+// and more chunk partials (k_post).
+constexpr int kFewSlots = 8;
 enum class Potential { kNone = 0, kBodies = 1, kEnergy = 2 };  // as sym::kPhi*
 constexpr double kSymMinBodies = 3000.0;    // typical system size from which the symmetric pass is a candidate
 constexpr double kSymOnlyBodies = 8192.0;  // ... and from which it is the only one (mixed path)
@@ -123,7 +127,7 @@ struct nbody_ctx : SymLayout {
   Chunk* d_chunks = nullptr;
   Chunk* d_vchunks = nullptr;  // same chunks, VJP tiling's slice counts
   int32_t* d_sys_chunk = nullptr;
-  int n_cchunks = 0;           // chunks of kChunk bodies of the staging origin's sums
+  std::vector<Chunk> wchunks;  // chunks of kChunk bodies: the staging origin's, and of a pass with few slots per body
   Chunk* d_cchunks = nullptr;
   int32_t* d_csys_chunk = nullptr;
   int64_t* d_off = nullptr;
@@ -134,6 +138,7 @@ struct nbody_ctx : SymLayout {
   int n_items = 0;
   int max_slices = 1;
   size_t fpart_bytes = 0;  // partial sums of the force pass
+  bool fwide = false, vwide = false;  // the O(N) kernels after the force (VJP) pass take chunks of kChunk bodies
   int sym_longest = 0;     // symmetric force list: j-bodies of its longest piece
   // VJP work list (built on first adjoint)
   Tiling vt;
@@ -149,7 +154,7 @@ struct nbody_ctx : SymLayout {
   bool vjp_params = false;  // VJP launches also form the G and eps gradient sums
 
   // scratch
-  DevBuf stage, stage_lo, stage_w, part, sysp, epart, status_counter, a_scratch;
+  DevBuf stage, stage_lo, stage_w, part, sysp, sys_done, epart, status_counter, a_scratch;
   unsigned* counter = nullptr;  // [2]
   unsigned* status = nullptr;   // [1]
 
@@ -417,6 +422,7 @@ nbody_status install_tiling(nbody_ctx* c, Tiling t, bool vjp) {
   std::vector<SymItem> sym_items;
   std::vector<WorkItem> items;
   int n_items = 0, max_slices = 1, longest = 1;
+  bool wide = false;
   size_t part_bytes = 0;
   if (is_sym(t)) {
     if (t.slice <= 0) t.slice = sym_slice(*c, t, occ * c->sm_count, kSymPieces);
@@ -433,7 +439,8 @@ nbody_status install_tiling(nbody_ctx* c, Tiling t, bool vjp) {
     t.slice = std::max(kSliceQuantum, (t.slice / kSliceQuantum) * kSliceQuantum);
     std::vector<int> sys_slices;
     build_items(c, t, items, sys_slices, max_slices);
-    chunks = c->chunks;
+    wide = prec == NBODY_MIXED && max_slices <= kFewSlots;
+    chunks = wide ? c->wchunks : c->chunks;
     for (auto& k : chunks) k.n_slices = sys_slices[k.sys], k.stride = (int32_t)c->n_total, k.row0 = 0;
     part_bytes = (size_t)max_slices * (size_t)c->n_total * per;
     n_items = (int)items.size();
@@ -459,10 +466,12 @@ nbody_status install_tiling(nbody_ctx* c, Tiling t, bool vjp) {
   if (vjp) {
     c->d_vitems = d_list, c->d_vchunks = static_cast<Chunk*>(d_chunks);
     c->vt = t, c->n_vitems = n_items, c->vmax_slices = max_slices, c->vpart_bytes = part_bytes, c->vjp_ready = true;
+    c->vwide = wide;
   } else {
     c->d_items = d_list, c->d_chunks = static_cast<Chunk*>(d_chunks);
     c->ft = t, c->n_items = n_items, c->max_slices = max_slices, c->fpart_bytes = part_bytes;
     c->sym_longest = longest;
+    c->fwide = wide;
   }
   return NBODY_OK;
 }
@@ -578,12 +587,18 @@ nbody_status run_force(nbody_ctx* c, cudaStream_t st, Potential phi) { return ru
 nbody_status run_vjp(nbody_ctx* c, cudaStream_t st) { return run_pair(c, st, true, Potential::kNone); }
 
 
+// Chunks of the O(N) kernels after a pass, and bodies of each.
+int32_t n_chunks(const nbody_ctx* c, bool wide) { return (int32_t)(wide ? c->wchunks : c->chunks).size(); }
+int chunk_size(const nbody_ctx* c, bool wide) { return wide ? kChunk : chunk_bodies(c->n_total); }
+
 // first_stage: the call's first staging (FP64: unequal masses are noted)
 PostLaunch post_launch(nbody_ctx* c, unsigned mode, double* x, double* v, const double* m, double* a, double* phi,
                        bool first_stage = false) {
   PostLaunch P{};
   P.chunks = c->d_chunks;
-  P.n_chunks = (int32_t)c->chunks.size();
+  P.n_chunks = n_chunks(c, c->fwide);
+  P.chunk = chunk_size(c, c->fwide);
+  P.few_slots = c->fwide;
   P.part = static_cast<const double*>(c->part.p);
   P.n_total = c->n_total;
   P.G = c->cfg.G;
@@ -608,7 +623,7 @@ PostLaunch post_launch(nbody_ctx* c, unsigned mode, double* x, double* v, const 
   P.status = c->status;
   P.eout = nullptr;
   P.u_weight = is_sym(c->ft) ? 1.0 : 0.5;  // energy passes: Potential::kEnergy
-  P.sys_chunk = c->d_sys_chunk;
+  P.sys_chunk = c->fwide ? c->d_csys_chunk : c->d_sys_chunk;
   P.n_sys = c->n_sys;
   P.done = c->counter + 4;
   P.part_rows = (int64_t)(c->part.bytes / 32);
@@ -639,7 +654,7 @@ nbody_status run_centre(nbody_ctx* c, const double* x, const double* m, cudaStre
   }
   CentreLaunch C{};
   C.chunks = c->d_cchunks;
-  C.n_chunks = c->n_cchunks;
+  C.n_chunks = (int32_t)c->wchunks.size();
   C.sys_chunk = c->d_csys_chunk;
   C.off = c->d_off;
   C.n_sys = c->n_sys;
@@ -649,6 +664,7 @@ nbody_status run_centre(nbody_ctx* c, const double* x, const double* m, cudaStre
   C.law = c->cfg.law;
   C.eps = c->cfg.eps, C.near_eps = kNearRadiusEps;
   C.done = c->counter + 5;
+  C.sys_done = static_cast<unsigned*>(c->sys_done.p);
   C.n_total = c->n_total;
   C.status = c->status;
   NB_CUDA(c, launch_centre(C, st));
@@ -814,7 +830,9 @@ nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
   };
   PostLaunch C{};
   C.chunks = vjp ? c->d_vchunks : c->d_chunks;
-  C.n_chunks = (int32_t)c->chunks.size();
+  C.n_chunks = n_chunks(c, vjp ? c->vwide : c->fwide);
+  C.chunk = chunk_size(c, vjp ? c->vwide : c->fwide);
+  C.few_slots = !vjp && c->fwide;
   C.part = static_cast<const double*>(c->part.p);
   C.n_total = c->n_total;
   C.G = 1.0;
@@ -1194,7 +1212,7 @@ void free_ctx(nbody_ctx* c) {
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   for (auto& u : c->ev_used) cudaEventDestroy(u.second.first), cudaEventDestroy(u.second.second);
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
-  for (DevBuf* b : {&c->stage, &c->stage_lo, &c->stage_w, &c->part, &c->sysp, &c->epart, &c->status_counter, &c->a_scratch,
+  for (DevBuf* b : {&c->stage, &c->stage_lo, &c->stage_w, &c->part, &c->sysp, &c->sys_done, &c->epart, &c->status_counter, &c->a_scratch,
                     &c->xw, &c->vw, &c->aw, &c->ckpt, &c->traj, &c->hx, &c->hv, &c->hm, &c->ha, &c->hlog})
     release(*b);
   if (c->h_status) cudaFreeHost(c->h_status);
@@ -1324,7 +1342,9 @@ nbody_status adjoint_sweep(nbody_ctx* c, const double* x0, const double* v0, con
   // x_s and the same weights), x_0 (coef dt/2).
   AdjLaunch A{};
   A.chunks = c->d_vchunks;
-  A.n_chunks = (int32_t)c->chunks.size();
+  A.n_chunks = n_chunks(c, c->vwide);
+  A.chunk = chunk_size(c, c->vwide);
+  A.few_slots = c->vwide;
   A.part = static_cast<const double*>(c->part.p);
   A.n_total = c->n_total;
   A.G = c->cfg.G;
@@ -1342,12 +1362,12 @@ nbody_status adjoint_sweep(nbody_ctx* c, const double* x0, const double* v0, con
   A.g_params = g_params;
   A.eps = c->cfg.eps;
   A.cpart = static_cast<double*>(c->epart.p);
-  A.sys_chunk = c->d_sys_chunk;
+  A.sys_chunk = c->vwide ? c->d_csys_chunk : c->d_sys_chunk;
   A.n_sys = c->n_sys;
   A.done = c->counter + 6;
   A.part_rows = (int64_t)(c->part.bytes / (size_t)vjp_bytes);
   const Chunk* vch = c->d_vchunks;
-  const int nch = (int)c->chunks.size();
+  const int nch = A.n_chunks;
   for (int k = nseg - 1; k >= 0; --k) {
     const int s0 = k * K, s1 = std::min(T, s0 + K), len = s1 - s0;
     double* cp = ck + (size_t)k * 3 * n3;
@@ -1359,12 +1379,12 @@ nbody_status adjoint_sweep(nbody_ctx* c, const double* x0, const double* v0, con
     // VJP that segment has already taken, so only the last segment steps to its end
     const int top = (k == nseg - 1) ? s1 : s1 - 1;
     if ((s = run_steps(top - s0, X + n3))) return s;
-    NB_CUDA(c, launch_stage_vec(vch, nch, c->cfg.precision, X + (size_t)(top - s0) * n3, m,
+    NB_CUDA(c, launch_stage_vec(vch, nch, A.chunk, c->cfg.precision, X + (size_t)(top - s0) * n3, m,
                                 A.sys, c->stage.p, c->stage_lo.p, 1, c->n_total,
                                 c->n_sys, c->status, st));
     ++c->launches;
     if (k == nseg - 1) {
-      NB_CUDA(c, launch_stage_vec(vch, nch, c->cfg.precision, g_v0, m, A.sys, c->stage_w.p, nullptr, 0, c->n_total, c->n_sys, c->status, st));
+      NB_CUDA(c, launch_stage_vec(vch, nch, A.chunk, c->cfg.precision, g_v0, m, A.sys, c->stage_w.p, nullptr, 0, c->n_total, c->n_sys, c->status, st));
       ++c->launches;
     }
     for (int t = top; t >= s0; --t) {
@@ -1472,10 +1492,8 @@ nbody_status nbody_init(nbody_ctx** out, const nbody_config* cfg, int64_t n_syst
 
   c->j_block = cfg->precision == NBODY_MIXED ? 64 : 32;
   cut_chunks(*c, chunk_bodies(c->n_total), c->chunks, c->sys_chunk);
-  std::vector<Chunk> cchunks;
   std::vector<int32_t> csys_chunk;
-  cut_chunks(*c, kChunk, cchunks, csys_chunk);
-  c->n_cchunks = (int)cchunks.size();
+  cut_chunks(*c, kChunk, c->wchunks, csys_chunk);
 
   nbody_status s;
   auto bail = [&](nbody_status st) {
@@ -1488,6 +1506,11 @@ nbody_status nbody_init(nbody_ctx** out, const nbody_config* cfg, int64_t n_syst
   if ((s = ensure(c, c->stage, stage_bytes))) return bail(s);
   if (cfg->precision == NBODY_MIXED && (s = ensure(c, c->stage_lo, n * sizeof(float4)))) return bail(s);
   if ((s = ensure(c, c->sysp, (size_t)c->n_sys * sizeof(SysParam)))) return bail(s);
+  if (cfg->precision == NBODY_MIXED && c->n_sys > 4) {
+    if ((s = ensure(c, c->sys_done, (size_t)c->n_sys * sizeof(unsigned)))) return bail(s);
+    if (cudaMemset(c->sys_done.p, 0, (size_t)c->n_sys * sizeof(unsigned)) != cudaSuccess)
+      return bail(fail(c, NBODY_ECUDA, "memset failed"));
+  }
   // two sets of chunk partials: a step's energy record may be finished by the next step's k_post
   if ((s = ensure(c, c->epart, 2 * std::max<size_t>(1, c->chunks.size()) * kEnergyVals * sizeof(double)))) return bail(s);
   // [0..1] work counter, [2] status word, [4] energy ticket, [5] centre ticket, [6] adjoint-parameter ticket
@@ -1515,7 +1538,7 @@ nbody_status nbody_init(nbody_ctx** out, const nbody_config* cfg, int64_t n_syst
           cudaSuccess)
     return bail(fail(c, NBODY_ECUDA, "upload of layout tables failed"));
   void* d_cchunks = nullptr;
-  if ((s = upload(c, cchunks.data(), cchunks.size() * sizeof(Chunk), &d_cchunks))) return bail(s);
+  if ((s = upload(c, c->wchunks.data(), c->wchunks.size() * sizeof(Chunk), &d_cchunks))) return bail(s);
   c->d_cchunks = static_cast<Chunk*>(d_cchunks);
 
   const bool fixed_variant = cfg->precision == NBODY_FP64 || cfg->variant != 0 || cfg->law == NBODY_LAW_LJ;

@@ -235,6 +235,8 @@ enum PostMode : unsigned {
 struct PostLaunch {
   const Chunk* chunks;
   int32_t n_chunks;
+  int chunk;               // bodies of a chunk at most (compiled: 16, 32, 64, 128)
+  int few_slots;           // at most eight slots per body
   const double* part;      // [slices][N] of fpair4 (mixed) or double4_32a (FP64)
   int64_t n_total;
   double G, half_dt, dt;
@@ -272,8 +274,8 @@ cudaError_t launch_post(const PostLaunch& P, cudaStream_t st);
 // Staging parameters of every system (mixed path): the origin c is the
 // mass-weighted mean position (plain mean if the mass is 0), and for gravity the
 // scales are set from the extent, the softening and the largest mass. Per-chunk sums into cpart
-// [n_chunks][kEnergyVals], then per system in a fixed order by the last CTA
-// (ticket `done`, zero between launches).
+// [n_chunks][kEnergyVals], then per system in a fixed order by the last CTA (of all, or of
+// the system; tickets).
 struct CentreLaunch {
   const Chunk* chunks;
   int32_t n_chunks;
@@ -287,6 +289,7 @@ struct CentreLaunch {
   int law;
   double eps, near_eps;  // gravity: softening length, near-pair radius in softening lengths
   unsigned* done;
+  unsigned* sys_done;    // [n_sys] tickets of the systems (more than four; zero between launches)
   int64_t n_total;
   unsigned* status;
 };
@@ -295,6 +298,8 @@ cudaError_t launch_centre(const CentreLaunch& C, cudaStream_t st);
 struct AdjLaunch {
   const Chunk* chunks;
   int32_t n_chunks;
+  int chunk;               // as in PostLaunch
+  int few_slots;
   const double* part;      // 2 (3 with g_params) x fpair4 (mixed) or double4_32a (FP64) [slices][N]
   int64_t n_total;
   double G, coef, dt;      // lam_x += coef * gx ; g_m += coef * gm ; lam_v += dt lam_x
@@ -331,7 +336,7 @@ cudaError_t launch_copy4(const Copy4& C, int n_sms, cudaStream_t st);
 
 // stage w = lam (float4 / double4_32a) or positions x (as_position; with their
 // float32 remainders into stage_lo when given) for a VJP without an update
-cudaError_t launch_stage_vec(const Chunk* chunks, int n_chunks, int precision, const double* vec, const double* m,
+cudaError_t launch_stage_vec(const Chunk* chunks, int n_chunks, int chunk, int precision, const double* vec, const double* m,
                              const SysParam* sys, void* stage, void* stage_lo, int as_position, int64_t n_total,
                              int n_sys, unsigned* status, cudaStream_t st);
 

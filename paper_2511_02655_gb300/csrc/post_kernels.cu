@@ -19,6 +19,13 @@ namespace {
 template <int CB>
 constexpr unsigned kSumThreads = CB < 32 ? 32 : CB;
 
+// The parameters of a chunk's system into shared memory (a barrier follows). Used from global memory they would be
+// read again after each store that might be to them, a round trip to L2 each time.
+__device__ __forceinline__ void load_params(SysParam& s, const SysParam* sys, const Chunk& c) {
+  if (threadIdx.x < sizeof(SysParam) / 4 && c.begin < c.end)
+    reinterpret_cast<uint32_t*>(&s)[threadIdx.x] = reinterpret_cast<const uint32_t*>(sys + c.sys)[threadIdx.x];
+}
+
 // One CTA per chunk, SG threads per body to add the slices and one to do
 // the rest (a CTA of one thread per body when the mode combines nothing). Adding
 // the slices is a chain of 32-byte loads from L2, and that latency and the FP64 pipe
@@ -26,13 +33,17 @@ constexpr unsigned kSumThreads = CB < 32 ? 32 : CB;
 // with one thread per body and 128-body chunks and 84 us with four and 64; with
 // 32-body chunks, eight threads and the body's own loads ahead of the slices' it went
 // from 70.5 to 69.1 us (on top of a faster force pass); 1024 bodies: 13.7 to 12.2 us.
-// At 65 536 bodies eight threads cost 1% (1024-thread CTAs), so chunks of 128 keep four.
+// At 65 536 bodies eight threads cost 1% (1024-thread CTAs), so chunks of 128 keep four. After a one-sided
+// pass of at most eight slots per body (ensembles of small systems) chunks are of 128 at any size, and above
+// 32 768 bodies two threads share a body's slots: a step of 64 systems of 512 bodies 29.4 us in chunks of 64
+// with eight threads, 27.2 so; of 64 systems of 2048 152.7 us with four threads, 148.7 with two.
 template <int CB, int SG>
 __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
   __shared__ union {
     SlotSums<CB, SG> f[4];
     double d[4][SG - 1][CB];
   } red;
+  __shared__ SysParam sp;
   Chunk c{};  // (the chunk list is as old as the context: read while the kernel before finishes)
   if ((int)blockIdx.x < P.n_chunks) c = P.chunks[blockIdx.x];
   pdl_wait();  // the force kernel before it has finished writing the partials
@@ -46,7 +57,6 @@ __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
   }
   if (!chunk_ok(c, P.n_total, P.n_sys, (P.mode & kCombine) ? P.part_rows : 0, P.status))
     c.begin = c.end = 0;  // NBODY_DEBUG builds only: processed as an empty chunk
-  SysParam& sp = P.sys[c.sys];
   double e[kEnergyVals];
 #pragma unroll
   for (int k = 0; k < kEnergyVals; ++k) e[k] = 0.0;
@@ -54,17 +64,14 @@ __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
   const int b = (int)threadIdx.x % CB, g = (int)threadIdx.x / CB;
   const int i = c.begin + b;
   const bool live = i < c.end && g < SG;  // (a chunk of 16 has half a warp without bodies in a pass that combines nothing)
+  load_params(sp, P.sys, c);
+  if (!(mode & kCombine)) __syncthreads();  // (else add_groups has a barrier)
   BodyIn in;
   if (g == 0 && live) in = load_body(P, mode, i);
-  double m_all = 1.0;  // FP64 gravity: the mass that a system's bodies share is left out of the sums
-  if (P.precision == 0 && P.law == 0 && P.off && (mode & (kCombine | kMasses))) {
-    const double m0 = P.m[P.off[c.sys]];
-    if (mode & kMasses) {
-      if (g == 0 && live && __double_as_longlong(in.m) != __double_as_longlong(m0)) sp.uniform = P.epoch;
-    } else if (sp.uniform != P.epoch) {
-      m_all = m0;
-    }
-  }
+  const bool masses = P.precision == 0 && P.law == 0 && P.off;
+  const double m0 = masses && (mode & (kCombine | kMasses)) && c.begin < c.end ? P.m[P.off[c.sys]] : 1.0;
+  if (masses && (mode & kMasses) && g == 0 && live && __double_as_longlong(in.m) != __double_as_longlong(m0))
+    P.sys[c.sys].uniform = P.epoch;
 
   double sx = 0.0, sy = 0.0, sz = 0.0, sphi = 0.0;
   if ((mode & kCombine) && P.precision == 1) {
@@ -90,6 +97,8 @@ __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
       }
     }
     add_groups(red.d, g, b, s4);
+    // FP64 gravity: the mass that a system's bodies share is left out of the sums
+    const double m_all = masses && sp.uniform != P.epoch ? m0 : 1.0;
     sx = m_all * s4[0], sy = m_all * s4[1], sz = m_all * s4[2], sphi = m_all * s4[3];
   }
   if (g == 0 && live && post_body(P, mode, i, sp, in, sx, sy, sz, sphi, e)) atomicOr(P.status, kFlagNonFinite);
@@ -153,42 +162,29 @@ __global__ void __launch_bounds__(kChunk) k_centre(const CentreLaunch C) {
     for (int k = 0; k < 7; ++k) o[k] = v[k];
     o[7] = q.pack();
   }
-  if (!last_of(C.done, gridDim.x)) return;
+  // The last CTA adds up to four systems' chunks; of more, each system's own last CTA does: one CTA for all of
+  // them takes 3 us for every four systems (512 systems of 128 bodies: 466 us, 15 us this way; a step of a
+  // twenty-step call 52 and 22.5 us).
+  const bool own = C.n_sys > 4;
+  const int sy0 = own ? c.sys : 0, sy1 = own ? c.sys + 1 : C.n_sys;
+  if (own && c.begin >= c.end) return;  // NBODY_DEBUG builds only
+  if (!last_of(own ? C.sys_done + c.sys : C.done,
+               own ? (unsigned)(C.sys_chunk[sy1] - C.sys_chunk[sy0]) : gridDim.x))
+    return;
   __threadfence();
-  auto emit = [&](const int sy, const double (&w)[7], const Extent& e) {
-    const int64_t first = C.off[sy], n = C.off[sy + 1] - first;
-    staging_params(C.sys[sy], w, e, n, C.x + 3 * first, n > 0 ? C.m[first] : 0.0, C.law == 0, C.eps, C.near_eps);
-  };
-  auto extent = [&](const int sy, const int first, const int step) {
+  for (int sy = sy0; sy < sy1; ++sy) {
     Extent e{0u, 0u, 1u};
-    for (int k = C.sys_chunk[sy] + first; k < C.sys_chunk[sy + 1]; k += step)
+    for (int k = C.sys_chunk[sy] + (int)threadIdx.x; k < C.sys_chunk[sy + 1]; k += CB)
       e.join(Extent::unpack(__ldcg(C.cpart + (int64_t)k * kEnergyVals + 7)));
     e.warp_join();
-    return e;
-  };
-  // up to four systems are reduced by the whole CTA, more by a warp each (as systems_final)
-  if (C.n_sys <= 4) {
-    for (int sy = 0; sy < C.n_sys; ++sy) {
-      Extent e = extent(sy, (int)threadIdx.x, CB);
-      __syncthreads();
-      if (lane == 0) ext[wid] = e;
-      __syncthreads();
-      for (int w = 0; w < NW; ++w) e.join(ext[w]);
-      systems_final<7, CB>(C.sys_chunk + sy, 1, C.cpart, gridDim.x, C.status,
-                           [&](int, const double (&w)[7]) { emit(sy, w, e); });
-    }
-    return;
-  }
-  for (int sy = wid; sy < C.n_sys; sy += NW) {
-    double w[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int k = C.sys_chunk[sy] + lane; k < C.sys_chunk[sy + 1]; k += 32) {
-#pragma unroll
-      for (int q = 0; q < 7; ++q) w[q] += __ldcg(C.cpart + (int64_t)k * kEnergyVals + q);
-    }
-#pragma unroll
-    for (int q = 0; q < 7; ++q) w[q] = warp_sum(w[q]);
-    const Extent e = extent(sy, lane, 32);
-    if (lane == 0) emit(sy, w, e);
+    __syncthreads();
+    if (lane == 0) ext[wid] = e;
+    __syncthreads();
+    for (int w = 0; w < NW; ++w) e.join(ext[w]);
+    systems_final<7, CB>(C.sys_chunk + sy, 1, C.cpart, gridDim.x, C.status, [&](int, const double (&w)[7]) {
+      const int64_t first = C.off[sy], n = C.off[sy + 1] - first;
+      staging_params(C.sys[sy], w, e, n, C.x + 3 * first, n > 0 ? C.m[first] : 0.0, C.law == 0, C.eps, C.near_eps);
+    });
   }
 }
 
@@ -198,10 +194,11 @@ __global__ void __launch_bounds__(SG * CB) k_adj_update(const AdjLaunch A) {
     SlotSums<CB, SG> f[10];
     double d[10][SG - 1][CB];
   } red;
+  __shared__ SysParam sp;  // (as in k_post)
   Chunk c = A.chunks[blockIdx.x];
   pdl_wait();  // the VJP kernel has finished writing the partials
   if (!chunk_ok(c, A.n_total, A.n_sys, A.part_rows, A.status)) c.begin = c.end = 0;  // NBODY_DEBUG builds only
-  const SysParam& sp = A.sys[c.sys];
+  load_params(sp, A.sys, c);
   const int kw = A.g_params ? 3 : 2;  // partials (fpair4 / double4_32a) per body and slice
   double pv[2] = {0.0, 0.0};          // this thread's w.da/dG and sum m (d.w) / s^5
   const int b = (int)threadIdx.x % CB, g = (int)threadIdx.x / CB;
@@ -254,16 +251,14 @@ __global__ void __launch_bounds__(SG * CB) k_adj_update(const AdjLaunch A) {
     add_groups(red.d, g, b, S);
   }
   if (g == 0 && live) {
-    // the staged sums carry powers of the staging scales
-    const double q = sp.scale, q2 = q * q, q3 = q2 * q, q3m = q3 * sp.inv_mscale;
-    const double a1x = q3 * S[0], a1y = q3 * S[1], a1z = q3 * S[2], a2 = q3m * S[3];
-    const double gbx = q3m * S[4], gby = q3m * S[5], gbz = q3m * S[6], gm = q2 * S[7];
-    if (A.g_params) pv[0] = q2 * sp.inv_mscale * S[8], pv[1] = q2 * q2 * sp.inv_mscale * S[9];
-    const double mi = A.m[i];
+    // the staged sums carry powers of the staging scales, and all but A1 and Gm a staged mass
+    const double q = sp.scale, q2 = q * q, q2m = q2 * sp.inv_mscale, K = A.G * (q2m * q);
+    if (A.g_params) pv[0] = q2m * S[8], pv[1] = q2 * q2m * S[9];
+    const double mi = A.m[i], ms = mi * sp.mscale, gm = q2 * S[7];
     double w0 = A.lam_v[3 * i + 0], w1 = A.lam_v[3 * i + 1], w2 = A.lam_v[3 * i + 2];
-    const double gx0 = A.G * (mi * a1x - a2 * w0 - 3.0 * gbx);
-    const double gx1 = A.G * (mi * a1y - a2 * w1 - 3.0 * gby);
-    const double gx2 = A.G * (mi * a1z - a2 * w2 - 3.0 * gbz);
+    const double gx0 = K * (ms * S[0] - S[3] * w0 - 3.0 * S[4]);
+    const double gx1 = K * (ms * S[1] - S[3] * w1 - 3.0 * S[5]);
+    const double gx2 = K * (ms * S[2] - S[3] * w2 - 3.0 * S[6]);
     const double gmi = -A.G * gm;
     if (!(isfinite(gx0) && isfinite(gx1) && isfinite(gx2) && isfinite(gmi))) atomicOr(A.status, kFlagNonFinite);
     const double l0 = A.lam_x[3 * i + 0] + A.coef * gx0;
@@ -345,12 +340,12 @@ cudaError_t launch_copy4(const Copy4& C, int n_sms, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// f(bodies per chunk of a layout of n_total bodies, slot groups of k_post, of k_adj_update), as
-// integral constants (the latter has ten sums per body to pass through shared memory)
+// f(bodies per chunk, slot groups of k_post, of k_adj_update), as integral constants (the latter has
+// ten sums per body to pass through shared memory)
 template <typename F>
-static cudaError_t with_chunk(const int64_t n_total, F f) {
+static cudaError_t with_chunk(const int chunk, F f) {
   using std::integral_constant;
-  switch (chunk_bodies(n_total)) {
+  switch (chunk) {
     case 16: return f(integral_constant<int, 16>(), integral_constant<int, 16>(), integral_constant<int, 16>());
     case 32: return f(integral_constant<int, 32>(), integral_constant<int, 8>(), integral_constant<int, 8>());
     case 64: return f(integral_constant<int, 64>(), integral_constant<int, 8>(), integral_constant<int, 8>());
@@ -358,14 +353,23 @@ static cudaError_t with_chunk(const int64_t n_total, F f) {
   }
 }
 
+// Few slots per body and chunks enough to fill the SMs: two threads a body, of four (or eight) the others would
+// find no slot.
+static bool two_groups(const int few_slots, const int chunk, const int64_t n_total) {
+  return few_slots && chunk == kChunk && n_total > 256 * kChunk;
+}
+
 cudaError_t launch_post(const PostLaunch& P, cudaStream_t st) {
   if (P.n_chunks <= 0) return cudaSuccess;
-  return with_chunk(P.n_total, [&](auto cb, auto sg, auto) {
+  auto launch = [&](auto cb, auto sg, auto) {
     constexpr int CB = decltype(cb)::value, SG = decltype(sg)::value;
     // a pass that combines nothing needs one thread per body only
     return launch_pdl(k_post<CB, SG>, (unsigned)P.n_chunks + (P.eprev_out ? 1u : 0u),
                       (P.mode & kCombine) ? SG * CB : (int)kSumThreads<CB>, st, P);
-  });
+  };
+  if (two_groups(P.few_slots, P.chunk, P.n_total))
+    return launch(std::integral_constant<int, kChunk>(), std::integral_constant<int, 2>(), 0);
+  return with_chunk(P.chunk, launch);
 }
 
 cudaError_t launch_centre(const CentreLaunch& C, cudaStream_t st) {
@@ -375,17 +379,20 @@ cudaError_t launch_centre(const CentreLaunch& C, cudaStream_t st) {
 
 cudaError_t launch_adj_update(const AdjLaunch& A, cudaStream_t st) {
   if (A.n_chunks <= 0) return cudaSuccess;
-  return with_chunk(A.n_total, [&](auto cb, auto, auto sg) {
+  auto launch = [&](auto cb, auto, auto sg) {
     constexpr int CB = decltype(cb)::value, SG = decltype(sg)::value;
     return launch_pdl(k_adj_update<CB, SG>, A.n_chunks, SG * CB, st, A);
-  });
+  };
+  if (two_groups(A.few_slots, A.chunk, A.n_total))
+    return launch(std::integral_constant<int, kChunk>(), 0, std::integral_constant<int, 2>());
+  return with_chunk(A.chunk, launch);
 }
 
-cudaError_t launch_stage_vec(const Chunk* chunks, int n_chunks, int precision, const double* vec, const double* m,
+cudaError_t launch_stage_vec(const Chunk* chunks, int n_chunks, int chunk, int precision, const double* vec, const double* m,
                              const SysParam* sys, void* stage, void* stage_lo, int as_position, int64_t n_total,
                              int n_sys, unsigned* status, cudaStream_t st) {
   if (n_chunks <= 0) return cudaSuccess;
-  return with_chunk(n_total, [&](auto cb, auto, auto) {
+  return with_chunk(chunk, [&](auto cb, auto, auto) {
     constexpr int CB = decltype(cb)::value;
     return launch_pdl(k_stage_vec<CB>, n_chunks, (int)kSumThreads<CB>, st, chunks, precision, vec, m, sys, stage, stage_lo, as_position,
                       n_total, n_sys, status);

@@ -10,8 +10,9 @@ from test_gpu_sym import _masses
 
 pytestmark = pytest.mark.gpu
 
-# Mixed gradients of 9000 and more bodies with random weights: elements below 1e-2 of the rms are sums that
-# cancel to less than float32 keeps to 1e-4 (the one-sided kernels have 2e-4 and 3.3e-4 at a guard of 1e-3)
+# Mixed gradients of 9000 and more bodies with random weights, or of widely spread masses: elements below 1e-2
+# of the rms are sums that cancel to less than float32 keeps to 1e-4 (the one-sided kernels have 2e-4, 3.3e-4 and
+# 1.3e-4 at a guard of 1e-3)
 GUARD = 1e-2
 
 
@@ -167,3 +168,46 @@ def test_sym64_replays_do_not_depend_on_earlier_masses(nb, tmp_path, monkeypatch
         torch.cuda.synchronize()
         for got, want in zip(r, e):
             assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("sizes", [[0, 130, 1, 300, 64, 1100, 0, 513, 2, 129, 128], [127, 300] * 120, [64] * 300],
+                         ids=["uneven", "240", "64x300"])
+@pytest.mark.parametrize("tiling", [{}, dict(block=128, i_per_thread=1, j_tile=128, slice=32, variant=2)],
+                         ids=["tuned", "many-slots"])
+def test_many_small_systems(nb, tiling, sizes):
+    """Every system's origin and scales, forces, energies, virials and gradients, with few slots per body (wide
+    chunks, two threads a body above 32 768 of them) and with many; a second call gives the same bits."""
+    import torch
+    G, eps, dt = 1.1, 0.05, 1e-3
+    ens = inputs.ensemble(len(sizes), seed=4, sizes=np.array(sizes))
+    off = [int(o) for o in ens.offsets]
+    x, v, m = ens.x + 30.0 * np.repeat(np.arange(len(sizes)), sizes)[:, None], ens.v, ens.m.copy()
+    m[off[1]:off[2]] *= np.exp(np.random.default_rng(1).standard_normal(sizes[1]))
+    rng = np.random.default_rng(2)
+    lx, lv = rng.standard_normal(x.shape), 0.1 * rng.standard_normal(x.shape)
+    ctx = nb.nbody_init(G=G, eps=eps, dt=dt, offsets=off, **tiling)
+    xt, vt, mt, lxt, lvt = to_dev(x, v, m, lx, lv)
+
+    def results():
+        a, phi = nb.nbody_forces(ctx, xt, mt)
+        out = [a, phi, nb.nbody_energy(ctx, xt, vt, mt), nb.nbody_virial(ctx, xt, vt, mt)]
+        return out + list(nb.nbody_adjoint_params(ctx, xt, vt, mt, 1, 1, lxt, lvt))
+
+    first, second = results(), results()
+    nb.nbody_sync(ctx)
+    assert all(torch.equal(s, t) for s, t in zip(first, second))
+    a, phi, en, vir, gx, gv, gm, gp = (t.cpu().numpy() for t in first)
+    for s in list(range(11)) + [len(sizes) - 1]:
+        k = slice(off[s], off[s + 1])
+        if sizes[s] < 2:
+            assert not a[k].any()
+            continue
+        a_ref, phi_ref = oracle.forces(x[k], m[k], G=G, eps=eps)
+        assert force_rel_err(a[k], a_ref).max() <= 1e-4, s
+        assert_elem_close(phi[k], phi_ref, 3e-5, f"phi {s}")
+        np.testing.assert_allclose(en[s, 1:3], oracle.energy(x[k], v[k], m[k], G=G, eps=eps)[1:3], rtol=1e-6)
+        ox, ov, om, (oG, oe) = oracle.adjoint_params(x[k], v[k], m[k], G, eps, dt, 1, lx[k], lv[k])
+        for g, o, what in ((gx, ox, "g_x0"), (gv, ov, "g_v0"), (gm, om, "g_m")):
+            assert elem_rel_err(g[k], o, guard=GUARD).max() <= 1e-4, f"{what} {s}"
+        scale = max(abs(oG), abs(oe) * eps)
+        assert abs(gp[s, 0] - oG) <= 1e-4 * scale and abs(gp[s, 1] - oe) * eps <= 1e-4 * scale, s
