@@ -32,6 +32,7 @@ constexpr size_t kMaxPartialBytes = size_t(1) << 30;  // cap on per-slice partia
 constexpr int kMinTilesPerSlice = 1;  // shortest slice in j-tiles (small systems need many items)
 constexpr double kTuneLargePairs = 4.0e10;  // above this many pairs per force pass, tune on short slices
 constexpr int kTuneSlice = 8192;
+constexpr double kLongPass = 20.0e-3, kLongPassPairs = 1.0e8;  // seconds (autotune); looked at above so many unordered pairs
 constexpr int kSliceQuantum = 4;  // slice lengths are multiples of this many bodies
 constexpr int64_t kTailMin = 64;   // shortest slice of a halving tail
 
@@ -845,23 +846,25 @@ nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
   cudaEvent_t ev[4];
   for (auto& e : ev) NB_CUDA(c, cudaEventCreate(&e));
   auto timed = [&](const PairLaunch& P, bool combine, float* best_ms) -> cudaError_t {
-    cudaError_t err = launch(P);  // warm-up; also writes every partial the combine reads
-    if (err == cudaSuccess && combine) err = launch_post(C, c->stream);
-    *best_ms = 1e30f;
-    // best of 3 launches, or of as many as fill ~2 ms (at most 20) for short ones
-    int reps = 3;
-    for (int rep = 0; rep < reps && err == cudaSuccess; ++rep) {
+    // an untimed pass (which also writes every partial the combine reads), then the best of 3, or of as many
+    // as fill ~2 ms (at most 20) for short ones; of passes of half a millisecond or more two, of 2 ms or
+    // more one (these repeat to 0.2%)
+    cudaError_t err = cudaSuccess;
+    float ms = 0.f, best = 1e30f;
+    int reps = 1;
+    for (int rep = 0; rep <= reps && err == cudaSuccess; ++rep) {
       err = cudaEventRecord(ev[0], c->stream);
       if (err == cudaSuccess) err = launch(P);
       if (err == cudaSuccess && combine) err = launch_post(C, c->stream);
       if (err == cudaSuccess) err = cudaEventRecord(ev[1], c->stream);
       if (err == cudaSuccess) err = cudaEventSynchronize(ev[1]);
-      float ms = 0.f;
       if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, ev[0], ev[1]);
-      if (err == cudaSuccess) *best_ms = std::min(*best_ms, ms);
-      if (rep == 0 && err == cudaSuccess) reps = std::max(3, std::min(20, (int)std::ceil(2.0 / std::max(ms, 1e-3f))));
+      if (err != cudaSuccess) break;
+      c->launches += combine ? 2 : 1;
+      if (rep > 0) best = std::min(best, ms);
+      if (rep < 2) reps = ms >= 2.f ? 1 : ms >= 0.5f ? 2 : std::max(3, std::min(20, (int)std::ceil(2.0 / std::max(ms, 1e-3f))));
     }
-    c->launches += (reps + 1) * (combine ? 2 : 1);
+    *best_ms = best;
     return err;
   };
   PairLaunch P = L;
@@ -871,7 +874,7 @@ nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
   if (P.n_items < L.n_items) err = timed(P, false, &ms);
   if (err == cudaSuccess && (P.n_items == L.n_items || ms * (double)L.n_items / std::max(1, P.n_items) < 60.0)) {
     P = L;
-    err = timed(P, !vjp || sym, &ms);  // (a gradient's slots: the force combine reads half of each entry)
+    err = timed(P, true, &ms);  // (a gradient's slots: the force combine reads half of each entry)
   }
   for (auto& e : ev) cudaEventDestroy(e);
   if (err != cudaSuccess) return fail(c, NBODY_ECUDA, "autotune launch failed: %s", cudaGetErrorString(err));
@@ -997,7 +1000,7 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
   }
   // Work lists of the symmetric tilings: one item per CTA of a full grid (or a few), cut evenly or
   // with shorter pieces for the end of the schedule. They are timed with the refined slicings below.
-  std::vector<Tiling> sym_settings;
+  std::vector<Tiling> sym_settings, sym_long;  // (sym_long: the cuts that long passes choose from)
   size_t room = 0, device = 0;  // memory that a list's partial sums can have
   NB_CUDA(c, cudaMemGetInfo(&room, &device));
   room += c->part.bytes;
@@ -1014,6 +1017,9 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
       if (n_ctas <= 0) continue;
       for (const auto& tk : std::vector<std::pair<int, int>>{
                {2, 1}, {2, 2}, {2, 3}, {2, 4}, {2, 6}, {0, 1}, {0, 2}, {0, 4}, {0, 6}, {1, 2}, {1, 4}, {1, 6}}) {
+        // (a gradient of one system was as fast with even pieces as with any at every size looked at, and its
+        // first call waits for this)
+        if (vjp && c->n_sys == 1 && tk.first != 2 && tk != std::make_pair(1, 4)) continue;
         t.tail = tk.first;
         t.slice = sym_slice(*c, t, n_ctas, tk.second);
         // FP64 lists of few large items need an even placement on the SMs, which the timing here has
@@ -1023,8 +1029,10 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
         if (!sym_fits(c, rows, vjp) || (size_t)rows * (vjp ? 64 : 32) > room) continue;
         if (!mixed && p.first > 64 && sym_item_count(*c, t, t.slice, c->sm_count) < c->sm_count) continue;
         if (sym_settings.empty() || sym_settings.back().tail != t.tail || sym_settings.back().block != t.block ||
-            sym_settings.back().ipt != t.ipt || sym_settings.back().slice != t.slice)
+            sym_settings.back().ipt != t.ipt || sym_settings.back().slice != t.slice) {
           sym_settings.push_back(t);
+          if (t.tail == 2 && tk.second >= 4) sym_long.push_back(t);
+        }
       }
     }
     // (where no list has room, as in layouts of very many bodies, the one-sided pass remains)
@@ -1118,7 +1126,16 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
   // of each other, and the one the tail favours must not be cut by that noise.
   // Every setting is timed once and those within 3% of the best once more.
   if ((vjp || g.slice == 0) && !large) {
-    std::vector<Tiling> settings = sym_settings;
+    // Passes of 20 ms and more take four or six even rounds of items: of 32 768 bodies in FP64 (17 ms, and a
+    // gradient 34) these came within 1% of the best of all cuts, which a 65 536-body gradient would time for half a minute.
+    bool long_pass = false;
+    if (!sym_long.empty() && total_pairs(*c) > kLongPassPairs) {
+      if ((s = install_tiling(c, sym_long[0], vjp)) && !no_room(s)) return s;
+      double cost = 0;
+      if (!s && (s = time_tiling(c, vjp, &cost))) return s;
+      long_pass = cost * 2.0 * total_pairs(*c) >= kLongPass;
+    }
+    std::vector<Tiling> settings = long_pass ? sym_long : sym_settings;
     for (size_t f = 0; f < top; ++f) {
       Tiling base = timed[f].second;
       if (vjp) {
@@ -1154,7 +1171,7 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
       }
     }
     std::vector<double> lc(settings.size(), 1e300);
-    for (int round = 0; round < 2 && !settings.empty(); ++round) {
+    for (int round = 0; round < (long_pass ? 1 : 2) && !settings.empty(); ++round) {
       const double limit = round == 0 ? 1e300 : 1.03 * *std::min_element(lc.begin(), lc.end());
       for (size_t k = 0; k < settings.size(); ++k) {
         if (round == 1 && lc[k] > limit) continue;
