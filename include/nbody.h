@@ -228,8 +228,9 @@ nbody_status nbody_sync(nbody_ctx* ctx);
  * kernel variant (as in nbody_config.variant: 1 scalar, 2 packed, 3 packed capped). Any pointer
  * may be NULL. The values can be handed back to nbody_init. Where the tuner chose the
  * symmetric pass (every unordered pair evaluated once; both precisions), which cannot
- * be requested, the nearest one-sided tiling and the longest piece's j-bodies as slice are
- * reported; nbody_get_slicing tells the two apart.
+ * be requested, the one-sided tiling that serves the layout is reported: a context that
+ * is given it runs slower, as one-sided passes are, and agrees to rounding;
+ * nbody_get_slicing tells the two apart, NBODY_TUNE_CACHE repeats the choice itself.
  */
 nbody_status nbody_get_tuning(const nbody_ctx* ctx, int32_t* block, int32_t* i_per_thread, int32_t* j_tile,
                               int32_t* slice, int32_t* n_ctas, int32_t* variant);
