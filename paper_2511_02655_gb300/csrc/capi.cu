@@ -1218,15 +1218,15 @@ Tiling one_sided(const nbody_ctx* c) {
   const int slice = auto_slice(c, t, t.n_ctas);
   t.slice = mixed ? std::max(256, slice / 2) : std::max(kSliceQuantum, std::min(slice, c->sym_longest));
   if (mixed && c->n_sys == 1 && largest > 16384) {
-    // whole waves of equal items instead, where a few of them have such (20 000 bodies: 208 us a step, 200 so)
+    // the number of equal slices, five to nine waves of the grid, that fills its last wave best
     const int64_t itile = (int64_t)t.block * t.ipt, tiles = (largest + itile - 1) / itile;
-    for (int64_t waves = 2; waves <= 9; ++waves) {
+    double best = 0.97;
+    for (int64_t waves = 5; waves <= 9; ++waves) {
       const int64_t ns = waves * t.n_ctas / tiles;
-      if (ns < 1 || (double)(tiles * ns) < 0.98 * (double)(waves * t.n_ctas)) continue;
-      const int64_t len = ((largest + ns - 1) / ns + kSliceQuantum - 1) / kSliceQuantum * kSliceQuantum;
-      if (len > 2 * (int64_t)slice) continue;
-      t.slice = (int)len;
-      break;
+      const double fill = (double)(tiles * ns) / (double)(waves * t.n_ctas);
+      if (ns < 1 || fill <= best) continue;
+      best = fill;
+      t.slice = (int)(((largest + ns - 1) / ns + kSliceQuantum - 1) / kSliceQuantum * kSliceQuantum);
     }
   }
   return t;
