@@ -32,7 +32,8 @@ constexpr size_t kMaxPartialBytes = size_t(1) << 30;  // cap on per-slice partia
 constexpr int kMinTilesPerSlice = 1;  // shortest slice in j-tiles (small systems need many items)
 constexpr double kTuneLargePairs = 4.0e10;  // above this many pairs per force pass, tune on short slices
 constexpr int kTuneSlice = 8192;
-constexpr double kLongPass = 20.0e-3, kLongPassPairs = 1.0e8;  // seconds (autotune); looked at above so many unordered pairs
+constexpr double kLongPass = 20.0e-3;      // seconds from which a symmetric pass chooses from fewer lists ...
+constexpr double kLongPassPairs = 1.0e8;  // ... asked above so many unordered pairs
 constexpr int kSliceQuantum = 4;  // slice lengths are multiples of this many bodies
 constexpr int64_t kTailMin = 64;   // shortest slice of a halving tail
 
@@ -794,7 +795,10 @@ nbody_status fill_synthetic(nbody_ctx* c, bool with_w) {
       const double X = pos[3 * i] * c->stage_scale, Y = pos[3 * i + 1] * c->stage_scale,
                    Z = pos[3 * i + 2] * c->stage_scale;
       const float hx = (float)X, hy = (float)Y, hz = (float)Z;
-      h[i] = make_float4(hx, hy, hz, c->cfg.law == NBODY_LAW_GRAVITY ? 1.f : (float)mass[i]);  // as SysParam::uniform says
+      // equal masses, staged as 1 (SysParam::uniform): with the masses kept in the sums instead the choice is 4%
+      // worse at 20 000 and 131 072 bodies of equal masses, and for unequal ones 5% better at 8000 bodies, 2%
+      // worse at 20 000 and within 1% elsewhere
+      h[i] = make_float4(hx, hy, hz, c->cfg.law == NBODY_LAW_GRAVITY ? 1.f : (float)mass[i]);
       hl[i] = make_float4((float)(X - hx), (float)(Y - hy), (float)(Z - hz), 0.f);
     }
     NB_CUDA(c, cudaMemcpy(c->stage.p, h.data(), n * sizeof(float4), cudaMemcpyHostToDevice));
@@ -847,8 +851,8 @@ nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
   for (auto& e : ev) NB_CUDA(c, cudaEventCreate(&e));
   auto timed = [&](const PairLaunch& P, bool combine, float* best_ms) -> cudaError_t {
     // an untimed pass (which also writes every partial the combine reads), then the best of 3, or of as many
-    // as fill ~2 ms (at most 20) for short ones; of passes of half a millisecond or more two, of 2 ms or
-    // more one (these repeat to 0.2%)
+    // as fill ~2 ms (at most 20) for short ones (a gradient's 1 ms: its first call waits); of passes of half a
+    // millisecond or more two, of 2 ms or more one (these repeat to 0.2%)
     cudaError_t err = cudaSuccess;
     float ms = 0.f, best = 1e30f;
     int reps = 1;
@@ -862,7 +866,8 @@ nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
       if (err != cudaSuccess) break;
       c->launches += combine ? 2 : 1;
       if (rep > 0) best = std::min(best, ms);
-      if (rep < 2) reps = ms >= 2.f ? 1 : ms >= 0.5f ? 2 : std::max(3, std::min(20, (int)std::ceil(2.0 / std::max(ms, 1e-3f))));
+      const int fill = (int)std::ceil((vjp ? 1.0 : 2.0) / std::max(ms, 1e-3f));
+      if (rep < 2) reps = ms >= 2.f ? 1 : ms >= 0.5f ? 2 : std::max(3, std::min(20, fill));
     }
     *best_ms = best;
     return err;
@@ -987,7 +992,9 @@ nbody_status autotune(nbody_ctx* c, bool vjp) {
   const bool any_tiling = !g.variant && (vjp || (!g.block && !g.i_per_thread && !g.j_tile && !g.slice));
   const bool mixed = g.precision == NBODY_MIXED;
   const bool sym = any_tiling && typical >= (mixed ? kSymMinBodies : kSymMinBodies64);
-  const bool sym_only = sym && typical >= (mixed ? kSymOnlyBodies : kSymOnlyBodies64);
+  // (mixed gradients: 8% ahead at 3001 bodies, 15% at 6500)
+  const double only = !mixed ? kSymOnlyBodies64 : vjp && !large ? kSymMinBodies : kSymOnlyBodies;
+  const bool sym_only = sym && typical >= only;
   if (sym_only && large) {
     // nothing to choose between: its cost per pair no longer depends on the tiling
     Tiling t;
@@ -1433,7 +1440,8 @@ nbody_status adjoint_sweep(nbody_ctx* c, const double* x0, const double* v0, con
                                 c->n_sys, c->status, st));
     ++c->launches;
     if (k == nseg - 1) {
-      NB_CUDA(c, launch_stage_vec(vch, nch, A.chunk, c->cfg.precision, g_v0, m, A.sys, c->stage_w.p, nullptr, 0, c->n_total, c->n_sys, c->status, st));
+      NB_CUDA(c, launch_stage_vec(vch, nch, A.chunk, c->cfg.precision, g_v0, m, A.sys, c->stage_w.p, nullptr, 0,
+                                  c->n_total, c->n_sys, c->status, st));
       ++c->launches;
     }
     for (int t = top; t >= s0; --t) {
