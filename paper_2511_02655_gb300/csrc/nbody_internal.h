@@ -336,8 +336,8 @@ cudaError_t launch_copy4(const Copy4& C, int n_sms, cudaStream_t st);
 
 // stage w = lam (float4 / double4_32a) or positions x (as_position; with their
 // float32 remainders into stage_lo when given) for a VJP without an update
-cudaError_t launch_stage_vec(const Chunk* chunks, int n_chunks, int chunk, int precision, const double* vec, const double* m,
-                             const SysParam* sys, void* stage, void* stage_lo, int as_position, int64_t n_total,
+cudaError_t launch_stage_vec(const Chunk* chunks, int n_chunks, int chunk, int precision, const double* vec,
+                             const double* m, const SysParam* sys, void* stage, void* stage_lo, int as_position, int64_t n_total,
                              int n_sys, unsigned* status, cudaStream_t st);
 
 }  // namespace nbody

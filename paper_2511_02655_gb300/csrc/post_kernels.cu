@@ -32,7 +32,8 @@ __device__ __forceinline__ void load_params(SysParam& s, const SysParam* sys, co
 // bound the kernel: on the 10 000-body Lennard-Jones gas (40 slices) a step took 89 us
 // with one thread per body and 128-body chunks and 84 us with four and 64; with
 // 32-body chunks, eight threads and the body's own loads ahead of the slices' it went
-// from 70.5 to 69.1 us (on top of a faster force pass); 1024 bodies: 13.7 to 12.2 us.
+// from 70.5 to 69.1 us (on top of a faster force pass); 1024 bodies: 13.7 to 12.2 us, and 11.7 with the chunk
+// read ahead of the wait.
 // At 65 536 bodies eight threads cost 1% (1024-thread CTAs), so chunks of 128 keep four. After a one-sided
 // pass of at most eight slots per body (ensembles of small systems) chunks are of 128 at any size, and above
 // 32 768 bodies two threads share a body's slots: a step of 64 systems of 512 bodies 29.4 us in chunks of 64
@@ -63,7 +64,8 @@ __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
   const unsigned mode = P.mode;
   const int b = (int)threadIdx.x % CB, g = (int)threadIdx.x / CB;
   const int i = c.begin + b;
-  const bool live = i < c.end && g < SG;  // (a chunk of 16 has half a warp without bodies in a pass that combines nothing)
+  // (a chunk of 16 has half a warp without bodies in a pass that combines nothing)
+  const bool live = i < c.end && g < SG;
   load_params(sp, P.sys, c);
   if (!(mode & kCombine)) __syncthreads();  // (else add_groups has a barrier)
   BodyIn in;
@@ -388,14 +390,14 @@ cudaError_t launch_adj_update(const AdjLaunch& A, cudaStream_t st) {
   return with_chunk(A.chunk, launch);
 }
 
-cudaError_t launch_stage_vec(const Chunk* chunks, int n_chunks, int chunk, int precision, const double* vec, const double* m,
-                             const SysParam* sys, void* stage, void* stage_lo, int as_position, int64_t n_total,
+cudaError_t launch_stage_vec(const Chunk* chunks, int n_chunks, int chunk, int precision, const double* vec,
+                             const double* m, const SysParam* sys, void* stage, void* stage_lo, int as_position, int64_t n_total,
                              int n_sys, unsigned* status, cudaStream_t st) {
   if (n_chunks <= 0) return cudaSuccess;
   return with_chunk(chunk, [&](auto cb, auto, auto) {
     constexpr int CB = decltype(cb)::value;
-    return launch_pdl(k_stage_vec<CB>, n_chunks, (int)kSumThreads<CB>, st, chunks, precision, vec, m, sys, stage, stage_lo, as_position,
-                      n_total, n_sys, status);
+    return launch_pdl(k_stage_vec<CB>, n_chunks, (int)kSumThreads<CB>, st, chunks, precision, vec, m, sys, stage,
+                      stage_lo, as_position, n_total, n_sys, status);
   });
 }
 

@@ -140,9 +140,9 @@ struct Smem {
 // integer operations, and small systems have few warps per scheduler to hide it.
 constexpr int kUnroll = 4;
 
-// The 32 steps of one block, or the 32 / KS from k0 on of a warp that shares it with KS - 1 others. FAST: returns whether the lane met an s^2 out of range, in which case
-// the sums are void and the block is to be repeated without FAST (there is no branch per pair, so
-// that the pairs of several steps overlap).
+// The 32 steps of one block, or the 32 / KS from k0 on of a warp that shares it with KS - 1 others. FAST:
+// returns whether the lane met an s^2 out of range, in which case the sums are void and the block is to be
+// repeated without FAST (there is no branch per pair, so that the pairs of several steps overlap).
 template <int LAW, bool SYM, bool MASK, int PHI, bool EQ, bool FAST, int R, int KS>
 __device__ __forceinline__ bool block32(const double (&q)[4][kTile / 32][64], const int b, const int k0, const int jg0,
                                         const int lane,
@@ -198,12 +198,12 @@ __device__ __forceinline__ void block(const double (&q)[4][kTile / 32][64], cons
   double bx[R], by[R], bz[R], bp[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) bx[r] = ax[r], by[r] = ay[r], bz[r] = az[r], bp[r] = pp[r];
-  const bool out = block32<LAW, SYM, MASK, PHI, EQ, true, R, KS>(q, b, k0, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, bx, by, bz, bp,
-                                                         jx, jy, jz, jp);
+  const bool out = block32<LAW, SYM, MASK, PHI, EQ, true, R, KS>(q, b, k0, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2,
+                                                                 bx, by, bz, bp, jx, jy, jz, jp);
   if (__any_sync(0xffffffffu, out)) {
     jx = jy = jz = jp = 0.0;
-    block32<LAW, SYM, MASK, PHI, EQ, false, R, KS>(q, b, k0, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp, jx, jy, jz,
-                                           jp);
+    block32<LAW, SYM, MASK, PHI, EQ, false, R, KS>(q, b, k0, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp,
+                                                   jx, jy, jz, jp);
   } else {
 #pragma unroll
     for (int r = 0; r < R; ++r) ax[r] = bx[r], ay[r] = by[r], az[r] = bz[r], pp[r] = bp[r];
@@ -256,7 +256,8 @@ __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Sme
           const double4_32a v = jt + t < it.j_end ? st[jt + t] : make_double4_32a(pad, pad, pad, 0.0);
           double* d = &sm.q[0][t >> 5][t & 31];
           constexpr int S = (kTile / 32) * 64;
-          d[0] = d[32] = v.x, d[S] = d[S + 32] = v.y, d[2 * S] = d[2 * S + 32] = v.z, d[3 * S] = d[3 * S + 32] = uniform && jt + t < it.j_end ? 1.0 : v.w;
+          d[0] = d[32] = v.x, d[S] = d[S + 32] = v.y, d[2 * S] = d[2 * S + 32] = v.z;
+          d[3 * S] = d[3 * S + 32] = uniform && jt + t < it.j_end ? 1.0 : v.w;
         }
         __syncthreads();
         for (int b = 0; b < kTile / 32; ++b) {
@@ -267,11 +268,11 @@ __device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Sme
             auto run = [&](auto eq) {
               constexpr bool EQ = decltype(eq)::value;
               if (both)
-                block<LAW, true, false, PHI, EQ, R, KS>(sm.q, b, k0, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp,
-                                                    jx, jy, jz, jp);
+                block<LAW, true, false, PHI, EQ, R, KS>(sm.q, b, k0, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay,
+                                                        az, pp, jx, jy, jz, jp);
               else if (jg0 + 32 > wi0)
-                block<LAW, false, true, PHI, EQ, R, KS>(sm.q, b, k0, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay, az, pp,
-                                                    jx, jy, jz, jp);
+                block<LAW, false, true, PHI, EQ, R, KS>(sm.q, b, k0, jg0, lane, ig0, xi, yi, zi, mi, eps2, s2, ax, ay,
+                                                        az, pp, jx, jy, jz, jp);
             };
             if (LAW == 0 && uniform && jg0 + 32 <= it.j_end && wi0 + 32 * R <= it.i_end)
               run(std::integral_constant<bool, LAW == 0>());

@@ -30,7 +30,8 @@ __global__ void __launch_bounds__(W * 32, MINB) k_force_sym(const SymLaunch L) {
 // With 4 warps to a block of the work 24 warps per SM are resident at most (short lists): left to
 // itself the compiler keeps to 64 registers and spills.
 template <int LAW, int W, int R, int PHI, int KS>
-__global__ void __launch_bounds__(W * KS * 32, KS < 4 ? 0 : std::max(1, 24 / (W * KS))) k_force_sym64(const SymLaunch L) {
+__global__ void __launch_bounds__(W * KS * 32, KS < 4 ? 0 : std::max(1, 24 / (W * KS)))
+    k_force_sym64(const SymLaunch L) {
   __shared__ sym64::Smem<W * KS> sm;
   pdl_wait();
   sym64::items<LAW, W, R, PHI, KS>(L, L.counter, sm);

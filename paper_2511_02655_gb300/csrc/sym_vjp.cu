@@ -41,7 +41,8 @@ int occupancy_of(K kern, int block, size_t smem) {
 
 }  // namespace
 
-// Compiled: warps, i-bodies per lane, resident CTAs (mixed); warps and warps to a block of the work (FP64, SymLaunch::split)
+// Compiled: warps, i-bodies per lane, resident CTAs (mixed); warps and warps to a block of the work (FP64,
+// SymLaunch::split)
 #define NBODY_SYM_VJP_TILINGS(X) X(4, 1, 5) X(4, 2, 3) X(8, 2, 1)
 #define NBODY_SYM_VJP64_TILINGS(X) X(2, 1) X(2, 2) X(2, 4) X(4, 1) X(4, 2) X(4, 4) X(8, 1)
 

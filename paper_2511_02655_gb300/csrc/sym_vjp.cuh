@@ -8,7 +8,7 @@
 // Seen from the other end d changes its sign and the weights change places, so the
 // bracket of Gb stays and the pair feeds both bodies from one set of powers and dot
 // products: 34 float32 operations and one MUFU.RSQ for two interactions instead of
-// 52 and two (FP64: 37 instead of about 86). Bound: the FP32 (FP64) pipe.
+// 52 and two (FP64: 36 instead of about 86). Bound: the FP32 (FP64) pipe.
 #pragma once
 
 #include "nbody_internal.h"
@@ -347,8 +347,8 @@ struct Body64 {
 };
 
 template <bool SYM, bool MASK, bool P, bool FAST, int KS>
-__device__ __forceinline__ bool block32(const double (&q)[7][kSymTile64 / 32][64], const int b, const int k0, const int jg0,
-                                        const int lane, const int ig, const Body64& B, const double eps2,
+__device__ __forceinline__ bool block32(const double (&q)[7][kSymTile64 / 32][64], const int b, const int k0,
+                                        const int jg0, const int lane, const int ig, const Body64& B, const double eps2,
                                         double (&si)[P ? 10 : 8], double (&sj)[P ? 10 : 8]) {
   constexpr int NC = P ? 10 : 8;
   const int src = (lane + 1) & 31;

@@ -14,7 +14,8 @@ DRIVER = r"""
 using namespace nbody;
 // out: bodies that read a slot written not exactly once, slots written and never read, bodies whose
 // pairs are not met exactly once, work items
-extern "C" int check(const int64_t* sizes, int n_sys, int j_block, int block, int ipt, int slice, int tail, int64_t* out) {
+extern "C" int check(const int64_t* sizes, int n_sys, int j_block, int block, int ipt, int slice, int tail,
+                     int64_t* out) {
   SymLayout c;
   c.n_sys = n_sys, c.j_block = j_block;
   c.offsets.push_back(0);
@@ -36,8 +37,10 @@ extern "C" int check(const int64_t* sizes, int n_sys, int j_block, int block, in
     for (int64_t i = w.i_begin; i < w.i_end; ++i) written[(size_t)(w.row0 + (int64_t)w.slot_i * w.stride + i)]++;
     for (int64_t j = w.j_begin; j < w.j_end; ++j) written[(size_t)(w.row0 + (int64_t)w.slot_j * w.stride + j)]++;
     // partners met as an i-body: the piece's later bodies; as a j-body: the row's earlier bodies
-    for (int64_t i = w.i_begin; i < w.i_end; ++i) met[(size_t)i] += std::max<int64_t>(0, w.j_end - std::max<int64_t>(w.j_begin, i + 1));
-    for (int64_t j = w.j_begin; j < w.j_end; ++j) met[(size_t)j] += std::max<int64_t>(0, std::min<int64_t>(w.i_end, j) - w.i_begin);
+    for (int64_t i = w.i_begin; i < w.i_end; ++i)
+      met[(size_t)i] += std::max<int64_t>(0, w.j_end - std::max<int64_t>(w.j_begin, i + 1));
+    for (int64_t j = w.j_begin; j < w.j_end; ++j)
+      met[(size_t)j] += std::max<int64_t>(0, std::min<int64_t>(w.i_end, j) - w.i_begin);
   }
   for (int k = 0; k < 4; ++k) out[k] = 0;
   for (const Chunk& k : chunks)
