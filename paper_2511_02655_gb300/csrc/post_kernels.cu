@@ -190,8 +190,9 @@ __global__ void __launch_bounds__(kChunk) k_centre(const CentreLaunch C) {
   }
 }
 
+// (64 registers: 1024 threads per SM, so that the 512 CTAs of 16 384 bodies run at once)
 template <int CB, int SG>
-__global__ void __launch_bounds__(SG * CB) k_adj_update(const AdjLaunch A) {
+__global__ void __launch_bounds__(SG * CB, 1024 / (SG * CB)) k_adj_update(const AdjLaunch A) {
   __shared__ union {
     SlotSums<CB, SG> f[10];
     double d[10][SG - 1][CB];
