@@ -83,6 +83,7 @@ __host__ __device__ inline Scratch scratch_of(unsigned char* p, const int n) {
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 void* g_scratch_addr[kMaxDevices] = {};
+int g_sm_count[kMaxDevices] = {};  // set with the address
 
 nbody_status fail(nbody_status s, const char* fmt, ...) {
   char buf[512];
@@ -300,7 +301,7 @@ cudaError_t launch_na_sym(const SymPlan& P, bool phi, unsigned char* sp, cudaStr
 }
 
 cudaError_t enqueue(const double* x, const double* m, const int n, const double G, const double eps, double* a,
-                    double* phi, unsigned char* sp, cudaStream_t st) {
+                    double* phi, unsigned char* sp, const int n_sms, cudaStream_t st) {
   cudaError_t e;
   const int n_sums = std::min(kSumCtas, (n + kSumThreads - 1) / kSumThreads);
   if ((e = launch_pdl(k_na_sums, n_sums, kSumThreads, st, x, m, n, sp))) return e;
@@ -311,7 +312,7 @@ cudaError_t enqueue(const double* x, const double* m, const int n, const double 
   if (n <= kMaxSymBodies) {
     // short i-tiles for small systems: their few tiles would leave SMs idle
     const int R = n <= 2048 ? 1 : n <= 8192 ? 2 : 4;
-    plan_sym(n, 128 * R, 152 * (R == 4 ? 4 : 6), std::min(room, kMaxSymSlots), P);
+    plan_sym(n, 128 * R, n_sms * (R == 4 ? 4 : 6), std::min(room, kMaxSymSlots), P);
     e = R == 1   ? launch_na_sym<1>(P, phi != nullptr, sp, st)
         : R == 2 ? launch_na_sym<2>(P, phi != nullptr, sp, st)
                  : launch_na_sym<4>(P, phi != nullptr, sp, st);
@@ -319,7 +320,7 @@ cudaError_t enqueue(const double* x, const double* m, const int n, const double 
     P = SymPlan{};
     // about eight items per resident CTA (3 per SM)
     const int tiles = (n + 255) / 256;
-    slices = std::max(1, std::min(room, (8 * 456 + tiles - 1) / tiles));
+    slices = std::max(1, std::min(room, (8 * 3 * n_sms + tiles - 1) / tiles));
     const int len = std::max(4, 4 * (int)(((int64_t)n + 4 * slices - 1) / (4 * slices)));
     slices = (n + len - 1) / len;
     const unsigned grid = (unsigned)tiles * (unsigned)slices;
@@ -370,12 +371,14 @@ extern "C" nbody_status nbody_forces_noalloc(const double* x, const double* m, i
       (s = check_dev_ptr(a, n3b, dev, "a", false)) || (s = check_dev_ptr(phi, n1b, dev, "phi", true)))
     return s;
   void* scratch = nullptr;
+  int n_sms = 0;
   {
     std::lock_guard<std::mutex> lk(g_mu);
     if (!g_scratch_addr[dev]) {
       void* p = nullptr;
       cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
       if (e == cudaSuccess) e = load_kernels();
+      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_sm_count[dev], cudaDevAttrMultiProcessorCount, dev);
       if (e != cudaSuccess || !p) {
         cudaGetLastError();
         return fail(NBODY_ECUDA, "nbody_forces_noalloc: loading the device code failed on device %d: %s", dev,
@@ -384,9 +387,10 @@ extern "C" nbody_status nbody_forces_noalloc(const double* x, const double* m, i
       g_scratch_addr[dev] = p;
     }
     scratch = g_scratch_addr[dev];
+    n_sms = g_sm_count[dev];
   }
   const cudaError_t e = enqueue(x, m, (int)n, G, eps, a, phi, static_cast<unsigned char*>(scratch),
-                                static_cast<cudaStream_t>(cuda_stream));
+                                n_sms, static_cast<cudaStream_t>(cuda_stream));
   if (e != cudaSuccess) return fail(NBODY_ECUDA, "nbody_forces_noalloc: launch failed: %s", cudaGetErrorString(e));
   return NBODY_OK;
 }
