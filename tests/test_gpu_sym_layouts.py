@@ -6,7 +6,7 @@ import pytest
 import oracle
 from paper_2511_02655_gb300 import inputs
 from helpers import assert_elem_close, elem_rel_err, force_rel_err, to_dev
-from test_gpu_sym import _masses
+from test_gpu_sym import _forced, _masses
 
 pytestmark = pytest.mark.gpu
 
@@ -211,3 +211,37 @@ def test_many_small_systems(nb, tiling, sizes):
             assert elem_rel_err(g[k], o, guard=GUARD).max() <= 1e-4, f"{what} {s}"
         scale = max(abs(oG), abs(oe) * eps)
         assert abs(gp[s, 0] - oG) <= 1e-4 * scale and abs(gp[s, 1] - oe) * eps <= 1e-4 * scale, s
+
+
+def test_sym64_pair_force_to_a_few_ulp(nb, tmp_path, monkeypatch):
+    """Two-body systems at separations over eight decades against 50-digit arithmetic. With u = 2^-53: s^2 has three
+    roundings, 4.5 u in s^-3, whose own steps are good to 1.5 ulp = 3 u; two products one each: 9.5 u in all,
+    and for the potential 6.5 u."""
+    from decimal import Decimal, getcontext
+    monkeypatch.setenv("NBODY_TUNE_CACHE", str(tmp_path / "tune"))
+    getcontext().prec = 50
+    systems = 500
+    rng = np.random.default_rng(3)
+    d = rng.standard_normal((systems, 3)) * 10.0 ** rng.uniform(-4, 4, (systems, 1))
+    x = np.zeros((2 * systems, 3))
+    x[1::2] = d
+    m = rng.uniform(0.5, 2.0, 2 * systems)
+    # (a third system size keeps the typical size above that of the symmetric pass)
+    big, _, big_m = inputs.plummer(200, seed=1)
+    off = list(range(0, 2 * systems + 1, 2)) + [2 * systems + 200]
+    ctx = _forced(nb, tmp_path / "tune", {"force": (64, 1, 64, 32, 3, 0)}, G=1.0, eps=0.0, dt=1e-3, offsets=off,
+                  precision=nb.FP64)
+    assert nb.nbody_get_slicing(ctx)["tail"] >= 2
+    a, phi = nb.nbody_forces(ctx, *to_dev(np.concatenate([x, big]), np.concatenate([m, _masses(big_m, "lognormal", 1)])))
+    nb.nbody_sync(ctx)
+    a, phi, u = a.cpu().numpy(), phi.cpu().numpy(), 2.0 ** -53
+    for k in range(systems):
+        q = [Decimal(float(v)) for v in d[k]]
+        r2 = sum(v * v for v in q)
+        for i, sign in ((0, 1), (1, -1)):
+            mj = Decimal(float(m[2 * k + 1 - i]))
+            for c in range(3):
+                want = sign * mj * q[c] / (r2 * r2.sqrt())
+                assert abs(Decimal(float(a[2 * k + i, c])) - want) <= abs(want) * Decimal(10 * u)
+            want = -mj / r2.sqrt()
+            assert abs(Decimal(float(phi[2 * k + i])) - want) <= abs(want) * Decimal(7 * u)
