@@ -53,7 +53,7 @@ namespace {
 using namespace nbody;
 
 constexpr int64_t kMaxBodies = NBODY_NOALLOC_MAX_BODIES;
-constexpr int kSumCtas = 64;  // CTAs of the staging origin's sums
+constexpr int kSumCtas = 96;  // CTAs of the staging origin's sums
 constexpr int kSumThreads = 256;
 constexpr size_t kHeaderBytes = 8192;
 constexpr size_t kSumsOffset = 256;  // header: SysParam, then the sums [kSumCtas][kEnergyVals]
