@@ -123,7 +123,7 @@ struct nbody_ctx : SymLayout {
   cudaStream_t cap_stream = nullptr;  // private stream used only to capture graphs
   std::string err = "no error";
   int64_t launches = 0;
-  uint32_t epoch = 0;  // number of the current call (SysParam::uniform), 0 before the first
+  bool new_number = false;  // FP64: the next force pass is a call's first (SymLaunch::call)
 
   // layout
   Chunk* d_chunks = nullptr;
@@ -507,7 +507,8 @@ SymLaunch sym_launch(nbody_ctx* c, bool vjp, Potential phi) {
   const int64_t warps = (int64_t)L.n_items * (t.block / 32), room = 16 * (int64_t)c->sm_count;
   L.split = 4 * warps <= room ? 4 : 2 * warps <= room ? 2 : 1;
   L.phi = (int)phi;
-  L.epoch = c->epoch;
+  L.call = c->counter + 7;
+  L.first = !vjp && c->new_number;
   L.status = c->status;
   return L;
 }
@@ -575,6 +576,7 @@ nbody_status run_pair(nbody_ctx* c, cudaStream_t st, bool vjp, Potential phi) {
     if (e0 && e1) NB_CUDA(c, cudaEventRecord(e0, st));
   }
   NB_CUDA(c, launch_pairs(c, vjp, phi, st));
+  if (!vjp) c->new_number = false;
   if (e0 && e1) {
     NB_CUDA(c, cudaEventRecord(e1, st));
     c->ev_used.push_back({vjp ? 1 : 0, {e0, e1}});
@@ -618,9 +620,10 @@ PostLaunch post_launch(nbody_ctx* c, unsigned mode, double* x, double* v, const 
   P.stage_lo = c->stage_lo.p;
   P.sys = static_cast<SysParam*>(c->sysp.p);
   // (one-sided kernels keep the masses in their sums: no system counts as uniform for them)
-  P.epoch = c->epoch;
   P.off = is_sym(c->ft) ? c->d_off : nullptr;
-  if (c->cfg.precision == NBODY_FP64 && is_sym(c->ft) && c->cfg.law == NBODY_LAW_GRAVITY && first_stage) P.mode |= kMasses;
+  P.call = c->counter + 7;
+  if (first_stage && c->cfg.precision == NBODY_FP64 && is_sym(c->ft) && c->cfg.law == NBODY_LAW_GRAVITY)
+    P.mode |= kMasses, c->new_number = true;
   P.epart = static_cast<double*>(c->epart.p);
   P.status = c->status;
   P.eout = nullptr;
@@ -639,21 +642,9 @@ nbody_status run_post(nbody_ctx* c, const PostLaunch& P, cudaStream_t st) {
   return NBODY_OK;
 }
 
-// Starts a call: its number (never 0), and on the mixed path the staging parameters. A captured call keeps its
-// number in every replay, so the marks of unequal masses that carry it are taken off first (one memset node; a
-// replay with unequal masses would leave them to one with equal masses, whose sums then differ in rounding).
+// Starts a call: on the mixed path the staging parameters.
 nbody_status run_centre(nbody_ctx* c, const double* x, const double* m, cudaStream_t st) {
-  if (++c->epoch == 0) c->epoch = 1;
-  if (c->n_total == 0) return NBODY_OK;
-  if (c->cfg.precision != NBODY_MIXED) {
-    if (c->cfg.law != NBODY_LAW_GRAVITY || !is_sym(c->ft)) return NBODY_OK;
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
-    if (capture == cudaStreamCaptureStatusActive)
-      NB_CUDA(c, cudaMemset2DAsync(&static_cast<SysParam*>(c->sysp.p)->uniform, sizeof(SysParam), 0, sizeof(uint32_t),
-                                   (size_t)c->n_sys, st));
-    return NBODY_OK;
-  }
+  if (c->cfg.precision != NBODY_MIXED || c->n_total == 0) return NBODY_OK;
   CentreLaunch C{};
   C.chunks = c->d_cchunks;
   C.n_chunks = (int32_t)c->wchunks.size();
@@ -1570,7 +1561,8 @@ nbody_status nbody_init(nbody_ctx** out, const nbody_config* cfg, int64_t n_syst
   }
   // two sets of chunk partials: a step's energy record may be finished by the next step's k_post
   if ((s = ensure(c, c->epart, 2 * std::max<size_t>(1, c->chunks.size()) * kEnergyVals * sizeof(double)))) return bail(s);
-  // [0..1] work counter, [2] status word, [4] energy ticket, [5] centre ticket, [6] adjoint-parameter ticket
+  // [0..1] work counter, [2] status word, [4] energy ticket, [5] centre ticket, [6] adjoint-parameter ticket,
+  // [7] number of the last call (FP64, SymLaunch::call)
   if ((s = ensure(c, c->status_counter, 8 * sizeof(unsigned)))) return bail(s);
   c->counter = static_cast<unsigned*>(c->status_counter.p);
   c->status = c->counter + 2;

@@ -32,7 +32,7 @@ struct __align__(16) SysParam {
   double scale, mscale, inv_mscale;
   float eps2, r2c;   // staged softening^2 and near-pair radius^2 (0: no refinement)
   uint32_t uniform;  // mixed: 1 if all masses are equal (staged as 1). FP64: the number of the last call that
-                     // met unequal masses (checked when a call first stages; PostLaunch::epoch)
+                     // met unequal masses (checked when a call first stages; SymLaunch::call)
   uint32_t pad;
 };
 
@@ -160,7 +160,11 @@ struct SymLaunch {
   int law, block, ipt, n_ctas;
   int split;               // FP64 force: warps that share a block's work (1, 2, 4; where compiled)
   int phi;                 // potential: 0 none, 1 of every body, 2 for an energy record (sym::kPhi*)
-  uint32_t epoch;          // FP64: number of the call (SysParam::uniform)
+  // FP64: number of the last call, and whether this is a new call's first pass. The number lives on the
+  // device, so that replays of a captured call have their own: the first staging marks systems of unequal masses
+  // with the number + 1, the first pass takes that for its number, and its last CTA stores it for the kernels after it.
+  unsigned* call;
+  int first;
   int params;              // VJP: also the sums for the G and eps gradients
   unsigned* status;
 };
@@ -255,7 +259,7 @@ struct PostLaunch {
   void* stage;             // float4 / double4_32a [N]
   void* stage_lo;          // mixed: float4 remainders of the staged coordinates [N] (nullable)
   SysParam* sys;           // [n_sys] staging origin and scales
-  uint32_t epoch;          // FP64: number of the call
+  const unsigned* call;    // FP64: number of the last call (kMasses) or of this one (kCombine), SymLaunch::call
   const int64_t* off;      // [n_sys + 1] first body of each system
   double* epart;           // [n_chunks][kEnergyVals]
   unsigned* status;        // device status word

@@ -72,8 +72,9 @@ __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
   if (g == 0 && live) in = load_body(P, mode, i);
   const bool masses = P.precision == 0 && P.law == 0 && P.off;
   const double m0 = masses && (mode & (kCombine | kMasses)) && c.begin < c.end ? P.m[P.off[c.sys]] : 1.0;
+  const unsigned number = masses && (mode & (kCombine | kMasses)) ? *P.call : 0u;
   if (masses && (mode & kMasses) && g == 0 && live && __double_as_longlong(in.m) != __double_as_longlong(m0))
-    P.sys[c.sys].uniform = P.epoch;
+    P.sys[c.sys].uniform = number + 1u;
 
   double sx = 0.0, sy = 0.0, sz = 0.0, sphi = 0.0;
   if ((mode & kCombine) && P.precision == 1) {
@@ -100,7 +101,7 @@ __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
     }
     add_groups(red.d, g, b, s4);
     // FP64 gravity: the mass that a system's bodies share is left out of the sums
-    const double m_all = masses && sp.uniform != P.epoch ? m0 : 1.0;
+    const double m_all = masses && sp.uniform != number ? m0 : 1.0;
     sx = m_all * s4[0], sy = m_all * s4[1], sz = m_all * s4[2], sphi = m_all * s4[3];
   }
   if (g == 0 && live && post_body(P, mode, i, sp, in, sx, sy, sz, sphi, e)) atomicOr(P.status, kFlagNonFinite);
