@@ -19,11 +19,15 @@ namespace {
 template <int CB>
 constexpr unsigned kSumThreads = CB < 32 ? 32 : CB;
 
-// The parameters of a chunk's system into shared memory (a barrier follows). Used from global memory they would be
-// read again after each store that might be to them, a round trip to L2 each time.
-__device__ __forceinline__ void load_params(SysParam& s, const SysParam* sys, const Chunk& c) {
-  if (threadIdx.x < sizeof(SysParam) / 4 && c.begin < c.end)
-    reinterpret_cast<uint32_t*>(&s)[threadIdx.x] = reinterpret_cast<const uint32_t*>(sys + c.sys)[threadIdx.x];
+// The parameters of a chunk's system for shared memory (used from global memory they would be read again after each
+// store that might be to them, a round trip to L2 each time): a word per thread, loaded with the body's own values
+// and stored ahead of the barrier that publishes it.
+__device__ __forceinline__ uint32_t load_param_word(const SysParam* sys, const Chunk& c) {
+  return threadIdx.x < sizeof(SysParam) / 4 && c.begin < c.end
+             ? reinterpret_cast<const uint32_t*>(sys + c.sys)[threadIdx.x] : 0u;
+}
+__device__ __forceinline__ void store_param_word(SysParam& s, const uint32_t word) {
+  if (threadIdx.x < sizeof(SysParam) / 4) reinterpret_cast<uint32_t*>(&s)[threadIdx.x] = word;
 }
 
 // One CTA per chunk, SG threads per body to add the slices and one to do
@@ -66,8 +70,7 @@ __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
   const int i = c.begin + b;
   // (a chunk of 16 has half a warp without bodies in a pass that combines nothing)
   const bool live = i < c.end && g < SG;
-  load_params(sp, P.sys, c);
-  if (!(mode & kCombine)) __syncthreads();  // (else add_groups has a barrier)
+  const uint32_t word = load_param_word(P.sys, c);
   BodyIn in;
   if (g == 0 && live) in = load_body(P, mode, i);
   const bool masses = P.precision == 0 && P.law == 0 && P.off;
@@ -75,6 +78,11 @@ __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
   const unsigned number = masses && (mode & (kCombine | kMasses)) ? *P.call : 0u;
   if (masses && (mode & kMasses) && g == 0 && live && __double_as_longlong(in.m) != __double_as_longlong(m0))
     P.sys[c.sys].uniform = number + 1u;
+
+  if (!(mode & kCombine)) {
+    store_param_word(sp, word);
+    __syncthreads();
+  }
 
   double sx = 0.0, sy = 0.0, sz = 0.0, sphi = 0.0;
   if ((mode & kCombine) && P.precision == 1) {
@@ -84,6 +92,7 @@ __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
 #pragma unroll 8
       for (int s = g; s < c.n_slices; s += SG) add_slot(fp[(int64_t)s * c.stride], h, l);
     }
+    store_param_word(sp, word);
     add_groups(red.f, g, b, h, l);
     if (g == 0) {
       sx = (double)h[0] + (double)l[0], sy = (double)h[1] + (double)l[1];
@@ -99,6 +108,7 @@ __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
         s4[0] += q.x, s4[1] += q.y, s4[2] += q.z, s4[3] += q.w;
       }
     }
+    store_param_word(sp, word);
     add_groups(red.d, g, b, s4);
     // FP64 gravity: the mass that a system's bodies share is left out of the sums
     const double m_all = masses && sp.uniform != number ? m0 : 1.0;
@@ -202,7 +212,7 @@ __global__ void __launch_bounds__(SG * CB, 1024 / (SG * CB)) k_adj_update(const 
   Chunk c = A.chunks[blockIdx.x];
   pdl_wait();  // the VJP kernel has finished writing the partials
   if (!chunk_ok(c, A.n_total, A.n_sys, A.part_rows, A.status)) c.begin = c.end = 0;  // NBODY_DEBUG builds only
-  load_params(sp, A.sys, c);
+  const uint32_t word = load_param_word(A.sys, c);
   const int kw = A.g_params ? 3 : 2;  // partials (fpair4 / double4_32a) per body and slice
   double pv[2] = {0.0, 0.0};          // this thread's w.da/dG and sum m (d.w) / s^5
   const int b = (int)threadIdx.x % CB, g = (int)threadIdx.x / CB;
@@ -232,6 +242,7 @@ __global__ void __launch_bounds__(SG * CB, 1024 / (SG * CB)) k_adj_update(const 
         }
       }
     }
+    store_param_word(sp, word);
     add_groups(red.f, g, b, h, l);
 #pragma unroll
     for (int q = 0; q < 10; ++q) S[q] = g == 0 ? (double)h[q] + (double)l[q] : 0.0;
@@ -252,6 +263,7 @@ __global__ void __launch_bounds__(SG * CB, 1024 / (SG * CB)) k_adj_update(const 
         }
       }
     }
+    store_param_word(sp, word);
     add_groups(red.d, g, b, S);
   }
   if (g == 0 && live) {
