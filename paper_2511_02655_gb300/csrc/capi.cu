@@ -123,7 +123,7 @@ struct nbody_ctx : SymLayout {
   cudaStream_t cap_stream = nullptr;  // private stream used only to capture graphs
   std::string err = "no error";
   int64_t launches = 0;
-  bool new_number = false;  // FP64: the next force pass is a call's first (SymLaunch::call)
+  uint32_t epoch = 0;  // number of the current call (SysParam::uniform), 0 before the first
 
   // layout
   Chunk* d_chunks = nullptr;
@@ -507,8 +507,7 @@ SymLaunch sym_launch(nbody_ctx* c, bool vjp, Potential phi) {
   const int64_t warps = (int64_t)L.n_items * (t.block / 32), room = 16 * (int64_t)c->sm_count;
   L.split = 4 * warps <= room ? 4 : 2 * warps <= room ? 2 : 1;
   L.phi = (int)phi;
-  L.call = c->counter + 7;
-  L.first = !vjp && c->new_number;
+  L.epoch = c->epoch;
   L.status = c->status;
   return L;
 }
@@ -576,7 +575,6 @@ nbody_status run_pair(nbody_ctx* c, cudaStream_t st, bool vjp, Potential phi) {
     if (e0 && e1) NB_CUDA(c, cudaEventRecord(e0, st));
   }
   NB_CUDA(c, launch_pairs(c, vjp, phi, st));
-  if (!vjp) c->new_number = false;
   if (e0 && e1) {
     NB_CUDA(c, cudaEventRecord(e1, st));
     c->ev_used.push_back({vjp ? 1 : 0, {e0, e1}});
@@ -620,10 +618,9 @@ PostLaunch post_launch(nbody_ctx* c, unsigned mode, double* x, double* v, const 
   P.stage_lo = c->stage_lo.p;
   P.sys = static_cast<SysParam*>(c->sysp.p);
   // (one-sided kernels keep the masses in their sums: no system counts as uniform for them)
+  P.epoch = c->epoch;
   P.off = is_sym(c->ft) ? c->d_off : nullptr;
-  P.call = c->counter + 7;
-  if (first_stage && c->cfg.precision == NBODY_FP64 && is_sym(c->ft) && c->cfg.law == NBODY_LAW_GRAVITY)
-    P.mode |= kMasses, c->new_number = true;
+  if (c->cfg.precision == NBODY_FP64 && is_sym(c->ft) && c->cfg.law == NBODY_LAW_GRAVITY && first_stage) P.mode |= kMasses;
   P.epart = static_cast<double*>(c->epart.p);
   P.status = c->status;
   P.eout = nullptr;
@@ -642,9 +639,22 @@ nbody_status run_post(nbody_ctx* c, const PostLaunch& P, cudaStream_t st) {
   return NBODY_OK;
 }
 
-// Starts a call: on the mixed path the staging parameters.
+// Starts a call: its number (never 0), and on the mixed path the staging parameters. A captured call keeps its
+// number in every replay, so the marks of unequal masses that carry it are taken off first (a replay with unequal
+// masses would leave them to one with equal masses, whose sums then differ in rounding).
 nbody_status run_centre(nbody_ctx* c, const double* x, const double* m, cudaStream_t st) {
-  if (c->cfg.precision != NBODY_MIXED || c->n_total == 0) return NBODY_OK;
+  if (++c->epoch == 0) c->epoch = 1;
+  if (c->n_total == 0) return NBODY_OK;
+  if (c->cfg.precision != NBODY_MIXED) {
+    if (c->cfg.law != NBODY_LAW_GRAVITY || !is_sym(c->ft)) return NBODY_OK;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
+    if (capture == cudaStreamCaptureStatusActive) {
+      NB_CUDA(c, launch_clear_marks(static_cast<SysParam*>(c->sysp.p), c->n_sys, st));
+      ++c->launches;
+    }
+    return NBODY_OK;
+  }
   CentreLaunch C{};
   C.chunks = c->d_cchunks;
   C.n_chunks = (int32_t)c->wchunks.size();
@@ -843,7 +853,7 @@ nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
   auto timed = [&](const PairLaunch& P, bool combine, float* best_ms) -> cudaError_t {
     // an untimed pass (which also writes every partial the combine reads), then the best of 3, or of as many
     // as fill ~2 ms (at most 20) for short ones (a gradient's 1 ms: its first call waits); of passes of half a
-    // millisecond or more two, of 2 ms or more one (these repeat to 0.2%)
+    // millisecond or more two, of 20 ms or more one (these repeat to 0.2%)
     cudaError_t err = cudaSuccess;
     float ms = 0.f, best = 1e30f;
     int reps = 1;
@@ -858,7 +868,7 @@ nbody_status time_tiling(nbody_ctx* c, bool vjp, double* cost) {
       c->launches += combine ? 2 : 1;
       if (rep > 0) best = std::min(best, ms);
       const int fill = (int)std::ceil((vjp ? 1.0 : 2.0) / std::max(ms, 1e-3f));
-      if (rep < 2) reps = ms >= 2.f ? 1 : ms >= 0.5f ? 2 : std::max(3, std::min(20, fill));
+      if (rep < 2) reps = ms >= 20.f ? 1 : ms >= 0.5f ? 2 : std::max(3, std::min(20, fill));
     }
     *best_ms = best;
     return err;
@@ -1561,8 +1571,7 @@ nbody_status nbody_init(nbody_ctx** out, const nbody_config* cfg, int64_t n_syst
   }
   // two sets of chunk partials: a step's energy record may be finished by the next step's k_post
   if ((s = ensure(c, c->epart, 2 * std::max<size_t>(1, c->chunks.size()) * kEnergyVals * sizeof(double)))) return bail(s);
-  // [0..1] work counter, [2] status word, [4] energy ticket, [5] centre ticket, [6] adjoint-parameter ticket,
-  // [7] number of the last call (FP64, SymLaunch::call)
+  // [0..1] work counter, [2] status word, [4] energy ticket, [5] centre ticket, [6] adjoint-parameter ticket
   if ((s = ensure(c, c->status_counter, 8 * sizeof(unsigned)))) return bail(s);
   c->counter = static_cast<unsigned*>(c->status_counter.p);
   c->status = c->counter + 2;

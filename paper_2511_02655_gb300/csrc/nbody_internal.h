@@ -32,7 +32,7 @@ struct __align__(16) SysParam {
   double scale, mscale, inv_mscale;
   float eps2, r2c;   // staged softening^2 and near-pair radius^2 (0: no refinement)
   uint32_t uniform;  // mixed: 1 if all masses are equal (staged as 1). FP64: the number of the last call that
-                     // met unequal masses (checked when a call first stages; SymLaunch::call)
+                     // met unequal masses (checked when a call first stages; PostLaunch::epoch)
   uint32_t pad;
 };
 
@@ -160,11 +160,7 @@ struct SymLaunch {
   int law, block, ipt, n_ctas;
   int split;               // FP64 force: warps that share a block's work (1, 2, 4; where compiled)
   int phi;                 // potential: 0 none, 1 of every body, 2 for an energy record (sym::kPhi*)
-  // FP64: number of the last call, and whether this is a new call's first pass. The number lives on the
-  // device, so that replays of a captured call have their own: the first staging marks systems of unequal masses
-  // with the number + 1, the first pass takes that for its number, and its last CTA stores it for the kernels after it.
-  unsigned* call;
-  int first;
+  uint32_t epoch;          // FP64: number of the call (SysParam::uniform)
   int params;              // VJP: also the sums for the G and eps gradients
   unsigned* status;
 };
@@ -259,7 +255,7 @@ struct PostLaunch {
   void* stage;             // float4 / double4_32a [N]
   void* stage_lo;          // mixed: float4 remainders of the staged coordinates [N] (nullable)
   SysParam* sys;           // [n_sys] staging origin and scales
-  const unsigned* call;    // FP64: number of the last call (kMasses) or of this one (kCombine), SymLaunch::call
+  uint32_t epoch;          // FP64: number of the call
   const int64_t* off;      // [n_sys + 1] first body of each system
   double* epart;           // [n_chunks][kEnergyVals]
   unsigned* status;        // device status word
@@ -274,6 +270,9 @@ struct PostLaunch {
   int64_t part_rows;       // entries the partial buffer holds (index checks of NBODY_DEBUG builds)
 };
 cudaError_t launch_post(const PostLaunch& P, cudaStream_t st);
+
+// SysParam::uniform = 0 of every system (FP64, at the start of a captured call).
+cudaError_t launch_clear_marks(SysParam* sys, int n_sys, cudaStream_t st);
 
 // Staging parameters of every system (mixed path): the origin c is the
 // mass-weighted mean position (plain mean if the mass is 0), and for gravity the

@@ -103,17 +103,16 @@ struct ItemSource {
   }
 };
 
-// True in thread 0 of the last CTA (every other one has finished its items).
-__device__ __forceinline__ bool retire_cta(unsigned* counter) {
-  if (threadIdx.x != 0) return false;
-  __threadfence();
-  const bool last = atomicAdd(&counter[1], 1u) == gridDim.x - 1;
-  if (last) {
-    counter[0] = 0u;
-    counter[1] = 0u;
+__device__ __forceinline__ void retire_cta(unsigned* counter) {
+  if (threadIdx.x == 0) {
     __threadfence();
+    const unsigned done = atomicAdd(&counter[1], 1u);
+    if (done == gridDim.x - 1) {
+      counter[0] = 0u;
+      counter[1] = 0u;
+      __threadfence();
+    }
   }
-  return last;
 }
 
 }  // namespace nbody

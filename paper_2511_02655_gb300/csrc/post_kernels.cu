@@ -75,9 +75,8 @@ __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
   if (g == 0 && live) in = load_body(P, mode, i);
   const bool masses = P.precision == 0 && P.law == 0 && P.off;
   const double m0 = masses && (mode & (kCombine | kMasses)) && c.begin < c.end ? P.m[P.off[c.sys]] : 1.0;
-  const unsigned number = masses && (mode & (kCombine | kMasses)) ? *P.call : 0u;
   if (masses && (mode & kMasses) && g == 0 && live && __double_as_longlong(in.m) != __double_as_longlong(m0))
-    P.sys[c.sys].uniform = number + 1u;
+    P.sys[c.sys].uniform = P.epoch;
 
   if (!(mode & kCombine)) {
     store_param_word(sp, word);
@@ -111,7 +110,7 @@ __global__ void __launch_bounds__(SG * CB) k_post(const PostLaunch P) {
     store_param_word(sp, word);
     add_groups(red.d, g, b, s4);
     // FP64 gravity: the mass that a system's bodies share is left out of the sums
-    const double m_all = masses && sp.uniform != number ? m0 : 1.0;
+    const double m_all = masses && sp.uniform != P.epoch ? m0 : 1.0;
     sx = m_all * s4[0], sy = m_all * s4[1], sz = m_all * s4[2], sphi = m_all * s4[3];
   }
   if (g == 0 && live && post_body(P, mode, i, sp, in, sx, sy, sz, sphi, e)) atomicOr(P.status, kFlagNonFinite);
@@ -331,6 +330,12 @@ __global__ void __launch_bounds__(kSumThreads<CB>) k_stage_vec(const Chunk* chun
   }
 }
 
+__global__ void __launch_bounds__(128) k_clear_marks(SysParam* sys, const int n_sys) {
+  pdl_wait();
+  const int s = (int)(blockIdx.x * 128 + threadIdx.x);
+  if (s < n_sys) sys[s].uniform = 0u;
+}
+
 // Up to four plain copies of float64 arrays in one launch (the host-buffer
 // step's transfers through mapped pinned host memory).
 __global__ void __launch_bounds__(256) k_copy4(const Copy4 C) {
@@ -386,6 +391,11 @@ cudaError_t launch_post(const PostLaunch& P, cudaStream_t st) {
   if (two_groups(P.few_slots, P.chunk, P.n_total))
     return launch(std::integral_constant<int, kChunk>(), std::integral_constant<int, 2>(), 0);
   return with_chunk(P.chunk, launch);
+}
+
+// (a memset node in its place is no part of the chain of dependent launches: 4.6 us of a captured call)
+cudaError_t launch_clear_marks(SysParam* sys, int n_sys, cudaStream_t st) {
+  return launch_pdl(k_clear_marks, (unsigned)(n_sys + 127) / 128, 128, st, sys, n_sys);
 }
 
 cudaError_t launch_centre(const CentreLaunch& C, cudaStream_t st) {

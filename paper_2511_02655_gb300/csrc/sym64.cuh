@@ -210,12 +210,12 @@ __device__ __forceinline__ void block(const double (&q)[4][kTile / 32][64], cons
   }
 }
 
-// Work items, taken from `counter` until none is left; number: the call's (SymLaunch::call).
+// Work items, taken from `counter` until none is left.
 // KS warps share the W warps' i-bodies and blocks, each a range of the rotation's steps (short lists,
 // SymLaunch::split): the j-sums need nothing new, as the CTA's warps' sums are added anyway, the i-sums
 // are added at the end of the i-tile.
 template <int LAW, int W, int R, int PHI, int KS>
-__device__ __forceinline__ void items(const SymLaunch& L, const unsigned number, unsigned* counter, Smem<W * KS>& sm) {
+__device__ __forceinline__ void items(const SymLaunch& L, unsigned* counter, Smem<W * KS>& sm) {
   constexpr int T = W * KS * 32, TI = W * 32 * R, NC = PHI == sym::kPhiBoth ? 4 : 3;  // sums of a j-body
   const int tid = (int)threadIdx.x, lane = tid & 31, w = tid >> 5, wi = w % W, k0 = w / W * (32 / KS);
   const double4_32a* __restrict__ st = static_cast<const double4_32a*>(L.stage_x);
@@ -235,7 +235,7 @@ __device__ __forceinline__ void items(const SymLaunch& L, const unsigned number,
     // that u^3 is exactly 0.
     // Equal masses are left out of the sums: bodies count 1, padding 0, and blocks without padding
     // need no products with them.
-    const bool uniform = LAW == 0 && L.sys[it.sys].uniform != number;
+    const bool uniform = LAW == 0 && L.sys[it.sys].uniform != L.epoch;
     const double4_32a q0 = st[it.i_begin];
     const double pad = LAW == 0 ? 1.0e30 * (1.0 + fabs(q0.x) + fabs(q0.y) + fabs(q0.z)) : 3.0e89;
 

@@ -34,10 +34,9 @@ __global__ void __launch_bounds__(W * KS * 32, KS < 4 ? 0 : std::max(1, 24 / (W 
     k_force_sym64(const SymLaunch L) {
   __shared__ sym64::Smem<W * KS> sm;
   pdl_wait();
-  const unsigned number = *L.call + (L.first ? 1u : 0u);
-  sym64::items<LAW, W, R, PHI, KS>(L, number, L.counter, sm);
+  sym64::items<LAW, W, R, PHI, KS>(L, L.counter, sm);
   pdl_trigger();
-  if (retire_cta(L.counter) && L.first) *L.call = number;
+  retire_cta(L.counter);
 }
 
 // More than 48 KB of shared memory per CTA has to be asked for, once per kernel and device.
