@@ -128,6 +128,7 @@ struct nbody_ctx : SymLayout {
   // layout
   Chunk* d_chunks = nullptr;
   Chunk* d_vchunks = nullptr;  // same chunks, VJP tiling's slice counts
+  size_t chunk_count = 0, vchunk_count = 0;
   int32_t* d_sys_chunk = nullptr;
   std::vector<Chunk> wchunks;  // chunks of kChunk bodies: the staging origin's, and of a pass with few slots per body
   Chunk* d_cchunks = nullptr;
@@ -455,7 +456,10 @@ nbody_status install_tiling(nbody_ctx* c, Tiling t, bool vjp) {
   void *d_list = nullptr, *d_chunks = nullptr;
   nbody_status s = is_sym(t) ? upload(c, sym_items.data(), sym_items.size() * sizeof(SymItem), &d_list)
                              : upload(c, items.data(), items.size() * sizeof(WorkItem), &d_list);
-  if (!s) s = upload(c, chunks.data(), chunks.size() * sizeof(Chunk), &d_chunks);
+  // (a chunk list of the old one's size is copied over it below: the tuner installs dozens of tilings)
+  const bool same_chunks =
+      (vjp ? c->d_vchunks : c->d_chunks) && chunks.size() == (vjp ? c->vchunk_count : c->chunk_count);
+  if (!s && !same_chunks) s = upload(c, chunks.data(), chunks.size() * sizeof(Chunk), &d_chunks);
   if (!s) s = ensure(c, c->part, part_bytes);
   if (s) {
     cudaFree(d_list);
@@ -463,13 +467,26 @@ nbody_status install_tiling(nbody_ctx* c, Tiling t, bool vjp) {
     return s;
   }
   cudaStreamSynchronize(c->stream);  // nothing reads the old lists any more
+  if (same_chunks) {
+    d_chunks = vjp ? c->d_vchunks : c->d_chunks;
+    const size_t bytes = chunks.size() * sizeof(Chunk);
+    cudaError_t e = bytes ? cudaMemcpy(d_chunks, chunks.data(), bytes, cudaMemcpyHostToDevice) : cudaSuccess;
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) {
+      cudaFree(d_list);
+      return fail(c, NBODY_ECUDA, "upload of the chunk list failed: %s", cudaGetErrorString(e));
+    }
+  } else {
+    cudaFree(vjp ? c->d_vchunks : c->d_chunks);
+  }
   cudaFree(vjp ? c->d_vitems : c->d_items);
-  cudaFree(vjp ? c->d_vchunks : c->d_chunks);
   if (vjp) {
+    c->vchunk_count = chunks.size();
     c->d_vitems = d_list, c->d_vchunks = static_cast<Chunk*>(d_chunks);
     c->vt = t, c->n_vitems = n_items, c->vmax_slices = max_slices, c->vpart_bytes = part_bytes, c->vjp_ready = true;
     c->vwide = wide;
   } else {
+    c->chunk_count = chunks.size();
     c->d_items = d_list, c->d_chunks = static_cast<Chunk*>(d_chunks);
     c->ft = t, c->n_items = n_items, c->max_slices = max_slices, c->fpart_bytes = part_bytes;
     c->sym_longest = longest;
